@@ -67,15 +67,17 @@ int dsfacto_create(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32_t p, 
  * (r,c) belongs to round s = (c-r) mod p; tiles ordered by (s, r); inside a tile entries ordered
  * by (column, row)), copies CSR and tiles to the device and runs the recompute pass once, so that
  * A, G and the objective of the initial parameters exist.  Replaces any earlier data set.
- * Non-empty loads are bucketed on the device itself when the packed entry layout
- * applies (local row and column ids fit 32 bits together, tile number and local column id too) and the
- * device has room for the buffers of a sort (about 25 bytes per stored entry for the duration of the call):
- * the CSR copy that the recompute pass needs anyway is turned into (tile, local column) keys, sorted by a
- * stable radix sort, packed into entry records, and a kernel cuts the chunks of the stratum SGD launch; only
- * the CSR arrays cross the link, and from 2^24 stored entries on they are sent while the host still checks them
- * (a data set that fails the checks leaves the handle as it was, as on every path).  On this path the
- * row-block sweep stores several consecutive row blocks of a column block as one slot (up to 8, for loads of
- * fewer than 2^24 entries up to 16; see DSFACTO_DEBUG_ROW_MERGE).  DSFACTO_LOAD=device asks for this way
+ * Non-empty loads are put in order on the device itself when it has room for the buffers of a sort (about 26
+ * bytes per stored entry for the duration of the call): the CSR copy that the recompute pass needs anyway is
+ * turned into (pass, column, phase) keys and sorted by a stable radix sort, and kernels list the runs of entries
+ * of a column and cut the entries into equal units of the update loop; only the CSR arrays cross the link, and
+ * from 2^24 stored entries on they are sent while the host still checks them (a data set that fails the checks
+ * leaves the handle as it was, as on every path).  A pass holds a band of rows whose auxiliaries fit L2; a data
+ * set of one band has every column as one run in its full stratified order (DSFACTO_BANDS=B asks for B bands).
+ * With row blocks per slot asked for (DSFACTO_DEBUG_ROW_MERGE, DSFACTO_ROW_MERGE) or a planted wait
+ * (DSFACTO_DEBUG_EXTRA_NEED), tile lists are bucketed on the device instead and swept tile by tile, as they are
+ * where the host has built them; in these, several consecutive row blocks of a column block make one slot (up to
+ * 8, for loads of fewer than 2^24 entries up to 16).  DSFACTO_LOAD=device asks for the device
  * explicitly.  Otherwise, and with any other value of DSFACTO_LOAD, the tile lists are built on the host; there,
  * loads of 2^24 stored entries and more (with p at least twice the number of host threads) are
  * streamed: each host thread buckets one row block at a time into page-locked staging memory and
@@ -169,10 +171,10 @@ int dsfacto_get_stats(dsfacto_t *h, double *mean_loss, double *sum_G);
  * NULL = the legacy default stream).  The stream stays owned by the caller. */
 int dsfacto_set_stream(dsfacto_t *h, void *cuda_stream);
 
-/* Device time of the last dsfacto_epoch from CUDA events on the handle's stream, in milliseconds:
+/* Device time of the last dsfacto_epoch, taken by its kernels from the device's clock, in milliseconds:
  * ms[0] whole epoch, ms[1] the p strata (update loop), ms[2] recompute pass (refresh + residual +
- * loss sums), ms[3] parameter norms + final reduction.  With dsfacto_set_refresh_every each figure is
- * the sum over the segments of the epoch. */
+ * loss sums, parameter norms, final reduction), ms[3] 0 (the norms are part of the recompute pass).
+ * With dsfacto_set_refresh_every each figure is the sum over the segments of the epoch. */
 int dsfacto_last_epoch_ms(dsfacto_t *h, float ms[4]);
 
 /* Test and debugging knobs of the stratum SGD launch.
@@ -184,8 +186,8 @@ int dsfacto_last_epoch_ms(dsfacto_t *h, float ms[4]);
  *                             wait for that many finished chunks more than its column block really has before
  *                             it; with a value larger than the number of chunks its wait runs out, so the
  *                             failure path above can be exercised without a fault or a hang.  0 = off.
- *   DSFACTO_DEBUG_CHUNK_LEN   (takes effect at the next dsfacto_load_csr) entries per chunk, 16 .. 4096, 0 = chosen
- *                             by the load; the environment variable DSFACTO_CHUNK does the same for every handle.
+ *   DSFACTO_DEBUG_CHUNK_LEN   (takes effect at the next dsfacto_load_csr) entries per chunk (per unit of the update loop
+ *                             by column runs: rounded up to a power of two), 16 .. 4096, 0 = chosen by the load; the environment variable DSFACTO_CHUNK does the same for every handle.
  *                             The sweep kernel reads a chunk's entries block by block; the environment variable
  *                             DSFACTO_BLOCK (a multiple of 32, 32 .. 256) sets the entries per block.
  *   DSFACTO_DEBUG_ROW_MERGE   (takes effect at the next dsfacto_load_csr that buckets on the device) row blocks per slot of

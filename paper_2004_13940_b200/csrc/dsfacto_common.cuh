@@ -51,4 +51,24 @@ __device__ __forceinline__ void block_sum2(double &a, double &b) {
     }
 }
 
+// the same for four
+__device__ __forceinline__ void block_sum4(double (&s)[4]) {
+    __shared__ double sh[4][kThreads / 32];
+    const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
+    __syncthreads();   // (an earlier call's reads)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        s[c] = warp_sum(s[c]);
+        if (ln == 0) sh[c][wid] = s[c];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            double x = 0.0;
+            for (int i = 0; i < kThreads / 32; ++i) x += sh[c][i];
+            s[c] = x;
+        }
+}
+
 }  // namespace dsf

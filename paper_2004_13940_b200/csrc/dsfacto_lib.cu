@@ -3,10 +3,13 @@
 #include "dsfacto.h"
 #include "dsfacto_bucket.cuh"
 #include "dsfacto_refresh.cuh"
+#include "dsfacto_runplan.cuh"
+#include "dsfacto_runs.cuh"
 #include "dsfacto_sgd.cuh"
 
 #include <cub/device/device_radix_sort.cuh>
 
+#include <immintrin.h>
 #include <omp.h>
 #include <sys/mman.h>
 
@@ -23,6 +26,12 @@
 namespace {
 
 using namespace dsf;
+
+// A pass of the update loop by column runs: its entries, runs and units in the handle's arrays.
+struct RunPass {
+    int64_t first = 0, run_first = 0, unit_first = 0;
+    int count = 0, nruns = 0, units = 0;
+};
 
 }  // namespace
 
@@ -55,7 +64,7 @@ struct dsfacto {
 
     // device
     float *d_w = nullptr, *d_V = nullptr, *d_A = nullptr, *d_G = nullptr, *d_y = nullptr, *d_val = nullptr, *d_xw = nullptr;
-    int64_t *d_indptr = nullptr, *d_tile_ptr = nullptr, *d_row_start = nullptr;
+    int64_t *d_indptr = nullptr, *d_row_start = nullptr;
     int32_t *d_idx = nullptr, *d_col_start = nullptr;
     uint2 *d_ent = nullptr;
     double *d_partials = nullptr, *d_scal = nullptr;
@@ -92,6 +101,20 @@ struct dsfacto {
     // changed since it was made (model_version counts the changes).
     float2 *d_pair = nullptr, *d_pair_s = nullptr;
     int64_t model_version = 1, pair_version = 0, slot_version = 0;
+
+    // scalars of an epoch on the device, and the mapped host memory its last kernel reports to
+    EpochState *d_state = nullptr;
+    EpochReport *report = nullptr;
+    unsigned long long report_seq = 0;
+    // update loop by column runs (dsfacto_runs.cuh): every load that is bucketed on the device with default settings
+    bool runs = false;
+    int bands = 1;                 // passes per segment
+    int unit_len = 0;
+    std::vector<RunPass> passes;   // segment by segment, band by band
+    int *d_run_start = nullptr, *d_unit_run = nullptr;
+    uint32_t *d_run_key = nullptr;
+    float4 *d_rec = nullptr, *d_part = nullptr;
+    int32_t *d_slot_of = nullptr;
 
     double loss_sum = 0, g_sum = 0, w2 = 0, v2 = 0, objective = 0;
 };
@@ -313,12 +336,58 @@ void unpack_merged_tiles(const dsfacto *h, const uint2 *ent, std::vector<int64_t
     }
 }
 
+// The same from the passes of the update loop by column runs: the tiles of a column block are listed column by
+// column, and inside a column the passes (segments, bands) in order, which keeps the rows of a tile ascending.
+void unpack_runs(const dsfacto *h, const uint2 *ent, const std::vector<int> &run_start, const std::vector<uint32_t> &run_key,
+                 std::vector<int64_t> &canon_ptr, int32_t *rows, int32_t *cols, float *vals) {
+    const int64_t p = h->p, n = h->n;
+    canon_ptr.assign((size_t)(p * p) + 1, 0);
+    std::vector<std::vector<int64_t>> cursor((size_t)omp_get_max_threads(), std::vector<int64_t>(h->passes.size()));
+    for (int write = 0; write < 2; ++write) {
+        std::vector<int64_t> fill;
+        if (write) {
+            for (int64_t t = 0; t < p * p; ++t) canon_ptr[(size_t)t + 1] += canon_ptr[(size_t)t];
+            if (!rows && !cols && !vals) return;
+            fill.assign(canon_ptr.begin(), canon_ptr.end() - 1);
+        }
+#pragma omp parallel for schedule(dynamic, 1)
+        for (int64_t c = 0; c < p; ++c) {   // (different column blocks hold different tiles)
+            std::vector<int64_t> &cur = cursor[(size_t)omp_get_thread_num()];
+            for (size_t q = 0; q < h->passes.size(); ++q) {
+                const uint32_t *k0 = run_key.data() + h->passes[q].run_first;
+                cur[q] = std::lower_bound(k0, k0 + h->passes[q].nruns, (uint32_t)h->col_start[(size_t)c] << 1) - k0;
+            }
+            for (int64_t j = h->col_start[(size_t)c]; j < h->col_start[(size_t)c + 1]; ++j)
+                for (size_t q = 0; q < h->passes.size(); ++q) {
+                    const RunPass &ps = h->passes[q];
+                    for (; cur[q] < ps.nruns && (int64_t)(run_key[(size_t)(ps.run_first + cur[q])] >> 1) == j; ++cur[q]) {
+                        const int64_t k = ps.run_first + cur[q];
+                        const int64_t end = cur[q] + 1 < ps.nruns ? run_start[(size_t)k + 1] : ps.count;
+                        for (int64_t e = run_start[(size_t)k]; e < end; ++e) {
+                            const uint2 rec = ent[ps.first + e];
+                            const int64_t i = (int64_t)(rec.x & ~kRunStart), r = i * p / n;
+                            const int64_t tile = (c >= r ? c - r : c - r + p) * p + r;
+                            if (!write) { canon_ptr[(size_t)tile + 1] += 1; continue; }
+                            const int64_t at = fill[(size_t)tile]++;
+                            if (rows) rows[at] = (int32_t)i;
+                            if (cols) cols[at] = (int32_t)j;
+                            if (vals) std::memcpy(&vals[at], &rec.y, 4);
+                        }
+                    }
+                }
+        }
+    }
+}
+
 void free_data(dsfacto *h) {
     h->rbits = 0;
     dev_free(h->d_A); dev_free(h->d_G); dev_free(h->d_y); dev_free(h->d_val); dev_free(h->d_xw);
-    dev_free(h->d_indptr); dev_free(h->d_tile_ptr); dev_free(h->d_idx); dev_free(h->d_ent);
+    dev_free(h->d_indptr); dev_free(h->d_idx); dev_free(h->d_ent);
     dev_free(h->d_partials); dev_free(h->d_desc); dev_free(h->d_records); dev_free(h->d_run_count);
-    dev_free(h->d_sync); dev_free(h->d_column_of); dev_free(h->d_Vs); dev_free(h->d_pair_s);
+    dev_free(h->d_sync); dev_free(h->d_column_of); dev_free(h->d_slot_of); dev_free(h->d_Vs); dev_free(h->d_pair_s);
+    dev_free(h->d_run_start); dev_free(h->d_run_key); dev_free(h->d_unit_run); dev_free(h->d_rec); dev_free(h->d_part);
+    h->runs = false;
+    h->passes.clear();
     h->slots = false;
     h->slot_version = 0;
     h->launch_ptr.clear();
@@ -354,12 +423,30 @@ void launch_sgd(dsfacto *h, const SgdArgs &a, int64_t chunks) {
     if (h->wide) sgd_sweep_kernel<LG, NV, true><<<grid, kSgdThreads, bytes, h->stream>>>(a);
     else sgd_sweep_kernel<LG, NV, false><<<grid, kSgdThreads, bytes, h->stream>>>(a);
 }
+// A launch that may start its prologue while the kernel before it on the stream is still running (programmatic
+// stream serialisation); every kernel launched this way waits (griddepcontrol.wait) before it reads what earlier
+// kernels wrote or writes what they read.
+template <typename... P, typename... A>
+void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threads, size_t smem, const A &...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);   // (an error is picked up by the cudaGetLastError at the end of the call)
+    h->launches += 1;
+}
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
-    if (mode == kTrain) refresh_kernel<LG, NV, kTrain><<<grid, kThreads, 0, h->stream>>>(a);
-    else if (mode == kEvaluate) refresh_kernel<LG, NV, kEvaluate><<<grid, kThreads, 0, h->stream>>>(a);
-    else if (mode == kPartial) refresh_kernel<LG, NV, kPartial><<<grid, kThreads, 0, h->stream>>>(a);
-    else refresh_kernel<LG, NV, kScore><<<grid, kThreads, 0, h->stream>>>(a);
+    if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, 0, a);
+    else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, 0, a);
+    else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, 0, a);
+    else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, 0, a);
 }
 
 #define DSF_DISPATCH(h, FN, ...)                                   \
@@ -688,6 +775,55 @@ void run_sgd_phase(dsfacto *h, int64_t L0, int64_t L1) {
     }
 }
 
+// ---- update loop by column runs ----
+template <int LG, int NV>
+void launch_run_pass(dsfacto *h, const RunPass &ps, RunSweepArgs &sw, RunApplyArgs &ap) {
+    const int64_t ctas = std::max<int64_t>(((int64_t)ps.units + kRunWarps - 1) / kRunWarps, 1);
+    launch_overlapped(h, runs_sweep_kernel<LG, NV>, ctas, kRunThreads, run_sweep_smem<LG, NV>(), sw);
+    // a warp per run while that leaves no more warps than the device holds: the runs are long then and have many pieces
+    const bool coop = (int64_t)ps.nruns <= (int64_t)h->sm_count * 64;
+    const int64_t per_cta = coop ? ApplyCfg<LG, NV, true>::RUNS : ApplyCfg<LG, NV, false>::RUNS;
+    const int64_t grid = std::max<int64_t>((ps.nruns + per_cta - 1) / per_cta, 1);
+    if (coop) launch_overlapped(h, runs_apply_kernel<LG, NV, true>, grid, kThreads, 0, ap);
+    else launch_overlapped(h, runs_apply_kernel<LG, NV, false>, grid, kThreads, 0, ap);
+}
+
+// The strata of segment `seg` (the whole epoch unless the second schedule is on).  share > 0: w0 takes that part of
+// its step first, from the multiplier sum on the device.
+void run_strata(dsfacto *h, int64_t seg, double share) {
+    const double ew = (double)h->h * (double)h->lambda_w, log1m_ew = std::log1p(-ew);
+    // The training rows' view of the model is kept up to date by the kernels that change the model.
+    h->model_version += 1;
+    (h->slots ? h->slot_version : h->pair_version) = h->model_version;
+    float2 *pair = h->slots ? h->d_pair_s : h->d_pair;
+    float4 *Vs = h->slots ? reinterpret_cast<float4 *>(h->d_Vs) : nullptr;
+    const int32_t *slot_of = h->slots ? h->d_slot_of : nullptr;
+    for (int b = 0; b < h->bands; ++b) {
+        const RunPass &ps = h->passes[(size_t)(seg * h->bands + b)];
+        RunSweepArgs sw{};
+        sw.ent = h->d_ent + ps.first; sw.count = ps.count; sw.unit_len = h->unit_len;
+        sw.run_start = h->d_run_start + ps.run_first; sw.unit_run = h->d_unit_run + ps.unit_first; sw.nruns = ps.nruns;
+        sw.stamp = b == 0; sw.A = h->d_A; sw.G = h->d_G; sw.n = h->n; sw.rec = h->d_rec; sw.part = h->d_part; sw.st = h->d_state;
+        sw.h = h->h; sw.lambda_v = h->lambda_v; sw.kappa_w = (float)(-log1m_ew / std::log(2.0));
+        RunApplyArgs ap{};
+        ap.run_key = h->d_run_key + ps.run_first; ap.run_start = sw.run_start; ap.nruns = ps.nruns; ap.count = ps.count;
+        ap.shift = bits_for((int64_t)kRunWarps * h->unit_len); ap.rec = h->d_rec; ap.part = h->d_part; ap.w = h->d_w; ap.V = h->d_V;
+        ap.Tw = h->d_Tw; ap.Tb = h->d_Tb; ap.TS = h->d_TS;
+        if (h->bands == 1) { ap.pair = pair; ap.Vs = Vs; ap.slot_of = slot_of; }
+        ap.st = h->d_state; ap.log1m_ew = log1m_ew;
+        if (b == 0 && share > 0.0) ap.w0_step = (double)h->h * share;
+        DSF_DISPATCH(h, launch_run_pass, h, ps, sw, ap);
+    }
+    if (h->bands > 1) {
+        const int kp4 = h->Kp / 4;
+        int gs = 1;
+        while (gs < kp4 && gs < 16) gs *= 2;
+        const int64_t grid = std::min<int64_t>(((int64_t)h->d * gs + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
+        launch_overlapped(h, runs_fold_kernel, grid, kThreads, 0, reinterpret_cast<float4 *>(h->d_V), h->d_w,
+                          reinterpret_cast<float4 *>(h->d_Tb), h->d_Tw, h->d_TS, (int64_t)h->d, kp4, gs, slot_of, Vs, pair, log1m_ew);
+    }
+}
+
 template <int LG, int NV>
 void launch_finish(dsfacto *h, int grid) {
     finish_kernel<LG, NV><<<grid, kThreads, 0, h->stream>>>(h->n, h->d_A, h->d_lin, h->d_q, h->d_y, h->d_G, h->d_partials,
@@ -704,7 +840,7 @@ void model_view(dsfacto *h, RefreshArgs &a, bool training_rows) {
     if (version != h->model_version) {
         const int kp4 = h->Kp / 4;
         int gs = 1;
-        while (gs < kp4 && gs < 32) gs *= 2;
+        while (gs < kp4 && gs < 16) gs *= 2;   // (as the update loop's lane groups: the same sums of squares, bit for bit)
         const int64_t groups_per_cta = kThreads / gs;
         const int grid = (int)std::min<int64_t>(((int64_t)h->d + groups_per_cta - 1) / groups_per_cta, (int64_t)h->sm_count * 16);
         model_view_kernel<<<grid, kThreads, 0, h->stream>>>(reinterpret_cast<const float4 *>(h->d_V), h->d_w,
@@ -734,7 +870,7 @@ int order_columns(dsfacto *h) {
     int32_t *d_col = nullptr, *d_slot_of = nullptr;
     void *tmp = nullptr;
     auto cleanup = [&]() {
-        dev_free(d_key); dev_free(d_key_out); dev_free(d_col); dev_free(d_slot_of);
+        dev_free(d_key); dev_free(d_key_out); dev_free(d_col); dev_free(d_slot_of);   // (d_slot_of: kept by the handle on success)
         if (tmp) cudaFree(tmp);
         tmp = nullptr;
     };
@@ -769,6 +905,8 @@ int order_columns(dsfacto *h) {
     column_rename_kernel<<<grid, kThreads, 0, h->stream>>>(h->d_idx, h->nnz, d_slot_of);
     h->launches += 4;
     if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    h->d_slot_of = d_slot_of;
+    d_slot_of = nullptr;
     cleanup();
     h->slots = true;
     return DSFACTO_OK;
@@ -783,7 +921,6 @@ int run_partial_refresh(dsfacto *h) {
     a.lin_out = h->d_lin; a.q_out = h->d_q;
     a.partials = h->d_partials; a.w0 = h->w0; a.loss = h->loss;
     DSF_DISPATCH_REFRESH(h, h, a, kPartial, h->refresh_grid);
-    h->launches += 1;
     cudaEventRecord(h->ev[2], h->stream);   // (the epoch's phase timers expect both marks)
     cudaEventRecord(h->ev[3], h->stream);
     CU_TRY(h, cudaStreamSynchronize(h->stream));
@@ -814,29 +951,51 @@ int run_finish(dsfacto *h) {
     return DSFACTO_OK;
 }
 
-// recompute pass + norms + objective; ends with a stream sync and the four sums on the host
-int run_refresh(dsfacto *h, bool timed) {
+// Waits until the kernel that was given report number h->report_seq has delivered it (the last thing that kernel
+// does).  The stream is asked now and then, so that a failed launch ends the wait.
+int wait_report(dsfacto *h) {
+    const volatile EpochReport *r = h->report;
+    for (unsigned spin = 1; r->seq != h->report_seq; ++spin) {
+        _mm_pause();
+        if ((spin & 0x3FFFu) != 0) continue;
+        const cudaError_t e = cudaStreamQuery(h->stream);
+        if (e == cudaErrorNotReady) continue;
+        if (e == cudaSuccess && r->seq == h->report_seq) break;
+        h->err = std::string("epoch: ") + (e == cudaSuccess ? "the last kernel left no report" : cudaGetErrorString(e));
+        return DSFACTO_ERR_CUDA;
+    }
+    CU_TRY(h, cudaGetLastError());
+    return DSFACTO_OK;
+}
+
+// Recompute pass with the squared norms of the objective; w0 is taken from the device.  report: the pass is the
+// last of its epoch, the sums come to the host.
+int run_refresh(dsfacto *h, bool first, bool report) {
     if (h->nshards > 1) return run_partial_refresh(h);
     RefreshArgs a{};
     a.n = h->n; a.indptr = h->d_indptr; a.idx = h->d_idx; a.val = h->d_val; a.y = h->d_y;
     model_view(h, a, true);
     a.A = h->d_A; a.G = h->d_G; a.f_out = nullptr;
-    a.partials = h->d_partials; a.w0 = h->w0; a.loss = h->loss;
+    a.partials = h->d_partials; a.loss = h->loss;
+    a.norm_w = h->d_w; a.norm_V = h->d_V; a.norm_d = h->d; a.norm_v4 = (int64_t)h->d * (h->Kp / 4);
+    a.done = &h->d_state->done; a.st = h->d_state; a.first = first ? 1 : 0;
+    if (report) { a.report = h->report; a.seq = ++h->report_seq; }
     DSF_DISPATCH_REFRESH(h, h, a, kTrain, h->refresh_grid);
-    reduce2_kernel<<<1, kThreads, 0, h->stream>>>(h->d_partials, h->refresh_grid, h->d_scal);
-    if (timed) cudaEventRecord(h->ev[2], h->stream);
-    double *np = h->d_partials + 2 * (size_t)h->refresh_grid;
-    sqnorm_kernel<<<h->norm_grid, kThreads, 0, h->stream>>>(h->d_w, h->d, h->d_V, (int64_t)h->d * h->Kp, np);
-    reduce2_kernel<<<1, kThreads, 0, h->stream>>>(np, h->norm_grid, h->d_scal + 2);
-    h->launches += 4;
-    if (timed) cudaEventRecord(h->ev[3], h->stream);
-    double s[4];
-    CU_TRY(h, cudaMemcpyAsync(s, h->d_scal, sizeof s, cudaMemcpyDeviceToHost, h->stream));
-    CU_TRY(h, cudaStreamSynchronize(h->stream));
-    CU_TRY(h, cudaGetLastError());
-    h->loss_sum = s[0]; h->g_sum = s[1]; h->w2 = s[2]; h->v2 = s[3];
-    h->objective = s[0] / (double)h->n + 0.5 * (double)h->lambda_w * s[2] + 0.5 * (double)h->lambda_v * s[3];
+    if (!report) return DSFACTO_OK;
+    const int rc = wait_report(h);
+    if (rc) return rc;
+    const EpochReport r = *h->report;
+    h->loss_sum = r.loss; h->g_sum = r.g; h->w2 = r.w2; h->v2 = r.v2; h->w0 = r.w0;
+    h->objective = r.loss / (double)h->n + 0.5 * (double)h->lambda_w * r.w2 + 0.5 * (double)h->lambda_v * r.v2;
     return DSFACTO_OK;
+}
+// ... with the host's w0
+int refresh_now(dsfacto *h) {
+    if (h->nshards == 1) {
+        epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
+        h->launches += 1;
+    }
+    return run_refresh(h, true, true);
 }
 
 // V padded (d x Kp) <-> caller layout (d x K)
@@ -1281,6 +1440,27 @@ const char *dsfacto_strerror(int status) {
 
 const char *dsfacto_last_error(dsfacto_t *h) { return h ? h->err.c_str() : ""; }
 
+// Column state beside w and V, zero outside the update loop: the tail composites (row-block sweep, several bands)
+// and the scale records of the tile sweep.  Allocated by the first load that needs them.
+static int column_state(dsfacto *h, bool tails, bool scales) {
+    int rc;
+    const size_t d = (size_t)h->d;
+    if (scales && !h->d_S) {
+        if ((rc = dev_alloc(h, &h->d_S, d))) return rc;
+        CU_TRY(h, cudaMemsetAsync(h->d_S, 0, sizeof(float4) * d, h->stream));
+    }
+    if (tails && !h->d_TS) {
+        if ((rc = dev_alloc(h, &h->d_Tb, d * h->Kp)) || (rc = dev_alloc(h, &h->d_Tw, d)) || (rc = dev_alloc(h, &h->d_TS, d))) {
+            dev_free(h->d_Tb); dev_free(h->d_Tw); dev_free(h->d_TS);
+            return rc;
+        }
+        CU_TRY(h, cudaMemsetAsync(h->d_Tb, 0, sizeof(float) * d * h->Kp, h->stream));
+        CU_TRY(h, cudaMemsetAsync(h->d_Tw, 0, sizeof(float) * d, h->stream));
+        CU_TRY(h, cudaMemsetAsync(h->d_TS, 0, sizeof(float4) * d, h->stream));
+    }
+    return DSFACTO_OK;
+}
+
 static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32_t p, int32_t loss, float lambda_w,
                          float lambda_v, float eta, uint64_t seed, int32_t shard, int32_t nshards) {
     if (!out) return DSFACTO_ERR_INVALID_ARG;
@@ -1349,17 +1529,11 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
         return fail(DSFACTO_ERR_CUDA);
     h->norm_grid = h->sm_count * 8;
     if (const char *env = std::getenv("DSFACTO_SWEEP")) h->sweep = (std::strcmp(env, "round") == 0) ? 0 : 1;
-    if ((rc = dev_alloc(h, &h->d_S, (size_t)d))) return fail(rc);
-    if (cudaMemset(h->d_S, 0, sizeof(float4) * (size_t)d) != cudaSuccess) return fail(DSFACTO_ERR_CUDA);
-    if (h->sweep == 1) {
-        if ((rc = dev_alloc(h, &h->d_Tb, (size_t)d * h->Kp)) || (rc = dev_alloc(h, &h->d_Tw, (size_t)d)) ||
-            (rc = dev_alloc(h, &h->d_TS, (size_t)d)))
-            return fail(rc);
-        if (cudaMemset(h->d_Tb, 0, sizeof(float) * (size_t)d * h->Kp) != cudaSuccess ||
-            cudaMemset(h->d_Tw, 0, sizeof(float) * (size_t)d) != cudaSuccess ||
-            cudaMemset(h->d_TS, 0, sizeof(float4) * (size_t)d) != cudaSuccess)
-            return fail(DSFACTO_ERR_CUDA);
-    }
+    if ((rc = dev_alloc(h, &h->d_state, 1))) return fail(rc);
+    if (cudaMemset(h->d_state, 0, sizeof(EpochState)) != cudaSuccess) return fail(DSFACTO_ERR_CUDA);
+    if (cudaHostAlloc((void **)&h->report, sizeof(EpochReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
+        return fail(DSFACTO_ERR_OOM);
+    std::memset(h->report, 0, sizeof(EpochReport));
     *out = h;
     return DSFACTO_OK;
 }
@@ -1386,6 +1560,8 @@ void dsfacto_destroy(dsfacto_t *h) {
     cudaStreamSynchronize(h->stream);
     free_data(h);
     dev_free(h->d_w); dev_free(h->d_V); dev_free(h->d_Tb); dev_free(h->d_Tw); dev_free(h->d_S); dev_free(h->d_TS); dev_free(h->d_row_start); dev_free(h->d_col_start); dev_free(h->d_scal); dev_free(h->d_pair);
+    dev_free(h->d_state);
+    if (h->report) cudaFreeHost(h->report);
     for (auto &e : h->ev)
         if (e) cudaEventDestroy(e);
     delete h;
@@ -1621,6 +1797,141 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     return DSFACTO_OK;
 }
 
+// ---- plan of the update loop by column runs (see dsfacto_runplan.cuh) ----
+// Whether this load takes it: every load that may be bucketed on the device, unless a knob asks for the tile sweep
+// (DSFACTO_SWEEP=round, row blocks per slot, the planted wait), as long as pass, column and phase fit a 32-bit key.
+static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env) {
+    if (nnz <= 0 || h->sweep != 1 || h->row_merge > 0 || h->debug_extra_need > 0 || std::getenv("DSFACTO_ROW_MERGE")) return false;
+    if (load_env) { if (std::strcmp(load_env, "device") != 0) return false; }
+    else {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+        // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs
+        if ((double)free_b < 1.1 * ((double)nnz * 26.0 + (double)h->n * 4.0 * (h->Kp + 2))) return false;
+    }
+    return true;
+}
+// Bands: rows per pass such that their auxiliary rows, which every column of the pass reads, stay in L2.
+static int64_t band_count(const dsfacto *h) {
+    if (const char *env = std::getenv("DSFACTO_BANDS")) {
+        const int64_t v = std::atoll(env);
+        if (v >= 1 && v <= h->n) return v;
+    }
+    const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
+    return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
+}
+// d_indptr, d_idx, d_val hold the CSR arrays (copies queued on the stream).  Fills the entries, runs and units of
+// the passes.  Returns 1 if the data set does not fit this plan (nothing is left behind then).
+static int plan_runs(dsfacto *h, int64_t nnz) {
+    const bool segmented = h->refresh_every > 0 && h->refresh_every < h->p;
+    const int64_t every = segmented ? h->refresh_every : h->p, nseg = ((int64_t)h->p + every - 1) / every;
+    const int64_t bands = band_count(h), npass = nseg * bands;
+    const int cbits = bits_for(h->d), low_bits = cbits + 1, kb = bits_for(npass) + low_bits;
+    if (kb > 32 || npass > (1 << 20)) return 1;
+    const int drop = bands == 1 ? 1 : 0;   // one band: a column is one run, whatever the phase
+    cudaStream_t st = h->stream;
+    uint32_t *key[2] = {nullptr, nullptr};
+    unsigned long long *pay[2] = {nullptr, nullptr};
+    void *tmp = nullptr;
+    int64_t *d_count = nullptr, *d_bounds = nullptr;   // run starts before each block; per pass its first entry, its first run
+    auto cleanup = [&]() {
+        dev_free(key[0]); dev_free(key[1]); dev_free(pay[0]); dev_free(pay[1]); dev_free(d_count); dev_free(d_bounds);
+        if (tmp) cudaFree(tmp);
+        tmp = nullptr;
+    };
+    auto fail = [&](cudaError_t e) {
+        h->err = std::string("run plan: ") + cudaGetErrorString(e);
+        cudaStreamSynchronize(st);
+        cleanup();
+        return e == cudaErrorMemoryAllocation ? DSFACTO_ERR_OOM : DSFACTO_ERR_CUDA;
+    };
+    const int64_t blocks = (nnz + kRunBlock - 1) / kRunBlock;
+    int rc;
+    if ((rc = dev_alloc(h, &key[0], (size_t)nnz)) || (rc = dev_alloc(h, &key[1], (size_t)nnz)) ||
+        (rc = dev_alloc(h, &pay[0], (size_t)nnz)) || (rc = dev_alloc(h, &pay[1], (size_t)nnz)) ||
+        (rc = dev_alloc(h, &d_count, (size_t)blocks + 1)) || (rc = dev_alloc(h, &d_bounds, 2 * ((size_t)npass + 1)))) {
+        cleanup();
+        return rc;
+    }
+    cudaError_t e;
+    cub::DoubleBuffer<uint32_t> kbuf(key[0], key[1]);
+    cub::DoubleBuffer<unsigned long long> pbuf(pay[0], pay[1]);
+    size_t tmp_bytes = 0;
+    if ((e = cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
+    if ((e = cudaMalloc(&tmp, tmp_bytes ? tmp_bytes : 1)) != cudaSuccess) return fail(e);
+    const int wide_grid = h->sm_count * 16;
+    RunKeyArgs ka{};
+    ka.n = h->n; ka.nnz = nnz; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p; ka.cbits = cbits;
+    ka.bands = (int32_t)bands; ka.band_rows = (h->n + bands - 1) / bands; ka.every = (int32_t)every; ka.row_start = h->d_row_start;
+    ka.key = key[0]; ka.payload = pay[0];
+    run_keys_kernel<<<(int)std::min<int64_t>((h->n + 7) / 8, wide_grid), kThreads, 0, st>>>(ka);
+    if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
+    const uint32_t *sorted = kbuf.Current();
+    pass_bounds_kernel<<<(int)((npass + kThreads) / kThreads), kThreads, 0, st>>>(nnz, sorted, low_bits, (int)npass, d_bounds);
+    run_count_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(nnz, sorted, drop, d_count);
+    run_scan_kernel<<<1, 1024, 0, st>>>(d_count, blocks);
+    pass_runs_kernel<<<(int)((npass * 32 + 32 + kThreads - 1) / kThreads), kThreads, 0, st>>>(nnz, sorted, drop, d_count, (int)npass, d_bounds,
+                                                                                             d_bounds + npass + 1);
+    h->launches += 5;
+    std::vector<int64_t> bounds;
+    try {
+        bounds.resize(2 * ((size_t)npass + 1));
+        h->passes.assign((size_t)npass, RunPass());
+    } catch (const std::bad_alloc &) { cudaStreamSynchronize(st); cleanup(); return DSFACTO_ERR_OOM; }
+    if ((e = cudaMemcpyAsync(bounds.data(), d_bounds, sizeof(int64_t) * bounds.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess)
+        return fail(e);
+    const int64_t *first = bounds.data(), *run_first = first + npass + 1;
+    int64_t longest = 0, most_runs = 1;
+    for (int64_t q = 0; q < npass; ++q) longest = std::max(longest, first[q + 1] - first[q]);
+    if (longest >= ((int64_t)1 << 31) - ((int64_t)1 << 17)) { cleanup(); h->passes.clear(); return 1; }   // positions inside a pass are 32-bit
+    // Units: long enough to amortise a unit's start and end, short enough that a small pass keeps every SM busy.
+    int64_t want = std::min<int64_t>(1024, longest / ((int64_t)h->sm_count * 32));
+    if (h->chunk_override > 0) want = h->chunk_override;
+    if (const char *env = std::getenv("DSFACTO_CHUNK")) {
+        const int v = std::atoi(env);
+        if (v >= 16 && v <= kUnitMax) want = v;
+    }
+    int64_t unit = 32;
+    while (unit < want) unit *= 2;
+    h->unit_len = (int)unit;
+    int64_t units = 0, most_units = 1;
+    for (int64_t q = 0; q < npass; ++q) {
+        RunPass &ps = h->passes[(size_t)q];
+        ps.first = first[q]; ps.count = (int)(first[q + 1] - first[q]);
+        ps.run_first = run_first[q]; ps.nruns = (int)(run_first[q + 1] - run_first[q]);
+        ps.unit_first = units; ps.units = (int)((ps.count + unit - 1) / unit);
+        units += ps.units;
+        most_runs = std::max<int64_t>(most_runs, ps.nruns);
+        most_units = std::max<int64_t>(most_units, ps.units);
+    }
+    const int64_t runs = run_first[npass], ctas = (most_units + kRunWarps - 1) / kRunWarps, rec4 = h->Kp / 4 + 1;
+    if ((rc = dev_alloc(h, &h->d_run_start, (size_t)runs)) || (rc = dev_alloc(h, &h->d_run_key, (size_t)runs)) ||
+        (rc = dev_alloc(h, &h->d_unit_run, (size_t)units)) || (rc = dev_alloc(h, &h->d_rec, (size_t)(most_runs * rec4))) ||
+        (rc = dev_alloc(h, &h->d_part, (size_t)(2 * ctas * rec4))) || (rc = column_state(h, bands > 1, false))) {
+        cleanup();
+        return rc;
+    }
+    RunWriteArgs wa{};
+    wa.nnz = nnz; wa.key = sorted; wa.drop = drop; wa.low_bits = low_bits; wa.cbits = cbits; wa.count = d_count; wa.bounds = d_bounds;
+    wa.ent = reinterpret_cast<uint2 *>(pbuf.Current()); wa.run_start = h->d_run_start; wa.run_key = h->d_run_key;
+    run_write_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(wa);
+    h->launches += 1;
+    for (const RunPass &ps : h->passes) {
+        if (ps.units == 0) continue;
+        const int grid = (int)std::min<int64_t>((ps.units + kThreads - 1) / kThreads, wide_grid);
+        unit_runs_kernel<<<grid, kThreads, 0, st>>>(h->d_run_start + ps.run_first, ps.nruns, ps.units, h->unit_len, h->d_unit_run + ps.unit_first);
+        h->launches += 1;
+    }
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    h->d_ent = reinterpret_cast<uint2 *>(pbuf.Current());   // the sorted payloads are the entry records
+    pay[pbuf.selector] = nullptr;
+    cleanup();
+    h->runs = true;
+    h->bands = (int)bands;
+    return DSFACTO_OK;
+}
+
 // the device copy of the CSR arrays and labels, made before the handle's old data set is let go
 struct PendingCsr {
     int64_t *indptr = nullptr;
@@ -1688,6 +1999,78 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
     return load_validated(h, indptr, indices, values, y, overlapped ? &pending : nullptr);
 }
 
+// Tile lists and launch plan of the tile sweep.  The CSR copies are queued on the stream; on an error the caller
+// lets the data set go.
+static int load_tiles(dsfacto_t *h, const int64_t *indptr, const int32_t *indices, const float *values, const char *load_env) {
+    const int64_t n = h->n, nnz = indptr[n];
+    const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
+    cudaStream_t st = h->stream;
+    int rc = column_state(h, h->sweep == 1, true);
+    if (rc) return rc;
+    // Tile lists.  With enough row blocks (row-block sweep) a row block is the unit of work; large
+    // loads are then streamed: bucketed into page-locked staging memory and copied to the device
+    // block by block, overlapping the bucketing of the other blocks.  DSFACTO_LOAD=stream takes that
+    // way for small loads too, DSFACTO_LOAD=simple never.
+    HostBuf<uint2> ent;
+    HostBuf<float> xw;
+    std::vector<int32_t> cb;
+    int64_t longest = 0;
+    choose_chunk_len(h, nnz, h->p);
+    SgdPlanBuild pb;   // the chunks of the stratum SGD launches are cut while the tiles are bucketed
+    if (!init_plan_build(h, pb, omp_get_max_threads())) return DSFACTO_ERR_OOM;
+    const bool by_row_block = use_row_block_bucketer(h);
+    const bool on_device = device_bucketing_wanted(h, nnz, load_env);
+    const bool streamed = !on_device && by_row_block && nnz > 0 &&
+                          (nnz >= kStreamedLoadMinEntries ||
+                           (load_env && (std::strcmp(load_env, "stream") == 0 || std::strcmp(load_env, "nostaging") == 0))) &&
+                          !(load_env && std::strcmp(load_env, "simple") == 0);
+    if (on_device) {
+        // bucketed below, once the entry array is allocated; the tile pointers get their size here
+        try { h->tile_ptr.assign((size_t)h->p * h->p + 1, 0); }
+        catch (const std::bad_alloc &) { return DSFACTO_ERR_OOM; }
+    } else if (streamed) {
+        try { column_blocks(h, cb); } catch (const std::bad_alloc &) { return DSFACTO_ERR_OOM; }
+        longest = count_tiles_by_row_block(h, cb, indptr, indices);
+        if (longest < 0) return DSFACTO_ERR_OOM;
+    } else {
+        rc = by_row_block ? bucket_tiles_by_row_block(h, indptr, indices, values, ent, xw, &pb)
+                          : bucket_tiles(h, indptr, indices, values, ent, xw, &pb);
+        if (rc) return rc;
+    }
+    if ((rc = dev_alloc(h, &h->d_ent, cnt + 4)) || (h->wide && (rc = dev_alloc(h, &h->d_xw, cnt + 4)))) return rc;
+    bool copy_from_host = !streamed && !on_device;
+    if (on_device) {
+        if ((rc = device_bucket_tiles(h, nnz, pb))) return rc;
+    }
+    if (streamed) {
+        bool no_staging = false;
+        rc = stream_tiles_by_row_block(h, cb, longest, indptr, indices, values, &no_staging, &pb);
+        if (rc && no_staging) {   // no page-locked memory to be had: bucket into pageable memory, one copy
+            if (!init_plan_build(h, pb, omp_get_max_threads())) return DSFACTO_ERR_OOM;
+            rc = bucket_tiles_by_row_block(h, indptr, indices, values, ent, xw, &pb);
+            copy_from_host = true;
+        }
+        if (rc) return rc;
+    }
+    if (copy_from_host && nnz > 0) {
+        CU_TRY(h, cudaMemcpyAsync(h->d_ent, ent.data(), sizeof(uint2) * (size_t)nnz, cudaMemcpyHostToDevice, st));
+        if (h->wide) CU_TRY(h, cudaMemcpyAsync(h->d_xw, xw.data(), sizeof(float) * (size_t)nnz, cudaMemcpyHostToDevice, st));
+    }
+    CU_TRY(h, cudaStreamSynchronize(st));
+    if (!pb.finished && (rc = finish_sgd_plan(h, pb))) return rc;
+    {
+        const int64_t nt1 = (int64_t)h->p * h->p + 1, plan_bytes = (int64_t)sizeof(ChunkDesc) * h->total_chunks;
+        const int64_t csr_bytes = 8 * (n + 1) + 8 * nnz + 4 * n;   // indptr, idx, val, y
+        const int64_t nt = nt1 - 1;
+        h->load_info[0] = on_device ? 2 : (copy_from_host ? 0 : 1);
+        // device bucketing: the per-tile counts come back, the per-tile starting values go out; only a plan
+        // that is cut into segments sends its descriptors to the host and back
+        h->load_info[1] = csr_bytes + 8 * nt1 + (on_device ? 8 * (4 * nt + 1) + (pb.finished ? 0 : plan_bytes) : plan_bytes + (h->wide ? 12 : 8) * nnz);
+        h->load_info[2] = on_device ? 8 * nt1 + 24 * nt + (pb.finished ? 0 : plan_bytes) : 0;
+    }
+    return DSFACTO_OK;
+}
+
 static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *indices, const float *values, const float *y,
                           PendingCsr *pending) {
     const int64_t n = h->n, nnz = indptr[n];
@@ -1695,7 +2078,9 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
     if (!pending) CU_TRY(h, cudaStreamSynchronize(h->stream));   // (the copies of a pending CSR are still under way)
     free_data(h);
     h->nnz = nnz;
-    h->refresh_grid = refresh_grid_for(h, n);
+    // the recompute pass also takes the squared norms of the parameters: CTAs for both
+    h->refresh_grid = std::max(refresh_grid_for(h, n),
+                               (int)std::min<int64_t>(((int64_t)h->d * (h->Kp / 4) + 8 * kThreads - 1) / (8 * kThreads), (int64_t)h->sm_count * 8));
     const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
     cudaStream_t st = h->stream;
     if (pending) {
@@ -1717,85 +2102,36 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
         CU_TRY_LOAD(h, cudaMemcpyAsync(h->d_y, y, sizeof(float) * (size_t)n, cudaMemcpyHostToDevice, st));
     }
 
-    // Tile lists.  With enough row blocks (row-block sweep) a row block is the unit of work; large
-    // loads are then streamed: bucketed into page-locked staging memory and copied to the device
-    // block by block, overlapping the bucketing of the other blocks.  DSFACTO_LOAD=stream takes that
-    // way for small loads too, DSFACTO_LOAD=simple never.
-    HostBuf<uint2> ent;
-    HostBuf<float> xw;
-    std::vector<int32_t> cb;
-    int64_t longest = 0;
-    choose_chunk_len(h, nnz, h->p);
-    SgdPlanBuild pb;   // the chunks of the stratum SGD launches are cut while the tiles are bucketed
-    if (!init_plan_build(h, pb, omp_get_max_threads())) { cudaStreamSynchronize(st); free_data(h); return DSFACTO_ERR_OOM; }
-    const bool by_row_block = use_row_block_bucketer(h);
-    const char *load_env = std::getenv("DSFACTO_LOAD");
-    const bool on_device = device_bucketing_wanted(h, nnz, load_env);
-    const bool streamed = !on_device && by_row_block && nnz > 0 &&
-                          (nnz >= kStreamedLoadMinEntries ||
-                           (load_env && (std::strcmp(load_env, "stream") == 0 || std::strcmp(load_env, "nostaging") == 0))) &&
-                          !(load_env && std::strcmp(load_env, "simple") == 0);
-    if (on_device) {
-        // bucketed below, once the entry array is allocated; the tile pointers get their size here
-        try { h->tile_ptr.assign((size_t)h->p * h->p + 1, 0); }
-        catch (const std::bad_alloc &) { cudaStreamSynchronize(st); free_data(h); return DSFACTO_ERR_OOM; }
-    } else if (streamed) {
-        try { column_blocks(h, cb); } catch (const std::bad_alloc &) { cudaStreamSynchronize(st); free_data(h); return DSFACTO_ERR_OOM; }
-        longest = count_tiles_by_row_block(h, cb, indptr, indices);
-        if (longest < 0) { cudaStreamSynchronize(st); free_data(h); return DSFACTO_ERR_OOM; }
-    } else {
-        rc = by_row_block ? bucket_tiles_by_row_block(h, indptr, indices, values, ent, xw, &pb)
-                          : bucket_tiles(h, indptr, indices, values, ent, xw, &pb);
-        if (rc) { cudaStreamSynchronize(st); free_data(h); return rc; }
-    }
-    h->nnz = nnz;   // (free_data on an error path above resets it)
     if ((rc = dev_alloc(h, &h->d_A, (size_t)n * h->Kp + (h->nshards > 1 ? 2 * (size_t)n : 0))) || (rc = dev_alloc(h, &h->d_G, (size_t)n)) ||
-        (rc = dev_alloc(h, &h->d_tile_ptr, h->tile_ptr.size())) || (rc = dev_alloc(h, &h->d_ent, cnt + 4)) ||
-        (rc = dev_alloc(h, &h->d_partials, 2 * ((size_t)h->refresh_grid + (size_t)h->norm_grid))) ||
-        (h->wide && (rc = dev_alloc(h, &h->d_xw, cnt + 4)))) {
+        (rc = dev_alloc(h, &h->d_partials, std::max(4 * (size_t)h->refresh_grid, 2 * ((size_t)h->refresh_grid + (size_t)h->norm_grid))))) {
         cudaStreamSynchronize(st);
         free_data(h);
         return rc;
     }
-    bool copy_from_host = !streamed && !on_device;
-    if (on_device) {
-        if ((rc = device_bucket_tiles(h, nnz, pb))) { cudaStreamSynchronize(st); free_data(h); return rc; }
+    const char *load_env = std::getenv("DSFACTO_LOAD");
+    bool by_runs = run_plan_wanted(h, nnz, load_env);
+    if (by_runs) {
+        rc = plan_runs(h, nnz);
+        if (rc < 0) { cudaStreamSynchronize(st); free_data(h); return rc; }
+        by_runs = rc == 0;
     }
-    if (streamed) {
-        bool no_staging = false;
-        rc = stream_tiles_by_row_block(h, cb, longest, indptr, indices, values, &no_staging, &pb);
-        if (rc && no_staging) {   // no page-locked memory to be had: bucket into pageable memory, one copy
-            if (!init_plan_build(h, pb, omp_get_max_threads())) { cudaStreamSynchronize(st); free_data(h); return DSFACTO_ERR_OOM; }
-            rc = bucket_tiles_by_row_block(h, indptr, indices, values, ent, xw, &pb);
-            copy_from_host = true;
-        }
-        if (rc) { cudaStreamSynchronize(st); free_data(h); return rc; }
+    if (by_runs) {
+        h->load_info[0] = 2;
+        h->load_info[1] = 8 * (n + 1) + 8 * nnz + 4 * n;                       // indptr, idx, val, y
+        h->load_info[2] = 16 * ((int64_t)h->passes.size() + 1);                // first entry and run of every pass
+    } else if ((rc = load_tiles(h, indptr, indices, values, load_env))) {
+        cudaStreamSynchronize(st);
+        free_data(h);
+        return rc;
     }
-    if (copy_from_host && nnz > 0) {
-        CU_TRY_LOAD(h, cudaMemcpyAsync(h->d_ent, ent.data(), sizeof(uint2) * (size_t)nnz, cudaMemcpyHostToDevice, st));
-        if (h->wide) CU_TRY_LOAD(h, cudaMemcpyAsync(h->d_xw, xw.data(), sizeof(float) * (size_t)nnz, cudaMemcpyHostToDevice, st));
-    }
-    CU_TRY_LOAD(h, cudaMemcpyAsync(h->d_tile_ptr, h->tile_ptr.data(), sizeof(int64_t) * h->tile_ptr.size(), cudaMemcpyHostToDevice, st));
-    CU_TRY_LOAD(h, cudaStreamSynchronize(st));
-    if (!pb.finished && (rc = finish_sgd_plan(h, pb))) { free_data(h); return rc; }
     if ((rc = order_columns(h))) { free_data(h); return rc; }
-    {
-        const int64_t nt1 = (int64_t)h->p * h->p + 1, plan_bytes = (int64_t)sizeof(ChunkDesc) * h->total_chunks;
-        const int64_t csr_bytes = 8 * (n + 1) + 8 * nnz + 4 * n;   // indptr, idx, val, y
-        const int64_t nt = nt1 - 1;
-        h->load_info[0] = on_device ? 2 : (copy_from_host ? 0 : 1);
-        // device bucketing: the per-tile counts come back, the per-tile starting values go out; only a plan
-        // that is cut into segments sends its descriptors to the host and back
-        h->load_info[1] = csr_bytes + 8 * nt1 + (on_device ? 8 * (4 * nt + 1) + (pb.finished ? 0 : plan_bytes) : plan_bytes + (h->wide ? 12 : 8) * nnz);
-        h->load_info[2] = on_device ? 8 * nt1 + 24 * nt + (pb.finished ? 0 : plan_bytes) : 0;
-    }
     h->failed = false;
     h->loaded = true;
     if (h->nshards > 1) {   // the partial sums sit right behind A, so that one buffer holds what the shards exchange
         h->d_lin = h->d_A + (size_t)n * h->Kp;
         h->d_q = h->d_lin + n;
     }
-    rc = run_refresh(h, false);
+    rc = refresh_now(h);
     if (rc) return rc;
     if (h->nshards > 1) return DSFACTO_OK;   // no objective before the shards' partial sums have been added up
     return std::isfinite(h->objective) ? DSFACTO_OK : DSFACTO_ERR_DIVERGED;
@@ -1813,9 +2149,12 @@ static int sgd_gave_up(dsfacto *h, const int code[3]) {
     else std::snprintf(buf, sizeof buf, "stratum SGD: debug check %d failed (value %d)", code[1], code[2]);
     h->err = buf;
     const size_t d = (size_t)h->d;
-    cudaMemsetAsync(h->d_run_count, 0, sizeof(int) * (size_t)std::max<int64_t>(h->long_runs, 1), h->stream);
-    cudaMemsetAsync(h->d_sync, 0, sizeof(int) * sync_words(h->p), h->stream);
-    cudaMemsetAsync(h->d_S, 0, sizeof(float4) * d, h->stream);
+    cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream);
+    if (!h->runs) {
+        cudaMemsetAsync(h->d_run_count, 0, sizeof(int) * (size_t)std::max<int64_t>(h->long_runs, 1), h->stream);
+        cudaMemsetAsync(h->d_sync, 0, sizeof(int) * sync_words(h->p), h->stream);
+        cudaMemsetAsync(h->d_S, 0, sizeof(float4) * d, h->stream);
+    }
     if (h->d_TS) {
         cudaMemsetAsync(h->d_TS, 0, sizeof(float4) * d, h->stream);
         cudaMemsetAsync(h->d_Tw, 0, sizeof(float) * d, h->stream);
@@ -1836,32 +2175,49 @@ int dsfacto_epoch(dsfacto_t *h) {
 }
 
 static int epoch_impl(dsfacto_t *h) {
-    cudaStream_t st = h->stream;
-    CU_TRY(h, cudaEventRecord(h->ev[0], st));
     const int64_t p = h->p;
     const int64_t every = (h->refresh_every > 0 && h->refresh_every < p) ? h->refresh_every : p;
-    float t01 = 0, t12 = 0, t23 = 0;
+    const bool shard = h->nshards > 1;
     int rc = DSFACTO_OK;
+    if (shard) CU_TRY(h, cudaEventRecord(h->ev[0], h->stream));
     for (int64_t L0 = 0; L0 < p; L0 += every) {
         const int64_t L1 = std::min(L0 + every, p);
-        if (L0 > 0) CU_TRY(h, cudaEventRecord(h->ev[0], st));
         // w0 step with the frozen multipliers: the share of the epoch's step that belongs to these rounds
-        h->w0 = (float)((double)h->w0 - (double)h->h * ((double)(L1 - L0) / (double)p) * h->g_sum);
-        run_sgd_phase(h, L0, L1);
-        CU_TRY(h, cudaEventRecord(h->ev[1], st));
-        rc = run_refresh(h, true);
+        const double share = (double)(L1 - L0) / (double)p;
+        const bool last = L1 == p;
+        if (h->runs && !shard) {
+            // the segments follow one another on the device; the host hears of the last one
+            run_strata(h, L0 / every, share);
+            rc = run_refresh(h, L0 == 0, last);
+        } else {
+            h->w0 = (float)((double)h->w0 - (double)h->h * share * h->g_sum);
+            if (!shard) {
+                epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
+                h->launches += 1;
+            }
+            if (h->runs) run_strata(h, 0, 0.0);
+            else run_sgd_phase(h, L0, L1);
+            if (shard) CU_TRY(h, cudaEventRecord(h->ev[1], h->stream));
+            rc = run_refresh(h, L0 == 0, true);
+        }
         if (rc) return rc;
-        float a01 = 0, a12 = 0, a23 = 0;
-        cudaEventElapsedTime(&a01, h->ev[0], h->ev[1]);
-        cudaEventElapsedTime(&a12, h->ev[1], h->ev[2]);
-        cudaEventElapsedTime(&a23, h->ev[2], h->ev[3]);
-        t01 += a01; t12 += a12; t23 += a23;
     }
-    int sgd_error[3] = {0, 0, 0};  // set by the SGD kernel if one of its bounded waits ran out
-    CU_TRY(h, cudaMemcpy(sgd_error, h->d_sync + kSyncError, sizeof sgd_error, cudaMemcpyDeviceToHost));
+    if (shard) {
+        float t01 = 0, t12 = 0;
+        cudaEventElapsedTime(&t01, h->ev[0], h->ev[1]);
+        cudaEventElapsedTime(&t12, h->ev[1], h->ev[2]);
+        h->ms[0] = t01 + t12; h->ms[1] = t01; h->ms[2] = t12; h->ms[3] = 0.f;
+    } else {
+        h->ms[1] = (float)(1e-6 * (double)h->report->ns[0]);
+        h->ms[2] = (float)(1e-6 * (double)h->report->ns[1]);
+        h->ms[0] = h->ms[1] + h->ms[2];
+        h->ms[3] = 0.f;
+    }
+    int sgd_error[3] = {0, 0, 0};  // set by the SGD kernel if a bounded wait ran out or a check of the debug build failed
+    if (!h->runs) CU_TRY(h, cudaMemcpy(sgd_error, h->d_sync + kSyncError, sizeof sgd_error, cudaMemcpyDeviceToHost));
+    else if (!shard) for (int c = 0; c < 3; ++c) sgd_error[c] = h->report->err[c];
     if (sgd_error[0]) return sgd_gave_up(h, sgd_error);
-    h->ms[0] = t01 + t12 + t23; h->ms[1] = t01; h->ms[2] = t12; h->ms[3] = t23;
-    if (h->nshards > 1) return DSFACTO_OK;   // the objective exists only after the shards' sums have been added up
+    if (shard) return DSFACTO_OK;   // the objective exists only after the shards' sums have been added up
     return std::isfinite(h->objective) ? DSFACTO_OK : DSFACTO_ERR_DIVERGED;
 }
 
@@ -1964,7 +2320,7 @@ int dsfacto_set_params(dsfacto_t *h, const float *w0, const float *w, const floa
     if (V) { int rc = upload_V(h, V); if (rc) return rc; }
     if (w && V) h->failed = false;   // a handle whose SGD launch gave up is usable again once w and V are replaced
     if (h->loaded) {
-        int rc = run_refresh(h, false);
+        int rc = refresh_now(h);
         if (rc) return rc;
         if (!std::isfinite(h->objective)) return DSFACTO_ERR_DIVERGED;
     }
@@ -1987,6 +2343,24 @@ int dsfacto_get_tiles(dsfacto_t *h, int64_t *tile_ptr, int32_t *rows, int32_t *c
     if (!h->loaded) return DSFACTO_ERR_NO_DATA;
     const int64_t nt = (int64_t)h->p * h->p;
     std::vector<int64_t> canon;
+    if (h->runs) {
+        HostBuf<uint2> ent;
+        if (!ent.alloc((size_t)h->nnz)) return DSFACTO_ERR_OOM;
+        std::vector<int> run_start;
+        std::vector<uint32_t> run_key;
+        try {
+            const RunPass &last = h->passes.back();
+            run_start.resize((size_t)(last.run_first + last.nruns));
+            run_key.resize(run_start.size());
+        } catch (const std::bad_alloc &) { return DSFACTO_ERR_OOM; }
+        CU_TRY(h, cudaMemcpyAsync(ent.data(), h->d_ent, sizeof(uint2) * (size_t)h->nnz, cudaMemcpyDeviceToHost, h->stream));
+        CU_TRY(h, cudaMemcpyAsync(run_start.data(), h->d_run_start, sizeof(int) * run_start.size(), cudaMemcpyDeviceToHost, h->stream));
+        CU_TRY(h, cudaMemcpyAsync(run_key.data(), h->d_run_key, sizeof(uint32_t) * run_key.size(), cudaMemcpyDeviceToHost, h->stream));
+        CU_TRY(h, cudaStreamSynchronize(h->stream));
+        try { unpack_runs(h, ent.data(), run_start, run_key, canon, rows, cols, vals); } catch (const std::bad_alloc &) { return DSFACTO_ERR_OOM; }
+        if (tile_ptr) std::memcpy(tile_ptr, canon.data(), sizeof(int64_t) * ((size_t)nt + 1));
+        return DSFACTO_OK;
+    }
     if (h->rbits == 0) {
         try { canon = canonical_tile_ptr(h); } catch (const std::bad_alloc &) { return DSFACTO_ERR_OOM; }
         if (tile_ptr) std::memcpy(tile_ptr, canon.data(), sizeof(int64_t) * ((size_t)nt + 1));
@@ -2075,21 +2449,19 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         if ((rc = dev_alloc(h, &d_f, (size_t)m))) { cleanup(); return rc; }
         a.f_out = d_f;
         DSF_DISPATCH_REFRESH(h, h, a, kScore, grid);
-        h->launches += 1;
         e = cudaMemcpyAsync(scores_out, d_f, sizeof(float) * (size_t)m, cudaMemcpyDeviceToHost, h->stream);
     } else {
-        if ((rc = dev_alloc(h, &d_yy, (size_t)m)) || (rc = dev_alloc(h, &d_part, 2 * (size_t)grid + 2))) { cleanup(); return rc; }
+        if ((rc = dev_alloc(h, &d_yy, (size_t)m)) || (rc = dev_alloc(h, &d_part, 4 * (size_t)grid))) { cleanup(); return rc; }
         cudaMemcpyAsync(d_yy, y, sizeof(float) * (size_t)m, cudaMemcpyHostToDevice, h->stream);
         a.y = d_yy; a.partials = d_part;
+        a.done = &h->d_state->done; a.report = h->report; a.seq = ++h->report_seq;
         DSF_DISPATCH_REFRESH(h, h, a, kEvaluate, grid);
-        reduce2_kernel<<<1, kThreads, 0, h->stream>>>(d_part, grid, d_part + 2 * (size_t)grid);
-        h->launches += 2;
-        e = cudaMemcpyAsync(sums2, d_part + 2 * (size_t)grid, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     cleanup();
     if (e != cudaSuccess) { h->err = cudaGetErrorString(e); return DSFACTO_ERR_CUDA; }
+    if (mode == kEvaluate) { sums2[0] = h->report->loss; sums2[1] = h->report->g; }
     return DSFACTO_OK;
 }
 

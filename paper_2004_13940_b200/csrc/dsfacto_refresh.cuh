@@ -2,6 +2,7 @@
 // fp64 sums behind the objective.
 #pragma once
 #include "dsfacto_common.cuh"
+#include "dsfacto_runs.cuh"
 
 namespace dsf {
 
@@ -34,10 +35,41 @@ struct RefreshArgs {
     float *G;
     float *f_out;
     float *lin_out, *q_out;  // kPartial: per-row partial sums
-    double *partials;  // 2 per CTA
+    double *partials;  // 4 per CTA: the two sums of the mode, sum w_j^2, sum v_jk^2
     float w0;
     int loss;
+    // the squared norms of eq. (fm_obj), shared out over the CTAs (kTrain; norm_d = 0: left out)
+    const float *norm_w, *norm_V;
+    int64_t norm_d, norm_v4;
+    // end of the pass: the last CTA adds the partial sums up
+    unsigned *done;        // CTAs that have delivered (zero between launches)
+    EpochState *st;        // kTrain: w0 comes from here and the sums go here; NULL: w0 above
+    EpochReport *report;   // mapped host memory: the sums and, behind them, seq (NULL: not the end of an epoch)
+    unsigned long long seq;
+    int first;             // kTrain: the first segment of an epoch (its times are set, not added)
 };
+
+// Sums of the whole launch in a fixed order: thread 0 of the last CTA to get here returns true and holds them.
+__device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, unsigned *done) {
+    __shared__ bool last;
+    block_sum4(s);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) partials[4 * (size_t)blockIdx.x + c] = s[c];
+        __threadfence();
+        last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[c] = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kThreads)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] += __ldcg(partials + 4 * (size_t)b + c);
+    block_sum4(s);
+    return threadIdx.x == 0;
+}
 
 // Rows of 128 bytes and more keep 8 float4s per lane in flight and would take 88 to 100 registers:
 // capped at 80 so that three CTAs stay resident (K = 128: 27.1 -> 22.3 ms per pass on 400 M entries;
@@ -56,6 +88,7 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
     // the fp64 sums of a lane group live in shared memory: only its first lane touches them, once per row
     __shared__ double sums[2][G];
     if (l == 0) { sums[0][g] = 0.0; sums[1][g] = 0.0; }
+    let_next_kernel_start();
 
     // The row pointers of the next row are requested while the current row is processed, and its
     // first batch of entries during the current row's last batch: a lane group never waits for the
@@ -71,6 +104,11 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
         nlen = (int)(__ldg(a.indptr + row_first + 1) - nbeg);
         if (l < nlen) { jn = __ldg(a.idx + nbeg + l); xn = __ldg(a.val + nbeg + l); }
     }
+    // (the rows do not change during an epoch; the model, which the kernel before this one writes, is read with
+    // plain loads: the read-only path assumes data that nobody writes during the whole life of a kernel)
+    wait_for_previous_kernel();
+    if (TRAIN && a.st && blockIdx.x == 0 && threadIdx.x == 0) a.st->t1 = device_ns();
+    const float w0 = TRAIN && a.st ? a.st->w0 : a.w0;
     for (int64_t row = row_first; row < a.n; row += row_step) {
         const int64_t beg = nbeg;
         const int len = nlen;
@@ -98,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             jn = 0; xn = 0.f;
             if (more) { jn = __ldg(a.idx + ahead); xn = __ldg(a.val + ahead); }
             if (t0 + l < len) {
-                const float2 ws = __ldg(a.pair + jm);
+                const float2 ws = a.pair[jm];
                 lin = fmaf(ws.x, xm, lin);
                 q = fmaf(xm * xm, ws.y, q);
             }
@@ -119,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
                     xs[u] = X_EARLY ? __shfl_sync(gm, xm, u0 + u, LG) : 0.f;
                     if (u0 + u < cnt) {
 #pragma unroll
-                        for (int v = 0; v < NV; ++v) vv[u][v] = __ldg(V4 + (size_t)j * KP4 + v * LG + l);
+                        for (int v = 0; v < NV; ++v) vv[u][v] = V4[(size_t)j * KP4 + v * LG + l];
                     }
                 }
 #pragma unroll
@@ -158,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             lin += __shfl_xor_sync(gm, lin, o, LG);
         }
         if (l == 0) {
-            const float f = a.w0 + lin + 0.5f * pair;
+            const float f = w0 + lin + 0.5f * pair;
             if (MODE != kScore) {
                 const float yy = a.y[row];
                 float li, gi;
@@ -184,12 +222,45 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             }
         }
     }
-    if (MODE != kScore && MODE != kPartial) {
-        double loss_sum = l == 0 ? sums[0][g] : 0.0, g_sum = l == 0 ? sums[1][g] : 0.0;
-        block_sum2(loss_sum, g_sum);
-        if (threadIdx.x == 0) {
-            a.partials[2 * blockIdx.x] = loss_sum;
-            a.partials[2 * blockIdx.x + 1] = g_sum;
+    if (MODE == kTrain || MODE == kEvaluate) {
+        double s[4] = {l == 0 ? sums[0][g] : 0.0, l == 0 ? sums[1][g] : 0.0, 0.0, 0.0};
+        if (TRAIN) {
+            const int64_t stride = (int64_t)gridDim.x * kThreads;
+            for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.norm_d; i += stride) {
+                const double x = (double)a.norm_w[i];
+                s[2] += x * x;
+            }
+            const float4 *N4 = reinterpret_cast<const float4 *>(a.norm_V);
+            for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.norm_v4; i += stride) {
+                const float4 x = N4[i];
+                s[3] += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
+            }
+        }
+        if (last_cta_sum4(s, a.partials, a.done)) {
+            if (TRAIN && a.st) {
+                EpochState &st = *a.st;
+                st.loss = s[0]; st.g = s[1]; st.w2 = s[2]; st.v2 = s[3];
+            }
+            if (a.report) {
+                volatile EpochReport *r = a.report;
+                r->loss = s[0]; r->g = s[1]; r->w2 = s[2]; r->v2 = s[3];
+            }
+            if (TRAIN && a.st) {
+                EpochState &st = *a.st;
+                const unsigned long long now = device_ns();
+                const unsigned long long ns0 = st.t1 - st.t0 + (a.first ? 0ull : st.ns[0]), ns1 = now - st.t1 + (a.first ? 0ull : st.ns[1]);
+                st.ns[0] = ns0; st.ns[1] = ns1;
+                if (a.report) {
+                    volatile EpochReport *r = a.report;
+                    r->w0 = st.w0;
+                    r->ns[0] = ns0; r->ns[1] = ns1;
+                    for (int c = 0; c < 3; ++c) r->err[c] = st.err[c];
+                }
+            }
+            if (a.report) {
+                __threadfence_system();
+                ((volatile EpochReport *)a.report)->seq = a.seq;
+            }
         }
     }
 }
