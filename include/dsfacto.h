@@ -213,6 +213,11 @@ int dsfacto_debug_set(dsfacto_t *h, int32_t key, int64_t value);
  * info[2] = bytes it copied device -> host.  DSFACTO_ERR_NO_DATA before the first load. */
 int dsfacto_last_load(dsfacto_t *h, int64_t info[3]);
 
+/* The library keeps freed device memory for its next calls (per device up to a 64th of its memory) and the
+ * page-locked mailboxes of up to eight destroyed handles.  This gives all of it back.  It is also given back when an
+ * allocation of the library fails.  Safe to call at any time, from any thread. */
+void dsfacto_trim(void);
+
 /* Number of kernels this handle has launched since creation. */
 int dsfacto_launch_count(dsfacto_t *h, int64_t *out);
 

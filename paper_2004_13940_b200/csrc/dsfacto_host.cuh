@@ -1,0 +1,364 @@
+// Host-side services of the library: the device memory pool and the transfers between pageable caller memory and
+// the device.
+#pragma once
+#include <cuda_runtime.h>
+#include <unistd.h>
+
+#include <algorithm>
+#include <atomic>
+#include <condition_variable>
+#include <cstdint>
+#include <cstring>
+#include <initializer_list>
+#include <map>
+#include <mutex>
+#include <new>
+#include <thread>
+#include <unordered_map>
+#include <vector>
+
+namespace dsf {
+
+// ------------------------------------------------------------------------------------------
+// Device memory.  cudaMalloc and cudaFree cost 0.4 and 0.3 ms whatever the size, and a load makes some thirty of
+// each: a load of 2.6 M entries spent nine tenths of its time there.  Freed blocks are kept per device, up to a
+// 64th of its memory, and handed out again for requests of about their size; they go back to the driver when an
+// allocation fails, when the bound is reached (the block at hand is freed at once), and with trim().
+// A block is freed only after the work that used it has finished (callers synchronise their stream first), so it may
+// be handed to any thread and stream.
+// ------------------------------------------------------------------------------------------
+class DevicePool {
+public:
+    static DevicePool &get() {
+        static DevicePool *pool = new DevicePool;   // (never destroyed: handles may outlive static destruction)
+        return *pool;
+    }
+    cudaError_t alloc(void **out, size_t bytes) {
+        *out = nullptr;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const size_t unit = bytes > ((size_t)1 << 20) ? (size_t)1 << 21 : 4096;   // large blocks are mapped in 2 MB pages anyway
+        const size_t size = (std::max<size_t>(bytes, 1) + unit - 1) / unit * unit;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            std::multimap<size_t, void *> &idle = idle_[dev];
+            const auto it = idle.lower_bound(size);
+            if (it != idle.end() && it->first <= size + size / 4) {
+                *out = it->second;
+                live_[it->second] = {it->first, dev};
+                idle_bytes_[dev] -= it->first;
+                idle.erase(it);
+                return cudaSuccess;
+            }
+        }
+        e = cudaMalloc(out, size);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            trim();
+            e = cudaMalloc(out, size);
+        }
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lock(mu_);
+        live_[*out] = {size, dev};
+        return cudaSuccess;
+    }
+    void free(void *ptr) {
+        if (!ptr) return;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            const auto it = live_.find(ptr);
+            if (it != live_.end()) {
+                const Block b = it->second;
+                live_.erase(it);
+                if (idle_bytes_[b.dev] + b.bytes <= bound(b.dev)) {
+                    idle_[b.dev].emplace(b.bytes, ptr);
+                    idle_bytes_[b.dev] += b.bytes;
+                    return;
+                }
+            }
+        }
+        cudaFree(ptr);
+    }
+    // idle bytes on the current device
+    size_t idle_bytes() {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        std::lock_guard<std::mutex> lock(mu_);
+        return idle_bytes_[dev];
+    }
+    void trim() {
+        std::vector<void *> go;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            for (auto &d : idle_) {
+                for (auto &b : d.second) go.push_back(b.second);
+                d.second.clear();
+                idle_bytes_[d.first] = 0;
+            }
+        }
+        for (void *p : go) cudaFree(p);
+    }
+
+private:
+    struct Block { size_t bytes; int dev; };
+    size_t bound(int dev) {   // (mu_ is held)
+        auto it = bound_.find(dev);
+        if (it == bound_.end()) {
+            size_t free_b = 0, total_b = 0;
+            if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) total_b = 0;
+            it = bound_.emplace(dev, total_b / 64).first;
+        }
+        return it->second;
+    }
+    std::mutex mu_;
+    std::map<int, std::multimap<size_t, void *>> idle_;
+    std::map<int, size_t> idle_bytes_, bound_;
+    std::unordered_map<void *, Block> live_;
+};
+
+// ------------------------------------------------------------------------------------------
+// Transfers.  A copy between pageable memory and the device goes through the driver's staging buffer in one
+// thread: 11 GB/s, and less into memory that has not been touched yet.  Large copies are therefore cut into regions
+// of 2 MB that the calling thread and a few helpers take one after another, each through two page-locked slots of
+// its own: 30 to 50 GB/s.  The helpers sleep between transfers; nobody waits for a helper that has not woken up yet,
+// so a busy machine costs bandwidth, not a stall.  One transfer at a time per process.
+// ------------------------------------------------------------------------------------------
+struct Piece {            // one array of a transfer
+    void *dev;
+    void *host;
+    size_t bytes;
+};
+class Courier {
+public:
+    static Courier &get() {
+        static Courier *c = new Courier;   // (never destroyed: its helpers sleep until the process ends)
+        return *c;
+    }
+    static constexpr size_t kSlot = (size_t)512 << 10, kRegion = (size_t)2 << 20;
+    static constexpr int kMostPieces = 8;
+    static constexpr size_t kWorth = (size_t)1 << 20;   // smaller arrays go through the driver
+    // Copies the pieces on the stream; on return host memory has been read (to the device) or written (from it).
+    // To the device, the last copies may still be under way on the stream.
+    cudaError_t move(bool to_device, std::initializer_list<Piece> pieces, cudaStream_t st) { return move(to_device, pieces.begin(), (int)pieces.size(), st); }
+    cudaError_t move(bool to_device, const Piece *pieces, int count, cudaStream_t st) {
+        cudaError_t e = cudaSuccess;
+        Piece large[kMostPieces];
+        int nlarge = 0;
+        for (int q = 0; q < count; ++q) {
+            const Piece &p = pieces[q];
+            if (p.bytes == 0) continue;
+            bool direct = p.bytes < kWorth;
+            if (!direct) {   // page-locked caller memory needs no detour
+                cudaPointerAttributes at{};
+                if (cudaPointerGetAttributes(&at, p.host) != cudaSuccess) cudaGetLastError();
+                else direct = at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged;
+            }
+            if (!direct && nlarge < kMostPieces) { large[nlarge++] = p; continue; }
+            e = to_device ? cudaMemcpyAsync(p.dev, p.host, p.bytes, cudaMemcpyHostToDevice, st)
+                          : cudaMemcpyAsync(p.host, p.dev, p.bytes, cudaMemcpyDeviceToHost, st);
+            if (e != cudaSuccess) return e;
+        }
+        if (nlarge > 0 && (e = staged(to_device, large, nlarge, st)) != cudaSuccess) return e;
+        return to_device ? cudaSuccess : cudaStreamSynchronize(st);
+    }
+
+private:
+    struct Lane {          // the page-locked slots of one thread
+        char *slot[2] = {nullptr, nullptr};
+        cudaEvent_t ev[2] = {nullptr, nullptr};
+        bool busy[2] = {false, false};
+    };
+    struct Region { char *dev, *host; size_t bytes; };
+    cudaError_t staged(bool to_device, const Piece *pieces, int count, cudaStream_t st) {
+        std::lock_guard<std::mutex> one(transfer_);
+        cudaError_t e;
+        try {
+            size_t most = 0;
+            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kRegion + 2;
+            regions_.reserve(most);
+            e = prepare();
+        } catch (const std::bad_alloc &) { e = cudaErrorMemoryAllocation; }
+        if (e != cudaSuccess) {   // no page-locked memory or threads to be had: the driver's way
+            cudaGetLastError();
+            for (int q = 0; q < count; ++q) {
+                const Piece &p = pieces[q];
+                if ((e = to_device ? cudaMemcpyAsync(p.dev, p.host, p.bytes, cudaMemcpyHostToDevice, st)
+                                   : cudaMemcpyAsync(p.host, p.dev, p.bytes, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+                    return e;
+            }
+            return cudaSuccess;
+        }
+        regions_.clear();
+        for (int q = 0; q < count; ++q) {
+            const Piece &p = pieces[q];
+            char *d = static_cast<char *>(p.dev), *h = static_cast<char *>(p.host), *end = h + p.bytes;
+            while (h < end) {   // regions end on 2 MB boundaries of host memory: a huge page is touched by one thread
+                char *stop = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(h) / kRegion + 1) * kRegion);
+                const size_t n = (size_t)(std::min(stop, end) - h);
+                regions_.push_back({d, h, n});
+                d += n;
+                h += n;
+            }
+        }
+        to_device_ = to_device;
+        stream_ = st;
+        next_.store(0);
+        error_.store(cudaSuccess);
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            open_ = true;
+            ++job_;
+        }
+        wake_.notify_all();
+        work(lanes_[0]);
+        std::unique_lock<std::mutex> lock(mu_);
+        open_ = false;                                   // helpers that wake up now find nothing
+        idle_.wait(lock, [&] { return active_ == 0; });   // those at work finish the region they have
+        return (cudaError_t)error_.load();
+    }
+    void work(Lane &lane) {
+        int turn = 0;
+        auto note = [&](cudaError_t e) { if (e != cudaSuccess) error_.store(e); return e == cudaSuccess; };
+        char *out[2] = {nullptr, nullptr};   // from the device: where the slot's contents go
+        size_t out_n[2] = {0, 0};
+        auto settle = [&](int t) {           // the copy that last used slot t has finished; its contents are passed on
+            if (!lane.busy[t]) return;
+            note(cudaEventSynchronize(lane.ev[t]));
+            lane.busy[t] = false;
+            if (out[t]) { std::memcpy(out[t], lane.slot[t], out_n[t]); out[t] = nullptr; }
+        };
+        for (size_t r; error_.load() == cudaSuccess && (r = next_.fetch_add(1)) < regions_.size();) {
+            const Region &g = regions_[r];
+            for (size_t at = 0; at < g.bytes; at += kSlot) {
+                const size_t n = std::min(kSlot, g.bytes - at);
+                settle(turn);
+                if (to_device_) {
+                    std::memcpy(lane.slot[turn], g.host + at, n);
+                    if (!note(cudaMemcpyAsync(g.dev + at, lane.slot[turn], n, cudaMemcpyHostToDevice, stream_))) break;
+                } else {
+                    if (!note(cudaMemcpyAsync(lane.slot[turn], g.dev + at, n, cudaMemcpyDeviceToHost, stream_))) break;
+                    out[turn] = g.host + at;
+                    out_n[turn] = n;
+                }
+                if (!note(cudaEventRecord(lane.ev[turn], stream_))) break;
+                lane.busy[turn] = true;
+                turn ^= 1;
+            }
+        }
+        if (!to_device_) { settle(turn); settle(turn ^ 1); }
+    }
+    cudaError_t prepare() {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (pid_ != getpid()) {   // first use, or the child of a fork, which has no helpers
+            pid_ = getpid();
+            lanes_.clear();
+        }
+        if (!lanes_.empty() && dev == device_) return cudaSuccess;
+        // (events belong to a device: a process that works on several gets new ones when it changes over)
+        const bool fresh = lanes_.empty();
+        if (fresh) {
+            const unsigned cores = std::max(2u, std::thread::hardware_concurrency());
+            lanes_.resize(std::min(8u, cores / 2));
+            if ((e = cudaHostAlloc((void **)&arena_, lanes_.size() * 2 * kSlot, cudaHostAllocPortable)) != cudaSuccess) { lanes_.clear(); return e; }
+            for (size_t k = 0; k < lanes_.size(); ++k)
+                for (int t = 0; t < 2; ++t) lanes_[k].slot[t] = arena_ + (2 * k + t) * kSlot;
+        }
+        for (Lane &l : lanes_)
+            for (int t = 0; t < 2; ++t) {
+                if (l.ev[t]) { cudaEventSynchronize(l.ev[t]); cudaEventDestroy(l.ev[t]); }
+                l.busy[t] = false;
+                l.ev[t] = nullptr;
+                if ((e = cudaEventCreateWithFlags(&l.ev[t], cudaEventDisableTiming)) != cudaSuccess) {
+                    if (fresh) lanes_.clear();
+                    device_ = -1;
+                    return e;
+                }
+            }
+        device_ = dev;
+        if (fresh)
+            for (size_t k = 1; k < lanes_.size(); ++k) {
+                try { std::thread([this, k] { help(k); }).detach(); } catch (...) { lanes_.resize(k); break; }
+            }
+        return cudaSuccess;
+    }
+    void help(size_t k) {
+        uint64_t seen = 0;
+        int dev = -1;
+        std::unique_lock<std::mutex> lock(mu_);
+        for (;;) {
+            wake_.wait(lock, [&] { return open_ && job_ != seen; });
+            seen = job_;
+            ++active_;
+            lock.unlock();
+            if (dev != device_) { dev = device_; cudaSetDevice(dev); }
+            work(lanes_[k]);
+            lock.lock();
+            if (--active_ == 0) idle_.notify_all();
+        }
+    }
+    std::mutex transfer_, mu_;
+    std::condition_variable wake_, idle_;
+    bool open_ = false;
+    uint64_t job_ = 0;
+    int active_ = 0, device_ = -1;
+    pid_t pid_ = 0;
+    char *arena_ = nullptr;
+    std::vector<Lane> lanes_;
+    std::vector<Region> regions_;
+    bool to_device_ = false;
+    cudaStream_t stream_ = nullptr;
+    std::atomic<size_t> next_{0};
+    std::atomic<int> error_{0};
+};
+
+// Page-locked, mapped memory of a handle: what kernels report to the host, and small inputs and results.  Page-locking
+// costs 0.45 ms per megabyte, so blocks of handles that are gone are kept for the next ones, eight of them at most.
+constexpr size_t kMailboxBytes = (size_t)128 << 10;
+class Mailboxes {
+public:
+    static Mailboxes &get() {
+        static Mailboxes *m = new Mailboxes;
+        return *m;
+    }
+    void *take() {
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (!idle_.empty()) {
+                void *p = idle_.back();
+                idle_.pop_back();
+                return p;
+            }
+        }
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, kMailboxBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return p;
+    }
+    void give(void *p) {
+        if (!p) return;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (idle_.size() < 8) { idle_.push_back(p); return; }
+        }
+        cudaFreeHost(p);
+    }
+    void trim() {
+        std::vector<void *> go;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            go.swap(idle_);
+        }
+        for (void *p : go) cudaFreeHost(p);
+    }
+
+private:
+    std::mutex mu_;
+    std::vector<void *> idle_;
+};
+
+}  // namespace dsf

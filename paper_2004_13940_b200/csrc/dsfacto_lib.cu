@@ -2,6 +2,8 @@
 // the tile bucketer, device memory, the epoch driver and the copy-out calls.
 #include "dsfacto.h"
 #include "dsfacto_bucket.cuh"
+#include "dsfacto_host.cuh"
+#include "dsfacto_prepare.cuh"
 #include "dsfacto_refresh.cuh"
 #include "dsfacto_runplan.cuh"
 #include "dsfacto_runs.cuh"
@@ -106,6 +108,8 @@ struct dsfacto {
     EpochState *d_state = nullptr;
     EpochReport *report = nullptr;
     unsigned long long report_seq = 0;
+    char *mail = nullptr;          // the rest of that memory: small inputs and results (mail_bytes of it)
+    size_t mail_bytes = 0;
     // update loop by column runs (dsfacto_runs.cuh): every load that is bucketed on the device with default settings
     bool runs = false;
     int bands = 1;                 // passes per segment
@@ -147,12 +151,12 @@ template <typename T>
 int dev_alloc(dsfacto *h, T **ptr, size_t count) {
     *ptr = nullptr;
     if (count == 0) count = 1;
-    CU_TRY(h, cudaMalloc((void **)ptr, count * sizeof(T)));
+    CU_TRY(h, DevicePool::get().alloc((void **)ptr, count * sizeof(T)));
     return DSFACTO_OK;
 }
 template <typename T>
 void dev_free(T *&ptr) {
-    if (ptr) cudaFree(ptr);
+    DevicePool::get().free(ptr);   // (nothing on the device may still be using it)
     ptr = nullptr;
 }
 
@@ -186,21 +190,6 @@ struct HostBuf {
     T *data() { return p; }
     T &operator[](size_t i) { return p[i]; }
 };
-
-// ---- SplitMix64 (Steele, Lea, Flood 2014), random access to the c-th output ----
-inline uint64_t splitmix64_output(uint64_t seed, uint64_t c) {
-    uint64_t z = seed + (c + 1) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-inline double open_unit(uint64_t u) { return ((double)(u >> 11) + 0.5) * (1.0 / 9007199254740992.0); }
-inline float init_factor(uint64_t seed, uint64_t e) {
-    const double u1 = open_unit(splitmix64_output(seed, 2 * e));
-    const double u2 = open_unit(splitmix64_output(seed, 2 * e + 1));
-    const double z = std::sqrt(-2.0 * std::log(u1)) * std::cos(2.0 * 3.14159265358979323846 * u2);
-    return (float)(0.01 * z);
-}
 
 constexpr int kMaxRowMerge = 16;   // most row blocks per slot of the device entry array (32 and 64 were no faster on any data set)
 constexpr int64_t kStreamedLoadMinEntries = (int64_t)1 << 24;   // smaller loads are not worth the staging set-up
@@ -871,7 +860,7 @@ int order_columns(dsfacto *h) {
     void *tmp = nullptr;
     auto cleanup = [&]() {
         dev_free(d_key); dev_free(d_key_out); dev_free(d_col); dev_free(d_slot_of);   // (d_slot_of: kept by the handle on success)
-        if (tmp) cudaFree(tmp);
+        DevicePool::get().free(tmp);
         tmp = nullptr;
     };
     int rc;
@@ -892,7 +881,7 @@ int order_columns(dsfacto *h) {
     if ((e = cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, d_key, d_key_out, d_col, h->d_column_of, (int64_t)d, 0, 32,
                                              h->stream)) != cudaSuccess)
         return fail(e);
-    if ((e = cudaMalloc(&tmp, tmp_bytes ? tmp_bytes : 1)) != cudaSuccess) return fail(e);
+    if ((e = DevicePool::get().alloc(&tmp, tmp_bytes)) != cudaSuccess) return fail(e);
     const int grid = (int)std::min<int64_t>((h->nnz + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     const int dgrid = (int)std::min<int64_t>(((int64_t)d + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     if ((e = cudaMemsetAsync(d_slot_of, 0, sizeof(int32_t) * d, h->stream)) != cudaSuccess) return fail(e);
@@ -998,31 +987,83 @@ int refresh_now(dsfacto *h) {
     return run_refresh(h, true, true);
 }
 
-// V padded (d x Kp) <-> caller layout (d x K)
-int upload_V(dsfacto *h, const float *V) {
-    h->model_version += 1;
-    if (h->Kp == h->K) {
-        CU_TRY(h, cudaMemcpyAsync(h->d_V, V, sizeof(float) * (size_t)h->d * h->K, cudaMemcpyHostToDevice, h->stream));
-    } else {
-        CU_TRY(h, cudaMemsetAsync(h->d_V, 0, sizeof(float) * (size_t)h->d * h->Kp, h->stream));
-        CU_TRY(h, cudaMemcpy2DAsync(h->d_V, sizeof(float) * h->Kp, V, sizeof(float) * h->K, sizeof(float) * h->K,
-                                    (size_t)h->d, cudaMemcpyHostToDevice, h->stream));
+// Results to the caller: small ones through the mailbox, with one wait for all of them.
+struct Fetch {   // at most two arrays
+    Piece piece[2];
+    int count = 0;
+    void add(void *dev, void *host, size_t bytes) { piece[count++] = {dev, host, bytes}; }
+    const Piece *begin() const { return piece; }
+    const Piece *end() const { return piece + count; }
+};
+int fetch(dsfacto *h, const Fetch &pieces) {
+    size_t all = 0;
+    for (const Piece &p : pieces) all += (p.bytes + 15) & ~(size_t)15;
+    if (all == 0) return DSFACTO_OK;
+    if (all > h->mail_bytes) {
+        CU_TRY(h, Courier::get().move(false, pieces.piece, pieces.count, h->stream));
+        return DSFACTO_OK;
+    }
+    size_t at = 0;
+    for (const Piece &p : pieces) {
+        CU_TRY(h, cudaMemcpyAsync(h->mail + at, p.dev, p.bytes, cudaMemcpyDeviceToHost, h->stream));
+        at += (p.bytes + 15) & ~(size_t)15;
     }
     CU_TRY(h, cudaStreamSynchronize(h->stream));
-    return DSFACTO_OK;
-}
-int download_rows(dsfacto *h, float *dst, const float *src_dev, int64_t rows) {
-    if (h->Kp == h->K) {
-        CU_TRY(h, cudaMemcpyAsync(dst, src_dev, sizeof(float) * (size_t)rows * h->K, cudaMemcpyDeviceToHost, h->stream));
-    } else {
-        CU_TRY(h, cudaMemcpy2DAsync(dst, sizeof(float) * h->K, src_dev, sizeof(float) * h->Kp, sizeof(float) * h->K,
-                                    (size_t)rows, cudaMemcpyDeviceToHost, h->stream));
+    at = 0;
+    for (const Piece &p : pieces) {
+        std::memcpy(p.host, h->mail + at, p.bytes);
+        at += (p.bytes + 15) & ~(size_t)15;
     }
-    CU_TRY(h, cudaStreamSynchronize(h->stream));
     return DSFACTO_OK;
 }
 
-// CSR checks shared by load_csr and predict.  Returns DSFACTO_OK or DSFACTO_ERR_INVALID_CSR.
+// rows of Kp floats on the device <-> the caller's rows of K floats
+int upload_rows(dsfacto *h, float *dst_dev, const float *src, int64_t rows) {
+    float *packed = dst_dev;
+    int rc;
+    if (h->Kp != h->K && (rc = dev_alloc(h, &packed, (size_t)rows * h->K))) return rc;
+    cudaError_t e = Courier::get().move(true, {{packed, const_cast<float *>(src), sizeof(float) * (size_t)rows * h->K}}, h->stream);
+    if (e == cudaSuccess && packed != dst_dev) {
+        const int grid = (int)std::min<int64_t>((rows * h->Kp + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
+        pad_rows_kernel<<<grid, kThreads, 0, h->stream>>>(packed, rows, h->K, h->Kp, dst_dev);
+        h->launches += 1;
+    }
+    const cudaError_t e2 = cudaStreamSynchronize(h->stream);
+    if (packed != dst_dev) dev_free(packed);
+    CU_TRY(h, e);
+    CU_TRY(h, e2);
+    return DSFACTO_OK;
+}
+int upload_V(dsfacto *h, const float *V) {
+    h->model_version += 1;
+    return upload_rows(h, h->d_V, V, h->d);
+}
+// (more: other arrays to fetch with the same wait)
+int download_rows(dsfacto *h, float *dst, float *src_dev, int64_t rows, Fetch more) {
+    float *packed = src_dev;
+    int rc;
+    if (h->Kp != h->K) {
+        if ((rc = dev_alloc(h, &packed, (size_t)rows * h->K))) return rc;
+        const int grid = (int)std::min<int64_t>((rows * h->K + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
+        unpad_rows_kernel<<<std::max(grid, 1), kThreads, 0, h->stream>>>(src_dev, rows, h->K, h->Kp, packed);
+        h->launches += 1;
+    }
+    more.add(packed, dst, sizeof(float) * (size_t)rows * h->K);
+    rc = fetch(h, more);
+    if (packed != src_dev) {
+        if (rc) cudaStreamSynchronize(h->stream);
+        dev_free(packed);
+    }
+    return rc;
+}
+
+void launch_validate(dsfacto *h, int64_t m, int64_t nnz, const int64_t *indptr, const int32_t *idx, const float *val, const float *y, int *bad) {
+    const int grid = (int)std::min<int64_t>((m + kThreads / 32 - 1) / (kThreads / 32), (int64_t)h->sm_count * 16);
+    validate_rows_kernel<<<grid, kThreads, 0, h->stream>>>(m, nnz, h->d, indptr, idx, val, y, bad);
+    h->launches += 1;
+}
+
+// CSR checks on the host (shards, the host bucketer).  Returns DSFACTO_OK or DSFACTO_ERR_INVALID_CSR.
 int validate_csr(int64_t m, int32_t d, const int64_t *indptr, const int32_t *indices, const float *values) {
     if (indptr[0] != 0) return DSFACTO_ERR_INVALID_CSR;
     int bad = 0;
@@ -1517,23 +1558,53 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
         (rc = dev_alloc(h, &h->d_scal, 4)) || (rc = dev_alloc(h, &h->d_pair, (size_t)d)))
         return fail(rc);
 
-    std::vector<float> V;
-    try { V.resize((size_t)d * K); } catch (const std::bad_alloc &) { return fail(DSFACTO_ERR_OOM); }
-#pragma omp parallel for schedule(static)
-    for (int64_t e = 0; e < (int64_t)d * K; ++e) V[(size_t)e] = init_factor(seed, (uint64_t)e);
+    if ((rc = dev_alloc(h, &h->d_state, 1))) return fail(rc);
+    h->report = static_cast<EpochReport *>(Mailboxes::get().take());
+    if (!h->report) return fail(DSFACTO_ERR_OOM);
+    std::memset(h->report, 0, sizeof(EpochReport));
+    constexpr size_t kReportBytes = (sizeof(EpochReport) + 255) & ~(size_t)255;
+    h->mail = reinterpret_cast<char *>(h->report) + kReportBytes;
+    h->mail_bytes = kMailboxBytes - kReportBytes;
+
     h->w0 = 0.f;
-    if (cudaMemset(h->d_w, 0, sizeof(float) * (size_t)d) != cudaSuccess) return fail(DSFACTO_ERR_CUDA);
-    if ((rc = upload_V(h, V.data()))) return fail(rc);
-    if (cudaMemcpy(h->d_row_start, h->row_start.data(), sizeof(int64_t) * ((size_t)p + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->d_col_start, h->col_start.data(), sizeof(int32_t) * ((size_t)p + 1), cudaMemcpyHostToDevice) != cudaSuccess)
-        return fail(DSFACTO_ERR_CUDA);
     h->norm_grid = h->sm_count * 8;
     if (const char *env = std::getenv("DSFACTO_SWEEP")) h->sweep = (std::strcmp(env, "round") == 0) ? 0 : 1;
-    if ((rc = dev_alloc(h, &h->d_state, 1))) return fail(rc);
-    if (cudaMemset(h->d_state, 0, sizeof(EpochState)) != cudaSuccess) return fail(DSFACTO_ERR_CUDA);
-    if (cudaHostAlloc((void **)&h->report, sizeof(EpochReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
-        return fail(DSFACTO_ERR_OOM);
-    std::memset(h->report, 0, sizeof(EpochReport));
+    constexpr int kListed = 4096;   // elements of V the host decides (one in four million)
+    int64_t *list = nullptr;
+    int listed = 0;
+    if ((rc = dev_alloc(h, &list, kListed + 1))) return fail(rc);
+    int *d_listed = reinterpret_cast<int *>(list + kListed);
+    const int init_grid = (int)std::min<int64_t>(((int64_t)d * h->Kp + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream)) == cudaSuccess &&
+        (e = cudaMemsetAsync(h->d_w, 0, sizeof(float) * (size_t)d, h->stream)) == cudaSuccess &&
+        (e = cudaMemsetAsync(d_listed, 0, sizeof(int), h->stream)) == cudaSuccess) {
+        init_factors_kernel<<<init_grid, kThreads, 0, h->stream>>>(seed, d, K, h->Kp, h->d_V, d_listed, list, kListed);
+        h->launches += 1;
+        if ((e = cudaMemcpyAsync(h->d_row_start, h->row_start.data(), sizeof(int64_t) * ((size_t)p + 1), cudaMemcpyHostToDevice, h->stream)) == cudaSuccess &&
+            (e = cudaMemcpyAsync(h->d_col_start, h->col_start.data(), sizeof(int32_t) * ((size_t)p + 1), cudaMemcpyHostToDevice, h->stream)) == cudaSuccess &&
+            (e = cudaMemcpyAsync(&listed, d_listed, sizeof(int), cudaMemcpyDeviceToHost, h->stream)) == cudaSuccess)
+            e = cudaStreamSynchronize(h->stream);
+    }
+    rc = e == cudaSuccess ? DSFACTO_OK : DSFACTO_ERR_CUDA;
+    if (!rc && listed > kListed) {   // (not with a generator that works) everything from the host
+        std::vector<float> V;
+        try { V.resize((size_t)d * K); } catch (const std::bad_alloc &) { rc = DSFACTO_ERR_OOM; }
+        if (!rc) {
+#pragma omp parallel for schedule(static)
+            for (int64_t q = 0; q < (int64_t)d * K; ++q) V[(size_t)q] = (float)init_factor(seed, (uint64_t)q);
+            rc = upload_V(h, V.data());
+        }
+    } else if (!rc && listed > 0) {
+        int64_t at[kListed];
+        if (cudaMemcpy(at, list, sizeof(int64_t) * (size_t)listed, cudaMemcpyDeviceToHost) != cudaSuccess) rc = DSFACTO_ERR_CUDA;
+        for (int q = 0; q < listed && !rc; ++q) {
+            const float v = (float)init_factor(seed, (uint64_t)at[q]);
+            if (cudaMemcpy(h->d_V + at[q] / K * h->Kp + at[q] % K, &v, sizeof v, cudaMemcpyHostToDevice) != cudaSuccess) rc = DSFACTO_ERR_CUDA;
+        }
+    }
+    dev_free(list);
+    if (rc) return fail(rc);
     *out = h;
     return DSFACTO_OK;
 }
@@ -1561,7 +1632,7 @@ void dsfacto_destroy(dsfacto_t *h) {
     free_data(h);
     dev_free(h->d_w); dev_free(h->d_V); dev_free(h->d_Tb); dev_free(h->d_Tw); dev_free(h->d_S); dev_free(h->d_TS); dev_free(h->d_row_start); dev_free(h->d_col_start); dev_free(h->d_scal); dev_free(h->d_pair);
     dev_free(h->d_state);
-    if (h->report) cudaFreeHost(h->report);
+    Mailboxes::get().give(h->report);
     for (auto &e : h->ev)
         if (e) cudaEventDestroy(e);
     delete h;
@@ -1613,6 +1684,7 @@ static bool device_bucketing_wanted(const dsfacto *h, int64_t nnz, const char *l
     // epoch on 20 k / 650 k / 3.7 M entries 1.4 / 8.4 / 15.9 ms against 19.8 / 15.7 / 17.7 ms on the host)
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+    free_b += DevicePool::get().idle_bytes();
     // sort buffers 2 x (4 + 8) bytes and their scratch, then entry records, A, G and the launch plan
     const double need = (double)nnz * (24.0 + 1.0 + 8.0 + 2.0) + (double)h->n * 4.0 * (h->Kp + 2);
     return (double)free_b > need * 1.1;
@@ -1672,7 +1744,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     ChunkDesc *d_out = nullptr;
     auto cleanup = [&]() {
         dev_free(key[0]); dev_free(key[1]); dev_free(pay[0]); dev_free(pay[1]);
-        if (tmp) cudaFree(tmp);
+        DevicePool::get().free(tmp);
         tmp = nullptr;
         dev_free(d_tp); dev_free(d_plan); dev_free(d_in); dev_free(d_out);
     };
@@ -1694,7 +1766,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     size_t tmp_bytes = 0;
     if ((e = cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, key[0], key[1], pay[0], pay[1], nnz, 0, kb, st)) != cudaSuccess)
         return fail(e);
-    if ((e = cudaMalloc(&tmp, tmp_bytes ? tmp_bytes : 1)) != cudaSuccess) return fail(e);
+    if ((e = DevicePool::get().alloc(&tmp, tmp_bytes)) != cudaSuccess) return fail(e);
 
     const int wide_grid = h->sm_count * 16;
     TileKeyArgs ka{};
@@ -1806,6 +1878,7 @@ static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env)
     else {
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+        free_b += DevicePool::get().idle_bytes();
         // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs
         if ((double)free_b < 1.1 * ((double)nnz * 26.0 + (double)h->n * 4.0 * (h->Kp + 2))) return false;
     }
@@ -1836,7 +1909,7 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     int64_t *d_count = nullptr, *d_bounds = nullptr;   // run starts before each block; per pass its first entry, its first run
     auto cleanup = [&]() {
         dev_free(key[0]); dev_free(key[1]); dev_free(pay[0]); dev_free(pay[1]); dev_free(d_count); dev_free(d_bounds);
-        if (tmp) cudaFree(tmp);
+        DevicePool::get().free(tmp);
         tmp = nullptr;
     };
     auto fail = [&](cudaError_t e) {
@@ -1858,7 +1931,7 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     cub::DoubleBuffer<unsigned long long> pbuf(pay[0], pay[1]);
     size_t tmp_bytes = 0;
     if ((e = cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc(&tmp, tmp_bytes ? tmp_bytes : 1)) != cudaSuccess) return fail(e);
+    if ((e = DevicePool::get().alloc(&tmp, tmp_bytes)) != cudaSuccess) return fail(e);
     const int wide_grid = h->sm_count * 16;
     RunKeyArgs ka{};
     ka.n = h->n; ka.nnz = nnz; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p; ka.cbits = cbits;
@@ -1949,42 +2022,44 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
     const int64_t nnz = indptr[n];
     if (nnz > 0 && (!indices || !values)) return DSFACTO_ERR_INVALID_ARG;
     int rc;
-    int bad = 0;
-    // A large load sends the CSR arrays to the device while the host checks them (0.1 s of checks against
-    // 0.27 s on the link for 1.755 G entries).  The row pointers are checked first, so that the copies read
-    // exactly the nnz entries they promise; the copies go into new device arrays, and the handle's old data
-    // set is let go only after the checks: a rejected data set leaves the handle as it was.
+    // The CSR arrays go to the device first and are checked there (a pass over them that costs next to nothing where
+    // they are; on the host it takes longer than the copy).  They go into new device arrays, and the handle's old
+    // data set is let go only after the checks: a rejected data set leaves the handle as it was.  A column shard
+    // keeps a part of the entries only, which the host picks out, so there the host checks as well.
     PendingCsr pending;
-    const bool overlapped = h->nshards == 1 && nnz >= kStreamedLoadMinEntries;
-    if (overlapped) {
-#pragma omp parallel for schedule(static) reduction(| : bad)
-        for (int64_t i = 0; i < n; ++i)
-            if (indptr[i + 1] < indptr[i]) bad |= 1;
-        if (bad) return DSFACTO_ERR_INVALID_CSR;
-        if ((rc = dev_alloc(h, &pending.indptr, (size_t)n + 1)) || (rc = dev_alloc(h, &pending.idx, (size_t)nnz)) ||
-            (rc = dev_alloc(h, &pending.val, (size_t)nnz)) || (rc = dev_alloc(h, &pending.y, (size_t)n))) {
+    if (h->nshards == 1) {
+        const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
+        if ((rc = dev_alloc(h, &pending.indptr, (size_t)n + 1)) || (rc = dev_alloc(h, &pending.idx, cnt)) ||
+            (rc = dev_alloc(h, &pending.val, cnt)) || (rc = dev_alloc(h, &pending.y, (size_t)n))) {
             pending.release();
             return rc;
         }
-        cudaError_t e;
-        if ((e = cudaMemcpyAsync(pending.indptr, indptr, sizeof(int64_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, h->stream)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(pending.idx, indices, sizeof(int32_t) * (size_t)nnz, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(pending.val, values, sizeof(float) * (size_t)nnz, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(pending.y, y, sizeof(float) * (size_t)n, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess) {
-            h->err = std::string("dsfacto_load_csr: ") + cudaGetErrorString(e);
+        cudaError_t e = Courier::get().move(true, {{pending.indptr, const_cast<int64_t *>(indptr), sizeof(int64_t) * ((size_t)n + 1)},
+                                                   {pending.idx, const_cast<int32_t *>(indices), sizeof(int32_t) * (size_t)nnz},
+                                                   {pending.val, const_cast<float *>(values), sizeof(float) * (size_t)nnz},
+                                                   {pending.y, const_cast<float *>(y), sizeof(float) * (size_t)n}}, h->stream);
+        if (e == cudaSuccess) {
+            launch_validate(h, n, nnz, pending.indptr, pending.idx, pending.val, pending.y, &h->report->bad);
+            e = cudaStreamSynchronize(h->stream);
+        }
+        if (e == cudaSuccess) e = cudaGetLastError();
+        const bool bad = h->report->bad != 0;
+        h->report->bad = 0;
+        if (e != cudaSuccess || bad) {
             cudaStreamSynchronize(h->stream);
             pending.release();
+            if (e == cudaSuccess) return DSFACTO_ERR_INVALID_CSR;
+            h->err = std::string("dsfacto_load_csr: ") + cudaGetErrorString(e);
             return DSFACTO_ERR_CUDA;
         }
-    }
-    rc = validate_csr(n, h->d, indptr, indices, values);
+    } else {
+        int bad = 0;
+        rc = validate_csr(n, h->d, indptr, indices, values);
 #pragma omp parallel for schedule(static) reduction(| : bad)
-    for (int64_t i = 0; i < n; ++i)
-        if (!std::isfinite(y[i])) bad |= 1;
-    if (!rc && bad) rc = DSFACTO_ERR_INVALID_CSR;
-    if (rc) {
-        if (overlapped) { cudaStreamSynchronize(h->stream); pending.release(); }
-        return rc;
+        for (int64_t i = 0; i < n; ++i)
+            if (!std::isfinite(y[i])) bad |= 1;
+        if (!rc && bad) rc = DSFACTO_ERR_INVALID_CSR;
+        if (rc) return rc;
     }
 
     // a column shard keeps only the stored entries of its own columns (all rows stay, some become empty)
@@ -1996,7 +2071,7 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
         if (rc) return rc;
         indptr = f_indptr.data(); indices = f_indices.data(); values = f_values.data();
     }
-    return load_validated(h, indptr, indices, values, y, overlapped ? &pending : nullptr);
+    return load_validated(h, indptr, indices, values, y, h->nshards == 1 ? &pending : nullptr);
 }
 
 // Tile lists and launch plan of the tile sweep.  The CSR copies are queued on the stream; on an error the caller
@@ -2075,7 +2150,7 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
                           PendingCsr *pending) {
     const int64_t n = h->n, nnz = indptr[n];
     int rc = DSFACTO_OK;
-    if (!pending) CU_TRY(h, cudaStreamSynchronize(h->stream));   // (the copies of a pending CSR are still under way)
+    CU_TRY(h, cudaStreamSynchronize(h->stream));
     free_data(h);
     h->nnz = nnz;
     // the recompute pass also takes the squared norms of the parameters: CTAs for both
@@ -2301,12 +2376,23 @@ int dsfacto_get_stats(dsfacto_t *h, double *mean_loss, double *sum_G) {
 int dsfacto_get_params(dsfacto_t *h, float *w0, float *w, float *V) {
     if (!h) return DSFACTO_ERR_INVALID_ARG;
     if (w0) *w0 = h->w0;
-    if (w) {
-        CU_TRY(h, cudaMemcpyAsync(w, h->d_w, sizeof(float) * (size_t)h->d, cudaMemcpyDeviceToHost, h->stream));
-        CU_TRY(h, cudaStreamSynchronize(h->stream));
+    const size_t w_bytes = w ? sizeof(float) * (size_t)h->d : 0, V_bytes = V ? sizeof(float) * (size_t)h->d * h->K : 0;
+    if (w_bytes + V_bytes == 0) return DSFACTO_OK;
+    if (w_bytes + V_bytes <= h->mail_bytes) {   // a small model: one kernel writes both into the mailbox
+        float *mw = reinterpret_cast<float *>(h->mail), *mV = reinterpret_cast<float *>(h->mail + w_bytes);
+        const int grid = (int)((std::max(w_bytes, V_bytes) / sizeof(float) + kThreads - 1) / kThreads);
+        launch_overlapped(h, copy_out_kernel, grid, kThreads, 0, (const float *)h->d_w, (int64_t)h->d, (const float *)h->d_V, (int)h->K, (int)h->Kp,
+                          w ? mw : nullptr, V ? mV : nullptr, &h->d_state->done, h->report, ++h->report_seq);
+        const int rc = wait_report(h);
+        if (rc) return rc;
+        if (w) std::memcpy(w, mw, w_bytes);
+        if (V) std::memcpy(V, mV, V_bytes);
+        return DSFACTO_OK;
     }
-    if (V) return download_rows(h, V, h->d_V, h->d);
-    return DSFACTO_OK;
+    Fetch pieces;
+    if (w) pieces.add(h->d_w, w, w_bytes);
+    if (V) return download_rows(h, V, h->d_V, h->d, pieces);
+    return fetch(h, pieces);
 }
 
 int dsfacto_set_params(dsfacto_t *h, const float *w0, const float *w, const float *V) {
@@ -2314,7 +2400,7 @@ int dsfacto_set_params(dsfacto_t *h, const float *w0, const float *w, const floa
     if (w0) { if (!std::isfinite(*w0)) return DSFACTO_ERR_INVALID_ARG; h->w0 = *w0; }
     if (w) {
         h->model_version += 1;
-        CU_TRY(h, cudaMemcpyAsync(h->d_w, w, sizeof(float) * (size_t)h->d, cudaMemcpyHostToDevice, h->stream));
+        CU_TRY(h, Courier::get().move(true, {{h->d_w, const_cast<float *>(w), sizeof(float) * (size_t)h->d}}, h->stream));
         CU_TRY(h, cudaStreamSynchronize(h->stream));
     }
     if (V) { int rc = upload_V(h, V); if (rc) return rc; }
@@ -2330,12 +2416,10 @@ int dsfacto_set_params(dsfacto_t *h, const float *w0, const float *w, const floa
 int dsfacto_get_aux(dsfacto_t *h, float *A, float *G) {
     if (!h) return DSFACTO_ERR_INVALID_ARG;
     if (!h->loaded) return DSFACTO_ERR_NO_DATA;
-    if (G) {
-        CU_TRY(h, cudaMemcpyAsync(G, h->d_G, sizeof(float) * (size_t)h->n, cudaMemcpyDeviceToHost, h->stream));
-        CU_TRY(h, cudaStreamSynchronize(h->stream));
-    }
-    if (A) return download_rows(h, A, h->d_A, h->n);
-    return DSFACTO_OK;
+    Fetch pieces;
+    if (G) pieces.add(h->d_G, G, sizeof(float) * (size_t)h->n);
+    if (A) return download_rows(h, A, h->d_A, h->n, pieces);
+    return fetch(h, pieces);
 }
 
 int dsfacto_get_tiles(dsfacto_t *h, int64_t *tile_ptr, int32_t *rows, int32_t *cols, float *vals) {
@@ -2407,62 +2491,110 @@ int dsfacto_bucket_host(int64_t n, int32_t d, int32_t p, const int64_t *indptr, 
     return DSFACTO_OK;
 }
 
-// Scores m rows (training rows when indptr is NULL, otherwise a caller CSR copied to the device for
-// the call).  mode kScore: scores_out fp32[m].  mode kEvaluate: labels y (host) and sums2 = {sum of
-// losses, sum of squared errors or number of correct signs}.
+// CSR and label checks of a small batch, on the calling thread
+static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_t *indices, const float *values, const float *y) {
+    const int64_t nnz = indptr[m];
+    for (int64_t i = 0; i < m; ++i) {
+        const int64_t b = indptr[i], e = indptr[i + 1];
+        if (b < 0 || e < b || e > nnz || (y && !std::isfinite(y[i]))) return false;
+        int32_t prev = -1;
+        for (int64_t t = b; t < e; ++t) {
+            if (indices[t] <= prev || indices[t] >= d || !std::isfinite(values[t])) return false;
+            prev = indices[t];
+        }
+    }
+    return true;
+}
+
+// Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
+// fp32[m].  mode kEvaluate: labels y (host) and sums2 = {sum of losses, sum of squared errors or number of correct
+// signs}.
 static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, const int32_t *indices,
                       const float *values, const float *y, float *scores_out, double sums2[2]) {
     RefreshArgs a{};
     a.w0 = h->w0; a.loss = h->loss; a.n = m;
-    int64_t *d_ip = nullptr;
-    int32_t *d_ix = nullptr;
-    float *d_vl = nullptr, *d_f = nullptr, *d_yy = nullptr;
-    double *d_part = nullptr;
+    a.done = &h->d_state->done; a.report = h->report; a.seq = h->report_seq + 1;
+    const int grid = refresh_grid_for(h, m);
+    // everything the call allocates on the device is one block: [indptr | indices | values | y | partial sums | scores]
+    char *block = nullptr;
+    size_t used = 0;
+    auto room = [&](size_t bytes) { const size_t at = used; used += (bytes + 255) & ~(size_t)255; return at; };
+    const size_t part_at = room(mode == kEvaluate ? 4 * sizeof(double) * (size_t)grid : 0);
     int rc = DSFACTO_OK;
-    auto cleanup = [&]() { dev_free(d_ip); dev_free(d_ix); dev_free(d_vl); dev_free(d_f); dev_free(d_yy); dev_free(d_part); };
+    bool mailed_out = false;   // the scores come through the mailbox
+    auto cleanup = [&]() { dev_free(block); };
     if (!indptr) {
         if (!h->loaded) return DSFACTO_ERR_NO_DATA;
         if (m != h->n) return DSFACTO_ERR_INVALID_ARG;
         a.indptr = h->d_indptr; a.idx = h->d_idx; a.val = h->d_val;
+        const size_t f_at = room(sizeof(float) * (size_t)m);
+        if ((rc = dev_alloc(h, &block, used))) return rc;
+        a.f_out = reinterpret_cast<float *>(block + f_at);
         model_view(h, a, true);
     } else {
         if (indptr[0] != 0 || indptr[m] < 0) return DSFACTO_ERR_INVALID_CSR;
         const int64_t nnz = indptr[m];
         if (nnz > 0 && (!indices || !values)) return DSFACTO_ERR_INVALID_ARG;
-        if ((rc = validate_csr(m, h->d, indptr, indices, values))) return rc;
-        const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
-        if ((rc = dev_alloc(h, &d_ip, (size_t)m + 1)) || (rc = dev_alloc(h, &d_ix, cnt)) || (rc = dev_alloc(h, &d_vl, cnt))) {
-            cleanup();
-            return rc;
+        const size_t ip_b = sizeof(int64_t) * ((size_t)m + 1), e_b = 4 * (size_t)nnz, y_b = sizeof(float) * (size_t)m;
+        const size_t mail = ip_b + 2 * e_b + y_b;   // (labels in, or scores out)
+        if (mail <= h->mail_bytes) {
+            // A request: the kernel reads the rows from the mailbox across the link and leaves the scores there, which
+            // takes less time than copies in and out before and behind it (32 rows: 60 us -> 20 us per call).
+            if (!sound_rows(m, h->d, indptr, indices, values, y)) return DSFACTO_ERR_INVALID_CSR;
+            char *p = h->mail;
+            std::memcpy(p, indptr, ip_b);
+            if (nnz > 0) { std::memcpy(p + ip_b, indices, e_b); std::memcpy(p + ip_b + e_b, values, e_b); }
+            a.indptr = reinterpret_cast<int64_t *>(p);
+            a.idx = reinterpret_cast<int32_t *>(p + ip_b);
+            a.val = reinterpret_cast<float *>(p + ip_b + e_b);
+            float *last = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
+            if (mode == kScore) { a.f_out = last; mailed_out = true; }
+            else { std::memcpy(last, y, y_b); a.y = last; }
+            if (used > 0 && (rc = dev_alloc(h, &block, used))) return rc;
+        } else {
+            const size_t ip_at = room(ip_b), ix_at = room(e_b), vl_at = room(e_b), yf_at = room(y_b);
+            if ((rc = dev_alloc(h, &block, used))) return rc;
+            float *yf = reinterpret_cast<float *>(block + yf_at);
+            a.indptr = reinterpret_cast<int64_t *>(block + ip_at);
+            a.idx = reinterpret_cast<int32_t *>(block + ix_at);
+            a.val = reinterpret_cast<float *>(block + vl_at);
+            if (mode == kScore) a.f_out = yf;
+            else a.y = yf;
+            const cudaError_t e = Courier::get().move(true, {{block + ip_at, const_cast<int64_t *>(indptr), ip_b},
+                                                             {block + ix_at, const_cast<int32_t *>(indices), e_b},
+                                                             {block + vl_at, const_cast<float *>(values), e_b},
+                                                             {yf, const_cast<float *>(y), y ? y_b : 0}}, h->stream);
+            if (e != cudaSuccess) {
+                cudaStreamSynchronize(h->stream);
+                cleanup();
+                h->err = cudaGetErrorString(e);
+                return DSFACTO_ERR_CUDA;
+            }
+            // checked where they are now; the scoring kernel leaves at once if they are not sound
+            a.bad = &h->d_state->bad;
+            launch_validate(h, m, nnz, a.indptr, a.idx, a.val, a.y, a.bad);
         }
-        cudaMemcpyAsync(d_ip, indptr, sizeof(int64_t) * ((size_t)m + 1), cudaMemcpyHostToDevice, h->stream);
-        if (nnz > 0) {
-            cudaMemcpyAsync(d_ix, indices, sizeof(int32_t) * (size_t)nnz, cudaMemcpyHostToDevice, h->stream);
-            cudaMemcpyAsync(d_vl, values, sizeof(float) * (size_t)nnz, cudaMemcpyHostToDevice, h->stream);
-        }
-        a.indptr = d_ip; a.idx = d_ix; a.val = d_vl;
         model_view(h, a, false);
     }
-    const int grid = refresh_grid_for(h, m);
-    cudaError_t e = cudaSuccess;
-    if (mode == kScore) {
-        if ((rc = dev_alloc(h, &d_f, (size_t)m))) { cleanup(); return rc; }
-        a.f_out = d_f;
-        DSF_DISPATCH_REFRESH(h, h, a, kScore, grid);
-        e = cudaMemcpyAsync(scores_out, d_f, sizeof(float) * (size_t)m, cudaMemcpyDeviceToHost, h->stream);
-    } else {
-        if ((rc = dev_alloc(h, &d_yy, (size_t)m)) || (rc = dev_alloc(h, &d_part, 4 * (size_t)grid))) { cleanup(); return rc; }
-        cudaMemcpyAsync(d_yy, y, sizeof(float) * (size_t)m, cudaMemcpyHostToDevice, h->stream);
-        a.y = d_yy; a.partials = d_part;
-        a.done = &h->d_state->done; a.report = h->report; a.seq = ++h->report_seq;
-        DSF_DISPATCH_REFRESH(h, h, a, kEvaluate, grid);
+    a.partials = reinterpret_cast<double *>(block + part_at);
+    ++h->report_seq;
+    if (mode == kScore) DSF_DISPATCH_REFRESH(h, h, a, kScore, grid);
+    else DSF_DISPATCH_REFRESH(h, h, a, kEvaluate, grid);
+    rc = wait_report(h);
+    if (!rc && h->report->bad) rc = DSFACTO_ERR_INVALID_CSR;
+    if (!rc && mode == kScore) {
+        if (mailed_out) std::memcpy(scores_out, a.f_out, sizeof(float) * (size_t)m);
+        else {
+            const Piece out = {a.f_out, scores_out, sizeof(float) * (size_t)m};
+            const cudaError_t e = Courier::get().move(false, &out, 1, h->stream);
+            if (e != cudaSuccess) { h->err = cudaGetErrorString(e); rc = DSFACTO_ERR_CUDA; }
+        }
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    if (rc == DSFACTO_ERR_CUDA) cudaStreamSynchronize(h->stream);
+    h->report->bad = 0;
+    if (!rc && mode == kEvaluate) { sums2[0] = h->report->loss; sums2[1] = h->report->g; }
     cleanup();
-    if (e != cudaSuccess) { h->err = cudaGetErrorString(e); return DSFACTO_ERR_CUDA; }
-    if (mode == kEvaluate) { sums2[0] = h->report->loss; sums2[1] = h->report->g; }
-    return DSFACTO_OK;
+    return rc;
 }
 
 int dsfacto_predict(dsfacto_t *h, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values,
@@ -2475,11 +2607,6 @@ int dsfacto_predict(dsfacto_t *h, int64_t m, const int64_t *indptr, const int32_
 int dsfacto_evaluate(dsfacto_t *h, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values,
                      const float *y, double *mean_loss, double *metric) {
     if (!h || !indptr || !y || m < 1) return DSFACTO_ERR_INVALID_ARG;
-    int bad = 0;
-#pragma omp parallel for schedule(static) reduction(| : bad)
-    for (int64_t i = 0; i < m; ++i)
-        if (!std::isfinite(y[i])) bad |= 1;
-    if (bad) return DSFACTO_ERR_INVALID_CSR;
     double s[2] = {0.0, 0.0};
     const int rc = score_rows(h, kEvaluate, m, indptr, indices, values, y, nullptr, s);
     if (rc) return rc;
@@ -2534,6 +2661,11 @@ int dsfacto_last_load(dsfacto_t *h, int64_t info[3]) {
     if (!h->loaded) return DSFACTO_ERR_NO_DATA;
     for (int k = 0; k < 3; ++k) info[k] = h->load_info[k];
     return DSFACTO_OK;
+}
+
+void dsfacto_trim(void) {
+    DevicePool::get().trim();
+    Mailboxes::get().trim();
 }
 
 int dsfacto_launch_count(dsfacto_t *h, int64_t *out) {

@@ -47,6 +47,7 @@ struct RefreshArgs {
     EpochReport *report;   // mapped host memory: the sums and, behind them, seq (NULL: not the end of an epoch)
     unsigned long long seq;
     int first;             // kTrain: the first segment of an epoch (its times are set, not added)
+    int *bad;              // caller rows that were checked on the device: no row is read if it is set (NULL: sound rows)
 };
 
 // Sums of the whole launch in a fixed order: thread 0 of the last CTA to get here returns true and holds them.
@@ -69,6 +70,15 @@ __device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, 
         for (int c = 0; c < 4; ++c) s[c] += __ldcg(partials + 4 * (size_t)b + c);
     block_sum4(s);
     return threadIdx.x == 0;
+}
+
+// The last thread of a kernel whose CTAs have all written their results (to memory of the host as well): thread 0
+// of the last CTA to get here.
+__device__ __forceinline__ bool last_thread(unsigned *done) {
+    __syncthreads();
+    if (threadIdx.x != 0) return false;
+    __threadfence_system();
+    return atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
 }
 
 // Rows of 128 bytes and more keep 8 float4s per lane in flight and would take 88 to 100 registers:
@@ -99,7 +109,14 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
     int nlen = 0;
     int32_t jn = 0;
     float xn = 0.f;
-    if (row_first < a.n) {
+    int64_t n = a.n;
+    int bad = 0;
+    if ((MODE == kScore || MODE == kEvaluate) && a.bad) {
+        wait_for_previous_kernel();
+        bad = *(volatile int *)a.bad;
+        if (bad) n = 0;
+    }
+    if (row_first < n) {
         nbeg = __ldg(a.indptr + row_first);
         nlen = (int)(__ldg(a.indptr + row_first + 1) - nbeg);
         if (l < nlen) { jn = __ldg(a.idx + nbeg + l); xn = __ldg(a.val + nbeg + l); }
@@ -109,11 +126,11 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
     wait_for_previous_kernel();
     if (TRAIN && a.st && blockIdx.x == 0 && threadIdx.x == 0) a.st->t1 = device_ns();
     const float w0 = TRAIN && a.st ? a.st->w0 : a.w0;
-    for (int64_t row = row_first; row < a.n; row += row_step) {
+    for (int64_t row = row_first; row < n; row += row_step) {
         const int64_t beg = nbeg;
         const int len = nlen;
         nlen = 0;
-        if (row + row_step < a.n) {
+        if (row + row_step < n) {
             nbeg = __ldg(a.indptr + row + row_step);
             nlen = (int)(__ldg(a.indptr + row + row_step + 1) - nbeg);
         }
@@ -222,6 +239,13 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             }
         }
     }
+    if (MODE == kScore && a.report && last_thread(a.done)) {
+        volatile EpochReport *r = a.report;
+        r->bad = bad;
+        if (a.bad) *a.bad = 0;
+        __threadfence_system();
+        r->seq = a.seq;
+    }
     if (MODE == kTrain || MODE == kEvaluate) {
         double s[4] = {l == 0 ? sums[0][g] : 0.0, l == 0 ? sums[1][g] : 0.0, 0.0, 0.0};
         if (TRAIN) {
@@ -244,6 +268,10 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             if (a.report) {
                 volatile EpochReport *r = a.report;
                 r->loss = s[0]; r->g = s[1]; r->w2 = s[2]; r->v2 = s[3];
+                if (MODE == kEvaluate) {
+                    r->bad = bad;
+                    if (a.bad) *a.bad = 0;
+                }
             }
             if (TRAIN && a.st) {
                 EpochState &st = *a.st;
@@ -263,6 +291,19 @@ __global__ void __launch_bounds__(kThreads, (LG >= 8 ? 3 : 4)) refresh_kernel(co
             }
         }
     }
+}
+
+// Parameters of a small model to mapped host memory, with a report behind them.
+__global__ void __launch_bounds__(kThreads) copy_out_kernel(const float *w, int64_t d, const float *V, int K, int Kp, float *out_w, float *out_V,
+                                                            unsigned *done, EpochReport *report, unsigned long long seq) {
+    const int64_t stride = (int64_t)gridDim.x * kThreads, first = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    let_next_kernel_start();
+    wait_for_previous_kernel();
+    if (out_w)
+        for (int64_t i = first; i < d; i += stride) out_w[i] = w[i];
+    if (out_V)
+        for (int64_t i = first; i < d * K; i += stride) out_V[i] = V[i / K * Kp + i % K];
+    if (last_thread(done)) ((volatile EpochReport *)report)->seq = seq;
 }
 
 // ------------------------------------------------------------------------------------------

@@ -33,6 +33,7 @@ struct EpochState {
     float w0;
     unsigned done;                 // CTAs of the recompute pass that have delivered their sums
     int err[3];                    // bounds-checked build: code and value of the first failed check
+    int bad;                       // caller data on the device has failed a check (zero between calls)
     unsigned long long t0, t1;     // device clock: start of the update loop, start of the recompute pass
     unsigned long long ns[2];      // update loop, recompute pass: sums over the segments of an epoch
 };
@@ -41,6 +42,7 @@ struct EpochReport {
     double loss, g, w2, v2;
     float w0;
     int err[3];
+    int bad;
     unsigned long long ns[2];
     unsigned long long seq;
 };

@@ -49,6 +49,7 @@ SIGNATURES = {
     "dsfacto_bucket_host_shard": (ctypes.c_int, [_c_i64, _c_i32, _c_i32, _c_i32, _c_i32, _vp, _vp, _vp,
                                                  ctypes.POINTER(_c_i64), _vp, _vp, _vp, _vp]),
     "dsfacto_launch_count": (ctypes.c_int, [_vp, ctypes.POINTER(_c_i64)]),
+    "dsfacto_trim": (None, []),
     "dsfacto_last_load": (ctypes.c_int, [_vp, ctypes.POINTER(_c_i64)]),
     "dsfacto_last_error": (ctypes.c_char_p, [_vp]),
     "dsfacto_strerror": (ctypes.c_char_p, [ctypes.c_int]),
@@ -154,6 +155,11 @@ def dsfacto_get_params(h, w0, w, V):
 
 def dsfacto_set_params(h, w0, w, V):
     return lib().dsfacto_set_params(h, _ptr(w0), _ptr(w), _ptr(V))
+
+
+def dsfacto_trim():
+    """Gives the device and page-locked memory back that the library keeps for its next calls."""
+    lib().dsfacto_trim()
 
 
 def dsfacto_destroy(h):
