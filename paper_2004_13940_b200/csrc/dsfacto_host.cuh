@@ -23,7 +23,7 @@ namespace dsf {
 // Device memory.  cudaMalloc and cudaFree cost 0.4 and 0.3 ms whatever the size, and a load makes some thirty of
 // each: a load of 2.6 M entries spent nine tenths of its time there.  Freed blocks are kept per device, up to a
 // 64th of its memory, and handed out again for requests of about their size; they go back to the driver when an
-// allocation fails, when the bound is reached (the block at hand is freed at once), and with trim().
+// allocation fails, when the bound is reached (those that have been idle longest), and with trim().
 // A block is freed only after the work that used it has finished (callers synchronise their stream first), so it may
 // be handed to any thread and stream.
 // ------------------------------------------------------------------------------------------
@@ -42,11 +42,11 @@ public:
         const size_t size = (std::max<size_t>(bytes, 1) + unit - 1) / unit * unit;
         {
             std::lock_guard<std::mutex> lock(mu_);
-            std::multimap<size_t, void *> &idle = idle_[dev];
+            std::multimap<size_t, Idle> &idle = idle_[dev];
             const auto it = idle.lower_bound(size);
             if (it != idle.end() && it->first <= size + size / 4) {
-                *out = it->second;
-                live_[it->second] = {it->first, dev};
+                *out = it->second.ptr;
+                live_[it->second.ptr] = {it->first, dev};
                 idle_bytes_[dev] -= it->first;
                 idle.erase(it);
                 return cudaSuccess;
@@ -65,20 +65,29 @@ public:
     }
     void free(void *ptr) {
         if (!ptr) return;
+        std::vector<void *> go;   // what has been idle longest makes room
         {
             std::lock_guard<std::mutex> lock(mu_);
             const auto it = live_.find(ptr);
-            if (it != live_.end()) {
-                const Block b = it->second;
-                live_.erase(it);
-                if (idle_bytes_[b.dev] + b.bytes <= bound(b.dev)) {
-                    idle_[b.dev].emplace(b.bytes, ptr);
-                    idle_bytes_[b.dev] += b.bytes;
-                    return;
+            const Block b = it != live_.end() ? it->second : Block{~(size_t)0, 0};
+            if (it != live_.end()) live_.erase(it);
+            if (b.bytes > bound(b.dev)) {
+                go.push_back(ptr);
+            } else {
+                std::multimap<size_t, Idle> &idle = idle_[b.dev];
+                idle.emplace(b.bytes, Idle{ptr, ++clock_});
+                idle_bytes_[b.dev] += b.bytes;
+                while (idle_bytes_[b.dev] > bound(b.dev)) {
+                    auto old = idle.begin();
+                    for (auto q = idle.begin(); q != idle.end(); ++q)
+                        if (q->second.since < old->second.since) old = q;
+                    go.push_back(old->second.ptr);
+                    idle_bytes_[b.dev] -= old->first;
+                    idle.erase(old);
                 }
             }
         }
-        cudaFree(ptr);
+        for (void *p : go) cudaFree(p);
     }
     // idle bytes on the current device
     size_t idle_bytes() {
@@ -92,7 +101,7 @@ public:
         {
             std::lock_guard<std::mutex> lock(mu_);
             for (auto &d : idle_) {
-                for (auto &b : d.second) go.push_back(b.second);
+                for (auto &b : d.second) go.push_back(b.second.ptr);
                 d.second.clear();
                 idle_bytes_[d.first] = 0;
             }
@@ -102,6 +111,7 @@ public:
 
 private:
     struct Block { size_t bytes; int dev; };
+    struct Idle { void *ptr; uint64_t since; };
     size_t bound(int dev) {   // (mu_ is held)
         auto it = bound_.find(dev);
         if (it == bound_.end()) {
@@ -112,16 +122,19 @@ private:
         return it->second;
     }
     std::mutex mu_;
-    std::map<int, std::multimap<size_t, void *>> idle_;
+    std::map<int, std::multimap<size_t, Idle>> idle_;
+    uint64_t clock_ = 0;
     std::map<int, size_t> idle_bytes_, bound_;
     std::unordered_map<void *, Block> live_;
 };
 
 // ------------------------------------------------------------------------------------------
 // Transfers.  A copy between pageable memory and the device goes through the driver's staging buffer in one
-// thread: 11 GB/s, and less into memory that has not been touched yet.  Large copies are therefore cut into regions
-// of 2 MB that the calling thread and a few helpers take one after another, each through two page-locked slots of
-// its own: 30 to 50 GB/s.  The helpers sleep between transfers; nobody waits for a helper that has not woken up yet,
+// thread: 11 GB/s, and 5 GB/s into memory that has not been touched yet.  Large copies are therefore cut into regions
+// that the calling thread and a few helpers take one after another, each through two page-locked slots of its own.
+// 328 MB to the device, 4 threads: 43 GB/s (8 threads: 40; slots of 512 / 256 / 128 KB instead of 1 MB: 32 / 22 /
+// 16, every copy costs the driver some 10 us); 67 MB into fresh memory, 8 threads: 34 GB/s (4 threads: 19, page
+// faults).  The helpers sleep between transfers; nobody waits for a helper that has not woken up yet,
 // so a busy machine costs bandwidth, not a stall.  One transfer at a time per process.
 // ------------------------------------------------------------------------------------------
 struct Piece {            // one array of a transfer
@@ -135,9 +148,11 @@ public:
         static Courier *c = new Courier;   // (never destroyed: its helpers sleep until the process ends)
         return *c;
     }
-    static constexpr size_t kSlot = (size_t)512 << 10, kRegion = (size_t)2 << 20;
+    static constexpr size_t kSlot = (size_t)1 << 20, kRegion = (size_t)2 << 20;   // of what one copy moves; of what a thread takes
     static constexpr int kMostPieces = 8;
-    static constexpr size_t kWorth = (size_t)1 << 20;   // smaller arrays go through the driver
+    // Smaller arrays go through the driver: 1 MB to the device takes 0.08 ms either way, 2.7 MB back 0.20 ms through
+    // the driver and 0.28 ms with helpers that have to wake up first.
+    static constexpr size_t kWorth = (size_t)1 << 20, kWorthBack = (size_t)6 << 20;
     // Copies the pieces on the stream; on return host memory has been read (to the device) or written (from it).
     // To the device, the last copies may still be under way on the stream.
     cudaError_t move(bool to_device, std::initializer_list<Piece> pieces, cudaStream_t st) { return move(to_device, pieces.begin(), (int)pieces.size(), st); }
@@ -148,7 +163,7 @@ public:
         for (int q = 0; q < count; ++q) {
             const Piece &p = pieces[q];
             if (p.bytes == 0) continue;
-            bool direct = p.bytes < kWorth;
+            bool direct = p.bytes < (to_device ? kWorth : kWorthBack);
             if (!direct) {   // page-locked caller memory needs no detour
                 cudaPointerAttributes at{};
                 if (cudaPointerGetAttributes(&at, p.host) != cudaSuccess) cudaGetLastError();
@@ -175,7 +190,7 @@ private:
         cudaError_t e;
         try {
             size_t most = 0;
-            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kRegion + 2;
+            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kSlot + 2;
             regions_.reserve(most);
             e = prepare();
         } catch (const std::bad_alloc &) { e = cudaErrorMemoryAllocation; }
@@ -193,8 +208,9 @@ private:
         for (int q = 0; q < count; ++q) {
             const Piece &p = pieces[q];
             char *d = static_cast<char *>(p.dev), *h = static_cast<char *>(p.host), *end = h + p.bytes;
-            while (h < end) {   // regions end on 2 MB boundaries of host memory: a huge page is touched by one thread
-                char *stop = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(h) / kRegion + 1) * kRegion);
+            while (h < end) {   // on the way back regions end on 2 MB boundaries: a huge page is touched by one thread
+                const size_t unit = to_device ? kSlot : kRegion;
+                char *stop = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(h) / unit + 1) * unit);
                 const size_t n = (size_t)(std::min(stop, end) - h);
                 regions_.push_back({d, h, n});
                 d += n;
@@ -291,6 +307,7 @@ private:
         for (;;) {
             wake_.wait(lock, [&] { return open_ && job_ != seen; });
             seen = job_;
+            if (to_device_ && k >= 4) continue;
             ++active_;
             lock.unlock();
             if (dev != device_) { dev = device_; cudaSetDevice(dev); }
