@@ -469,13 +469,12 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
         }                                                          \
     } while (0)
 
+// CTAs of the recompute kernel: as many as stay resident (each lane group then fetches its next row while it works
+// on the present one), fewer for few rows.
 int refresh_grid_for(const dsfacto *h, int64_t rows) {
     const int G = kThreads / h->LGr;
-    int64_t want = (rows + G - 1) / G;
-    const int64_t cap = (int64_t)h->sm_count * 16;
-    if (want > cap) want = cap;
-    if (want < 1) want = 1;
-    return (int)want;
+    const int64_t want = (rows + G - 1) / G, cap = (int64_t)h->sm_count * (h->LGr >= 8 ? 3 : 4);
+    return (int)std::max<int64_t>(1, std::min(want, cap));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2155,7 +2154,7 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
     h->nnz = nnz;
     // the recompute pass also takes the squared norms of the parameters: CTAs for both
     h->refresh_grid = std::max(refresh_grid_for(h, n),
-                               (int)std::min<int64_t>(((int64_t)h->d * (h->Kp / 4) + 8 * kThreads - 1) / (8 * kThreads), (int64_t)h->sm_count * 8));
+                               (int)std::min<int64_t>(((int64_t)h->d * (h->Kp / 4) + 8 * kThreads - 1) / (8 * kThreads), (int64_t)h->sm_count * (h->LGr >= 8 ? 3 : 4)));
     const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
     cudaStream_t st = h->stream;
     if (pending) {
