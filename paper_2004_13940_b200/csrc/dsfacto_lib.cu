@@ -432,10 +432,11 @@ void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threa
 }
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
-    if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, 0, a);
-    else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, 0, a);
-    else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, 0, a);
-    else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, 0, a);
+    const size_t smem = sizeof(float2) * (size_t)a.hot;
+    if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, smem, a);
+    else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, smem, a);
+    else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, smem, a);
+    else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, smem, a);
 }
 
 #define DSF_DISPATCH(h, FN, ...)                                   \
@@ -461,7 +462,7 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
         case 21: launch_refresh<2, 1>(__VA_ARGS__); break;         \
         case 41: launch_refresh<4, 1>(__VA_ARGS__); break;         \
         case 81: launch_refresh<8, 1>(__VA_ARGS__); break;         \
-        case 161: launch_refresh<16, 1>(__VA_ARGS__); break;       \
+        case 82: launch_refresh<8, 2>(__VA_ARGS__); break;         \
         case 84: launch_refresh<8, 4>(__VA_ARGS__); break;         \
         case 86: launch_refresh<8, 6>(__VA_ARGS__); break;         \
         case 88: launch_refresh<8, 8>(__VA_ARGS__); break;         \
@@ -473,7 +474,7 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
 // on the present one), fewer for few rows.
 int refresh_grid_for(const dsfacto *h, int64_t rows) {
     const int G = kThreads / h->LGr;
-    const int64_t want = (rows + G - 1) / G, cap = (int64_t)h->sm_count * (h->LGr >= 8 ? 3 : 4);
+    const int64_t want = (rows + G - 1) / G, cap = (int64_t)h->sm_count * (h->LGr < 8 ? 4 : h->NVr >= 4 ? 2 : 3);
     return (int)std::max<int64_t>(1, std::min(want, cap));
 }
 
@@ -818,6 +819,8 @@ void launch_finish(dsfacto *h, int grid) {
                                                             h->w0, h->loss);
 }
 
+constexpr int kHotPairs = 2048;   // pairs of the most frequent columns a CTA of the recompute pass keeps (16 KB)
+
 // V and the pairs (w_j, s_j) as the recompute pass reads them: by slot for the training rows when the load
 // renumbered the columns of the device CSR, by column index otherwise (and always for rows a caller passes).
 // Rebuilt only when the parameters changed since the last time: one pass over V (4 d Kp bytes read, twice
@@ -840,6 +843,7 @@ void model_view(dsfacto *h, RefreshArgs &a, bool training_rows) {
     }
     a.V = by_slot ? h->d_Vs : h->d_V;
     a.pair = by_slot ? h->d_pair_s : h->d_pair;
+    a.hot = by_slot ? std::min(h->d, kHotPairs) : 0;
 }
 
 // Renumbers the columns of the device CSR by frequency (see the kernels).  Decided per load: it pays when
@@ -1528,10 +1532,10 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
     h->LG = LG;
     h->NV = (q4 + LG - 1) / LG;
     h->Kp = 4 * h->LG * h->NV;
-    // The recompute kernel gives a row of 512 bytes and more to 8 lanes (four rows per warp instruction):
-    // K = 128 per pass on 400 M entries, 22.3 ms as 32 x 1, 19.8 ms as 16 x 2, 17.5 ms as 8 x 4 float4.
+    // The recompute kernel gives a row of 128 bytes and more to 8 lanes, a 128-byte line per load and row: four rows
+    // share the instructions that hand out columns and values.
     h->LGr = h->LG; h->NVr = h->NV;
-    if (h->Kp >= 128) { h->LGr = 8; h->NVr = h->Kp / 32; }
+    if (h->Kp >= 64) { h->LGr = 8; h->NVr = h->Kp / 32; }
 
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2154,7 +2158,7 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
     h->nnz = nnz;
     // the recompute pass also takes the squared norms of the parameters: CTAs for both
     h->refresh_grid = std::max(refresh_grid_for(h, n),
-                               (int)std::min<int64_t>(((int64_t)h->d * (h->Kp / 4) + 8 * kThreads - 1) / (8 * kThreads), (int64_t)h->sm_count * (h->LGr >= 8 ? 3 : 4)));
+                               (int)std::min<int64_t>(((int64_t)h->d * (h->Kp / 4) + 8 * kThreads - 1) / (8 * kThreads), (int64_t)h->sm_count * 2));
     const size_t cnt = (size_t)std::max<int64_t>(nnz, 1);
     cudaStream_t st = h->stream;
     if (pending) {

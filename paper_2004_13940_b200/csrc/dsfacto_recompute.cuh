@@ -1,0 +1,340 @@
+// The recompute pass of the DS-FACTO epoch for sm_100a: auxiliaries, scores, multipliers, and the fp64 sums behind
+// the objective.
+#pragma once
+#include <type_traits>
+
+#include "dsfacto_common.cuh"
+#include "dsfacto_epoch.cuh"
+
+namespace dsf {
+
+// ------------------------------------------------------------------------------------------
+// Recompute pass (eq. (compute_a_jk), eq. (fm_model2), multiplier G).
+//   a_ik = sum_j v_jk x_ij ; lin_i = sum_j w_j x_ij ; q_i = sum_j sum_k (v_jk x_ij)^2
+//   f_i = w0 + lin_i + 1/2 (sum_k a_ik^2 - q_i)
+// q_i is taken as sum_j x_ij^2 s_j with s_j = sum_k v_jk^2, which is the same sum regrouped: s_j is computed
+// once per column after the parameters changed (model_view_kernel) and sits next to w_j, so the lane that
+// owns an entry gets both with one 8-byte load and the K-wide part of an entry is K multiply-adds.
+// MODE kScore: writes f only.  kTrain: writes A, G and per-CTA fp64 partial sums {sum l_i, sum G_i}.
+// kEvaluate (held-out rows with labels; the quantities of the convergence figures of Section 5):
+// writes nothing per row, per-CTA fp64 partial sums {sum l_i, sum t_i} with t_i = (f_i - y_i)^2 for
+// the squared loss (RMSE) and t_i = [y_i f_i > 0] for the logistic loss (accuracy).
+// kPartial (a handle that owns only a range of columns, Section 4.2's column blocks spread over
+// workers): the sums run over the handle's own columns, so they are partial; writes a_ik, lin_i and
+// q_i per row and stops there.  The partial sums of all shards are added outside and finish_kernel
+// turns the totals into f_i, l_i and G_i.
+// ------------------------------------------------------------------------------------------
+// kScoreSums (the entry point that allocates nothing): f and the sums {sum l_i, sum G_i}.
+enum { kScore = 0, kTrain = 1, kEvaluate = 2, kPartial = 3, kScoreSums = 4 };
+struct RefreshArgs {
+    int64_t n;
+    const int64_t *indptr;
+    const int32_t *idx;
+    const float *val;
+    const float *y;
+    const float2 *pair;  // per column (w_j, s_j = sum_k v_jk^2)
+    int hot;             // pairs of the first columns that are worth keeping in shared memory
+    const float *w;      // RAW: w instead of the pairs
+    double *sums_out;    // kScoreSums
+    const float *V;
+    float *A;
+    float *G;
+    float *f_out;
+    float *lin_out, *q_out;  // kPartial: per-row partial sums
+    double *partials;  // 4 per CTA: the two sums of the mode, sum w_j^2, sum v_jk^2
+    float w0;
+    int loss;
+    // the squared norms of eq. (fm_obj), shared out over the CTAs (kTrain; norm_d = 0: left out)
+    const float *norm_w, *norm_V;
+    int64_t norm_d, norm_v4;
+    // end of the pass: the last CTA adds the partial sums up
+    unsigned *done;        // CTAs that have delivered (zero between launches)
+    EpochState *st;        // kTrain: w0 comes from here and the sums go here; NULL: w0 above
+    EpochReport *report;   // mapped host memory: the sums and, behind them, seq (NULL: not the end of an epoch)
+    unsigned long long seq;
+    int first;             // kTrain: the first segment of an epoch (its times are set, not added)
+    int *bad;              // caller rows that were checked on the device: no row is read if it is set (NULL: sound rows)
+};
+
+// Sums of the whole launch in a fixed order: thread 0 of the last CTA to get here returns true and holds them.
+__device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, unsigned *done) {
+    __shared__ bool last;
+    block_sum4(s);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) partials[4 * (size_t)blockIdx.x + c] = s[c];
+        __threadfence();
+        last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[c] = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kThreads)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] += __ldcg(partials + 4 * (size_t)b + c);
+    block_sum4(s);
+    return threadIdx.x == 0;
+}
+
+// The last thread of a kernel whose CTAs have all written their results (to memory of the host as well): thread 0
+// of the last CTA to get here.
+__device__ __forceinline__ bool last_thread(unsigned *done) {
+    __syncthreads();
+    if (threadIdx.x != 0) return false;
+    __threadfence_system();
+    return atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+}
+
+// A warp takes GW = 32 / LG consecutive rows at a time, one per lane group, and stays converged: the loop over the
+// entries runs to the longest of the rows (an earlier form in which every group looped on its own took 9.3 warp
+// instructions per entry of 128-byte rows, most of them for the masks and branches of the divergent groups).  A batch
+// is B = LG * E entries of each row, every lane owns E of them: it takes their (w_j, s_j) and hands column and value
+// to its group; entries are requested two batches ahead.  Factor rows are requested UB entries at a time, always one
+// step ahead of the multiply-adds (two sets of registers).  Behind the end of a row its last entry is repeated with
+// x = 0.
+// RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
+// The pairs of the first `hot` columns (the most frequent ones, when the columns are numbered that way) sit in shared
+// memory.
+template <int LG, int NV>
+struct RefreshCfg {
+    static constexpr int GW = 32 / LG;
+    static constexpr int E = LG == 1 ? 4 : LG <= 4 ? 2 : 1;                 // entries per lane and batch
+    static constexpr int B = LG * E;
+    static constexpr int UB = NV >= 6 || LG == 1 ? 1 : NV >= 2 || LG == 4 ? 2 : B / 2;            // entries whose rows are requested together
+    static constexpr int S = B / UB;                                        // steps per batch (an even number)
+    static constexpr int CTAS = LG < 8 ? 4 : NV >= 4 ? 2 : 3;               // resident per SM (register cap)
+    static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
+};
+template <int LG, int NV, int MODE, bool RAW = false>
+__global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_kernel(const RefreshArgs a) {
+    typedef RefreshCfg<LG, NV> C;
+    constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, KP4 = LG * NV;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const int g = threadIdx.x / LG, l = threadIdx.x % LG, gw = (threadIdx.x & 31) / LG;
+    const float4 *V4 = reinterpret_cast<const float4 *>(a.V) + l;
+    float4 *A4 = reinterpret_cast<float4 *>(a.A);
+    constexpr bool TRAIN = MODE == kTrain;
+    constexpr bool STORE_A = MODE == kTrain || MODE == kPartial;
+    extern __shared__ __align__(16) float2 hot_pair[];
+    // the fp64 sums of a lane group live in shared memory: only its first lane touches them, once per row
+    __shared__ double sums[2][C::ROWS];
+    if (l == 0) { sums[0][g] = 0.0; sums[1][g] = 0.0; }
+    let_next_kernel_start();
+
+    int64_t n = a.n;
+    int bad = 0;
+    if ((MODE == kScore || MODE == kEvaluate) && a.bad) {
+        wait_for_previous_kernel();
+        bad = *(volatile int *)a.bad;
+        if (bad) n = 0;
+    }
+    const int64_t step = (int64_t)gridDim.x * C::ROWS;
+    int64_t base = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * GW;   // first row of the warp's set
+    int64_t nbeg = 0;      // this group's row of the next set: its first entry and its length (at most d < 2^31)
+    int nlen = 0;
+    int32_t j0[E], j1[E], jn[E];   // entries of the batch at work, of the next one, of the next rows' first one
+    float x0[E], x1[E], xn[E];
+    auto next_pointers = [&](int64_t row) {
+        nlen = 0;
+        if (row < n) {
+            nbeg = __ldg(a.indptr + row);
+            nlen = (int)(__ldg(a.indptr + row + 1) - nbeg);
+        }
+    };
+    auto load_entries = [&](int64_t beg, int t0, int len, int32_t (&j)[E], float (&x)[E]) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int t = t0 + e * LG + l;
+            j[e] = 0; x[e] = 0.f;
+            if (len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
+            if (t < len) x[e] = __ldg(a.val + beg + t);
+        }
+    };
+    next_pointers(base + gw);
+    load_entries(nbeg, 0, nlen, jn, xn);
+    // (the rows do not change during an epoch; the model, which the kernel before this one writes, is read with
+    // plain loads: the read-only path assumes data that nobody writes during the whole life of a kernel)
+    wait_for_previous_kernel();
+    if (TRAIN && a.st && blockIdx.x == 0 && threadIdx.x == 0) a.st->t1 = device_ns();
+    const float w0 = TRAIN && a.st ? a.st->w0 : a.w0;
+    if (!RAW && a.hot > 0) {
+        for (int i = threadIdx.x; i < a.hot; i += kThreads) hot_pair[i] = a.pair[i];
+        __syncthreads();
+    }
+    for (; base < n; base += step) {
+        const int64_t row = base + gw, beg = nbeg;
+        const int len = nlen;
+        next_pointers(row + step);
+        const int longest = __reduce_max_sync(FULL, len);
+        float4 acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        float q = 0.f, lin = 0.f;
+        float4 vv[2][UB][NV];
+        auto load_rows = [&](const int32_t (&j)[E], int u0, float4 (&r)[UB][NV]) {
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int32_t ju = __shfl_sync(FULL, j[(u0 + u) / LG], (u0 + u) % LG, LG);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) r[u][v] = V4[(size_t)ju * KP4 + v * LG];
+            }
+        };
+#pragma unroll
+        for (int e = 0; e < E; ++e) { j0[e] = jn[e]; x0[e] = xn[e]; }
+        load_rows(j0, 0, vv[0]);
+        load_entries(beg, B, len, j1, x1);
+        if (longest <= B) load_entries(nbeg, 0, nlen, jn, xn);
+        for (int t0 = 0; t0 < longest; t0 += B) {
+            int32_t j2[E];
+            float x2[E];
+            if (t0 + 2 * B < longest) load_entries(beg, t0 + 2 * B, len, j2, x2);
+            else if (t0 + B < longest) load_entries(nbeg, 0, nlen, jn, xn);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (t0 + e * LG + l < len) {
+                    if (RAW) {
+                        lin = fmaf(a.w[j0[e]], x0[e], lin);
+                    } else {
+                        const float2 ws = j0[e] < a.hot ? hot_pair[j0[e]] : a.pair[j0[e]];
+                        lin = fmaf(ws.x, x0[e], lin);
+                        q = fmaf(x0[e] * x0[e], ws.y, q);
+                    }
+                }
+#pragma unroll
+            for (int st = 0; st < S; ++st) {
+                if (st + 1 < S) load_rows(j0, (st + 1) * UB, vv[(st + 1) & 1]);
+                else if (t0 + B < longest) load_rows(j1, 0, vv[0]);
+#pragma unroll
+                for (int u = 0; u < UB; ++u) {
+                    const float x = __shfl_sync(FULL, x0[(st * UB + u) / LG], (st * UB + u) % LG, LG);
+                    const float4 (&r)[NV] = vv[st & 1][u];
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        acc[v].x = fmaf(r[v].x, x, acc[v].x); acc[v].y = fmaf(r[v].y, x, acc[v].y);
+                        acc[v].z = fmaf(r[v].z, x, acc[v].z); acc[v].w = fmaf(r[v].w, x, acc[v].w);
+                    }
+                    if (RAW) {
+                        float sv = 0.f;
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) {
+                            sv = fmaf(r[v].x, r[v].x, sv); sv = fmaf(r[v].y, r[v].y, sv);
+                            sv = fmaf(r[v].z, r[v].z, sv); sv = fmaf(r[v].w, r[v].w, sv);
+                        }
+                        q = fmaf(x * x, sv, q);
+                    }
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) { j0[e] = j1[e]; x0[e] = x1[e]; j1[e] = j2[e]; x1[e] = x2[e]; }
+        }
+        if (len == 0) {   // (a row without entries has added nothing but zeros times whatever row 0 holds)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            q = 0.f;
+        }
+        float sq = 0.f;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (STORE_A && row < n) A4[(size_t)row * KP4 + v * LG + l] = acc[v];
+            sq = fmaf(acc[v].x, acc[v].x, sq); sq = fmaf(acc[v].y, acc[v].y, sq);
+            sq = fmaf(acc[v].z, acc[v].z, sq); sq = fmaf(acc[v].w, acc[v].w, sq);
+        }
+        if (MODE == kPartial) {
+#pragma unroll
+            for (int o = LG / 2; o > 0; o >>= 1) {
+                q += __shfl_xor_sync(FULL, q, o);
+                lin += __shfl_xor_sync(FULL, lin, o);
+            }
+            if (l == 0 && row < n) { a.lin_out[row] = lin; a.q_out[row] = q; }
+            continue;
+        }
+        float pair = sq - q;
+#pragma unroll
+        for (int o = LG / 2; o > 0; o >>= 1) {
+            pair += __shfl_xor_sync(FULL, pair, o);
+            lin += __shfl_xor_sync(FULL, lin, o);
+        }
+        if (l == 0 && row < n) {
+            const float f = w0 + lin + 0.5f * pair;
+            if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
+            if (MODE != kScore) {
+                const float yy = a.y[row];
+                float li, gi;
+                if (a.loss == 0) {
+                    gi = f - yy;
+                    li = 0.5f * gi * gi;
+                } else {
+                    const float m = yy * f;
+                    li = fmaxf(-m, 0.f) + log1pf(expf(-fabsf(m)));
+                    gi = -yy / (1.f + expf(m));
+                }
+                sums[0][g] += (double)li;
+                if (TRAIN) a.G[row] = gi;
+                if (TRAIN || MODE == kScoreSums) {
+                    sums[1][g] += (double)gi;
+                } else if (a.loss == 0) {
+                    sums[1][g] += (double)gi * (double)gi;      // (f - y)^2 for the RMSE
+                } else {
+                    sums[1][g] += (yy * f > 0.f) ? 1.0 : 0.0;   // the sign of the score is the predicted class
+                }
+            }
+        }
+    }
+    if (MODE == kScore && a.report && last_thread(a.done)) {
+        volatile EpochReport *r = a.report;
+        r->bad = bad;
+        if (a.bad) *a.bad = 0;
+        __threadfence_system();
+        r->seq = a.seq;
+    }
+    if (MODE == kTrain || MODE == kEvaluate || MODE == kScoreSums) {
+        double s[4] = {l == 0 ? sums[0][g] : 0.0, l == 0 ? sums[1][g] : 0.0, 0.0, 0.0};
+        if (TRAIN) {
+            const int64_t stride = (int64_t)gridDim.x * kThreads;
+            for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.norm_d; i += stride) {
+                const double x = (double)a.norm_w[i];
+                s[2] += x * x;
+            }
+            const float4 *N4 = reinterpret_cast<const float4 *>(a.norm_V);
+            for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < a.norm_v4; i += stride) {
+                const float4 x = N4[i];
+                s[3] += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
+            }
+        }
+        if (last_cta_sum4(s, a.partials, a.done)) {
+            if (TRAIN && a.st) {
+                EpochState &st = *a.st;
+                st.loss = s[0]; st.g = s[1]; st.w2 = s[2]; st.v2 = s[3];
+            }
+            if (MODE == kScoreSums) { a.sums_out[0] = s[0]; a.sums_out[1] = s[1]; }
+            if (a.report) {
+                volatile EpochReport *r = a.report;
+                r->loss = s[0]; r->g = s[1]; r->w2 = s[2]; r->v2 = s[3];
+                if (MODE == kEvaluate) {
+                    r->bad = bad;
+                    if (a.bad) *a.bad = 0;
+                }
+            }
+            if (TRAIN && a.st) {
+                EpochState &st = *a.st;
+                const unsigned long long now = device_ns();
+                const unsigned long long ns0 = st.t1 - st.t0 + (a.first ? 0ull : st.ns[0]), ns1 = now - st.t1 + (a.first ? 0ull : st.ns[1]);
+                st.ns[0] = ns0; st.ns[1] = ns1;
+                if (a.report) {
+                    volatile EpochReport *r = a.report;
+                    r->w0 = st.w0;
+                    r->ns[0] = ns0; r->ns[1] = ns1;
+                    for (int c = 0; c < 3; ++c) r->err[c] = st.err[c];
+                }
+            }
+            if (a.report) {
+                __threadfence_system();
+                ((volatile EpochReport *)a.report)->seq = a.seq;
+            }
+        }
+    }
+}
+
+}  // namespace dsf
