@@ -12,6 +12,7 @@ struct EpochState {
     unsigned done;                 // CTAs of the recompute pass that have delivered their sums
     int err[3];                    // bounds-checked build: code and value of the first failed check
     int bad;                       // caller data on the device has failed a check (zero between calls)
+    unsigned long long epochs;     // reports of epochs (and other recompute passes) so far
     unsigned long long t0, t1;     // device clock: start of the update loop, start of the recompute pass
     unsigned long long ns[2];      // update loop, recompute pass: sums over the segments of an epoch
 };
@@ -22,7 +23,7 @@ struct EpochReport {
     int err[3];
     int bad;
     unsigned long long ns[2];
-    unsigned long long seq;
+    unsigned long long seq, epochs;   // last number reported by scoring and copying kernels; by recompute passes
 };
 
 __device__ __forceinline__ unsigned long long device_ns() {

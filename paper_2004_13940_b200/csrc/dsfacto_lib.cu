@@ -107,7 +107,10 @@ struct dsfacto {
     // scalars of an epoch on the device, and the mapped host memory its last kernel reports to
     EpochState *d_state = nullptr;
     EpochReport *report = nullptr;
-    unsigned long long report_seq = 0;
+    unsigned long long report_seq = 0, epoch_seq = 0;
+    cudaGraphExec_t epoch_graph = nullptr;   // the launches of an epoch (all but the sweep over tiles and shards)
+    int epochs_run = 0;
+    int64_t epoch_launches = 0;
     char *mail = nullptr;          // the rest of that memory: small inputs and results (mail_bytes of it)
     size_t mail_bytes = 0;
     // update loop by column runs (dsfacto_runs.cuh): every load that is bucketed on the device with default settings
@@ -368,7 +371,14 @@ void unpack_runs(const dsfacto *h, const uint2 *ent, const std::vector<int> &run
     }
 }
 
+void drop_epoch_graph(dsfacto *h) {
+    if (h->epoch_graph) cudaGraphExecDestroy(h->epoch_graph);
+    h->epoch_graph = nullptr;
+    h->epochs_run = 0;
+}
+
 void free_data(dsfacto *h) {
+    drop_epoch_graph(h);
     h->rbits = 0;
     dev_free(h->d_A); dev_free(h->d_G); dev_free(h->d_y); dev_free(h->d_val); dev_free(h->d_xw);
     dev_free(h->d_indptr); dev_free(h->d_idx); dev_free(h->d_ent);
@@ -432,8 +442,10 @@ void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threa
 }
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
-    const size_t smem = sizeof(float2) * (size_t)a.hot;
-    if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, smem, a);
+    const size_t smem = a.stage ? (size_t)a.stage_bytes : sizeof(float2) * (size_t)a.hot;
+    if (a.stage && mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate, false, true>, grid, kThreads, smem, a);
+    else if (a.stage) launch_overlapped(h, refresh_kernel<LG, NV, kScore, false, true>, grid, kThreads, smem, a);
+    else if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, smem, a);
     else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, smem, a);
     else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, smem, a);
     else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, smem, a);
@@ -943,17 +955,16 @@ int run_finish(dsfacto *h) {
     return DSFACTO_OK;
 }
 
-// Waits until the kernel that was given report number h->report_seq has delivered it (the last thing that kernel
-// does).  The stream is asked now and then, so that a failed launch ends the wait.
-int wait_report(dsfacto *h) {
-    const volatile EpochReport *r = h->report;
-    for (unsigned spin = 1; r->seq != h->report_seq; ++spin) {
+// Waits until a kernel has delivered its report (the last thing it does): number `want` in `at`.  The stream is
+// asked now and then, so that a failed launch ends the wait.
+int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long long want) {
+    for (unsigned spin = 1; at != want; ++spin) {
         _mm_pause();
         if ((spin & 0x3FFFu) != 0) continue;
         const cudaError_t e = cudaStreamQuery(h->stream);
         if (e == cudaErrorNotReady) continue;
-        if (e == cudaSuccess && r->seq == h->report_seq) break;
-        h->err = std::string("epoch: ") + (e == cudaSuccess ? "the last kernel left no report" : cudaGetErrorString(e));
+        if (e == cudaSuccess && at == want) break;
+        h->err = std::string("report: ") + (e == cudaSuccess ? "the last kernel left none" : cudaGetErrorString(e));
         return DSFACTO_ERR_CUDA;
     }
     CU_TRY(h, cudaGetLastError());
@@ -971,10 +982,14 @@ int run_refresh(dsfacto *h, bool first, bool report) {
     a.partials = h->d_partials; a.loss = h->loss;
     a.norm_w = h->d_w; a.norm_V = h->d_V; a.norm_d = h->d; a.norm_v4 = (int64_t)h->d * (h->Kp / 4);
     a.done = &h->d_state->done; a.st = h->d_state; a.first = first ? 1 : 0;
-    if (report) { a.report = h->report; a.seq = ++h->report_seq; }
+    if (report) a.report = h->report;
     DSF_DISPATCH_REFRESH(h, h, a, kTrain, h->refresh_grid);
-    if (!report) return DSFACTO_OK;
-    const int rc = wait_report(h);
+    return DSFACTO_OK;
+}
+// ... and its sums on the host
+int collect(dsfacto *h) {
+    if (h->nshards > 1) return DSFACTO_OK;
+    const int rc = wait_report(h, h->report->epochs, ++h->epoch_seq);
     if (rc) return rc;
     const EpochReport r = *h->report;
     h->loss_sum = r.loss; h->g_sum = r.g; h->w2 = r.w2; h->v2 = r.v2; h->w0 = r.w0;
@@ -987,7 +1002,8 @@ int refresh_now(dsfacto *h) {
         epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
         h->launches += 1;
     }
-    return run_refresh(h, true, true);
+    const int rc = run_refresh(h, true, true);
+    return rc ? rc : collect(h);
 }
 
 // Results to the caller: small ones through the mailbox, with one wait for all of them.
@@ -2228,6 +2244,8 @@ static int sgd_gave_up(dsfacto *h, const int code[3]) {
     h->err = buf;
     const size_t d = (size_t)h->d;
     cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream);
+    h->epoch_seq = 0;
+    h->report->epochs = 0;
     if (!h->runs) {
         cudaMemsetAsync(h->d_run_count, 0, sizeof(int) * (size_t)std::max<int64_t>(h->long_runs, 1), h->stream);
         cudaMemsetAsync(h->d_sync, 0, sizeof(int) * sync_words(h->p), h->stream);
@@ -2252,6 +2270,59 @@ int dsfacto_epoch(dsfacto_t *h) {
     return epoch_impl(h);
 }
 
+// The launches of an epoch by column runs.  The segments follow one another on the device; the host hears of the last.
+static int enqueue_epoch(dsfacto_t *h) {
+    const int64_t p = h->p;
+    const int64_t every = (h->refresh_every > 0 && h->refresh_every < p) ? h->refresh_every : p;
+    for (int64_t L0 = 0; L0 < p; L0 += every) {
+        const int64_t L1 = std::min(L0 + every, p);
+        run_strata(h, L0 / every, (double)(L1 - L0) / (double)p);
+        const int rc = run_refresh(h, L0 == 0, L1 == p);
+        if (rc) return rc;
+    }
+    return DSFACTO_OK;
+}
+// A handle that goes on training runs the same launches every epoch: from its 17th epoch on they are one graph (three
+// launches cost the host 7 us, one graph of three 3 us; making it takes as long as several epochs of a small data set).
+constexpr int kEpochsBeforeGraph = 16, kMostGraphLaunches = 256;
+static int run_epoch(dsfacto_t *h) {
+    if (h->epoch_graph) {
+        h->model_version += 1;   // (as run_strata)
+        (h->slots ? h->slot_version : h->pair_version) = h->model_version;
+        h->launches += h->epoch_launches;
+        CU_TRY(h, cudaGraphLaunch(h->epoch_graph, h->stream));
+        return DSFACTO_OK;
+    }
+    if (h->epochs_run < kEpochsBeforeGraph) {
+        const int64_t before = h->launches;
+        const int rc = enqueue_epoch(h);
+        h->epoch_launches = h->launches - before;
+        h->epochs_run += h->epoch_launches <= kMostGraphLaunches ? 1 : 0;
+        return rc;
+    }
+    cudaStream_t own = h->stream, cap = nullptr;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess && (e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal)) == cudaSuccess) {
+        const int64_t before = h->launches;
+        h->stream = cap;
+        const int rc = enqueue_epoch(h);
+        h->stream = own;
+        h->launches = before;
+        e = cudaStreamEndCapture(cap, &graph);
+        if (e == cudaSuccess && rc == DSFACTO_OK) e = cudaGraphInstantiate(&h->epoch_graph, graph, 0);
+    }
+    if (graph) cudaGraphDestroy(graph);
+    if (cap) cudaStreamDestroy(cap);
+    if (e != cudaSuccess) {   // no graph, then: the launches one by one
+        cudaGetLastError();
+        h->epoch_graph = nullptr;
+        h->epochs_run = 0;
+        return enqueue_epoch(h);
+    }
+    return run_epoch(h);
+}
+
 static int epoch_impl(dsfacto_t *h) {
     const int64_t p = h->p;
     const int64_t every = (h->refresh_every > 0 && h->refresh_every < p) ? h->refresh_every : p;
@@ -2262,24 +2333,18 @@ static int epoch_impl(dsfacto_t *h) {
         const int64_t L1 = std::min(L0 + every, p);
         // w0 step with the frozen multipliers: the share of the epoch's step that belongs to these rounds
         const double share = (double)(L1 - L0) / (double)p;
-        const bool last = L1 == p;
-        if (h->runs && !shard) {
-            // the segments follow one another on the device; the host hears of the last one
-            run_strata(h, L0 / every, share);
-            rc = run_refresh(h, L0 == 0, last);
-        } else {
-            h->w0 = (float)((double)h->w0 - (double)h->h * share * h->g_sum);
-            if (!shard) {
-                epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
-                h->launches += 1;
-            }
-            if (h->runs) run_strata(h, 0, 0.0);
-            else run_sgd_phase(h, L0, L1);
-            if (shard) CU_TRY(h, cudaEventRecord(h->ev[1], h->stream));
-            rc = run_refresh(h, L0 == 0, true);
+        if (h->runs && !shard) break;   // (below)
+        h->w0 = (float)((double)h->w0 - (double)h->h * share * h->g_sum);
+        if (!shard) {
+            epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
+            h->launches += 1;
         }
-        if (rc) return rc;
+        if (h->runs) run_strata(h, 0, 0.0);
+        else run_sgd_phase(h, L0, L1);
+        if (shard) CU_TRY(h, cudaEventRecord(h->ev[1], h->stream));
+        if ((rc = run_refresh(h, L0 == 0, true)) || (rc = collect(h))) return rc;
     }
+    if (h->runs && !shard && ((rc = run_epoch(h)) || (rc = collect(h)))) return rc;
     if (shard) {
         float t01 = 0, t12 = 0;
         cudaEventElapsedTime(&t01, h->ev[0], h->ev[1]);
@@ -2386,7 +2451,7 @@ int dsfacto_get_params(dsfacto_t *h, float *w0, float *w, float *V) {
         const int grid = (int)((std::max(w_bytes, V_bytes) / sizeof(float) + kThreads - 1) / kThreads);
         launch_overlapped(h, copy_out_kernel, grid, kThreads, 0, (const float *)h->d_w, (int64_t)h->d, (const float *)h->d_V, (int)h->K, (int)h->Kp,
                           w ? mw : nullptr, V ? mV : nullptr, &h->d_state->done, h->report, ++h->report_seq);
-        const int rc = wait_report(h);
+        const int rc = wait_report(h, h->report->seq, h->report_seq);
         if (rc) return rc;
         if (w) std::memcpy(w, mw, w_bytes);
         if (V) std::memcpy(V, mV, V_bytes);
@@ -2512,6 +2577,7 @@ static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_
 // Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
 // fp32[m].  mode kEvaluate: labels y (host) and sums2 = {sum of losses, sum of squared errors or number of correct
 // signs}.
+constexpr size_t kStagedMost = (size_t)24 << 10;   // a batch of up to this size is copied to shared memory by every CTA
 static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, const int32_t *indices,
                       const float *values, const float *y, float *scores_out, double sums2[2]) {
     RefreshArgs a{};
@@ -2553,6 +2619,13 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
             float *last = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
             if (mode == kScore) { a.f_out = last; mailed_out = true; }
             else { std::memcpy(last, y, y_b); a.y = last; }
+            if (mail <= kStagedMost) {
+                a.stage = reinterpret_cast<const uint4 *>(p);
+                a.stage_bytes = (int)((mail + 15) & ~(size_t)15);
+                a.idx = reinterpret_cast<int32_t *>(ip_b);
+                a.val = reinterpret_cast<float *>(ip_b + e_b);
+                a.y = reinterpret_cast<float *>(ip_b + 2 * e_b);
+            }
             if (used > 0 && (rc = dev_alloc(h, &block, used))) return rc;
         } else {
             const size_t ip_at = room(ip_b), ix_at = room(e_b), vl_at = room(e_b), yf_at = room(y_b);
@@ -2583,7 +2656,7 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
     ++h->report_seq;
     if (mode == kScore) DSF_DISPATCH_REFRESH(h, h, a, kScore, grid);
     else DSF_DISPATCH_REFRESH(h, h, a, kEvaluate, grid);
-    rc = wait_report(h);
+    rc = wait_report(h, h->report->seq, h->report_seq);
     if (!rc && h->report->bad) rc = DSFACTO_ERR_INVALID_CSR;
     if (!rc && mode == kScore) {
         if (mailed_out) std::memcpy(scores_out, a.f_out, sizeof(float) * (size_t)m);
@@ -2622,6 +2695,7 @@ int dsfacto_set_eta(dsfacto_t *h, float eta) {
     if (!h || !(eta > 0.f) || !std::isfinite(eta)) return DSFACTO_ERR_INVALID_ARG;
     h->eta = eta;
     h->h = (float)((double)eta / (double)h->n);
+    drop_epoch_graph(h);   // (its kernels hold the old step)
     return DSFACTO_OK;
 }
 

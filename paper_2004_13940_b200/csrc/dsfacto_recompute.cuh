@@ -50,9 +50,12 @@ struct RefreshArgs {
     // end of the pass: the last CTA adds the partial sums up
     unsigned *done;        // CTAs that have delivered (zero between launches)
     EpochState *st;        // kTrain: w0 comes from here and the sums go here; NULL: w0 above
-    EpochReport *report;   // mapped host memory: the sums and, behind them, seq (NULL: not the end of an epoch)
-    unsigned long long seq;
+    EpochReport *report;   // mapped host memory: the sums and, behind them, a number (NULL: not the end of an epoch)
+    unsigned long long seq;   // ... which is this one (kTrain: the number of such reports, counted on the device)
     int first;             // kTrain: the first segment of an epoch (its times are set, not added)
+    // STAGED: a small batch in mapped host memory, [indptr | idx | val | y]; indptr, idx, val, y are then offsets into it
+    const uint4 *stage;
+    int stage_bytes;       // (a multiple of 16)
     int *bad;              // caller rows that were checked on the device: no row is read if it is set (NULL: sound rows)
 };
 
@@ -107,7 +110,9 @@ struct RefreshCfg {
     static constexpr int CTAS = LG < 8 ? 4 : NV >= 4 ? 2 : 3;               // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
 };
-template <int LG, int NV, int MODE, bool RAW = false>
+// STAGED: every CTA first copies the whole batch from the host's memory to shared memory, all of it at once: one
+// trip across the link instead of one for the row pointers and one for every two batches of entries.
+template <int LG, int NV, int MODE, bool RAW = false, bool STAGED = false>
 __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_kernel(const RefreshArgs a) {
     typedef RefreshCfg<LG, NV> C;
     constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, KP4 = LG * NV;
@@ -123,6 +128,20 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
     if (l == 0) { sums[0][g] = 0.0; sums[1][g] = 0.0; }
     let_next_kernel_start();
 
+    const int64_t *indptr = a.indptr;
+    const int32_t *idx = a.idx;
+    const float *val = a.val, *lab = a.y;
+    if (STAGED) {
+        uint4 *to = reinterpret_cast<uint4 *>(hot_pair);
+        for (int i = threadIdx.x; i < a.stage_bytes / 16; i += kThreads) to[i] = a.stage[i];
+        const char *p = reinterpret_cast<const char *>(to);
+        indptr = reinterpret_cast<const int64_t *>(p);
+        idx = reinterpret_cast<const int32_t *>(p + reinterpret_cast<size_t>(a.idx));
+        val = reinterpret_cast<const float *>(p + reinterpret_cast<size_t>(a.val));
+        lab = reinterpret_cast<const float *>(p + reinterpret_cast<size_t>(a.y));
+        __syncthreads();
+    }
+    auto fixed = [](const auto *q) { return STAGED ? *q : __ldg(q); };   // data that does not change during the kernel
     int64_t n = a.n;
     int bad = 0;
     if ((MODE == kScore || MODE == kEvaluate) && a.bad) {
@@ -139,8 +158,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
     auto next_pointers = [&](int64_t row) {
         nlen = 0;
         if (row < n) {
-            nbeg = __ldg(a.indptr + row);
-            nlen = (int)(__ldg(a.indptr + row + 1) - nbeg);
+            nbeg = fixed(indptr + row);
+            nlen = (int)(fixed(indptr + row + 1) - nbeg);
         }
     };
     auto load_entries = [&](int64_t beg, int t0, int len, int32_t (&j)[E], float (&x)[E]) {
@@ -148,8 +167,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
         for (int e = 0; e < E; ++e) {
             const int t = t0 + e * LG + l;
             j[e] = 0; x[e] = 0.f;
-            if (len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
-            if (t < len) x[e] = __ldg(a.val + beg + t);
+            if (len > 0) j[e] = fixed(idx + beg + min(t, len - 1));
+            if (t < len) x[e] = fixed(val + beg + t);
         }
     };
     next_pointers(base + gw);
@@ -260,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
             const float f = w0 + lin + 0.5f * pair;
             if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
             if (MODE != kScore) {
-                const float yy = a.y[row];
+                const float yy = lab[row];
                 float li, gi;
                 if (a.loss == 0) {
                     gi = f - yy;
@@ -331,7 +350,9 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
             }
             if (a.report) {
                 __threadfence_system();
-                ((volatile EpochReport *)a.report)->seq = a.seq;
+                volatile EpochReport *r = a.report;
+                if (TRAIN) r->epochs = ++a.st->epochs;
+                else r->seq = a.seq;
             }
         }
     }

@@ -99,7 +99,8 @@ class DSFactoError(RuntimeError):
 
 
 def _ptr(a: Optional[np.ndarray]):
-    return None if a is None else ctypes.c_void_p(a.ctypes.data)
+    # (the address as an int: a.ctypes.data and a c_void_p object take 0.8 us more per argument)
+    return None if a is None else a.__array_interface__["data"][0]
 
 
 # ---- the C calls under their own names (thin wrappers: numpy arrays in, status out) ----
