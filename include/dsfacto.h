@@ -213,8 +213,15 @@ int dsfacto_debug_set(dsfacto_t *h, int32_t key, int64_t value);
  * info[2] = bytes it copied device -> host.  DSFACTO_ERR_NO_DATA before the first load. */
 int dsfacto_last_load(dsfacto_t *h, int64_t info[3]);
 
-/* The library keeps freed device memory for its next calls (per device up to a 64th of its memory) and the
- * page-locked mailboxes of up to eight destroyed handles.  This gives all of it back.  It is also given back when an
+/* Page-locked host memory for arrays that results are copied into again and again (dsfacto_get_params,
+ * dsfacto_predict, ...; any host memory will do there, results reach this kind faster).  NULL when the library holds
+ * 512 MB of it already or none can be had: use ordinary memory then.  Any thread may free it. */
+void *dsfacto_host_alloc(uint64_t bytes);
+void dsfacto_host_free(void *ptr);
+
+/* The library keeps freed device memory for its next calls (per device up to a 64th of its memory), the
+ * page-locked mailboxes of up to eight destroyed handles and up to 256 MB of freed dsfacto_host_alloc memory.  This
+ * gives all of it back.  It is also given back when an
  * allocation of the library fails.  Safe to call at any time, from any thread. */
 void dsfacto_trim(void);
 

@@ -2,6 +2,7 @@
 // the device.
 #pragma once
 #include <cuda_runtime.h>
+#include <sys/mman.h>
 #include <unistd.h>
 
 #include <algorithm>
@@ -126,6 +127,123 @@ private:
     uint64_t clock_ = 0;
     std::map<int, size_t> idle_bytes_, bound_;
     std::unordered_map<void *, Block> live_;
+};
+
+// Page-locked host memory on 2 MB pages: 64 MB take 5 ms (touched by several threads, then registered) against 29 ms
+// of cudaHostAlloc, which locks 4 KB pages.  bytes: a multiple of 2 MB.  NULL if it cannot be had.
+constexpr size_t kHugePage = (size_t)2 << 20;
+inline char *locked_alloc(size_t bytes) {
+    char *raw = static_cast<char *>(mmap(nullptr, bytes + kHugePage, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0));
+    if (raw == MAP_FAILED) return nullptr;
+    char *p = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(raw) + kHugePage - 1) / kHugePage * kHugePage);
+    if (p > raw) munmap(raw, (size_t)(p - raw));
+    if (raw + kHugePage > p) munmap(p + bytes, (size_t)(raw + kHugePage - p));
+    madvise(p, bytes, MADV_HUGEPAGE);
+    const int pages = (int)(bytes / kHugePage), workers = pages >= 8 ? 4 : 1;
+    auto touch = [=](int w) { for (int k = w; k < pages; k += workers) p[(size_t)k * kHugePage] = 0; };
+    std::thread team[4];
+    for (int w = 1; w < workers; ++w)
+        try { team[w] = std::thread(touch, w); } catch (...) {}   // (registering touches what is left)
+    touch(0);
+    for (std::thread &t : team)
+        if (t.joinable()) t.join();
+    if (cudaHostRegister(p, bytes, cudaHostRegisterPortable | cudaHostRegisterMapped) != cudaSuccess) {
+        cudaGetLastError();
+        munmap(p, bytes);
+        return nullptr;
+    }
+    return p;
+}
+inline void locked_free(char *p, size_t bytes) {
+    cudaHostUnregister(p);
+    munmap(p, bytes);
+}
+
+// ------------------------------------------------------------------------------------------
+// Result buffers: page-locked memory that the Python binding hands out as arrays, so that results arrive at the
+// link's speed and no page is touched for the first time on the way (71 MB of parameters: 2.5 -> 1.4 ms, 2.7 MB: 0.20
+// -> 0.06 ms).  At most 512 MB exist at a time, in use or idle (beyond that a caller gets NULL and takes ordinary
+// memory), at most 256 MB of them idle; trim() gives the idle ones back.
+// ------------------------------------------------------------------------------------------
+class ResultBuffers {
+public:
+    static ResultBuffers &get() {
+        static ResultBuffers *r = new ResultBuffers;
+        return *r;
+    }
+    void *alloc(size_t bytes) {
+        const size_t size = size_of(bytes);
+        std::lock_guard<std::mutex> lock(mu_);
+        auto it = idle_.lower_bound(size);
+        if (it == idle_.end() || (size > kSmallMost ? it->first > size + size / 4 : it->first != size)) {
+            const size_t region = std::max(size, kHugePage);
+            if (total_ + region > kMost) return nullptr;
+            char *p = locked_alloc(region);
+            if (!p) return nullptr;
+            total_ += region;
+            const int parts = (int)(region / size);
+            for (int k = 0; k < parts; ++k) idle_.emplace(size, Part{p + (size_t)k * size, p});
+            regions_[p] = {region, 0};
+            idle_bytes_ += region;
+            it = idle_.lower_bound(size);
+        }
+        const Part part = it->second;
+        live_[part.ptr] = {it->first, part.region};
+        regions_[part.region].live += 1;
+        idle_bytes_ -= it->first;
+        idle_.erase(it);
+        return part.ptr;
+    }
+    void free(void *ptr) {
+        std::lock_guard<std::mutex> lock(mu_);
+        const auto it = live_.find(static_cast<char *>(ptr));
+        if (it == live_.end()) return;
+        idle_.emplace(it->second.bytes, Part{it->first, it->second.region});
+        idle_bytes_ += it->second.bytes;
+        regions_[it->second.region].live -= 1;
+        live_.erase(it);
+        if (idle_bytes_ > kMostIdle) release_idle();
+    }
+    void trim() {
+        std::lock_guard<std::mutex> lock(mu_);
+        release_idle();
+    }
+
+private:
+    static constexpr size_t kMost = (size_t)512 << 20, kMostIdle = (size_t)256 << 20, kSmallMost = (size_t)1 << 20;
+    struct Part { char *ptr, *region; };
+    struct Live { size_t bytes; char *region; };
+    struct RegionUse { size_t bytes; int live; };
+    static size_t size_of(size_t bytes) {   // up to 1 MB a power of two (several share a page), then whole pages
+        if (bytes > kSmallMost) return (bytes + kHugePage - 1) / kHugePage * kHugePage;
+        size_t s = (size_t)32 << 10;
+        while (s < bytes) s *= 2;
+        return s;
+    }
+    void release_idle() {   // (mu_ is held) every region no part of which is in use
+        for (auto it = idle_.begin(); it != idle_.end();) {
+            if (regions_[it->second.region].live == 0) {
+                idle_bytes_ -= it->first;
+                it = idle_.erase(it);
+            } else {
+                ++it;
+            }
+        }
+        for (auto it = regions_.begin(); it != regions_.end();) {
+            if (it->second.live == 0) {
+                locked_free(it->first, it->second.bytes);
+                total_ -= it->second.bytes;
+                it = regions_.erase(it);
+            } else {
+                ++it;
+            }
+        }
+    }
+    std::mutex mu_;
+    std::multimap<size_t, Part> idle_;
+    std::unordered_map<char *, Live> live_;
+    std::map<char *, RegionUse> regions_;
+    size_t total_ = 0, idle_bytes_ = 0;
 };
 
 // ------------------------------------------------------------------------------------------
@@ -278,7 +396,7 @@ private:
         if (fresh) {
             const unsigned cores = std::max(2u, std::thread::hardware_concurrency());
             lanes_.resize(std::min(8u, cores / 2));
-            if ((e = cudaHostAlloc((void **)&arena_, lanes_.size() * 2 * kSlot, cudaHostAllocPortable)) != cudaSuccess) { lanes_.clear(); return e; }
+            if (!(arena_ = locked_alloc(lanes_.size() * 2 * kSlot))) { lanes_.clear(); return cudaErrorMemoryAllocation; }
             for (size_t k = 0; k < lanes_.size(); ++k)
                 for (int t = 0; t < 2; ++t) lanes_[k].slot[t] = arena_ + (2 * k + t) * kSlot;
         }

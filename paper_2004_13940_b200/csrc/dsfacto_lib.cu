@@ -1112,7 +1112,7 @@ void column_blocks(const dsfacto *h, std::vector<int32_t> &cb);
 int bucket_tiles(dsfacto *h, const int64_t *indptr, const int32_t *indices, const float *values,
                  HostBuf<uint2> &ent, HostBuf<float> &xw, SgdPlanBuild *pb) {
     const int64_t n = h->n, nnz = indptr[n];
-    const int32_t d = h->d, p = h->p;
+    const int32_t p = h->p;
     const int64_t nt = (int64_t)p * p;
     const bool wide = h->wide;
     const int jbits = h->jbits;
@@ -2743,6 +2743,17 @@ int dsfacto_last_load(dsfacto_t *h, int64_t info[3]) {
 void dsfacto_trim(void) {
     DevicePool::get().trim();
     Mailboxes::get().trim();
+    ResultBuffers::get().trim();
+}
+
+void *dsfacto_host_alloc(uint64_t bytes) {
+    if (bytes == 0) return nullptr;
+    try { return ResultBuffers::get().alloc((size_t)bytes); } catch (const std::bad_alloc &) { return nullptr; }
+}
+
+void dsfacto_host_free(void *ptr) {
+    if (!ptr) return;
+    try { ResultBuffers::get().free(ptr); } catch (const std::bad_alloc &) {}
 }
 
 int dsfacto_launch_count(dsfacto_t *h, int64_t *out) {

@@ -6,6 +6,7 @@ device is usable, dsfacto_create returns DSFACTO_ERR_CUDA and `DSFacto(...)` rai
 from __future__ import annotations
 
 import ctypes
+import weakref
 from typing import Optional
 
 import numpy as np
@@ -50,6 +51,8 @@ SIGNATURES = {
                                                  ctypes.POINTER(_c_i64), _vp, _vp, _vp, _vp]),
     "dsfacto_launch_count": (ctypes.c_int, [_vp, ctypes.POINTER(_c_i64)]),
     "dsfacto_trim": (None, []),
+    "dsfacto_host_alloc": (_vp, [_c_u64]),
+    "dsfacto_host_free": (None, [_vp]),
     "dsfacto_last_load": (ctypes.c_int, [_vp, ctypes.POINTER(_c_i64)]),
     "dsfacto_last_error": (ctypes.c_char_p, [_vp]),
     "dsfacto_strerror": (ctypes.c_char_p, [ctypes.c_int]),
@@ -99,8 +102,36 @@ class DSFactoError(RuntimeError):
 
 
 def _ptr(a: Optional[np.ndarray]):
-    # (the address as an int: a.ctypes.data and a c_void_p object take 0.8 us more per argument)
-    return None if a is None else a.__array_interface__["data"][0]
+    if a is None:
+        return None
+    try:   # 0.4 us; a.ctypes.data takes 1.0 us, which five arrays of a small request would feel
+        return ctypes.byref(ctypes.c_char.from_buffer(a))
+    except (TypeError, ValueError, BufferError):   # read-only or empty
+        return a.ctypes.data
+
+
+_asked = {}          # result sizes asked for so far, and how often (bounded: emptied when it grows)
+_LOCKED_FROM = 1 << 16
+
+
+def _result(*shape) -> np.ndarray:
+    """An uninitialised float32 array for results.  From the second time a size of 64 KB or more is asked for,
+    page-locked memory of the library (it goes back when the array dies); making that takes as long as two copies
+    into ordinary memory, so a program that asks once gets ordinary memory."""
+    nbytes = 4
+    for k in shape:
+        nbytes *= k
+    if nbytes < _LOCKED_FROM:
+        return np.empty(shape, np.float32)
+    if len(_asked) > 256:
+        _asked.clear()
+    _asked[nbytes] = _asked.get(nbytes, 0) + 1
+    p = lib().dsfacto_host_alloc(nbytes) if _asked[nbytes] >= 2 else None
+    if not p:
+        return np.empty(shape, np.float32)
+    buf = (ctypes.c_char * nbytes).from_address(p)
+    weakref.finalize(buf, lib().dsfacto_host_free, p).atexit = False
+    return np.frombuffer(buf, np.float32).reshape(shape)
 
 
 # ---- the C calls under their own names (thin wrappers: numpy arrays in, status out) ----
@@ -295,8 +326,8 @@ class DSFacto:
 
     def get_params(self):
         w0 = np.zeros(1, np.float32)
-        w = np.empty(self.d, np.float32)
-        V = np.empty((self.d, self.K), np.float32)
+        w = _result(self.d)
+        V = _result(self.d, self.K)
         self._check(dsfacto_get_params(self._h, w0, w, V), "dsfacto_get_params")
         return float(w0[0]), w, V
 
@@ -312,14 +343,14 @@ class DSFacto:
 
     def predict(self, indptr=None, indices=None, values=None):
         if indptr is None:
-            out = np.empty(self.n, np.float32)
+            out = _result(self.n)
             self._check(dsfacto_predict(self._h, self.n, None, None, None, out), "dsfacto_predict")
             return out
         indptr = np.ascontiguousarray(indptr, np.int64)
         indices = np.ascontiguousarray(indices, np.int32)
         values = np.ascontiguousarray(values, np.float32)
         m = indptr.shape[0] - 1
-        out = np.empty(max(m, 1), np.float32)[:m]
+        out = _result(max(m, 1))[:m]
         self._check(dsfacto_predict(self._h, m, indptr, indices, values, out), "dsfacto_predict")
         return out
 
@@ -353,8 +384,8 @@ class DSFacto:
         return tile_ptr, rows, cols, vals
 
     def get_aux(self):
-        A = np.empty((self.n, self.K), np.float32)
-        G = np.empty(self.n, np.float32)
+        A = _result(self.n, self.K)
+        G = _result(self.n)
         self._check(lib().dsfacto_get_aux(self._h, _ptr(A), _ptr(G)), "dsfacto_get_aux")
         return A, G
 
