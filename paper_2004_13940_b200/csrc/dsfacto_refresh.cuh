@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThreads) column_rename_kernel(int32_t *__rest
 }
 // The model as the recompute pass reads it: pair[s] = (w_j, sum_k v_jk^2) and, when the columns are
 // renumbered (column_of != NULL: j = column_of[s], and Vs is given), Vs[s] = V[j]; else j = s.  A group of gs
-// lanes (a power of two <= 32) takes a row of kp4 float4s.
+// lanes (a power of two <= 16) takes a row of kp4 float4s.
 __global__ void __launch_bounds__(kThreads) model_view_kernel(const float4 *__restrict__ V, const float *__restrict__ w,
                                                               const int32_t *__restrict__ column_of, int64_t d, int kp4, int gs,
                                                               float4 *__restrict__ Vs, float2 *__restrict__ pair) {
@@ -68,16 +68,20 @@ __global__ void __launch_bounds__(kThreads) model_view_kernel(const float4 *__re
     const int64_t rounds = (d + groups - 1) / groups;   // the same for every lane of a warp: the shuffles below stay converged
     for (int64_t it = 0; it < rounds; ++it) {
         const int64_t s = g0 + it * groups;
-        float sum = 0.f;
+        float sums[2] = {0.f, 0.f};   // of even and odd float4s of a lane (the tree over 32 lanes would start with these two)
         int64_t j = 0;
         if (s < d) {
             j = column_of ? (int64_t)__ldg(column_of + s) : s;
             for (int v = gl; v < kp4; v += gs) {
                 const float4 x = V[j * kp4 + v];
                 if (Vs) Vs[s * kp4 + v] = x;
+                const bool odd = ((v / gs) & 1) != 0;
+                float sum = odd ? sums[1] : sums[0];
                 sum = fmaf(x.x, x.x, sum); sum = fmaf(x.y, x.y, sum); sum = fmaf(x.z, x.z, sum); sum = fmaf(x.w, x.w, sum);
+                if (odd) sums[1] = sum; else sums[0] = sum;
             }
         }
+        float sum = sums[0] + sums[1];
         for (int o = gs >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         if (s < d && gl == 0) pair[s] = make_float2(w[j], sum);
     }

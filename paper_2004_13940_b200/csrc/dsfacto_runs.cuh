@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const bool mine = q[r] >= 0 && (!COOP || g == 0);
-        float sum = 0.f;
+        float sums[2] = {0.f, 0.f};   // of even and odd float4s: the order in which model_view_kernel adds
         if (mine) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
@@ -483,9 +483,11 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
                 t.x = fmaf(D[r], t.x, t.x); t.y = fmaf(D[r], t.y, t.y); t.z = fmaf(D[r], t.z, t.z); t.w = fmaf(D[r], t.w, t.w);
                 row_of(r)[v * LG] = t;
                 if (a.Vs) a.Vs[(int64_t)slot[r] * KP4 + v * LG + l] = t;
+                float &sum = sums[v & 1];
                 sum = fmaf(t.x, t.x, sum); sum = fmaf(t.y, t.y, sum); sum = fmaf(t.z, t.z, sum); sum = fmaf(t.w, t.w, sum);
             }
         }
+        float sum = NV > 1 ? sums[0] + sums[1] : sums[0];
         if (a.pair) {
 #pragma unroll
             for (int o = LG / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
@@ -516,7 +518,7 @@ __global__ void __launch_bounds__(kThreads) runs_fold_kernel(float4 *V, float *w
     wait_for_previous_kernel();
     for (int64_t it = 0; it < rounds; ++it) {
         const int64_t j = g0 + it * groups;
-        float sum = 0.f;
+        float sums[2] = {0.f, 0.f};
         int64_t slot = j;
         float4 t = zero4();
         if (j < d) {
@@ -533,9 +535,13 @@ __global__ void __launch_bounds__(kThreads) runs_fold_kernel(float4 *V, float *w
                     Tb[j * kp4 + v] = zero4();
                 }
                 if (Vs) Vs[slot * kp4 + v] = y;
+                const bool odd = ((v / gs) & 1) != 0;
+                float sum = odd ? sums[1] : sums[0];
                 sum = fmaf(y.x, y.x, sum); sum = fmaf(y.y, y.y, sum); sum = fmaf(y.z, y.z, sum); sum = fmaf(y.w, y.w, sum);
+                if (odd) sums[1] = sum; else sums[0] = sum;
             }
         }
+        float sum = sums[0] + sums[1];
         for (int o = gs >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         if (j < d && gl == 0) {
             float wj = w[j];
