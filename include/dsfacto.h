@@ -187,7 +187,7 @@ int dsfacto_last_epoch_ms(dsfacto_t *h, float ms[4]);
  *                             it; with a value larger than the number of chunks its wait runs out, so the
  *                             failure path above can be exercised without a fault or a hang.  0 = off.
  *   DSFACTO_DEBUG_CHUNK_LEN   (takes effect at the next dsfacto_load_csr) entries per chunk (per unit of the update loop
- *                             by column runs: rounded up to a power of two), 16 .. 4096, 0 = chosen by the load; the environment variable DSFACTO_CHUNK does the same for every handle.
+ *                             by column runs: rounded up to a multiple of 32), 16 .. 4096, 0 = chosen by the load; the environment variable DSFACTO_CHUNK does the same for every handle.
  *                             The sweep kernel reads a chunk's entries block by block; the environment variable
  *                             DSFACTO_BLOCK (a multiple of 32, 32 .. 256) sets the entries per block.
  *   DSFACTO_DEBUG_ROW_MERGE   (takes effect at the next dsfacto_load_csr that buckets on the device) row blocks per slot of

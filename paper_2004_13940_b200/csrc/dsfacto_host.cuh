@@ -308,7 +308,7 @@ private:
         cudaError_t e;
         try {
             size_t most = 0;
-            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kSlot + 2;
+            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kSlot + 32;
             regions_.reserve(most);
             e = prepare();
         } catch (const std::bad_alloc &) { e = cudaErrorMemoryAllocation; }
@@ -323,13 +323,20 @@ private:
             return cudaSuccess;
         }
         regions_.clear();
+        size_t all = 0, total = 0;
+        for (int q = 0; q < count; ++q) total += pieces[q].bytes;
         for (int q = 0; q < count; ++q) {
             const Piece &p = pieces[q];
             char *d = static_cast<char *>(p.dev), *h = static_cast<char *>(p.host), *end = h + p.bytes;
-            while (h < end) {   // on the way back regions end on 2 MB boundaries: a huge page is touched by one thread
-                const size_t unit = to_device ? kSlot : kRegion;
-                char *stop = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(h) / unit + 1) * unit);
-                const size_t n = (size_t)(std::min(stop, end) - h);
+            while (h < end) {
+                size_t n;
+                if (to_device) {   // small ones at the start, so that the link has work soon, and at the end, so that little is left then
+                    n = all < ((size_t)2 << 20) ? kSlot / 4 : total - all < ((size_t)6 << 20) ? kSlot / 2 : kSlot;
+                } else {           // on 2 MB boundaries: a huge page is touched by one thread
+                    n = kRegion - reinterpret_cast<uintptr_t>(h) % kRegion;
+                }
+                n = std::min(n, (size_t)(end - h));
+                all += n;
                 regions_.push_back({d, h, n});
                 d += n;
                 h += n;

@@ -777,6 +777,7 @@ void run_sgd_phase(dsfacto *h, int64_t L0, int64_t L1) {
 }
 
 // ---- update loop by column runs ----
+int run_ctas_per_sm(const dsfacto *h) { return h->LG * h->NV <= 4 ? 8 : h->LG * h->NV <= 8 ? 6 : 4; }   // as runs_sweep_kernel is bounded
 template <int LG, int NV>
 void launch_run_pass(dsfacto *h, const RunPass &ps, RunSweepArgs &sw, RunApplyArgs &ap) {
     const int64_t ctas = std::max<int64_t>(((int64_t)ps.units + kRunWarps - 1) / kRunWarps, 1);
@@ -808,7 +809,7 @@ void run_strata(dsfacto *h, int64_t seg, double share) {
         sw.h = h->h; sw.lambda_v = h->lambda_v; sw.kappa_w = (float)(-log1m_ew / std::log(2.0));
         RunApplyArgs ap{};
         ap.run_key = h->d_run_key + ps.run_first; ap.run_start = sw.run_start; ap.nruns = ps.nruns; ap.count = ps.count;
-        ap.shift = bits_for((int64_t)kRunWarps * h->unit_len); ap.rec = h->d_rec; ap.part = h->d_part; ap.w = h->d_w; ap.V = h->d_V;
+        ap.chunk = kRunWarps * h->unit_len; ap.chunk_inv = chunk_inverse(ap.chunk); ap.rec = h->d_rec; ap.part = h->d_part; ap.w = h->d_w; ap.V = h->d_V;
         ap.Tw = h->d_Tw; ap.Tb = h->d_Tb; ap.TS = h->d_TS;
         if (h->bands == 1) { ap.pair = pair; ap.Vs = Vs; ap.slot_of = slot_of; }
         ap.st = h->d_state; ap.log1m_ew = log1m_ew;
@@ -1895,11 +1896,12 @@ static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env)
     if (nnz <= 0 || h->sweep != 1 || h->row_merge > 0 || h->debug_extra_need > 0 || std::getenv("DSFACTO_ROW_MERGE")) return false;
     if (load_env) { if (std::strcmp(load_env, "device") != 0) return false; }
     else {
+        // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs
+        const double need = 1.1 * ((double)nnz * 26.0 + (double)h->n * 4.0 * (h->Kp + 2));
+        if (need <= (double)h->l2_bytes * 8.0) return true;   // (asking for the free memory takes 0.25 ms; a gigabyte is simply tried)
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-        free_b += DevicePool::get().idle_bytes();
-        // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs
-        if ((double)free_b < 1.1 * ((double)nnz * 26.0 + (double)h->n * 4.0 * (h->Kp + 2))) return false;
+        if ((double)(free_b + DevicePool::get().idle_bytes()) < need) return false;
     }
     return true;
 }
@@ -1978,14 +1980,17 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     for (int64_t q = 0; q < npass; ++q) longest = std::max(longest, first[q + 1] - first[q]);
     if (longest >= ((int64_t)1 << 31) - ((int64_t)1 << 17)) { cleanup(); h->passes.clear(); return 1; }   // positions inside a pass are 32-bit
     // Units: long enough to amortise a unit's start and end, short enough that a small pass keeps every SM busy.
-    int64_t want = std::min<int64_t>(1024, longest / ((int64_t)h->sm_count * 32));
-    if (h->chunk_override > 0) want = h->chunk_override;
+    // A pass is cut so that its units fill whole waves of resident warps, as few as units of 1024 entries allow (2.6 M
+    // entries of 128-byte rows, in 0.75 / 1.5 waves: 47 / 49 us, in one: 42 us).
+    const int64_t resident = (int64_t)h->sm_count * kRunWarps * run_ctas_per_sm(h);
+    const int64_t waves = std::max<int64_t>(1, (longest + 1024 * resident - 1) / (1024 * resident));
+    int64_t unit = (longest + waves * resident - 1) / (waves * resident);
+    if (h->chunk_override > 0) unit = h->chunk_override;
     if (const char *env = std::getenv("DSFACTO_CHUNK")) {
         const int v = std::atoi(env);
-        if (v >= 16 && v <= kUnitMax) want = v;
+        if (v >= 16 && v <= kUnitMax) unit = v;
     }
-    int64_t unit = 32;
-    while (unit < want) unit *= 2;
+    unit = std::max<int64_t>(32, (unit + 31) & ~(int64_t)31);
     h->unit_len = (int)unit;
     int64_t units = 0, most_units = 1;
     for (int64_t q = 0; q < npass; ++q) {
@@ -2206,6 +2211,12 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
     bool by_runs = run_plan_wanted(h, nnz, load_env);
     if (by_runs) {
         rc = plan_runs(h, nnz);
+        if (rc == DSFACTO_ERR_OOM && !load_env) {   // no room for the sort: the host buckets the entries
+            cudaStreamSynchronize(st);
+            dev_free(h->d_run_start); dev_free(h->d_run_key); dev_free(h->d_unit_run); dev_free(h->d_rec); dev_free(h->d_part);
+            h->passes.clear();
+            rc = 1;
+        }
         if (rc < 0) { cudaStreamSynchronize(st); free_data(h); return rc; }
         by_runs = rc == 0;
     }

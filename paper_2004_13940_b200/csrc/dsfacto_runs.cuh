@@ -31,7 +31,7 @@ constexpr uint32_t kRunStart = 0x80000000u;       // bit of an entry's row word:
 struct RunSweepArgs {
     const uint2 *ent;          // entries of the pass: {row | kRunStart, bits of x}
     int count;                 // their number
-    int unit_len;              // entries per unit (a power of two, at least 32)
+    int unit_len;              // entries per unit (a multiple of 32)
     const int *run_start;      // per run of the pass: its first entry
     const int *unit_run;       // per unit: the run that holds its first entry
     int nruns;
@@ -346,10 +346,21 @@ __global__ void __launch_bounds__(kRunThreads, (LG * NV <= 4 ? 8 : LG * NV <= 8 
     }
 }
 
+// Position of an entry -> CTA of the sweep that has it: division by the CTA's entries, 128 k of them with k <= 128.
+// q = p / 128 is below 2^24, so q / k = (q * ceil(2^32 / k)) >> 32 exactly (the inverse is too large by less than k / 2^32).
+static_assert(kRunWarps * 32 == 128 && kUnitMax <= 128 * 32, "see chunk_of");
+inline uint32_t chunk_inverse(int chunk) { return (uint32_t)((((uint64_t)1 << 32) + chunk / 128 - 1) / (uint64_t)(chunk / 128)); }   // (k = 1: 0)
+__device__ __forceinline__ int chunk_of(int p, uint32_t inv) {
+    const uint32_t q = (uint32_t)p >> 7;
+    return (int)(inv == 0u ? q : __umulhi(q, inv));
+}
+
 struct RunApplyArgs {
     const uint32_t *run_key;   // per run: (column << 1) | acts on the tail composite
     const int *run_start;
-    int nruns, count, shift;   // runs and entries of the pass; log2 of the entries per CTA of the sweep
+    int nruns, count;          // runs and entries of the pass
+    int chunk;                 // entries per CTA of the sweep
+    uint32_t chunk_inv;        // chunk_inverse(chunk)
     const float4 *rec, *part;
     float *w, *V;
     float *Tw, *Tb;            // tail composite: q_j and its part for w (several bands only)
@@ -414,8 +425,8 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
     auto w_of = [&](int r) { return ((key[r] & 1u) ? a.Tw : a.w) + (key[r] >> 1); };
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int c0 = s[r] >> a.shift;
-        np[r] = q[r] >= 0 ? ((e[r] - 1) >> a.shift) - c0 + 1 : 0;
+        const int c0 = chunk_of(s[r], a.chunk_inv);
+        np[r] = q[r] >= 0 ? chunk_of(e[r] - 1, a.chunk_inv) - c0 + 1 : 0;
         D[r] = 0.f; W[r] = 0.f; yw[r] = 0.f;
 #pragma unroll
         for (int v = 0; v < NV; ++v) { y[r][v] = zero4(); U[r][v] = zero4(); }
@@ -436,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
     // ---- the other pieces ----
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int c0 = s[r] >> a.shift;
+        const int c0 = chunk_of(s[r], a.chunk_inv);
         int lo = 1, hi = np[r];
         if (COOP) {
             const int per = (np[r] + GW - 1) / GW;
