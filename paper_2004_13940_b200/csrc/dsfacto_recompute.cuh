@@ -94,8 +94,8 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // entries runs to the longest of the rows (an earlier form in which every group looped on its own took 9.3 warp
 // instructions per entry of 128-byte rows, most of them for the masks and branches of the divergent groups).  A batch
 // is B = LG * E entries of each row, every lane owns E of them: it takes their (w_j, s_j) and hands column and value
-// to its group; entries are requested two batches ahead.  Factor rows are requested UB entries at a time, always one
-// step ahead of the multiply-adds (two sets of registers).  Behind the end of a row its last entry is repeated with
+// to its group; entries are requested two batches ahead.  Factor rows are requested UB entries at a time, NB - 1 steps
+// ahead of the multiply-adds.  Behind the end of a row its last entry is repeated with
 // x = 0.
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
 // The pairs of the first `hot` columns (the most frequent ones, when the columns are numbered that way) sit in shared
@@ -107,8 +107,10 @@ struct RefreshCfg {
     static constexpr int B = LG * E;
     // entries whose rows are requested together; a small batch (STAGED) has the GPU to itself and waits for nothing
     // but the latency of these requests, so it makes fewer and larger ones (32 rows of 39 entries: 25 -> 22 us per call)
-    static constexpr int UB = STAGED && NV <= 4 ? B / 2 : NV >= 6 || LG == 1 ? 1 : NV >= 2 || LG == 4 ? 2 : B / 2;
-    static constexpr int S = B / UB;                                        // steps per batch (an even number)
+    static constexpr int UB = STAGED && NV <= 4 ? B / 2 : LG == 8 && NV == 1 ? 2 : 1;
+    static constexpr int S = B / UB;                                        // steps per batch
+    static constexpr int NB = STAGED || NV >= 6 || LG == 1 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
+    static_assert(S % NB == 0, "a step keeps its registers from batch to batch");
     static constexpr int CTAS = STAGED ? 1 : LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
 };
@@ -117,7 +119,7 @@ struct RefreshCfg {
 template <int LG, int NV, int MODE, bool RAW = false, bool STAGED = false>
 __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) refresh_kernel(const RefreshArgs a) {
     typedef RefreshCfg<LG, NV, STAGED> C;
-    constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, KP4 = LG * NV;
+    constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, NB = C::NB, KP4 = LG * NV;
     constexpr unsigned FULL = 0xFFFFFFFFu;
     const int g = threadIdx.x / LG, l = threadIdx.x % LG, gw = (threadIdx.x & 31) / LG;
     const float4 *V4 = reinterpret_cast<const float4 *>(a.V) + l;
@@ -193,7 +195,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
         float q = 0.f, lin = 0.f;
-        float4 vv[2][UB][NV];
+        float2 q2 = make_float2(0.f, 0.f);   // (RAW)
+        float4 vv[NB][UB][NV];
         auto load_rows = [&](const int32_t (&j)[E], int u0, float4 (&r)[UB][NV]) {
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
@@ -204,7 +207,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
         };
 #pragma unroll
         for (int e = 0; e < E; ++e) { j0[e] = jn[e]; x0[e] = xn[e]; }
-        load_rows(j0, 0, vv[0]);
+#pragma unroll
+        for (int st = 0; st + 1 < NB; ++st) load_rows(j0, st * UB, vv[st]);
         load_entries(beg, B, len, j1, x1);
         if (longest <= B) load_entries(nbeg, 0, nlen, jn, xn);
         for (int t0 = 0; t0 < longest; t0 += B) {
@@ -225,31 +229,30 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
                 }
 #pragma unroll
             for (int st = 0; st < S; ++st) {
-                if (st + 1 < S) load_rows(j0, (st + 1) * UB, vv[(st + 1) & 1]);
-                else if (t0 + B < longest) load_rows(j1, 0, vv[0]);
+                const int ahead = st + NB - 1;
+                if (ahead < S) load_rows(j0, ahead * UB, vv[ahead % NB]);
+                else if (t0 + B < longest) load_rows(j1, (ahead - S) * UB, vv[ahead % NB]);
 #pragma unroll
                 for (int u = 0; u < UB; ++u) {
                     const float x = __shfl_sync(FULL, x0[(st * UB + u) / LG], (st * UB + u) % LG, LG);
-                    const float4 (&r)[NV] = vv[st & 1][u];
+                    const float4 (&r)[NV] = vv[st % NB][u];
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        acc[v].x = fmaf(r[v].x, x, acc[v].x); acc[v].y = fmaf(r[v].y, x, acc[v].y);
-                        acc[v].z = fmaf(r[v].z, x, acc[v].z); acc[v].w = fmaf(r[v].w, x, acc[v].w);
-                    }
+                    for (int v = 0; v < NV; ++v) fma4(acc[v], x, r[v]);
                     if (RAW) {
-                        float sv = 0.f;
+                        float2 sv = make_float2(0.f, 0.f);
 #pragma unroll
                         for (int v = 0; v < NV; ++v) {
-                            sv = fmaf(r[v].x, r[v].x, sv); sv = fmaf(r[v].y, r[v].y, sv);
-                            sv = fmaf(r[v].z, r[v].z, sv); sv = fmaf(r[v].w, r[v].w, sv);
+                            sv = __ffma2_rn(make_float2(r[v].x, r[v].y), make_float2(r[v].x, r[v].y), sv);
+                            sv = __ffma2_rn(make_float2(r[v].z, r[v].w), make_float2(r[v].z, r[v].w), sv);
                         }
-                        q = fmaf(x * x, sv, q);
+                        q2 = __ffma2_rn(sv, make_float2(x * x, x * x), q2);
                     }
                 }
             }
 #pragma unroll
             for (int e = 0; e < E; ++e) { j0[e] = j1[e]; x0[e] = x1[e]; j1[e] = j2[e]; x1[e] = x2[e]; }
         }
+        if (RAW) q = q2.x + q2.y;
         if (len == 0) {   // (a row without entries has added nothing but zeros times whatever row 0 holds)
 #pragma unroll
             for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
