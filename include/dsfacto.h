@@ -70,9 +70,9 @@ int dsfacto_create(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32_t p, 
  * Non-empty loads are put in order on the device itself when it has room for the buffers of a sort (about 26
  * bytes per stored entry for the duration of the call): the CSR copy that the recompute pass needs anyway is
  * turned into (pass, column, phase) keys and sorted by a stable radix sort, and kernels list the runs of entries
- * of a column and cut the entries into equal units of the update loop; only the CSR arrays cross the link, and
- * from 2^24 stored entries on they are sent while the host still checks them (a data set that fails the checks
- * leaves the handle as it was, as on every path).  A pass holds a band of rows whose auxiliaries fit L2; a data
+ * of a column and cut the entries into equal units of the update loop; only the CSR arrays cross the link.
+ * The arrays are checked on the device, where they lie beside the old data set until they have passed: a data set
+ * that fails the checks leaves the handle as it was (column shards: checked on the host).  A pass holds a band of rows whose auxiliaries fit L2; a data
  * set of one band has every column as one run in its full stratified order (DSFACTO_BANDS=B asks for B bands).
  * With row blocks per slot asked for (DSFACTO_DEBUG_ROW_MERGE, DSFACTO_ROW_MERGE) or a planted wait
  * (DSFACTO_DEBUG_EXTRA_NEED), tile lists are bucketed on the device instead and swept tile by tile, as they are
@@ -86,8 +86,8 @@ int dsfacto_create(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32_t p, 
  * for later loads; streamed loads of one process run one at a time.  The environment variable
  * DSFACTO_LOAD=stream streams smaller loads too, DSFACTO_LOAD=simple never streams; if the staging
  * memory cannot be had, the load falls back to one copy from pageable memory.  The resulting tile
- * lists are the same bit for bit on every path.  Page-locked caller arrays make the CSR copy overlap
- * the bucketing. */
+ * lists are the same bit for bit on every path.  Arrays in pageable memory are sent by several threads through
+ * page-locked slots; page-locked caller arrays are read by the device directly. */
 int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices,
                      const float *values, const float *y);
 

@@ -1,8 +1,7 @@
-// Tile bucketing on the device for large loads (Section 4.2's partition of the data into p x p blocks, the
-// order inside a block by (column, row)).  The host path of the library does the same with counting
-// sorts per row block; for a data set of a billion entries the host's scatter is slower than the link
-// (about 1.2 s against 0.3 s for the CSR arrays alone), so from 2^24 entries on the CSR copy that the
-// recompute pass needs anyway is bucketed where it already is:
+// Tile bucketing on the device (Section 4.2's partition of the data into p x p blocks, the order inside a block by
+// (column, row)) for the sweep over tiles (dsfacto_sgd.cuh).  Ordinary loads take the update loop by column runs
+// instead (dsfacto_runplan.cuh); this path serves the knobs that ask for tiles (row blocks per slot, a planted wait)
+// and data sets whose (pass, column, phase) does not fit a 32-bit key.
 //   1. tile_keys_kernel: per stored entry (i, j, x) a 32-bit key (slot, phase, local column, row block inside
 //      the slot) and a 64-bit payload (local row, bits of x), in CSR order;
 //   2. a stable radix sort of the pairs by key (cub::DeviceRadixSort, a library primitive): inside a

@@ -21,8 +21,7 @@ __device__ __forceinline__ uint32_t group_mask() {
 }
 
 // acc += c * r on four floats with two packed fp32x2 multiply-adds (each half rounds exactly as a scalar fmaf).
-// Used by the stratum SGD sweep (512-byte rows: 21.3 -> 19.4 ms per sweep of 400 M entries; 64-byte rows: no
-// change); the recompute pass got slower with it (14.4 -> 15.3 ms) and keeps scalar multiply-adds.
+// (512-byte rows in the tile sweep: 21.3 -> 19.4 ms per sweep of 400 M entries; 64-byte rows: no change.)
 __device__ __forceinline__ void fma4(float4 &acc, const float c, const float4 r) {
     const float2 cc = make_float2(c, c);
     const float2 lo = __ffma2_rn(make_float2(r.x, r.y), cc, make_float2(acc.x, acc.y));

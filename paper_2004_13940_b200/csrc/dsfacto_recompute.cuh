@@ -100,6 +100,12 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
 // The pairs of the first `hot` columns (the most frequent ones, when the columns are numbered that way) sit in shared
 // memory.
+// What bounds it: 64-byte rows of click logs (78 M entries, 615 us), the data and look-up stages of L1 (85 and 89 %
+// busy: every entry costs one look-up for its row and one for its pair) at 40 % issue; 128-byte rows (2.6 M entries,
+// 63 -> 44 us) a last round of rows that fills the SMs unevenly and latency; 512-byte rows (30 M entries, 1.0 ms) the
+// latency of gathers from L2 (47 % of its rate) with 16 resident warps.  Not kept: columns and values as records of 8
+// bytes (click logs 2.97 -> 3.35 ms per 390 M entries), rows taken longest first inside blocks of 256 (44 -> 42.5 us,
+// but click logs 2.97 -> 3.09 ms), two or four resident CTAs for 128-byte rows (46 and 43 us).
 template <int LG, int NV, bool STAGED = false>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;

@@ -1,4 +1,6 @@
-// Stratum SGD kernels of the DS-FACTO epoch for sm_100a.
+// Stratum SGD of the DS-FACTO epoch as a sweep over tiles, for sm_100a.  Data sets that are put in order on the device
+// take the update loop by column runs (dsfacto_runs.cuh), which uses the same algebra and has no waits; this sweep
+// serves tile lists that the host has built and the knobs that ask for tiles.
 //
 // With G_i and a_i frozen, one stored entry (i,j,x) maps (w_j, v_j) affinely
 // (eqs. (dsfacto_sgdupdatew), (dsfacto_sgdupdatev) regrouped):
