@@ -6,7 +6,7 @@ C4 synthetic workload (hashed categorical, n = 45M, d = 2^20, 39 entries per row
   value      inputs resident in HBM; CUDA events around exactly K epochs on the library's stream
   e2e        dsfacto_load_csr from host buffers (host->device copies, tile bucketing) + one epoch +
              the objective read back, through the C ABI
-  roofline   dominant kernel (stratum SGD): algorithmic bytes / measured launch time vs the
+  roofline   dominant phase (stratum SGD): algorithmic bytes / measured launch time vs the
              measured HBM copy peak
   cpu_baseline   the CPU oracle, as it stands, on a bounded row sample of the same workload
 
@@ -32,10 +32,10 @@ sys.path.insert(0, str(ROOT))
 METRIC = "nonzero-updates/sec"
 UNIT = "updates/s"
 ORACLE_SAMPLE_ROWS = 1_000_000
-# dram__bytes_read.sum + dram__bytes_write.sum of sgd_sweep_kernel per stored entry, by factor width K, from
-# the ncu captures summarised in profiles/ (scaled cases; DRAM traffic of the sweep grows with the entries).
-# A width without a capture of the current kernel reports traffic = null.
-SGD_DRAM_BYTES_PER_ENTRY = {16: 22.0, 128: 186.0}
+# dram__bytes_read.sum + dram__bytes_write.sum of the update loop's kernels (runs_sweep_kernel, runs_apply_kernel,
+# runs_fold_kernel) per stored entry, by factor width K, from the ncu captures summarised in profiles/ (scaled cases;
+# the DRAM traffic of the loop grows with the entries).  A width without a capture reports traffic = null.
+SGD_DRAM_BYTES_PER_ENTRY = {}
 
 
 def peaks():
@@ -305,9 +305,9 @@ def run_ours(args):
     peak, peak_kind = peaks()
     K, n, d, p = wl.K, wl.n, wl.d, wl.p
     # Stratum SGD, algorithmic bytes per epoch.  Row-block sweep (default): every array once - the 8-byte
-    # entry records, A and G once (all entries of a row meet in one launch), w and V read + written.
+    # entry records, A and G once (the entries of a band of rows meet in one pass), w and V read + written.
     # Round sweep: the p tiles of a round own disjoint row blocks, so every entry re-reads G_i and a_i.
-    # A plan cut into segments (--refresh-every) keeps the row-block sweep: one launch per segment, each of
+    # A plan cut into segments (--refresh-every) has passes of its own per segment, each segment of
     # which reads A and G of all rows and reads and writes w and V once.
     sweep = os.environ.get("DSFACTO_SWEEP", "rowblock")
     segments = -(-p // args.refresh_every) if 0 < args.refresh_every < p else 1
@@ -316,16 +316,18 @@ def run_ours(args):
     sgd_bytes = sgd_gather if sweep == "round" else sgd_floor
     ref_bytes = 8 * nnz + 8 * (n + 1) + 4 * d * (K + 2) + 4 * n * K + 8 * n
     sgd_s, ref_s = phase[1] * 1e-3, phase[2] * 1e-3
-    # the counters were taken on the default schedule (row-block sweep, one launch per sweep)
+    # the counters were taken on the default schedule
     per_entry = SGD_DRAM_BYTES_PER_ENTRY.get(K)
     traffic = None if (per_entry is None or sweep != "rowblock" or segments != 1) else per_entry * nnz
-    roof = {"bound": "hbm", "kernel": "sgd_sweep_kernel", "launches_per_step": segments, "sweep": sweep,
+    # the update loop of an epoch: everything but the recompute pass of each segment
+    loop_launches = max(1, round(launches / args.steps) - segments)
+    loop = "sgd_sweep_kernel" if sweep == "round" else "update loop (runs_sweep_kernel, runs_apply_kernel, runs_fold_kernel)"
+    roof = {"bound": "hbm", "kernel": loop, "launches_per_step": loop_launches, "sweep": sweep,
             "achieved": sgd_bytes / sgd_s / 1e9, "peak": peak, "unit": "GB/s", "frac": sgd_bytes / sgd_s / 1e9 / peak,
             "peak_kind": "of " + peak_kind, "traffic": traffic,
-            "algorithmic_bytes_per_launch": sgd_bytes / segments, "avg_launch_us": 1e6 * sgd_s / segments,
+            "algorithmic_bytes_per_launch": sgd_bytes / loop_launches, "avg_launch_us": 1e6 * sgd_s / loop_launches,
             "model": ("gather: nnz*(8+4K+4) + 8d(K+1)" if sweep == "round" else "stream floor: 8nnz + 4n(K+1) + 8d(K+1)")
-                     + ("; one launch covers the whole sweep" if segments == 1 else
-                        "; %d launches per sweep, A, G, w, V once per launch" % segments),
+                     + ("" if segments == 1 else "; %d segments per epoch, A, G, w, V once per segment" % segments),
             # bytes the sweep asks its caches for when nothing is reused in registers; most of them are served
             # by L2, so this rate is NOT a fraction of the HBM peak and is given for context only
             "cache_request_model": {"bytes_per_step": sgd_gather, "rate_GBps": sgd_gather / sgd_s / 1e9},
