@@ -1,0 +1,111 @@
+"""Edges of the ways a call takes between host and device: scoring batches that are staged through shared memory, read
+from mapped memory or copied; launches of an epoch one by one and as a graph; results in ordinary and in page-locked
+arrays; the entry point that allocates nothing at every factor width it takes."""
+import numpy as np
+import pytest
+
+from oracle import dsfacto_oracle as O
+from paper_2004_13940_b200 import dsfacto as D
+from paper_2004_13940_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("K", [5, 16, 32, 64, 128, 200])
+@pytest.mark.parametrize("m", [1, 40, 63, 64, 65, 290, 300, 310, 4000])
+def test_scoring_batches_of_every_size(m, K):
+    # 50 entries per row: 24 KB (staged) is passed between 58 and 60 rows, 127 KB (mapped) near 310; larger ones are copied
+    wl = W.make("C3", n=4000)
+    ip = wl.indptr[: m + 1].copy()
+    ix, v, y = wl.indices[: ip[-1]].copy(), wl.values[: ip[-1]].copy(), wl.y[:m].copy()
+    rng = np.random.default_rng(K)
+    w, V = (0.1 * rng.standard_normal(wl.d)).astype(np.float32), (0.1 * rng.standard_normal((wl.d, K))).astype(np.float32)
+    with D.DSFacto(1, wl.d, K, 1, D.LOGISTIC, 0.0, 0.0, 0.1, 1) as g:
+        g.set_params(0.25, w, V)
+        rows = np.repeat(np.arange(m), np.diff(ip))
+        x, Vx = v.astype(np.float64), v[:, None].astype(np.float64) * V[ix]
+        A = np.add.reduceat(Vx, ip[:-1], axis=0)      # (no row is empty)
+        f = 0.25 + np.bincount(rows, x * w[ix], m) + 0.5 * ((A * A).sum(1) - np.bincount(rows, (Vx * Vx).sum(1), m))
+        for _ in range(3):
+            np.testing.assert_allclose(g.predict(ip, ix, v), f, rtol=0, atol=2e-5 * (1 + np.abs(f).max()))
+        loss, acc = g.evaluate(ip, ix, v, y)
+        assert loss == pytest.approx(np.logaddexp(0.0, -y * f).mean(), rel=1e-5)
+        assert abs(acc - np.mean(y * f > 0)) * m <= np.count_nonzero(np.abs(f) <= 2e-5 * (1 + np.abs(f).max())) + 1e-9
+        # an unsound batch is refused on every way, and the next sound one is served
+        bad_ix, bad_v, bad_y = ix.copy(), v.copy(), y.copy()
+        bad_ix[-1], bad_v[-1], bad_y[-1] = wl.d, np.inf, np.nan
+        out = np.empty(m, np.float32)
+        assert D.dsfacto_predict(g._h, m, ip, bad_ix, v, out) == D.ERR_INVALID_CSR
+        assert D.dsfacto_predict(g._h, m, ip, ix, bad_v, out) == D.ERR_INVALID_CSR
+        assert D.dsfacto_evaluate(g._h, m, ip, ix, v, bad_y)[0] == D.ERR_INVALID_CSR
+        assert D.dsfacto_predict(g._h, m, ip, ix, v, out) == D.OK
+        np.testing.assert_allclose(out, f, rtol=0, atol=2e-5 * (1 + np.abs(f).max()))
+
+
+@pytest.mark.parametrize("every", [0, 2])
+def test_epochs_before_and_after_they_become_a_graph(every):
+    wl = W.make("C1")
+    o = O.Oracle(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, wl.init_seed)
+    o.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+    with D.DSFacto(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, wl.init_seed) as g:
+        g.set_refresh_every(every)
+        g.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+        before = g.launch_count()
+        g.epoch(), (o.epoch_segmented(every) if every else o.epoch())
+        per_epoch = g.launch_count() - before
+        for e in range(60):
+            if e == 25:      # other kernel arguments: the graph has to go
+                o.set_eta(0.5), g.set_eta(0.5)
+            if e == 45:      # other parameters: the graph stays
+                w, V = (0.9 * o.w).astype(np.float32), (0.9 * o.V).astype(np.float32)
+                g.set_params(0.1, w, V)
+                o.w0, o.w[:], o.V[:] = float(np.float32(0.1)), w, V
+                o.refresh()
+            before = g.launch_count()
+            want, got = (o.epoch_segmented(every) if every else o.epoch()), g.epoch()
+            assert got == pytest.approx(want, rel=1e-4), e
+            assert g.launch_count() - before == per_epoch
+        w0, w, V = g.get_params()
+        assert np.abs(w - o.w).max() <= 1e-4 * (1 + np.abs(o.w).max()) and np.all(np.abs(V - o.V) <= 1e-4 * (1 + np.abs(o.V)))
+
+
+@pytest.mark.parametrize("d,K", [(700, 45), (40_000, 20), (300_001, 7)])
+def test_parameters_come_back_whole(d, K):
+    # through the mailbox, through the driver, through several threads; several arrays alive at a time, and after a trim
+    rng = np.random.default_rng(d)
+    with D.DSFacto(1, d, K, 1, D.SQUARED, 0.0, 0.0, 0.1, 1) as g:
+        kept = []
+        for k in range(5):
+            w, V = rng.standard_normal(d).astype(np.float32), rng.standard_normal((d, K)).astype(np.float32)
+            g.set_params(float(k), w, V)
+            kept.append((g.get_params(), (float(k), w, V)))
+            if k == 2:
+                D.dsfacto_trim()
+        for (w0, w, V), (rw0, rw, rV) in kept:
+            assert w0 == rw0 and np.array_equal(w, rw) and np.array_equal(V, rV)
+
+
+@pytest.mark.parametrize("K", [4, 8, 16, 32, 64, 128, 256])
+@pytest.mark.parametrize("m", [1, 1003])
+def test_allocation_free_scoring_at_every_width(K, m):
+    import torch
+
+    wl = W.make("C3", n=1003)
+    ip = wl.indptr[: m + 1].copy()
+    ip[m // 2 + 1:] -= ip[m // 2 + 1] - ip[m // 2] if m > 1 else 0      # one row in the middle is empty
+    ix, v, y = wl.indices[: ip[-1]].copy(), wl.values[: ip[-1]].copy(), wl.y[:m].copy()
+    for i in range(m // 2, m):                                           # (rows behind it take what lies there)
+        ix[ip[i]:ip[i + 1]] = np.sort(np.random.default_rng(i).choice(wl.d, ip[i + 1] - ip[i], replace=False))
+    rng = np.random.default_rng(K)
+    w, V = (0.1 * rng.standard_normal(wl.d)).astype(np.float32), (0.1 * rng.standard_normal((wl.d, K))).astype(np.float32)
+    with D.DSFacto(1, wl.d, K, 1, D.LOGISTIC, 0.0, 0.0, 0.1, 1) as g:
+        g.set_params(0.25, w, V)
+        want = g.predict(ip, ix, v)
+        loss, _ = g.evaluate(ip, ix, v, y)
+    t = [torch.from_numpy(a).cuda() for a in (ip, ix, v, y, w, V)]
+    scores, sums = torch.empty(m, device="cuda"), torch.empty(2, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    assert D.dsfacto_score_loss_noalloc(m, wl.d, K, D.LOGISTIC, *[a.data_ptr() for a in t[:4]], 0.25, t[4].data_ptr(),
+                                        t[5].data_ptr(), scores.data_ptr(), sums.data_ptr()) == D.OK
+    np.testing.assert_allclose(scores.cpu().numpy(), want, rtol=0, atol=2e-5 * (1 + np.abs(want).max()))
+    assert float(sums[0]) == pytest.approx(loss * m, rel=1e-5)
