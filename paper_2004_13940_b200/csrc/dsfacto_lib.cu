@@ -442,7 +442,7 @@ void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threa
 }
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
-    const size_t smem = a.stage ? (size_t)a.stage_bytes : sizeof(float2) * (size_t)a.hot;
+    const size_t smem = a.stage ? (size_t)a.stage_bytes : 0;
     if (a.stage && mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate, false, true>, grid, kThreads, smem, a);
     else if (a.stage) launch_overlapped(h, refresh_kernel<LG, NV, kScore, false, true>, grid, kThreads, smem, a);
     else if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, smem, a);
@@ -832,8 +832,6 @@ void launch_finish(dsfacto *h, int grid) {
                                                             h->w0, h->loss);
 }
 
-constexpr int kHotPairs = 2048;   // pairs of the most frequent columns a CTA of the recompute pass keeps (16 KB)
-
 // V and the pairs (w_j, s_j) as the recompute pass reads them: by slot for the training rows when the load
 // renumbered the columns of the device CSR, by column index otherwise (and always for rows a caller passes).
 // Rebuilt only when the parameters changed since the last time: one pass over V (4 d Kp bytes read, twice
@@ -856,7 +854,6 @@ void model_view(dsfacto *h, RefreshArgs &a, bool training_rows) {
     }
     a.V = by_slot ? h->d_Vs : h->d_V;
     a.pair = by_slot ? h->d_pair_s : h->d_pair;
-    a.hot = by_slot ? std::min(h->d, kHotPairs) : 0;
 }
 
 // Renumbers the columns of the device CSR by frequency (see the kernels).  Decided per load: it pays when

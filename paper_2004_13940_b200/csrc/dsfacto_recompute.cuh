@@ -33,7 +33,6 @@ struct RefreshArgs {
     const float *val;
     const float *y;
     const float2 *pair;  // per column (w_j, s_j = sum_k v_jk^2)
-    int hot;             // pairs of the first columns that are worth keeping in shared memory
     const float *w;      // RAW: w instead of the pairs
     double *sums_out;    // kScoreSums
     const float *V;
@@ -98,14 +97,14 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // ahead of the multiply-adds.  Behind the end of a row its last entry is repeated with
 // x = 0.
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
-// The pairs of the first `hot` columns (the most frequent ones, when the columns are numbered that way) sit in shared
-// memory.
-// What bounds it: 64-byte rows of click logs (78 M entries, 615 us), the data and look-up stages of L1 (85 and 89 %
+// What bounds it: 64-byte rows of click logs (78 M entries, 0.60 ms), the data and look-up stages of L1 (85 and 89 %
 // busy: every entry costs one look-up for its row and one for its pair) at 40 % issue; 128-byte rows (2.6 M entries,
 // 63 -> 44 us) a last round of rows that fills the SMs unevenly and latency; 512-byte rows (30 M entries, 1.0 ms) the
 // latency of gathers from L2 (47 % of its rate) with 16 resident warps.  Not kept: columns and values as records of 8
-// bytes (click logs 2.97 -> 3.35 ms per 390 M entries), rows taken longest first inside blocks of 256 (44 -> 42.5 us,
-// but click logs 2.97 -> 3.09 ms), two or four resident CTAs for 128-byte rows (46 and 43 us).
+// bytes (2.97 -> 3.35 ms per 390 M entries of click logs); the pairs of the 2048 most frequent columns in shared memory,
+// which the L1 then lacks (2.95 -> 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms);
+// rows taken longest first inside blocks of 256 (text 44 -> 42.5 us, but click logs 2.97 -> 3.09 ms); two or four
+// resident CTAs for 128-byte rows (46 and 43 us).
 template <int LG, int NV, bool STAGED = false>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;
@@ -113,9 +112,9 @@ struct RefreshCfg {
     static constexpr int B = LG * E;
     // entries whose rows are requested together; a small batch (STAGED) has the GPU to itself and waits for nothing
     // but the latency of these requests, so it makes fewer and larger ones (32 rows of 39 entries: 25 -> 22 us per call)
-    static constexpr int UB = STAGED && NV <= 4 ? B / 2 : LG == 8 && NV == 1 ? 2 : 1;
+    static constexpr int UB = STAGED && NV <= 4 ? B / 2 : (LG == 8 && NV == 1) || LG == 4 ? 2 : 1;
     static constexpr int S = B / UB;                                        // steps per batch
-    static constexpr int NB = STAGED || NV >= 6 || LG == 1 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
+    static constexpr int NB = STAGED || NV >= 6 || LG == 1 || LG == 4 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
     static_assert(S % NB == 0, "a step keeps its registers from batch to batch");
     static constexpr int CTAS = STAGED ? 1 : LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
@@ -132,7 +131,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     float4 *A4 = reinterpret_cast<float4 *>(a.A);
     constexpr bool TRAIN = MODE == kTrain;
     constexpr bool STORE_A = MODE == kTrain || MODE == kPartial;
-    extern __shared__ __align__(16) float2 hot_pair[];
+    extern __shared__ __align__(16) uint4 staged[];   // STAGED: the batch
     // the fp64 sums of a lane group live in shared memory: only its first lane touches them, once per row
     __shared__ double sums[2][C::ROWS];
     if (l == 0) { sums[0][g] = 0.0; sums[1][g] = 0.0; }
@@ -142,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     const int32_t *idx = a.idx;
     const float *val = a.val, *lab = a.y;
     if (STAGED) {
-        uint4 *to = reinterpret_cast<uint4 *>(hot_pair);
+        uint4 *to = staged;
         for (int i = threadIdx.x; i < a.stage_bytes / 16; i += kThreads) to[i] = a.stage[i];
         const char *p = reinterpret_cast<const char *>(to);
         indptr = reinterpret_cast<const int64_t *>(p);
@@ -188,10 +187,6 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     wait_for_previous_kernel();
     if (TRAIN && a.st && blockIdx.x == 0 && threadIdx.x == 0) a.st->t1 = device_ns();
     const float w0 = TRAIN && a.st ? a.st->w0 : a.w0;
-    if (!RAW && a.hot > 0) {
-        for (int i = threadIdx.x; i < a.hot; i += kThreads) hot_pair[i] = a.pair[i];
-        __syncthreads();
-    }
     for (; base < n; base += step) {
         const int64_t row = base + gw, beg = nbeg;
         const int len = nlen;
@@ -228,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
                     if (RAW) {
                         lin = fmaf(a.w[j0[e]], x0[e], lin);
                     } else {
-                        const float2 ws = j0[e] < a.hot ? hot_pair[j0[e]] : a.pair[j0[e]];
+                        const float2 ws = a.pair[j0[e]];
                         lin = fmaf(ws.x, x0[e], lin);
                         q = fmaf(x0[e] * x0[e], ws.y, q);
                     }
