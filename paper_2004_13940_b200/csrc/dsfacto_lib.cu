@@ -1887,10 +1887,32 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
 }
 
 // ---- plan of the update loop by column runs (see dsfacto_runplan.cuh) ----
+// Bands: rows per pass such that their auxiliary rows, which every column of the pass reads, stay in L2.
+static int64_t band_count(const dsfacto *h) {
+    if (const char *env = std::getenv("DSFACTO_BANDS")) {
+        const int64_t v = std::atoll(env);
+        if (v >= 1 && v <= h->n) return v;
+    }
+    const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
+    return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
+}
+// Many bands of wide rows make many short runs, each of which moves its column's row and its record through memory
+// once per band, while the tile sweep only adds to it.  400 M entries of 512-byte rows over 2^20 columns in 30 bands (13
+// entries per column and band): update loop 23.3 ms by runs (8 / 16 / 22 bands: 25.9 / 23.1 / 22.8 ms), 18.7 ms by tiles;
+// 30 M entries of such rows with 77 entries per column and band: 1.25 ms against 2.24 ms; 1.755 G entries of 64-byte
+// rows, 40 entries per column and band: 19.0 ms against 20.0 ms.  The tile sweep needs a large data set and grid, or its
+// warps wait for one another.
+static bool tiles_move_less(const dsfacto *h, int64_t nnz) {
+    const bool segmented = h->refresh_every > 0 && h->refresh_every < h->p;
+    return h->Kp >= 64 && nnz >= ((int64_t)1 << 27) && h->p >= 128 && h->nshards == 1 && !segmented && !h->wide &&
+           bits_for((int64_t)h->p * h->p) + 1 + h->jbits <= 32 && !std::getenv("DSFACTO_BANDS") &&
+           (double)nnz < 24.0 * (double)h->d * (double)band_count(h);
+}
 // Whether this load takes it: every load that may be bucketed on the device, unless a knob asks for the tile sweep
 // (DSFACTO_SWEEP=round, row blocks per slot, the planted wait), as long as pass, column and phase fit a 32-bit key.
 static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env) {
     if (nnz <= 0 || h->sweep != 1 || h->row_merge > 0 || h->debug_extra_need > 0 || std::getenv("DSFACTO_ROW_MERGE")) return false;
+    if (tiles_move_less(h, nnz)) return false;
     if (load_env) { if (std::strcmp(load_env, "device") != 0) return false; }
     else {
         // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs
@@ -1901,15 +1923,6 @@ static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env)
         if ((double)(free_b + DevicePool::get().idle_bytes()) < need) return false;
     }
     return true;
-}
-// Bands: rows per pass such that their auxiliary rows, which every column of the pass reads, stay in L2.
-static int64_t band_count(const dsfacto *h) {
-    if (const char *env = std::getenv("DSFACTO_BANDS")) {
-        const int64_t v = std::atoll(env);
-        if (v >= 1 && v <= h->n) return v;
-    }
-    const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
-    return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
 }
 // d_indptr, d_idx, d_val hold the CSR arrays (copies queued on the stream).  Fills the entries, runs and units of
 // the passes.  Returns 1 if the data set does not fit this plan (nothing is left behind then).
