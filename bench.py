@@ -35,7 +35,7 @@ ORACLE_SAMPLE_ROWS = 1_000_000
 # dram__bytes_read.sum + dram__bytes_write.sum of the update loop's kernels (runs_sweep_kernel, runs_apply_kernel,
 # runs_fold_kernel) per stored entry, by factor width K, from the ncu captures summarised in profiles/ (scaled cases;
 # the DRAM traffic of the loop grows with the entries).  A width without a capture reports traffic = null.
-SGD_DRAM_BYTES_PER_ENTRY = {}
+SGD_DRAM_BYTES_PER_ENTRY = {16: 33.3}
 
 
 def peaks():
