@@ -97,7 +97,11 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
  *       w_j  <- w_j  - (eta/n) (G_i x + lambda_w w_j)                          eq. (dsfacto_sgdupdatew)
  *       v_jk <- v_jk - (eta/n) (G_i (x a_ik - v_jk x^2) + lambda_v v_jk)       eq. (dsfacto_sgdupdatev)
  *   recompute a_ik (eq. (compute_a_jk)), f_i (eq. (fm_model2)), G_i and the objective (eq. (fm_obj)).
- * Returns DSFACTO_ERR_DIVERGED if the new objective is not finite (state is kept). */
+ * Returns DSFACTO_ERR_DIVERGED if the new objective is not finite (state is kept).  If a launch is refused
+ * (DSFACTO_ERR_CUDA) before anything has run, the handle is as it was; if an epoch breaks off later, w and V are
+ * part of the way and the handle refuses further epochs until dsfacto_set_params replaces both or
+ * dsfacto_load_csr loads a data set.  (The same after a dsfacto_set_params or dsfacto_load_csr whose recompute
+ * pass was refused: A and G are then not those of the parameters.) */
 int dsfacto_epoch(dsfacto_t *h);
 
 /* Raw scores f(x_i), eq. (fm_model2), of m rows given as CSR (same rules as dsfacto_load_csr) with
@@ -202,10 +206,13 @@ int dsfacto_last_epoch_ms(dsfacto_t *h, float ms[4]);
  *                             entries and 1 MB of factors), 1 = always, 2 = never; the environment variable
  *                             DSFACTO_COLUMN_ORDER=0/1 does the same for every handle.  Nothing a caller passes
  *                             or receives is renumbered.
+ *   DSFACTO_DEBUG_REFUSE_LAUNCH the k-th kernel launch of this handle from now on (the launch of an epoch as a graph
+ *                             counts as one) is refused on the host, as if the driver had returned an error for
+ *                             it: the call it belongs to returns DSFACTO_ERR_CUDA.  0 = off.
  * The environment variable DSFACTO_SWEEP=round (read by dsfacto_create) stores and sweeps the tiles round by
  * round, exactly Algorithm 1's order, instead of row block by row block. */
 enum { DSFACTO_DEBUG_SPIN_LIMIT = 0, DSFACTO_DEBUG_EXTRA_NEED = 1, DSFACTO_DEBUG_CHUNK_LEN = 2, DSFACTO_DEBUG_COLUMN_ORDER = 3,
-       DSFACTO_DEBUG_ROW_MERGE = 4 };
+       DSFACTO_DEBUG_ROW_MERGE = 4, DSFACTO_DEBUG_REFUSE_LAUNCH = 5 };
 int dsfacto_debug_set(dsfacto_t *h, int32_t key, int64_t value);
 
 /* How the last dsfacto_load_csr built the tile lists: info[0] = 0 on the host with one copy, 1 on the host

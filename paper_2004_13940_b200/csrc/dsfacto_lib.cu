@@ -84,7 +84,7 @@ struct dsfacto {
     int sgd_grid = 0;           // CTAs of the persistent stratum SGD launch
     int spin_limit = kSgdSpinLimit;  // polls before a wait for an earlier tile gives up
     int debug_extra_need = 0;   // tests: added to the `need` of the first chunk at the next load, so that its wait runs out
-    bool failed = false;        // an SGD launch gave up; the parameters are unusable until they are set again
+    bool failed = false;        // an epoch broke off half-way; the parameters are unusable until they are set again
     float *d_records = nullptr, *d_Tb = nullptr, *d_Tw = nullptr;
     float4 *d_S = nullptr, *d_TS = nullptr;  // scale records of the scaled column state (zero outside the SGD phase)
     int *d_run_count = nullptr;
@@ -107,7 +107,9 @@ struct dsfacto {
     // scalars of an epoch on the device, and the mapped host memory its last kernel reports to
     EpochState *d_state = nullptr;
     EpochReport *report = nullptr;
-    unsigned long long report_seq = 0, epoch_seq = 0;
+    unsigned long long report_seq = 0, epoch_seq = 0;   // last number of a scoring or copying kernel; of a recompute pass (before_report)
+    cudaError_t launch_error = cudaSuccess;   // of the first launch that was refused since the last look (launch_status)
+    int refuse_launch = 0;                    // tests: the launch that this counts down to is refused
     cudaGraphExec_t epoch_graph = nullptr;   // the launches of an epoch (all but the sweep over tiles and shards)
     int epochs_run = 0;
     int64_t epoch_launches = 0;
@@ -399,6 +401,55 @@ void free_data(dsfacto *h) {
 // ---------------------------------------------------------------------------------------------
 // kernel dispatch over the factor-row layout
 // ---------------------------------------------------------------------------------------------
+// Launches.  A refused launch is noted in the handle, and the launches behind it are left out: they would work on what
+// the refused one has not written.  launch_status tells afterwards, and starts afresh.
+inline bool refused(dsfacto *h, cudaError_t e) {
+    if (e == cudaSuccess) return false;
+    cudaGetLastError();
+    h->launch_error = e;
+    return true;
+}
+inline bool planted_refusal(dsfacto *h) { return h->refuse_launch > 0 && --h->refuse_launch == 0; }
+template <typename... P, typename... A>
+void launch_as(dsfacto *h, bool overlapped, void (*kernel)(P...), int64_t grid, int threads, size_t smem, const A &...args) {
+    if (h->launch_error != cudaSuccess) return;
+    if (planted_refusal(h)) { h->launch_error = cudaErrorLaunchOutOfResources; return; }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlapped ? 1 : 0;
+    if (!refused(h, cudaLaunchKernelEx(&cfg, kernel, args...))) h->launches += 1;
+}
+// A launch that may start its prologue while the kernel before it on the stream is still running (programmatic
+// stream serialisation); every kernel launched this way waits (griddepcontrol.wait) before it reads what earlier
+// kernels wrote or writes what they read.
+template <typename... P, typename... A>
+void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threads, size_t smem, const A &...args) {
+    launch_as(h, true, kernel, grid, threads, smem, args...);
+}
+template <typename... P, typename... A>
+void launch(dsfacto *h, void (*kernel)(P...), int64_t grid, int threads, size_t smem, const A &...args) {
+    launch_as(h, false, kernel, grid, threads, smem, args...);
+}
+// Whether every launch since the last look was accepted.
+cudaError_t launch_error(dsfacto *h) {
+    const cudaError_t noted = h->launch_error, left = cudaGetLastError();   // (left: by a sort)
+    h->launch_error = cudaSuccess;
+    return noted != cudaSuccess ? noted : left;
+}
+int launch_status(dsfacto *h) {
+    const cudaError_t e = launch_error(h);
+    if (e == cudaSuccess) return DSFACTO_OK;
+    h->err = std::string("kernel launch: ") + cudaGetErrorString(e);
+    return DSFACTO_ERR_CUDA;
+}
+
 template <int LG, int NV>
 void launch_sgd(dsfacto *h, const SgdArgs &a, int64_t chunks) {
     const size_t bytes = (size_t)kSgdWarps * sgd_warp_smem<LG, NV>(h->wide, h->block_len);
@@ -419,26 +470,8 @@ void launch_sgd(dsfacto *h, const SgdArgs &a, int64_t chunks) {
     }
     const int64_t want = (chunks + kSgdWarps - 1) / kSgdWarps;
     const int grid = (int)std::min<int64_t>(h->sgd_grid, std::max<int64_t>(want, 1));
-    if (h->wide) sgd_sweep_kernel<LG, NV, true><<<grid, kSgdThreads, bytes, h->stream>>>(a);
-    else sgd_sweep_kernel<LG, NV, false><<<grid, kSgdThreads, bytes, h->stream>>>(a);
-}
-// A launch that may start its prologue while the kernel before it on the stream is still running (programmatic
-// stream serialisation); every kernel launched this way waits (griddepcontrol.wait) before it reads what earlier
-// kernels wrote or writes what they read.
-template <typename... P, typename... A>
-void launch_overlapped(dsfacto *h, void (*kernel)(P...), int64_t grid, int threads, size_t smem, const A &...args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = h->stream;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);   // (an error is picked up by the cudaGetLastError at the end of the call)
-    h->launches += 1;
+    if (h->wide) launch(h, sgd_sweep_kernel<LG, NV, true>, grid, kSgdThreads, bytes, a);
+    else launch(h, sgd_sweep_kernel<LG, NV, false>, grid, kSgdThreads, bytes, a);
 }
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
@@ -764,15 +797,11 @@ void run_sgd_phase(dsfacto *h, int64_t L0, int64_t L1) {
     const int64_t chunks = h->launch_ptr[(size_t)last] - h->launch_ptr[(size_t)first];
     a.desc = h->d_desc + h->launch_ptr[(size_t)first];
     a.nchunks = (int)chunks;
-    if (chunks > 0) {
-        DSF_DISPATCH(h, launch_sgd, h, a, chunks);
-        h->launches += 1;
-    }
+    if (chunks > 0) DSF_DISPATCH(h, launch_sgd, h, a, chunks);
     {   // back from the scaled state to plain (w, V); folds the tail composites in after a row-block sweep
         const int grid = h->sm_count * 8;
-        sgd_finalize_v_kernel<<<grid, kThreads, 0, h->stream>>>(h->d_V, h->d_Tb, h->d_S, h->d_TS, h->d, h->Kp / 4);
-        sgd_finalize_w_kernel<<<grid, kThreads, 0, h->stream>>>(h->d_w, h->d_Tw, h->d_S, h->d_TS, h->d, log1m_ew);
-        h->launches += 2;
+        launch(h, sgd_finalize_v_kernel, grid, kThreads, 0, h->d_V, h->d_Tb, h->d_S, h->d_TS, h->d, h->Kp / 4);
+        launch(h, sgd_finalize_w_kernel, grid, kThreads, 0, h->d_w, h->d_Tw, h->d_S, h->d_TS, h->d, log1m_ew);
     }
 }
 
@@ -828,8 +857,7 @@ void run_strata(dsfacto *h, int64_t seg, double share) {
 
 template <int LG, int NV>
 void launch_finish(dsfacto *h, int grid) {
-    finish_kernel<LG, NV><<<grid, kThreads, 0, h->stream>>>(h->n, h->d_A, h->d_lin, h->d_q, h->d_y, h->d_G, h->d_partials,
-                                                            h->w0, h->loss);
+    launch(h, finish_kernel<LG, NV>, grid, kThreads, 0, h->n, h->d_A, h->d_lin, h->d_q, h->d_y, h->d_G, h->d_partials, h->w0, h->loss);
 }
 
 // V and the pairs (w_j, s_j) as the recompute pass reads them: by slot for the training rows when the load
@@ -845,12 +873,10 @@ void model_view(dsfacto *h, RefreshArgs &a, bool training_rows) {
         while (gs < kp4 && gs < 16) gs *= 2;   // (as the update loop's lane groups: the same sums of squares, bit for bit)
         const int64_t groups_per_cta = kThreads / gs;
         const int grid = (int)std::min<int64_t>(((int64_t)h->d + groups_per_cta - 1) / groups_per_cta, (int64_t)h->sm_count * 16);
-        model_view_kernel<<<grid, kThreads, 0, h->stream>>>(reinterpret_cast<const float4 *>(h->d_V), h->d_w,
-                                                             by_slot ? h->d_column_of : nullptr, (int64_t)h->d, kp4, gs,
-                                                             by_slot ? reinterpret_cast<float4 *>(h->d_Vs) : nullptr,
-                                                             by_slot ? h->d_pair_s : h->d_pair);
-        h->launches += 1;
-        version = h->model_version;
+        launch(h, model_view_kernel, grid, kThreads, 0, reinterpret_cast<const float4 *>(h->d_V), h->d_w,
+               by_slot ? h->d_column_of : nullptr, (int64_t)h->d, kp4, gs, by_slot ? reinterpret_cast<float4 *>(h->d_Vs) : nullptr,
+               by_slot ? h->d_pair_s : h->d_pair);
+        if (h->launch_error == cudaSuccess) version = h->model_version;
     }
     a.V = by_slot ? h->d_Vs : h->d_V;
     a.pair = by_slot ? h->d_pair_s : h->d_pair;
@@ -886,6 +912,7 @@ int order_columns(dsfacto *h) {
     auto fail = [&](cudaError_t e) {
         h->err = std::string("column order: ") + cudaGetErrorString(e);
         cudaStreamSynchronize(h->stream);
+        launch_error(h);
         cleanup();
         return e == cudaErrorMemoryAllocation ? DSFACTO_ERR_OOM : DSFACTO_ERR_CUDA;
     };
@@ -898,15 +925,14 @@ int order_columns(dsfacto *h) {
     const int grid = (int)std::min<int64_t>((h->nnz + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     const int dgrid = (int)std::min<int64_t>(((int64_t)d + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     if ((e = cudaMemsetAsync(d_slot_of, 0, sizeof(int32_t) * d, h->stream)) != cudaSuccess) return fail(e);
-    column_count_kernel<<<grid, kThreads, 0, h->stream>>>(h->d_idx, h->nnz, d_slot_of);
-    column_keys_kernel<<<dgrid, kThreads, 0, h->stream>>>(d_slot_of, (int64_t)d, d_key, d_col);
+    launch(h, column_count_kernel, grid, kThreads, 0, h->d_idx, h->nnz, d_slot_of);
+    launch(h, column_keys_kernel, dgrid, kThreads, 0, d_slot_of, (int64_t)d, d_key, d_col);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, d_key, d_key_out, d_col, h->d_column_of, (int64_t)d, 0, 32,
                                              h->stream)) != cudaSuccess)
         return fail(e);
-    column_slots_kernel<<<dgrid, kThreads, 0, h->stream>>>(h->d_column_of, (int64_t)d, d_slot_of);
-    column_rename_kernel<<<grid, kThreads, 0, h->stream>>>(h->d_idx, h->nnz, d_slot_of);
-    h->launches += 4;
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    launch(h, column_slots_kernel, dgrid, kThreads, 0, h->d_column_of, (int64_t)d, d_slot_of);
+    launch(h, column_rename_kernel, grid, kThreads, 0, h->d_idx, h->nnz, d_slot_of);
+    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess || (e = launch_error(h)) != cudaSuccess) return fail(e);
     h->d_slot_of = d_slot_of;
     d_slot_of = nullptr;
     cleanup();
@@ -926,7 +952,8 @@ int run_partial_refresh(dsfacto *h) {
     cudaEventRecord(h->ev[2], h->stream);   // (the epoch's phase timers expect both marks)
     cudaEventRecord(h->ev[3], h->stream);
     CU_TRY(h, cudaStreamSynchronize(h->stream));
-    CU_TRY(h, cudaGetLastError());
+    const int rc = launch_status(h);
+    if (rc) return rc;
     h->awaiting_sum = true;
     return DSFACTO_OK;
 }
@@ -935,17 +962,16 @@ int run_partial_refresh(dsfacto *h) {
 // norms of the shard's own columns.
 int run_finish(dsfacto *h) {
     DSF_DISPATCH(h, launch_finish, h, h->refresh_grid);
-    reduce2_kernel<<<1, kThreads, 0, h->stream>>>(h->d_partials, h->refresh_grid, h->d_scal);
+    launch(h, reduce2_kernel, 1, kThreads, 0, h->d_partials, h->refresh_grid, h->d_scal);
     double *np = h->d_partials + 2 * (size_t)h->refresh_grid;
     const int64_t cols = h->col_hi - h->col_lo;
-    sqnorm_kernel<<<h->norm_grid, kThreads, 0, h->stream>>>(h->d_w + h->col_lo, cols, h->d_V + (size_t)h->col_lo * h->Kp,
-                                                            cols * h->Kp, np);
-    reduce2_kernel<<<1, kThreads, 0, h->stream>>>(np, h->norm_grid, h->d_scal + 2);
-    h->launches += 4;
+    launch(h, sqnorm_kernel, h->norm_grid, kThreads, 0, h->d_w + h->col_lo, cols, h->d_V + (size_t)h->col_lo * h->Kp, cols * h->Kp, np);
+    launch(h, reduce2_kernel, 1, kThreads, 0, np, h->norm_grid, h->d_scal + 2);
     double s[4];
     CU_TRY(h, cudaMemcpyAsync(s, h->d_scal, sizeof s, cudaMemcpyDeviceToHost, h->stream));
     CU_TRY(h, cudaStreamSynchronize(h->stream));
-    CU_TRY(h, cudaGetLastError());
+    const int rc = launch_status(h);
+    if (rc) return rc;
     h->loss_sum = s[0]; h->g_sum = s[1]; h->w2 = s[2]; h->v2 = s[3];
     // the regulariser share of the other shards is missing here: the caller adds the shares up
     h->objective = s[0] / (double)h->n + 0.5 * (double)h->lambda_w * s[2] + 0.5 * (double)h->lambda_v * s[3];
@@ -953,9 +979,15 @@ int run_finish(dsfacto *h) {
     return DSFACTO_OK;
 }
 
-// Waits until a kernel has delivered its report (the last thing it does): number `want` in `at`.  The stream is
-// asked now and then, so that a failed launch ends the wait.
+// Waits until a kernel has delivered its report (the last thing it does): number `want` in `at`.  If a launch was
+// refused there will be none: what was launched is waited for instead.  The stream is asked now and then, so that a
+// kernel that failed ends the wait as well.
 int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long long want) {
+    const int rc = launch_status(h);
+    if (rc) {
+        cudaStreamSynchronize(h->stream);
+        return rc;
+    }
     for (unsigned spin = 1; at != want; ++spin) {
         _mm_pause();
         if ((spin & 0x3FFFu) != 0) continue;
@@ -965,7 +997,6 @@ int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long
         h->err = std::string("report: ") + (e == cudaSuccess ? "the last kernel left none" : cudaGetErrorString(e));
         return DSFACTO_ERR_CUDA;
     }
-    CU_TRY(h, cudaGetLastError());
     return DSFACTO_OK;
 }
 
@@ -984,24 +1015,27 @@ int run_refresh(dsfacto *h, bool first, bool report) {
     DSF_DISPATCH_REFRESH(h, h, a, kTrain, h->refresh_grid);
     return DSFACTO_OK;
 }
+// The device counts the reports of recompute passes.  What the host waits for is the number after the one that lies in
+// the report before the launches, so a pass that never ran leaves the two counts in step.
+void before_report(dsfacto *h) { h->epoch_seq = *const_cast<const volatile unsigned long long *>(&h->report->epochs); }
 // ... and its sums on the host
 int collect(dsfacto *h) {
     if (h->nshards > 1) return DSFACTO_OK;
-    const int rc = wait_report(h, h->report->epochs, ++h->epoch_seq);
+    const int rc = wait_report(h, h->report->epochs, h->epoch_seq + 1);
     if (rc) return rc;
     const EpochReport r = *h->report;
     h->loss_sum = r.loss; h->g_sum = r.g; h->w2 = r.w2; h->v2 = r.v2; h->w0 = r.w0;
     h->objective = r.loss / (double)h->n + 0.5 * (double)h->lambda_w * r.w2 + 0.5 * (double)h->lambda_v * r.v2;
     return DSFACTO_OK;
 }
-// ... with the host's w0
+// ... with the host's w0.  If it cannot be had, the auxiliaries are not those of the parameters.
 int refresh_now(dsfacto *h) {
-    if (h->nshards == 1) {
-        epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
-        h->launches += 1;
-    }
-    const int rc = run_refresh(h, true, true);
-    return rc ? rc : collect(h);
+    before_report(h);
+    if (h->nshards == 1) launch(h, epoch_begin_kernel, 1, 1, 0, h->d_state, h->w0);
+    int rc = run_refresh(h, true, true);
+    if (!rc) rc = collect(h);
+    if (rc) h->failed = true;
+    return rc;
 }
 
 // Results to the caller: small ones through the mailbox, with one wait for all of them.
@@ -1042,14 +1076,14 @@ int upload_rows(dsfacto *h, float *dst_dev, const float *src, int64_t rows) {
     cudaError_t e = Courier::get().move(true, {{packed, const_cast<float *>(src), sizeof(float) * (size_t)rows * h->K}}, h->stream);
     if (e == cudaSuccess && packed != dst_dev) {
         const int grid = (int)std::min<int64_t>((rows * h->Kp + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
-        pad_rows_kernel<<<grid, kThreads, 0, h->stream>>>(packed, rows, h->K, h->Kp, dst_dev);
-        h->launches += 1;
+        launch(h, pad_rows_kernel, grid, kThreads, 0, packed, rows, h->K, h->Kp, dst_dev);
     }
     const cudaError_t e2 = cudaStreamSynchronize(h->stream);
     if (packed != dst_dev) dev_free(packed);
+    rc = launch_status(h);
     CU_TRY(h, e);
     CU_TRY(h, e2);
-    return DSFACTO_OK;
+    return rc;
 }
 int upload_V(dsfacto *h, const float *V) {
     h->model_version += 1;
@@ -1062,11 +1096,11 @@ int download_rows(dsfacto *h, float *dst, float *src_dev, int64_t rows, Fetch mo
     if (h->Kp != h->K) {
         if ((rc = dev_alloc(h, &packed, (size_t)rows * h->K))) return rc;
         const int grid = (int)std::min<int64_t>((rows * h->K + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
-        unpad_rows_kernel<<<std::max(grid, 1), kThreads, 0, h->stream>>>(src_dev, rows, h->K, h->Kp, packed);
-        h->launches += 1;
+        launch(h, unpad_rows_kernel, std::max(grid, 1), kThreads, 0, src_dev, rows, h->K, h->Kp, packed);
     }
     more.add(packed, dst, sizeof(float) * (size_t)rows * h->K);
-    rc = fetch(h, more);
+    rc = launch_status(h);
+    if (!rc) rc = fetch(h, more);
     if (packed != src_dev) {
         if (rc) cudaStreamSynchronize(h->stream);
         dev_free(packed);
@@ -1076,8 +1110,7 @@ int download_rows(dsfacto *h, float *dst, float *src_dev, int64_t rows, Fetch mo
 
 void launch_validate(dsfacto *h, int64_t m, int64_t nnz, const int64_t *indptr, const int32_t *idx, const float *val, const float *y, int *bad) {
     const int grid = (int)std::min<int64_t>((m + kThreads / 32 - 1) / (kThreads / 32), (int64_t)h->sm_count * 16);
-    validate_rows_kernel<<<grid, kThreads, 0, h->stream>>>(m, nnz, h->d, indptr, idx, val, y, bad);
-    h->launches += 1;
+    launch(h, validate_rows_kernel, grid, kThreads, 0, m, nnz, h->d, indptr, idx, val, y, bad);
 }
 
 // CSR checks on the host (shards, the host bucketer).  Returns DSFACTO_OK or DSFACTO_ERR_INVALID_CSR.
@@ -1596,14 +1629,14 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
     if ((e = cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream)) == cudaSuccess &&
         (e = cudaMemsetAsync(h->d_w, 0, sizeof(float) * (size_t)d, h->stream)) == cudaSuccess &&
         (e = cudaMemsetAsync(d_listed, 0, sizeof(int), h->stream)) == cudaSuccess) {
-        init_factors_kernel<<<init_grid, kThreads, 0, h->stream>>>(seed, d, K, h->Kp, h->d_V, d_listed, list, kListed);
-        h->launches += 1;
+        launch(h, init_factors_kernel, init_grid, kThreads, 0, seed, d, K, h->Kp, h->d_V, d_listed, list, kListed);
         if ((e = cudaMemcpyAsync(h->d_row_start, h->row_start.data(), sizeof(int64_t) * ((size_t)p + 1), cudaMemcpyHostToDevice, h->stream)) == cudaSuccess &&
             (e = cudaMemcpyAsync(h->d_col_start, h->col_start.data(), sizeof(int32_t) * ((size_t)p + 1), cudaMemcpyHostToDevice, h->stream)) == cudaSuccess &&
             (e = cudaMemcpyAsync(&listed, d_listed, sizeof(int), cudaMemcpyDeviceToHost, h->stream)) == cudaSuccess)
             e = cudaStreamSynchronize(h->stream);
     }
-    rc = e == cudaSuccess ? DSFACTO_OK : DSFACTO_ERR_CUDA;
+    rc = launch_status(h);   // (V is not drawn if the launch was refused)
+    if (e != cudaSuccess) rc = DSFACTO_ERR_CUDA;
     if (!rc && listed > kListed) {   // (not with a generator that works) everything from the host
         std::vector<float> V;
         try { V.resize((size_t)d * K); } catch (const std::bad_alloc &) { rc = DSFACTO_ERR_OOM; }
@@ -1768,6 +1801,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     auto fail = [&](cudaError_t e) {
         h->err = std::string("device bucketing: ") + cudaGetErrorString(e);
         cudaStreamSynchronize(st);
+        launch_error(h);
         cleanup();
         return e == cudaErrorMemoryAllocation ? DSFACTO_ERR_OOM : DSFACTO_ERR_CUDA;
     };
@@ -1791,11 +1825,11 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     ka.sweep = h->sweep; ka.jbits = h->jbits; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start;
     ka.rbits = h->rbits; ka.slot_rows = (int32_t)slot_rows;
     ka.key = key[0]; ka.payload = pay[0];
-    tile_keys_kernel<<<wide_grid, kThreads, 0, st>>>(ka);
+    launch(h, tile_keys_kernel, wide_grid, kThreads, 0, ka);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, key[0], key[1], pay[0], pay[1], nnz, 0, kb, st)) != cudaSuccess)
         return fail(e);
-    pack_entries_kernel<<<wide_grid, kThreads, 0, st>>>(nnz, key[1], pay[1], h->jbits, h->rbits, h->d_ent);
-    tile_bounds_kernel<<<(int)std::min<int64_t>((nt + kThreads) / kThreads, wide_grid), kThreads, 0, st>>>(nnz, key[1], low_bits, nt, d_tp);
+    launch(h, pack_entries_kernel, wide_grid, kThreads, 0, nnz, key[1], pay[1], h->jbits, h->rbits, h->d_ent);
+    launch(h, tile_bounds_kernel, (int)std::min<int64_t>((nt + kThreads) / kThreads, wide_grid), kThreads, 0, nnz, key[1], low_bits, nt, d_tp);
     // the chunk plan: count per tile, then write.  The plain plan visits the tiles in slot order, so the kernel
     // can write complete descriptors straight into the handle's array; a plan cut into segments (second
     // schedule) gets the per-tile pieces and is put in order on the host as in the host path.
@@ -1806,8 +1840,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     pa.rbits = h->rbits; pa.slot_rows = (int32_t)slot_rows;
     pa.count = d_plan; pa.runs = d_plan + nt; pa.recs = d_plan + 2 * nt;
     pa.p = h->p; pa.sweep = h->sweep; pa.row_start = h->d_row_start; pa.col_start = h->d_col_start;
-    plan_tiles_kernel<kPlanCount><<<wide_grid, kThreads, 0, st>>>(pa);
-    h->launches += 4;
+    launch(h, plan_tiles_kernel<kPlanCount>, wide_grid, kThreads, 0, pa);
     std::vector<int64_t> cnt, in;   // cnt: counts, runs, recs per tile; in: first (nt + 1), need, run0, rec0
     try {
         h->tile_ptr.assign((size_t)nt + 1, 0);
@@ -1816,7 +1849,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     } catch (const std::bad_alloc &) { cudaStreamSynchronize(st); cleanup(); return DSFACTO_ERR_OOM; }
     if ((e = cudaMemcpyAsync(h->tile_ptr.data(), d_tp, sizeof(int64_t) * ((size_t)nt + 1), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(cnt.data(), d_plan, sizeof(int64_t) * 3 * (size_t)nt, cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess)
+        (e = cudaStreamSynchronize(st)) != cudaSuccess || (e = launch_error(h)) != cudaSuccess)
         return fail(e);
     int64_t *first = in.data(), *need = first + nt + 1, *run0 = need + nt, *rec0 = run0 + nt;
     int64_t total = 0, runs = 0, recs = 0;
@@ -1852,8 +1885,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
         if (total > 0) {
             if ((rc = dev_alloc(h, &d_out, (size_t)total))) { cudaStreamSynchronize(st); cleanup(); return rc; }
             pa.out = d_out;
-            plan_tiles_kernel<kPlanPieces><<<wide_grid, kThreads, 0, st>>>(pa);
-            h->launches += 1;
+            launch(h, plan_tiles_kernel<kPlanPieces>, wide_grid, kThreads, 0, pa);
             if ((e = cudaMemcpyAsync(pb.bulk.data(), d_out, sizeof(ChunkDesc) * (size_t)total, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
                 return fail(e);
         }
@@ -1875,13 +1907,12 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
             return fail(e);
         if (total > 0) {
             pa.out = h->d_desc;
-            plan_tiles_kernel<kPlanFull><<<wide_grid, kThreads, 0, st>>>(pa);
-            h->launches += 1;
-            if (h->debug_extra_need > 0) plan_extra_need_kernel<<<1, 1, 0, st>>>(h->d_desc, h->debug_extra_need);
+            launch(h, plan_tiles_kernel<kPlanFull>, wide_grid, kThreads, 0, pa);
+            if (h->debug_extra_need > 0) launch(h, plan_extra_need_kernel, 1, 1, 0, h->d_desc, h->debug_extra_need);
         }
         pb.finished = true;
     }
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess || (e = launch_error(h)) != cudaSuccess) return fail(e);
     cleanup();
     return DSFACTO_OK;
 }
@@ -1946,6 +1977,7 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     auto fail = [&](cudaError_t e) {
         h->err = std::string("run plan: ") + cudaGetErrorString(e);
         cudaStreamSynchronize(st);
+        launch_error(h);
         cleanup();
         return e == cudaErrorMemoryAllocation ? DSFACTO_ERR_OOM : DSFACTO_ERR_CUDA;
     };
@@ -1968,22 +2000,21 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     ka.n = h->n; ka.nnz = nnz; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p; ka.cbits = cbits;
     ka.bands = (int32_t)bands; ka.band_rows = (h->n + bands - 1) / bands; ka.every = (int32_t)every; ka.row_start = h->d_row_start;
     ka.key = key[0]; ka.payload = pay[0];
-    run_keys_kernel<<<(int)std::min<int64_t>((h->n + 7) / 8, wide_grid), kThreads, 0, st>>>(ka);
+    launch(h, run_keys_kernel, (int)std::min<int64_t>((h->n + 7) / 8, wide_grid), kThreads, 0, ka);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
     const uint32_t *sorted = kbuf.Current();
-    pass_bounds_kernel<<<(int)((npass + kThreads) / kThreads), kThreads, 0, st>>>(nnz, sorted, low_bits, (int)npass, d_bounds);
-    run_count_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(nnz, sorted, drop, d_count);
-    run_scan_kernel<<<1, 1024, 0, st>>>(d_count, blocks);
-    pass_runs_kernel<<<(int)((npass * 32 + 32 + kThreads - 1) / kThreads), kThreads, 0, st>>>(nnz, sorted, drop, d_count, (int)npass, d_bounds,
+    launch(h, pass_bounds_kernel, (int)((npass + kThreads) / kThreads), kThreads, 0, nnz, sorted, low_bits, (int)npass, d_bounds);
+    launch(h, run_count_kernel, (unsigned)blocks, kThreads, 0, nnz, sorted, drop, d_count);
+    launch(h, run_scan_kernel, 1, 1024, 0, d_count, blocks);
+    launch(h, pass_runs_kernel, (int)((npass * 32 + 32 + kThreads - 1) / kThreads), kThreads, 0, nnz, sorted, drop, d_count, (int)npass, d_bounds,
                                                                                              d_bounds + npass + 1);
-    h->launches += 5;
     std::vector<int64_t> bounds;
     try {
         bounds.resize(2 * ((size_t)npass + 1));
         h->passes.assign((size_t)npass, RunPass());
     } catch (const std::bad_alloc &) { cudaStreamSynchronize(st); cleanup(); return DSFACTO_ERR_OOM; }
     if ((e = cudaMemcpyAsync(bounds.data(), d_bounds, sizeof(int64_t) * bounds.size(), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess)
+        (e = cudaStreamSynchronize(st)) != cudaSuccess || (e = launch_error(h)) != cudaSuccess)
         return fail(e);
     const int64_t *first = bounds.data(), *run_first = first + npass + 1;
     int64_t longest = 0, most_runs = 1;
@@ -2022,15 +2053,13 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     RunWriteArgs wa{};
     wa.nnz = nnz; wa.key = sorted; wa.drop = drop; wa.low_bits = low_bits; wa.cbits = cbits; wa.count = d_count; wa.bounds = d_bounds;
     wa.ent = reinterpret_cast<uint2 *>(pbuf.Current()); wa.run_start = h->d_run_start; wa.run_key = h->d_run_key;
-    run_write_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(wa);
-    h->launches += 1;
+    launch(h, run_write_kernel, (unsigned)blocks, kThreads, 0, wa);
     for (const RunPass &ps : h->passes) {
         if (ps.units == 0) continue;
         const int grid = (int)std::min<int64_t>((ps.units + kThreads - 1) / kThreads, wide_grid);
-        unit_runs_kernel<<<grid, kThreads, 0, st>>>(h->d_run_start + ps.run_first, ps.nruns, ps.units, h->unit_len, h->d_unit_run + ps.unit_first);
-        h->launches += 1;
+        launch(h, unit_runs_kernel, grid, kThreads, 0, h->d_run_start + ps.run_first, ps.nruns, ps.units, h->unit_len, h->d_unit_run + ps.unit_first);
     }
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess || (e = launch_error(h)) != cudaSuccess) return fail(e);
     h->d_ent = reinterpret_cast<uint2 *>(pbuf.Current());   // the sorted payloads are the entry records
     pay[pbuf.selector] = nullptr;
     cleanup();
@@ -2076,7 +2105,8 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
             launch_validate(h, n, nnz, pending.indptr, pending.idx, pending.val, pending.y, &h->report->bad);
             e = cudaStreamSynchronize(h->stream);
         }
-        if (e == cudaSuccess) e = cudaGetLastError();
+        const cudaError_t launched = launch_error(h);
+        if (e == cudaSuccess) e = launched;
         const bool bad = h->report->bad != 0;
         h->report->bad = 0;
         if (e != cudaSuccess || bad) {
@@ -2252,20 +2282,14 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
     return std::isfinite(h->objective) ? DSFACTO_OK : DSFACTO_ERR_DIVERGED;
 }
 
-// An SGD launch gave up (a bounded wait ran out, or a check of the debug build failed): the warps left
-// in the middle of the sweep, so the parameters and the scaled state are a mixture.  The bookkeeping of
-// the sweep is cleared and the handle refuses further epochs until the parameters are set again
-// (dsfacto_set_params with w and V) or a data set is loaded after that.
-static int sgd_gave_up(dsfacto *h, const int code[3]) {
+// An epoch broke off: parameters and scaled state are a mixture.  The bookkeeping of the update loop is cleared and
+// the handle refuses further epochs until the parameters are set again (dsfacto_set_params with w and V) or a data
+// set is loaded after that.
+static int broke_off(dsfacto *h) {
     h->failed = true;
-    char buf[160];
-    if (code[0] == 1) std::snprintf(buf, sizeof buf, "stratum SGD: a wait for an earlier tile of the same column block timed out");
-    else if (code[0] == 2) std::snprintf(buf, sizeof buf, "stratum SGD: a copy of entry records into shared memory did not arrive");
-    else std::snprintf(buf, sizeof buf, "stratum SGD: debug check %d failed (value %d)", code[1], code[2]);
-    h->err = buf;
+    drop_epoch_graph(h);
     const size_t d = (size_t)h->d;
     cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream);
-    h->epoch_seq = 0;
     h->report->epochs = 0;
     if (!h->runs) {
         cudaMemsetAsync(h->d_run_count, 0, sizeof(int) * (size_t)std::max<int64_t>(h->long_runs, 1), h->stream);
@@ -2280,15 +2304,31 @@ static int sgd_gave_up(dsfacto *h, const int code[3]) {
     cudaStreamSynchronize(h->stream);
     return DSFACTO_ERR_CUDA;
 }
+// An SGD launch gave up: a bounded wait ran out, or a check of the debug build failed.
+static int sgd_gave_up(dsfacto *h, const int code[3]) {
+    char buf[160];
+    if (code[0] == 1) std::snprintf(buf, sizeof buf, "stratum SGD: a wait for an earlier tile of the same column block timed out");
+    else if (code[0] == 2) std::snprintf(buf, sizeof buf, "stratum SGD: a copy of entry records into shared memory did not arrive");
+    else std::snprintf(buf, sizeof buf, "stratum SGD: debug check %d failed (value %d)", code[1], code[2]);
+    h->err = buf;
+    return broke_off(h);
+}
 
 static int epoch_impl(dsfacto_t *h);
 
 int dsfacto_epoch(dsfacto_t *h) {
     if (!h) return DSFACTO_ERR_INVALID_ARG;
     if (!h->loaded) return DSFACTO_ERR_NO_DATA;
-    if (h->failed) { h->err = "the last stratum SGD launch gave up: set the parameters again (dsfacto_set_params) first"; return DSFACTO_ERR_CUDA; }
+    if (h->failed) { h->err = "the last epoch or recompute pass gave up: set the parameters again (dsfacto_set_params) first"; return DSFACTO_ERR_CUDA; }
     if (h->nshards > 1) return DSFACTO_ERR_INVALID_ARG;   // a column shard advances with dsfacto_shard_epoch_begin / _end
-    return epoch_impl(h);
+    const int64_t launched = h->launches;
+    const float w0 = h->w0;
+    int rc = epoch_impl(h);
+    if (rc == DSFACTO_ERR_CUDA && !h->failed) {
+        if (h->launches != launched) rc = broke_off(h);
+        else h->w0 = w0;   // nothing has run: the handle is as it was
+    }
+    return rc;
 }
 
 // The launches of an epoch by column runs.  The segments follow one another on the device; the host hears of the last.
@@ -2308,18 +2348,21 @@ static int enqueue_epoch(dsfacto_t *h) {
 constexpr int kEpochsBeforeGraph = 16, kMostGraphLaunches = 256;
 static int run_epoch(dsfacto_t *h) {
     if (h->epoch_graph) {
-        h->model_version += 1;   // (as run_strata)
-        (h->slots ? h->slot_version : h->pair_version) = h->model_version;
-        h->launches += h->epoch_launches;
-        CU_TRY(h, cudaGraphLaunch(h->epoch_graph, h->stream));
+        if (planted_refusal(h)) h->launch_error = cudaErrorLaunchOutOfResources;
+        else if (!refused(h, cudaGraphLaunch(h->epoch_graph, h->stream))) {
+            h->model_version += 1;   // (as run_strata)
+            (h->slots ? h->slot_version : h->pair_version) = h->model_version;
+            h->launches += h->epoch_launches;
+        }
         return DSFACTO_OK;
     }
     if (h->epochs_run < kEpochsBeforeGraph) {
         const int64_t before = h->launches;
         const int rc = enqueue_epoch(h);
+        if (rc || h->launch_error != cudaSuccess) return rc;   // (collect tells)
         h->epoch_launches = h->launches - before;
         h->epochs_run += h->epoch_launches <= kMostGraphLaunches ? 1 : 0;
-        return rc;
+        return DSFACTO_OK;
     }
     cudaStream_t own = h->stream, cap = nullptr;
     cudaGraph_t graph = nullptr;
@@ -2330,15 +2373,16 @@ static int run_epoch(dsfacto_t *h) {
         const int rc = enqueue_epoch(h);
         h->stream = own;
         h->launches = before;
+        const cudaError_t launched = launch_error(h);
         e = cudaStreamEndCapture(cap, &graph);
-        if (e == cudaSuccess && rc == DSFACTO_OK) e = cudaGraphInstantiate(&h->epoch_graph, graph, 0);
+        if (e == cudaSuccess) e = launched;
+        if (e == cudaSuccess && rc == DSFACTO_OK && cudaGraphInstantiate(&h->epoch_graph, graph, 0) != cudaSuccess) h->epoch_graph = nullptr;
     }
     if (graph) cudaGraphDestroy(graph);
     if (cap) cudaStreamDestroy(cap);
-    if (e != cudaSuccess) {   // no graph, then: the launches one by one
+    if (e != cudaSuccess || !h->epoch_graph) {   // no graph, then: the launches one by one
         cudaGetLastError();
-        h->epoch_graph = nullptr;
-        h->epochs_run = 0;
+        drop_epoch_graph(h);
         return enqueue_epoch(h);
     }
     return run_epoch(h);
@@ -2357,15 +2401,18 @@ static int epoch_impl(dsfacto_t *h) {
         if (h->runs && !shard) break;   // (below)
         h->w0 = (float)((double)h->w0 - (double)h->h * share * h->g_sum);
         if (!shard) {
-            epoch_begin_kernel<<<1, 1, 0, h->stream>>>(h->d_state, h->w0);
-            h->launches += 1;
+            before_report(h);
+            launch(h, epoch_begin_kernel, 1, 1, 0, h->d_state, h->w0);
         }
         if (h->runs) run_strata(h, 0, 0.0);
         else run_sgd_phase(h, L0, L1);
         if (shard) CU_TRY(h, cudaEventRecord(h->ev[1], h->stream));
         if ((rc = run_refresh(h, L0 == 0, true)) || (rc = collect(h))) return rc;
     }
-    if (h->runs && !shard && ((rc = run_epoch(h)) || (rc = collect(h)))) return rc;
+    if (h->runs && !shard) {
+        before_report(h);
+        if ((rc = run_epoch(h)) || (rc = collect(h))) return rc;
+    }
     if (shard) {
         float t01 = 0, t12 = 0;
         cudaEventElapsedTime(&t01, h->ev[0], h->ev[1]);
@@ -2687,7 +2734,10 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
             if (e != cudaSuccess) { h->err = cudaGetErrorString(e); rc = DSFACTO_ERR_CUDA; }
         }
     }
-    if (rc == DSFACTO_ERR_CUDA) cudaStreamSynchronize(h->stream);
+    if (rc == DSFACTO_ERR_CUDA) {
+        if (a.bad) cudaMemsetAsync(a.bad, 0, sizeof(int), h->stream);   // (the kernel that did not run would have)
+        cudaStreamSynchronize(h->stream);
+    }
     h->report->bad = 0;
     if (!rc && mode == kEvaluate) { sums2[0] = h->report->loss; sums2[1] = h->report->g; }
     cleanup();
@@ -2744,6 +2794,10 @@ int dsfacto_debug_set(dsfacto_t *h, int32_t key, int64_t value) {
     case DSFACTO_DEBUG_ROW_MERGE:
         if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8 && value != kMaxRowMerge) return DSFACTO_ERR_INVALID_ARG;
         h->row_merge = (int)value;
+        return DSFACTO_OK;
+    case DSFACTO_DEBUG_REFUSE_LAUNCH:
+        if (value < 0 || value > (1 << 20)) return DSFACTO_ERR_INVALID_ARG;
+        h->refuse_launch = (int)value;
         return DSFACTO_OK;
     case DSFACTO_DEBUG_COLUMN_ORDER:
         if (value < 0 || value > 2) return DSFACTO_ERR_INVALID_ARG;

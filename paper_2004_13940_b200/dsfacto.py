@@ -168,7 +168,7 @@ def dsfacto_set_refresh_every(h, rounds):
     return lib().dsfacto_set_refresh_every(h, rounds)
 
 
-DEBUG_SPIN_LIMIT, DEBUG_EXTRA_NEED, DEBUG_CHUNK_LEN, DEBUG_COLUMN_ORDER, DEBUG_ROW_MERGE = 0, 1, 2, 3, 4
+DEBUG_SPIN_LIMIT, DEBUG_EXTRA_NEED, DEBUG_CHUNK_LEN, DEBUG_COLUMN_ORDER, DEBUG_ROW_MERGE, DEBUG_REFUSE_LAUNCH = range(6)
 
 
 def dsfacto_debug_set(h, key, value):
