@@ -253,7 +253,8 @@ private:
 // 328 MB to the device, 4 threads: 43 GB/s (8 threads: 40; slots of 512 / 256 / 128 KB instead of 1 MB: 32 / 22 /
 // 16, every copy costs the driver some 10 us); 67 MB into fresh memory, 8 threads: 34 GB/s (4 threads: 19, page
 // faults).  The helpers sleep between transfers; nobody waits for a helper that has not woken up yet,
-// so a busy machine costs bandwidth, not a stall.  One transfer at a time per process.
+// so a busy machine costs bandwidth, not a stall.  One transfer at a time has the helpers; another thread's that
+// finds them taken goes through the driver, beside the first (a request must not wait for a data set to pass).
 // ------------------------------------------------------------------------------------------
 struct Piece {            // one array of a transfer
     void *dev;
@@ -271,8 +272,9 @@ public:
     // Smaller arrays go through the driver: 1 MB to the device takes 0.08 ms either way, 2.7 MB back 0.20 ms through
     // the driver and 0.28 ms with helpers that have to wake up first.
     static constexpr size_t kWorth = (size_t)1 << 20, kWorthBack = (size_t)6 << 20;
-    // Copies the pieces on the stream; on return host memory has been read (to the device) or written (from it).
-    // To the device, the last copies may still be under way on the stream.
+    // Copies the pieces on the stream.  From the device: on return host memory has been written.  To the device: copies
+    // may still be under way, and page-locked host memory of the caller's is read by them, so the caller waits for the
+    // stream before it gives host memory back.
     cudaError_t move(bool to_device, std::initializer_list<Piece> pieces, cudaStream_t st) { return move(to_device, pieces.begin(), (int)pieces.size(), st); }
     cudaError_t move(bool to_device, const Piece *pieces, int count, cudaStream_t st) {
         cudaError_t e = cudaSuccess;
@@ -304,16 +306,18 @@ private:
     };
     struct Region { char *dev, *host; size_t bytes; };
     cudaError_t staged(bool to_device, const Piece *pieces, int count, cudaStream_t st) {
-        std::lock_guard<std::mutex> one(transfer_);
-        cudaError_t e;
-        try {
-            size_t most = 0;
-            for (int q = 0; q < count; ++q) most += pieces[q].bytes / kSlot + 32;
-            regions_.reserve(most);
-            e = prepare();
-        } catch (const std::bad_alloc &) { e = cudaErrorMemoryAllocation; }
-        if (e != cudaSuccess) {   // no page-locked memory or threads to be had: the driver's way
-            cudaGetLastError();
+        std::unique_lock<std::mutex> one(transfer_, std::try_to_lock);
+        cudaError_t e = cudaErrorNotReady;
+        if (one.owns_lock()) {
+            try {
+                size_t most = 0;
+                for (int q = 0; q < count; ++q) most += pieces[q].bytes / kSlot + 32;
+                regions_.reserve(most);
+                e = prepare();
+            } catch (const std::bad_alloc &) { e = cudaErrorMemoryAllocation; }
+            if (e != cudaSuccess) cudaGetLastError();
+        }
+        if (e != cudaSuccess) {   // another thread's transfer has them, or no page-locked memory or threads to be had: the driver's way
             for (int q = 0; q < count; ++q) {
                 const Piece &p = pieces[q];
                 if ((e = to_device ? cudaMemcpyAsync(p.dev, p.host, p.bytes, cudaMemcpyHostToDevice, st)
