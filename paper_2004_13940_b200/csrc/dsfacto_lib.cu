@@ -8,10 +8,10 @@
 #include "dsfacto_runplan.cuh"
 #include "dsfacto_runs.cuh"
 #include "dsfacto_sgd.cuh"
+#include "dsfacto_spin.h"
 
 #include <cub/device/device_radix_sort.cuh>
 
-#include <immintrin.h>
 #include <omp.h>
 #include <sys/mman.h>
 
@@ -989,7 +989,7 @@ int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long
         return rc;
     }
     for (unsigned spin = 1; at != want; ++spin) {
-        _mm_pause();
+        spin_pause();
         if ((spin & 0x3FFFu) != 0) continue;
         const cudaError_t e = cudaStreamQuery(h->stream);
         if (e == cudaErrorNotReady) continue;
@@ -997,6 +997,7 @@ int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long
         h->err = std::string("report: ") + (e == cudaSuccess ? "the last kernel left none" : cudaGetErrorString(e));
         return DSFACTO_ERR_CUDA;
     }
+    spin_done();
     return DSFACTO_OK;
 }
 

@@ -13,6 +13,7 @@
 #include "dsfacto_recompute.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 
@@ -31,9 +32,10 @@ constexpr int kMaxDevices = 64;
 static __device__ __align__(256) double g_noalloc_partials[4 * kMaxCtas];
 static __device__ unsigned g_noalloc_done;
 
-// their device addresses per device (the symbols themselves are only host-side stand-ins)
-double *g_partials_addr[kMaxDevices] = {nullptr};
-unsigned *g_done_addr[kMaxDevices] = {nullptr};
+// their device addresses per device (the symbols themselves are only host-side stand-ins); every writer stores the
+// same value, and the second is stored before the first is published
+std::atomic<double *> g_partials_addr[kMaxDevices];
+std::atomic<unsigned *> g_done_addr[kMaxDevices];
 
 // The recompute kernel of the epoch (eq. (fm_model2), the multiplier G, the loss) without its stores of the
 // auxiliaries and without per-column pairs, for which there is no room: w_j and sum_k v_jk^2 come from w and V.

@@ -100,3 +100,18 @@ def test_csr_validation_rejects_malformed_input():
     assert ok(np.array([0, 3, 2], np.int64), good, vals) == D.ERR_INVALID_CSR           # not monotone
     assert ok(np.array([1, 2, 4], np.int64), good, vals) == D.ERR_INVALID_CSR           # indptr[0] != 0
     assert ok(indptr, good, np.array([0, 1, 1, 1], np.float32)) == D.OK                 # stored zero is legal
+
+
+def test_host_code_builds_on_other_processors_than_x86():
+    # a Grace-Blackwell board has an Arm host: no x86 header or builtin outside a guarded branch
+    import subprocess
+    from paper_2004_13940_b200 import build as B
+    sources = [f for f in sorted(B.CSRC.iterdir()) if f.suffix in (".cu", ".cuh", ".h", ".c")]
+    assert len(sources) > 8
+    for f in sources:
+        text = f.read_text()
+        assert not re.search(r"#\s*include\s*[<\"]\w*intrin(_\w+)?\.h|_mm\d*_|__rdtsc", text), f.name
+    spin = (B.CSRC / "dsfacto_spin.h").read_text().replace("#include <atomic>", "namespace std { enum { memory_order_acquire }; void atomic_thread_fence(int); }")
+    r = subprocess.run(["g++", "-std=c++17", "-U__x86_64__", "-U__i386__", "-D__aarch64__", "-S", "-O1", "-x", "c++", "-o", "-", "-"],
+                       input=spin.replace("inline ", "") + "\n", capture_output=True, text=True)
+    assert r.returncode == 0 and "yield" in r.stdout, r.stderr
