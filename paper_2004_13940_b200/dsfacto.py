@@ -125,8 +125,8 @@ def _result(*shape) -> np.ndarray:
         return np.empty(shape, np.float32)
     if len(_asked) > 256:
         _asked.clear()
-    _asked[nbytes] = _asked.get(nbytes, 0) + 1
-    p = lib().dsfacto_host_alloc(nbytes) if _asked[nbytes] >= 2 else None
+    times = _asked[nbytes] = _asked.get(nbytes, 0) + 1   # (another thread may empty it in the meantime)
+    p = lib().dsfacto_host_alloc(nbytes) if times >= 2 else None
     if not p:
         return np.empty(shape, np.float32)
     buf = (ctypes.c_char * nbytes).from_address(p)

@@ -115,3 +115,13 @@ def test_host_code_builds_on_other_processors_than_x86():
     r = subprocess.run(["g++", "-std=c++17", "-U__x86_64__", "-U__i386__", "-D__aarch64__", "-S", "-O1", "-x", "c++", "-o", "-", "-"],
                        input=spin.replace("inline ", "") + "\n", capture_output=True, text=True)
     assert r.returncode == 0 and "yield" in r.stdout, r.stderr
+
+
+def test_result_arrays_while_another_thread_empties_the_count_of_sizes(monkeypatch):
+    class Emptied(dict):        # the other thread comes in at the worst moment
+        def __setitem__(self, key, value):
+            super().__setitem__(key, value)
+            self.clear()
+
+    monkeypatch.setattr(D, "_asked", Emptied())
+    assert D._result(1 << 15).shape == (1 << 15,)
