@@ -43,15 +43,17 @@ public:
         const size_t size = (std::max<size_t>(bytes, 1) + unit - 1) / unit * unit;
         {
             std::lock_guard<std::mutex> lock(mu_);
-            std::multimap<size_t, Idle> &idle = idle_[dev];
-            const auto it = idle.lower_bound(size);
-            if (it != idle.end() && it->first <= size + size / 4) {
-                *out = it->second.ptr;
-                live_[it->second.ptr] = {it->first, dev};
-                idle_bytes_[dev] -= it->first;
-                idle.erase(it);
-                return cudaSuccess;
-            }
+            try {
+                std::multimap<size_t, Idle> &idle = idle_[dev];
+                const auto it = idle.lower_bound(size);
+                if (it != idle.end() && it->first <= size + size / 4) {
+                    live_[it->second.ptr] = {it->first, dev};
+                    *out = it->second.ptr;
+                    idle_bytes_[dev] -= it->first;
+                    idle.erase(it);
+                    return cudaSuccess;
+                }
+            } catch (const std::bad_alloc &) { return cudaErrorMemoryAllocation; }
         }
         e = cudaMalloc(out, size);
         if (e == cudaErrorMemoryAllocation) {
@@ -60,54 +62,68 @@ public:
             e = cudaMalloc(out, size);
         }
         if (e != cudaSuccess) return e;
-        std::lock_guard<std::mutex> lock(mu_);
-        live_[*out] = {size, dev};
+        try {
+            std::lock_guard<std::mutex> lock(mu_);
+            live_[*out] = {size, dev};
+        } catch (const std::bad_alloc &) {
+            cudaFree(*out);
+            *out = nullptr;
+            return cudaErrorMemoryAllocation;
+        }
         return cudaSuccess;
     }
     void free(void *ptr) {
         if (!ptr) return;
-        std::vector<void *> go;   // what has been idle longest makes room
-        {
-            std::lock_guard<std::mutex> lock(mu_);
-            const auto it = live_.find(ptr);
-            const Block b = it != live_.end() ? it->second : Block{~(size_t)0, 0};
-            if (it != live_.end()) live_.erase(it);
-            if (b.bytes > bound(b.dev)) {
-                go.push_back(ptr);
-            } else {
-                std::multimap<size_t, Idle> &idle = idle_[b.dev];
-                idle.emplace(b.bytes, Idle{ptr, ++clock_});
-                idle_bytes_[b.dev] += b.bytes;
-                while (idle_bytes_[b.dev] > bound(b.dev)) {
-                    auto old = idle.begin();
-                    for (auto q = idle.begin(); q != idle.end(); ++q)
-                        if (q->second.since < old->second.since) old = q;
-                    go.push_back(old->second.ptr);
-                    idle_bytes_[b.dev] -= old->first;
-                    idle.erase(old);
+        for (;;) {
+            void *go = ptr;   // back to the driver: this block, or the ones that have been idle longest, to make room for it
+            {
+                std::lock_guard<std::mutex> lock(mu_);
+                const auto it = live_.find(ptr);
+                if (it != live_.end()) {
+                    const Block b = it->second;
+                    try {
+                        const size_t most = bound(b.dev);
+                        size_t &held = idle_bytes_[b.dev];
+                        std::multimap<size_t, Idle> &idle = idle_[b.dev];
+                        if (held + b.bytes <= most) {
+                            idle.emplace(b.bytes, Idle{ptr, ++clock_});
+                            held += b.bytes;
+                            live_.erase(it);
+                            return;
+                        }
+                        if (b.bytes <= most) {
+                            auto old = idle.begin();
+                            for (auto q = idle.begin(); q != idle.end(); ++q)
+                                if (q->second.since < old->second.since) old = q;
+                            go = old->second.ptr;
+                            held -= old->first;
+                            idle.erase(old);
+                        }
+                    } catch (const std::bad_alloc &) {}   // (no room in the lists)
+                    if (go == ptr) live_.erase(it);
                 }
             }
+            cudaFree(go);
+            if (go == ptr) return;
         }
-        for (void *p : go) cudaFree(p);
     }
     // idle bytes on the current device
     size_t idle_bytes() {
         int dev = 0;
         cudaGetDevice(&dev);
         std::lock_guard<std::mutex> lock(mu_);
-        return idle_bytes_[dev];
+        const auto it = idle_bytes_.find(dev);
+        return it == idle_bytes_.end() ? 0 : it->second;
     }
     void trim() {
-        std::vector<void *> go;
+        std::map<int, std::multimap<size_t, Idle>> go;
         {
             std::lock_guard<std::mutex> lock(mu_);
-            for (auto &d : idle_) {
-                for (auto &b : d.second) go.push_back(b.second.ptr);
-                d.second.clear();
-                idle_bytes_[d.first] = 0;
-            }
+            go.swap(idle_);
+            for (auto &held : idle_bytes_) held.second = 0;
         }
-        for (void *p : go) cudaFree(p);
+        for (auto &d : go)
+            for (auto &b : d.second) cudaFree(b.second.ptr);
     }
 
 private:
@@ -489,7 +505,7 @@ public:
         if (!p) return;
         {
             std::lock_guard<std::mutex> lock(mu_);
-            if (idle_.size() < 8) { idle_.push_back(p); return; }
+            try { if (idle_.size() < 8) { idle_.push_back(p); return; } } catch (const std::bad_alloc &) {}
         }
         cudaFreeHost(p);
     }

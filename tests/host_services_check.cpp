@@ -8,6 +8,9 @@
 #include <cstdlib>
 #include <random>
 
+// memory of the host may run out at any allocation of the library
+static thread_local int t_left = -1;   // allocations until then (-1: never)
+
 // ---- the runtime ----
 static std::mutex g_mu;
 static std::condition_variable g_cv;
@@ -26,7 +29,7 @@ cudaError_t cudaMalloc(void **p, size_t n) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (g_device_bytes + n > kDeviceTotal) return cudaErrorMemoryAllocation;
     *p = std::malloc(n);
-    g_device[(char *)*p] = n;
+    { const int left = t_left; t_left = -1; g_device[(char *)*p] = n; t_left = left; }   // (the runtime has its own memory)
     g_device_bytes += n;
     return cudaSuccess;
 }
@@ -58,6 +61,16 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { std::free((void *)e); return cudaS
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 }
+
+void *operator new(size_t n) {
+    if (t_left == 0) throw std::bad_alloc();
+    if (t_left > 0) --t_left;
+    void *p = std::malloc(n);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
 
 #define NEED(cond)                                                         \
     do {                                                                   \
@@ -136,10 +149,38 @@ static int threads() {
     return 0;
 }
 
+// Without host memory for its lists the pool reports an allocation as failed and gives a freed block back: nothing is
+// thrown, nothing is lost.
+static int no_host_memory() {
+    using dsf::DevicePool;
+    dsf::Mailboxes::get();
+    DevicePool::get();
+    for (int left = 0; left < 8; ++left) {
+        void *p = nullptr, *q = nullptr;
+        t_left = left;
+        const cudaError_t e = DevicePool::get().alloc(&p, 5000);
+        t_left = -1;
+        NEED((e == cudaSuccess) == (p != nullptr));
+        if (!p) NEED(e == cudaErrorMemoryAllocation && DevicePool::get().alloc(&p, 5000) == cudaSuccess);
+        NEED(DevicePool::get().alloc(&q, 100000) == cudaSuccess);
+        std::memset(p, 1, 5000);
+        t_left = left;
+        DevicePool::get().free(p);
+        DevicePool::get().free(q);
+        void *box = dsf::Mailboxes::get().take();
+        dsf::Mailboxes::get().give(box);
+        DevicePool::get().trim();
+        t_left = -1;
+        NEED(DevicePool::get().idle_bytes() == 0 && g_device.empty() && g_device_bytes == 0);
+    }
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "transfers-in") return transfers(true);
     if (what == "transfers-out") return transfers(false);
     if (what == "threads") return threads();
+    if (what == "no-host-memory") return no_host_memory();
     return 2;
 }
