@@ -500,27 +500,32 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
     } while (0)
 
 // the recompute kernel has its own lane layout (4 * LGr * NVr = Kp as well)
-#define DSF_DISPATCH_REFRESH(h, ...)                               \
+#define DSF_DISPATCH_REFRESH(h, FN, ...)                           \
     do {                                                           \
         switch ((h)->LGr * 10 + (h)->NVr) {                        \
-        case 11: launch_refresh<1, 1>(__VA_ARGS__); break;         \
-        case 21: launch_refresh<2, 1>(__VA_ARGS__); break;         \
-        case 41: launch_refresh<4, 1>(__VA_ARGS__); break;         \
-        case 81: launch_refresh<8, 1>(__VA_ARGS__); break;         \
-        case 82: launch_refresh<8, 2>(__VA_ARGS__); break;         \
-        case 84: launch_refresh<8, 4>(__VA_ARGS__); break;         \
-        case 86: launch_refresh<8, 6>(__VA_ARGS__); break;         \
-        case 88: launch_refresh<8, 8>(__VA_ARGS__); break;         \
+        case 11: FN<1, 1>(__VA_ARGS__); break;                     \
+        case 21: FN<2, 1>(__VA_ARGS__); break;                     \
+        case 41: FN<4, 1>(__VA_ARGS__); break;                     \
+        case 81: FN<8, 1>(__VA_ARGS__); break;                     \
+        case 82: FN<8, 2>(__VA_ARGS__); break;                     \
+        case 84: FN<8, 4>(__VA_ARGS__); break;                     \
+        case 86: FN<8, 6>(__VA_ARGS__); break;                     \
+        case 88: FN<8, 8>(__VA_ARGS__); break;                     \
         default: break;                                            \
         }                                                          \
     } while (0)
 
 // CTAs of the recompute kernel: as many as stay resident (each lane group then fetches its next row while it works
 // on the present one), fewer for few rows.
+template <int LG, int NV>
+void refresh_grid_of(int sm_count, int64_t rows, int &grid) {
+    typedef RefreshCfg<LG, NV> C;
+    grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + C::ROWS - 1) / C::ROWS, (int64_t)sm_count * C::CTAS));
+}
 int refresh_grid_for(const dsfacto *h, int64_t rows) {
-    const int G = kThreads / h->LGr;
-    const int64_t want = (rows + G - 1) / G, cap = (int64_t)h->sm_count * (h->LGr < 8 ? 4 : h->NVr >= 4 ? 2 : 3);
-    return (int)std::max<int64_t>(1, std::min(want, cap));
+    int grid = 1;
+    DSF_DISPATCH_REFRESH(h, refresh_grid_of, h->sm_count, rows, grid);
+    return grid;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -806,7 +811,13 @@ void run_sgd_phase(dsfacto *h, int64_t L0, int64_t L1) {
 }
 
 // ---- update loop by column runs ----
-int run_ctas_per_sm(const dsfacto *h) { return h->LG * h->NV <= 4 ? 8 : h->LG * h->NV <= 8 ? 6 : 4; }   // as runs_sweep_kernel is bounded
+template <int LG, int NV>
+void run_ctas_of(int &per_sm) { per_sm = RunCfg<LG, NV>::CTAS; }
+int run_ctas_per_sm(const dsfacto *h) {
+    int per_sm = 1;
+    DSF_DISPATCH(h, run_ctas_of, per_sm);
+    return per_sm;
+}
 template <int LG, int NV>
 void launch_run_pass(dsfacto *h, const RunPass &ps, RunSweepArgs &sw, RunApplyArgs &ap) {
     const int64_t ctas = std::max<int64_t>(((int64_t)ps.units + kRunWarps - 1) / kRunWarps, 1);
@@ -948,7 +959,7 @@ int run_partial_refresh(dsfacto *h) {
     a.A = h->d_A; a.G = h->d_G; a.f_out = nullptr;
     a.lin_out = h->d_lin; a.q_out = h->d_q;
     a.partials = h->d_partials; a.w0 = h->w0; a.loss = h->loss;
-    DSF_DISPATCH_REFRESH(h, h, a, kPartial, h->refresh_grid);
+    DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kPartial, h->refresh_grid);
     cudaEventRecord(h->ev[2], h->stream);   // (the epoch's phase timers expect both marks)
     cudaEventRecord(h->ev[3], h->stream);
     CU_TRY(h, cudaStreamSynchronize(h->stream));
@@ -1013,7 +1024,7 @@ int run_refresh(dsfacto *h, bool first, bool report) {
     a.norm_w = h->d_w; a.norm_V = h->d_V; a.norm_d = h->d; a.norm_v4 = (int64_t)h->d * (h->Kp / 4);
     a.done = &h->d_state->done; a.st = h->d_state; a.first = first ? 1 : 0;
     if (report) a.report = h->report;
-    DSF_DISPATCH_REFRESH(h, h, a, kTrain, h->refresh_grid);
+    DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kTrain, h->refresh_grid);
     return DSFACTO_OK;
 }
 // The device counts the reports of recompute passes.  What the host waits for is the number after the one that lies in
@@ -2723,8 +2734,8 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
     }
     a.partials = reinterpret_cast<double *>(block + part_at);
     ++h->report_seq;
-    if (mode == kScore) DSF_DISPATCH_REFRESH(h, h, a, kScore, grid);
-    else DSF_DISPATCH_REFRESH(h, h, a, kEvaluate, grid);
+    if (mode == kScore) DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kScore, grid);
+    else DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kEvaluate, grid);
     rc = wait_report(h, h->report->seq, h->report_seq);
     if (!rc && h->report->bad) rc = DSFACTO_ERR_INVALID_CSR;
     if (!rc && mode == kScore) {

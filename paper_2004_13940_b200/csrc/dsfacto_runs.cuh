@@ -64,6 +64,7 @@ struct RunCfg {
     static constexpr int ST = U * GW;        // entries per stage
     static constexpr int SP = 32 / ST;       // stages per pass of 32 entries
     static constexpr int REC = KP4 + 1;      // float4s of a record
+    static constexpr int CTAS = KP4 <= 4 ? 8 : KP4 <= 8 ? 6 : 4;   // of the sweep, resident per SM (register cap; the load cuts units by it)
 };
 template <int LG, int NV>
 constexpr size_t run_sweep_smem() { return (size_t)kRunWarps * 2 * RunCfg<LG, NV>::REC * sizeof(float4); }
@@ -109,7 +110,7 @@ __device__ __forceinline__ void sum_groups(float4 (&x)[NV]) {
 // against 250 G for plain loads.
 // ------------------------------------------------------------------------------------------
 template <int LG, int NV>
-__global__ void __launch_bounds__(kRunThreads, (LG * NV <= 4 ? 8 : LG * NV <= 8 ? 6 : 4)) runs_sweep_kernel(const RunSweepArgs a) {
+__global__ void __launch_bounds__(kRunThreads, (RunCfg<LG, NV>::CTAS)) runs_sweep_kernel(const RunSweepArgs a) {
     typedef RunCfg<LG, NV> C;
     constexpr int GW = C::GW, KP4 = C::KP4, U = C::U, ST = C::ST, SP = C::SP, REC = C::REC;
     constexpr unsigned FULL = 0xFFFFFFFFu;
