@@ -2654,10 +2654,19 @@ static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_
     return true;
 }
 
+// Whether a batch in the mailbox is staged: every CTA copies all of it to shared memory in one trip across the link,
+// instead of one trip for its row pointers and one for every two batches of its rows' entries.  That saves trips, the more
+// the longer the rows, and costs the link (CTAs x size).  Calls of dsfacto_predict, staged / not, in us: 32 factors, rows
+// of 39 entries, 2 CTAs x 12 KB 23.1 / 25.5, 3 x 24 KB 25.6 / 27.8; of 8 entries, 2 x 3 KB 17.6 / 18.5, 5 x 12 KB 24.1 /
+// 21.4; of one entry, 3 x 1.5 KB 17.9 / 18.9, 10 x 6 KB 23.2 / 20.7, 38 x 24 KB 47.7 / 23.9; 8 factors, rows of 39 entries,
+// 1 x 24 KB 25.6 / 34.6; of 20 entries, 2 x 24 KB 24.8 / 28.1; of one entry, 2 x 3 KB 18.8 / 19.8, 5 x 12 KB 24.4 / 21.7.
+static bool staging_pays(size_t size, int ctas, int64_t m, int64_t nnz) {
+    return size <= (size_t)24 << 10 && (double)size * ctas <= 12288.0 + 1800.0 * (double)nnz / (double)m;
+}
+
 // Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
 // fp32[m].  mode kEvaluate: labels y (host) and sums2 = {sum of losses, sum of squared errors or number of correct
 // signs}.
-constexpr size_t kStagedMost = (size_t)24 << 10;   // a batch of up to this size is copied to shared memory by every CTA
 static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, const int32_t *indices,
                       const float *values, const float *y, float *scores_out, double sums2[2]) {
     RefreshArgs a{};
@@ -2699,7 +2708,7 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
             float *last = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
             if (mode == kScore) { a.f_out = last; mailed_out = true; }
             else { std::memcpy(last, y, y_b); a.y = last; }
-            if (mail <= kStagedMost) {
+            if (staging_pays(mail, grid, m, nnz)) {
                 a.stage = reinterpret_cast<const uint4 *>(p);
                 a.stage_bytes = (int)((mail + 15) & ~(size_t)15);
                 a.idx = reinterpret_cast<int32_t *>(ip_b);

@@ -109,3 +109,43 @@ def test_allocation_free_scoring_at_every_width(K, m):
                                         t[5].data_ptr(), scores.data_ptr(), sums.data_ptr()) == D.OK
     np.testing.assert_allclose(scores.cpu().numpy(), want, rtol=0, atol=2e-5 * (1 + np.abs(want).max()))
     assert float(sums[0]) == pytest.approx(loss * m, rel=1e-5)
+
+
+def _short_rows(m, per_row, d, seed):
+    rng = np.random.default_rng(seed)
+    ix = (np.sort(rng.integers(0, d // per_row, (m, per_row)), axis=1) + np.arange(per_row) * (d // per_row)).astype(np.int32)
+    return np.arange(m + 1, dtype=np.int64) * per_row, ix.ravel(), rng.standard_normal(m * per_row).astype(np.float32)
+
+
+@pytest.mark.parametrize("K,per_row", [(8, 1), (32, 1), (32, 3), (128, 8)])
+@pytest.mark.parametrize("m", [33, 96, 129, 160, 256, 300, 1200])
+def test_batches_of_short_rows(K, per_row, m):
+    # both sides of the rule that lets every CTA copy the whole batch: few CTAs, and many (a CTA takes 32 rows, 128 at K = 8)
+    d = 4096
+    ip, ix, v = _short_rows(m, per_row, d, m)
+    rng = np.random.default_rng(K)
+    w, V = rng.standard_normal(d).astype(np.float32), (0.3 * rng.standard_normal((d, K))).astype(np.float32)
+    with D.DSFacto(1, d, K, 1, D.SQUARED, 0.0, 0.0, 0.1, 1) as g:
+        g.set_params(0.25, w, V)
+        f = O.score(ip, ix, v, 0.25, w.astype(np.float64), V.astype(np.float64))
+        for _ in range(2):
+            np.testing.assert_allclose(g.predict(ip, ix, v), f, rtol=0, atol=2e-5 * (1 + np.abs(f).max()))
+
+
+def test_many_short_rows_do_not_wait_for_copies_of_the_whole_batch():
+    # 1200 rows of one entry are 24 KB in 38 CTAs (47 us when every CTA copied them), 1300 rows are too large for that (24 us)
+    import time
+
+    d, K = 4096, 32
+    with D.DSFacto(1, d, K, 1, D.SQUARED, 0.0, 0.0, 0.1, 1) as g:
+        def median_us(m):
+            ip, ix, v = _short_rows(m, 1, d, 1)
+            out, took = np.empty(m, np.float32), []
+            for _ in range(300):
+                t = time.perf_counter()
+                assert D.dsfacto_predict(g._h, m, ip, ix, v, out) == D.OK
+                took.append(time.perf_counter() - t)
+            return 1e6 * float(np.median(took[50:]))
+
+        median_us(1300)
+        assert min(median_us(1200) for _ in range(3)) <= 1.5 * min(median_us(1300) for _ in range(3))
