@@ -1939,23 +1939,33 @@ static int64_t band_count(const dsfacto *h) {
     const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
     return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
 }
-// Many bands of wide rows make many short runs, each of which moves its column's row and its record through memory
-// once per band, while the tile sweep only adds to it.  400 M entries of 512-byte rows over 2^20 columns in 30 bands (13
-// entries per column and band): update loop 23.3 ms by runs (8 / 16 / 22 bands: 25.9 / 23.1 / 22.8 ms), 18.7 ms by tiles;
-// 30 M entries of such rows with 77 entries per column and band: 1.25 ms against 2.24 ms; 1.755 G entries of 64-byte
-// rows, 40 entries per column and band: 19.0 ms against 20.0 ms.  The tile sweep needs a large data set and grid, or its
-// warps wait for one another.
-static bool tiles_move_less(const dsfacto *h, int64_t nnz) {
+// Wide rows in many bands with short runs: every run moves its column's row and its record through memory once per
+// band, while the tile sweep only adds to the row.  Update loop by runs / by tiles, in ms (columns with power-law
+// frequencies; "short" = entries per column and band):
+//   bands    128 factors: 63 M entries in 6 bands 4.6 / 5.0, 118 M in 11 bands 8.0 / 7.1 (p = 128) to 9.1 (p = 512), 158 M in
+//            15 bands 10.4 / 8.8, 221 M in 20 bands 14.8 / 12.0, 400 M in 30 bands 23.3 / 18.7; 256 factors: 30 M in 6 bands
+//            3.7 / 3.6 to 4.5, 60 M in 12 bands 7.1 / 5.7, 113 M in 22 bands 12.9 / 10.3
+//   short    128 factors: 20 of them 11.4 / 10.2, 39 6.7 / 7.1, 77 5.5 / 6.5; 192 factors: 7 8.6 / 7.0, 106 5.8 / 5.9; 256
+//            factors: 5 25.3 / 15.1, 20 17.1 / 11.3, 39 12.9 / 10.3, 78 12.1 / 11.8
+//   size     in 12 or 13 bands: 30 to 34 M entries of 128 factors 2.3 / 2.4, 3.5 / 3.9, 6.2 / 6.2; 18 M of 192 factors 1.5 /
+//            1.8; 18, 20, 27 M of 256 factors 2.4 / 2.4 and 2.8 / 2.5, 6.7 / 6.6, 5.0 / 4.4
+//   entries  per row block, which the dependent tiles of a column block share: 60 M entries of 256 factors, p = 12 / 48 /
+//            128 6.9 / 5.3, 7.0 / 6.2, 7.1 / 5.7, but p = 512 7.1 / 8.7; 158 M of 128 factors, p = 128 10.4 / 8.8, p = 512 10.9 /
+//            10.7, p = 1024 10.6 / 13.5
+//   width    64 factors: 118 M in 6 bands 4.6 / 6.3, 239 M in 11 bands 11.0 / 11.6, 315 M in 15 bands 11.6 / 10.6 (p = 128),
+//            11.5 (256), 14.1 (48), 16.2 (1024); 1.755 G entries of 16 factors 19.0 / 20.0
+static bool tiles_move_less(const dsfacto *h, int64_t nnz, const char *load_env) {
     const bool segmented = h->refresh_every > 0 && h->refresh_every < h->p;
-    return h->Kp >= 64 && nnz >= ((int64_t)1 << 27) && h->p >= 128 && h->nshards == 1 && !segmented && !h->wide &&
-           bits_for((int64_t)h->p * h->p) + 1 + h->jbits <= 32 && !std::getenv("DSFACTO_BANDS") &&
-           (double)nnz < 24.0 * (double)h->d * (double)band_count(h);
+    const int64_t bands = band_count(h);
+    return h->Kp >= 128 && bands >= 12 && (double)nnz * h->Kp >= 6e9 && h->p >= 12 && nnz >= (int64_t)300000 * h->p &&
+           (double)nnz < 24.0 * (h->Kp / 128.0) * (double)h->d * (double)bands && h->nshards == 1 && !segmented &&
+           !std::getenv("DSFACTO_BANDS") && device_bucketing_wanted(h, nnz, load_env);   // (on the host the tiles take longer to build than they save)
 }
 // Whether this load takes it: every load that may be bucketed on the device, unless a knob asks for the tile sweep
 // (DSFACTO_SWEEP=round, row blocks per slot, the planted wait), as long as pass, column and phase fit a 32-bit key.
 static bool run_plan_wanted(const dsfacto *h, int64_t nnz, const char *load_env) {
     if (nnz <= 0 || h->sweep != 1 || h->row_merge > 0 || h->debug_extra_need > 0 || std::getenv("DSFACTO_ROW_MERGE")) return false;
-    if (tiles_move_less(h, nnz)) return false;
+    if (tiles_move_less(h, nnz, load_env)) return false;
     if (load_env) { if (std::strcmp(load_env, "device") != 0) return false; }
     else {
         // sort buffers 2 x (4 + 8) bytes (8 of them stay as the entry records), then A, G and the runs

@@ -46,3 +46,46 @@ def test_bands_units_and_widths(monkeypatch, bands, chunk, K, p, every):
         A, G = g.get_aux()
         np.testing.assert_allclose(A, o.A, rtol=0, atol=2e-5 * (1 + np.abs(o.A).max()))
         np.testing.assert_allclose(G, o.G, rtol=0, atol=2e-5)
+
+
+def _wide_rows(n, d, per_row, seed):
+    rng = np.random.default_rng(seed)
+    idx = rng.integers(0, d // per_row, (n, per_row), dtype=np.int32) + (np.arange(per_row, dtype=np.int32) * (d // per_row))
+    indptr = np.arange(n + 1, dtype=np.int64) * per_row
+    return indptr, idx.ravel(), rng.standard_normal(n * per_row, dtype=np.float32), rng.standard_normal(n, dtype=np.float32)
+
+
+def _launches_per_epoch(g):
+    g.epoch()
+    before = g.launch_count()
+    g.epoch()
+    return g.launch_count() - before
+
+
+_TILES = 6      # w0, sweep, two kernels back to plain parameters, views, recompute; by runs two per band and more
+
+
+# a data set that just goes by tiles, and one step over each line of the rule
+@pytest.mark.parametrize("K,n,d,per_row,p,tiles", [(256, 800_000, 60_000, 30, 48, True), (130, 1_200_000, 80_000, 27, 13, True),
+                                                   (256, 800_000, 60_000, 30, 81, False), (256, 800_000, 60_000, 29, 12, False),
+                                                   (256, 700_000, 60_000, 35, 12, False), (256, 800_000, 40_000, 30, 48, False),
+                                                   (256, 800_000, 60_000, 30, 11, False), (64, 3_400_000, 1_000_000, 28, 48, False)])
+def test_many_short_runs_of_wide_rows_go_by_tiles(K, n, d, per_row, p, tiles):
+    indptr, idx, val, y = _wide_rows(n, d, per_row, K)
+    with D.DSFacto(n, d, K, p, D.SQUARED, 1e-3, 1e-3, 20.0, 11) as g:
+        g.load_csr(indptr, idx, val, y)
+        first = _launches_per_epoch(g)
+        assert first == _TILES if tiles else first >= 2 * 10
+        if not tiles:
+            return
+        w0, w, V = g.get_params()
+        objective = g.objective()
+    o = O.Oracle(n, d, K, p, O.SQUARED, 1e-3, 1e-3, 20.0, 11)
+    o.load_csr(indptr, idx, val, y)
+    before = o.V.copy()
+    o.epoch()
+    assert objective == pytest.approx(o.epoch(), rel=1e-4)
+    assert w0 == pytest.approx(o.w0, abs=1e-6)
+    assert np.abs(w - o.w).max() <= 1e-4 * (1 + np.abs(o.w).max())
+    assert np.abs(o.V - before).max() > 1e-5
+    assert np.abs(V - o.V).max() <= 2e-3 * np.abs(o.V - before).max() + 4e-7     # (two epochs: twice the rounding of one)
