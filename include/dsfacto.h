@@ -74,6 +74,7 @@ int dsfacto_create(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32_t p, 
  * The arrays are checked on the device, where they lie beside the old data set until they have passed: a data set
  * that fails the checks leaves the handle as it was (column shards: checked on the host).  A pass holds a band of rows whose auxiliaries fit L2; a data
  * set of one band has every column as one run in its full stratified order (DSFACTO_BANDS=B asks for B bands).
+ * Large data sets of wide rows whose runs would be short take the tile lists below instead.
  * With row blocks per slot asked for (DSFACTO_DEBUG_ROW_MERGE, DSFACTO_ROW_MERGE) or a planted wait
  * (DSFACTO_DEBUG_EXTRA_NEED), tile lists are bucketed on the device instead and swept tile by tile, as they are
  * where the host has built them; in these, several consecutive row blocks of a column block make one slot (up to

@@ -1931,13 +1931,17 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
 
 // ---- plan of the update loop by column runs (see dsfacto_runplan.cuh) ----
 // Bands: rows per pass such that their auxiliary rows, which every column of the pass reads, stay in L2.
+static int64_t bands_by_size(const dsfacto *h) {
+    const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
+    return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
+}
+// ... of this plan (DSFACTO_BANDS: as many as asked for)
 static int64_t band_count(const dsfacto *h) {
     if (const char *env = std::getenv("DSFACTO_BANDS")) {
         const int64_t v = std::atoll(env);
         if (v >= 1 && v <= h->n) return v;
     }
-    const double fit = 0.55 * (double)h->l2_bytes / ((double)h->Kp * 4.0);
-    return std::max<int64_t>(1, (int64_t)std::ceil((double)h->n / std::max(fit, 1.0)));
+    return bands_by_size(h);
 }
 // Wide rows in many bands with short runs: every run moves its column's row and its record through memory once per
 // band, while the tile sweep only adds to the row.  Update loop by runs / by tiles, in ms (columns with power-law
@@ -1956,10 +1960,10 @@ static int64_t band_count(const dsfacto *h) {
 //            11.5 (256), 14.1 (48), 16.2 (1024); 1.755 G entries of 16 factors 19.0 / 20.0
 static bool tiles_move_less(const dsfacto *h, int64_t nnz, const char *load_env) {
     const bool segmented = h->refresh_every > 0 && h->refresh_every < h->p;
-    const int64_t bands = band_count(h);
+    const int64_t bands = bands_by_size(h);   // (by the data set alone: DSFACTO_BANDS cuts the plan by runs, it does not choose it)
     return h->Kp >= 128 && bands >= 12 && (double)nnz * h->Kp >= 6e9 && h->p >= 12 && nnz >= (int64_t)300000 * h->p &&
            (double)nnz < 24.0 * (h->Kp / 128.0) * (double)h->d * (double)bands && h->nshards == 1 && !segmented &&
-           !std::getenv("DSFACTO_BANDS") && device_bucketing_wanted(h, nnz, load_env);   // (on the host the tiles take longer to build than they save)
+           device_bucketing_wanted(h, nnz, load_env);   // (on the host the tiles take longer to build than they save)
 }
 // Whether this load takes it: every load that may be bucketed on the device, unless a knob asks for the tile sweep
 // (DSFACTO_SWEEP=round, row blocks per slot, the planted wait), as long as pass, column and phase fit a 32-bit key.

@@ -89,3 +89,15 @@ def test_many_short_runs_of_wide_rows_go_by_tiles(K, n, d, per_row, p, tiles):
     assert np.abs(w - o.w).max() <= 1e-4 * (1 + np.abs(o.w).max())
     assert np.abs(o.V - before).max() > 1e-5
     assert np.abs(V - o.V).max() <= 2e-3 * np.abs(o.V - before).max() + 4e-7     # (two epochs: twice the rounding of one)
+
+
+@pytest.mark.parametrize("bands", ["2", "12", "40"])
+def test_the_number_of_bands_does_not_choose_the_update_loop(monkeypatch, bands):
+    n, d, K, p = 800_000, 60_000, 256, 48
+    indptr, idx, val, y = _wide_rows(n, d, 30, 4)
+    with D.DSFacto(n, d, K, p, D.SQUARED, 1e-3, 1e-3, 20.0, 11) as g:
+        g.load_csr(indptr, idx, val, y)
+        assert _launches_per_epoch(g) == _TILES
+        monkeypatch.setenv("DSFACTO_BANDS", bands)
+        g.load_csr(indptr, idx, val, y)
+        assert _launches_per_epoch(g) == _TILES
