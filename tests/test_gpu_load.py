@@ -1,9 +1,9 @@
 """The ways dsfacto_load_csr builds the tile lists on the device give the same lists, bit for bit, as the
 oracle's bucketing: the plain host bucketer, the row-block bucketer, the streamed load (row blocks
 bucketed into page-locked staging memory and copied block by block; DSFACTO_LOAD=stream forces it on small
-loads), and the bucketing on the device itself (keys, a stable radix sort, the chunk plan cut by a kernel),
-which loads take by default when the packed entry layout applies (DSFACTO_LOAD=device asks for it by name).  DSFACTO_LOAD=nostaging
-makes the streamed load behave as if no page-locked memory could be had, which must end in the row-block
+loads), the plan by column runs that loads take by default (DSFACTO_LOAD=device asks for the device by name), and the
+bucketing of tiles on the device (keys, a stable radix sort, the chunk plan cut by a kernel), which DSFACTO_ROW_MERGE or
+DEBUG_ROW_MERGE asks for.  DSFACTO_LOAD=nostaging makes the streamed load behave as if no page-locked memory could be had, which must end in the row-block
 bucketer with one copy, not in an error."""
 import numpy as np
 import pytest
@@ -95,8 +95,8 @@ def test_device_bucketing_gives_the_same_bits_as_the_host(monkeypatch, sweep, na
 
 
 def test_a_rejected_large_load_leaves_the_handle_as_it_was():
-    # from 2^24 entries on the CSR arrays travel to the device while the host still checks them; a data set
-    # that fails the checks must not replace the one the handle holds
+    # the CSR arrays are checked where they lie on the device, beside the data set that the handle holds: one that fails
+    # the checks must not replace it
     wl = W.make("C4", n=600_000, p=64)
     assert wl.nnz >= 1 << 24
     with D.DSFacto(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, wl.init_seed) as g, \
