@@ -321,7 +321,10 @@ def run_ours(args):
     traffic = None if (per_entry is None or sweep != "rowblock" or segments != 1) else per_entry * nnz
     # the update loop of an epoch: everything but the recompute pass of each segment
     loop_launches = max(1, round(launches / args.steps) - segments)
-    loop = "sgd_sweep_kernel" if sweep == "round" else "update loop (runs_sweep_kernel, runs_apply_kernel, runs_fold_kernel)"
+    # an epoch by tiles is six launches (w0, sweep, two kernels back to plain parameters, views, recompute); by runs only
+    # one in two bands of rows is, whose auxiliaries are far smaller than those of data sets that go by tiles
+    by_tiles = sweep == "round" or (round(launches / args.steps / segments) == 6 and 4 * n * K > 5e8)
+    loop = "sgd_sweep_kernel" if by_tiles else "update loop (runs_sweep_kernel, runs_apply_kernel, runs_fold_kernel)"
     roof = {"bound": "hbm", "kernel": loop, "launches_per_step": loop_launches, "sweep": sweep,
             "achieved": sgd_bytes / sgd_s / 1e9, "peak": peak, "unit": "GB/s", "frac": sgd_bytes / sgd_s / 1e9 / peak,
             "peak_kind": "of " + peak_kind, "traffic": traffic,

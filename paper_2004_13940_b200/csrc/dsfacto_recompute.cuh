@@ -97,14 +97,18 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // ahead of the multiply-adds.  Behind the end of a row its last entry is repeated with
 // x = 0.
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
-// What bounds it: 64-byte rows of click logs (78 M entries, 0.60 ms), the data and look-up stages of L1 (85 and 89 %
-// busy: every entry costs one look-up for its row and one for its pair) at 40 % issue; 128-byte rows (2.6 M entries,
-// 63 -> 44 us) a last round of rows that fills the SMs unevenly and latency; 512-byte rows (30 M entries, 1.0 ms) the
-// latency of gathers from L2 (47 % of its rate) with 16 resident warps.  Not kept: columns and values as records of 8
-// bytes (2.97 -> 3.35 ms per 390 M entries of click logs); the pairs of the 2048 most frequent columns in shared memory,
-// which the L1 then lacks (2.95 -> 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms);
-// rows taken longest first inside blocks of 256 (text 44 -> 42.5 us, but click logs 2.97 -> 3.09 ms); two or four
-// resident CTAs for 128-byte rows (46 and 43 us).
+// What bounds it: 64-byte rows of click logs (390 M entries, 2.8 to 2.9 ms), the data and look-up stages of L1 (85 and 89 %
+// busy: every entry costs one look-up for its row and one for its pair) at 40 % issue.  Wider rows reach no rate of any
+// unit: 128-byte rows (2.6 M entries, 63 -> 44 us) 52 % of the L1 data stage, 40 % issue; 256-byte rows without pairs
+// (500 k rows, 0.40 ms) 66 % and 49 %; 512-byte rows (30 M entries, 1.0 ms) 62 % and 27 %, L2 47 %, with 16 resident
+// warps that wait for their gathers.  Ragged rows pay for the common loop besides: rows of 26 to 76 and 20 to 60 entries
+// issue 1.37 and 1.39 row gathers per stored entry (1.27 and 1.29 from the longest of four rows, the rest from whole
+// batches; 39 entries in every row: 1.03).
+// Not kept (each against the version it was tried on): columns and values as records of 8 bytes (2.97 -> 3.35 ms per 390 M
+// entries of click logs); the pairs of the 2048 most frequent columns in shared memory, which the L1 then lacks (2.95 ->
+// 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms); rows taken longest first inside
+// blocks of 256 (text 44 -> 42.5 us, but click logs 2.97 -> 3.09 ms); two or four resident CTAs for 128-byte rows (46 and
+// 43 us).
 template <int LG, int NV, bool STAGED = false>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;

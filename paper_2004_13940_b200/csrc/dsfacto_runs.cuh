@@ -102,12 +102,12 @@ __device__ __forceinline__ void sum_groups(float4 (&x)[NV]) {
 //                 that lie inside it, and a segmented scan over the groups closes the others.
 // A finished run goes to its record; the piece of the run that was open at the unit's start and the one left open
 // at its end go to shared memory, where the CTA joins them.
-// What bounds it (39 M entries of click logs, 64-byte rows, 365 us = 8.5 entries per clock of the GPU): the load /
-// store data pipe is 79 % busy (one slot per gathered row, as many again for shuffles and the gathers of G), L2 62 %
-// of its rate (a 64-byte row gather reaches 16 TB/s), instruction issue 50 %.  A row ring that is copied from register to register (instead of requested
-// into the registers that have just been used up) took 470 us; rows and coefficients handed to the groups through
-// shared memory 365 us (a 16-byte broadcast load takes eight slots); tile::gather4 copies reach 114 G rows/s
-// against 250 G for plain loads.
+// What bounds it (39 M entries of click logs, 64-byte rows, 365 us = 54 entries per clock of the GPU): the load / store
+// data pipe is 79 % busy with 2.1 slots per entry: 0.68 shuffles and shared memory, 0.77 the gathered rows and words of
+// G, the rest their look-ups.  L2 is at 62 % of its rate (a 64-byte row gather reaches 16 TB/s), instruction issue at
+// 50 %.  A row ring that is copied from register to register (instead of requested into the registers that have just
+// been used up) took 470 us; rows and coefficients handed to the groups through shared memory 365 us (a 16-byte
+// broadcast load takes 2.05 slots); tile::gather4 copies reach 114 G rows/s against 250 G for plain loads.
 // ------------------------------------------------------------------------------------------
 template <int LG, int NV>
 __global__ void __launch_bounds__(kRunThreads, (RunCfg<LG, NV>::CTAS)) runs_sweep_kernel(const RunSweepArgs a) {
