@@ -100,7 +100,7 @@ int dsfacto_load_csr(dsfacto_t *h, const int64_t *indptr, const int32_t *indices
  *   recompute a_ik (eq. (compute_a_jk)), f_i (eq. (fm_model2)), G_i and the objective (eq. (fm_obj)).
  * Returns DSFACTO_ERR_DIVERGED if the new objective is not finite (state is kept).  If a launch is refused
  * (DSFACTO_ERR_CUDA) before anything has run, the handle is as it was; if an epoch breaks off later, w and V are
- * part of the way and the handle refuses further epochs until dsfacto_set_params replaces both or
+ * part of the way (w0 is as it was) and the handle refuses further epochs until dsfacto_set_params replaces both or
  * dsfacto_load_csr loads a data set.  (The same after a dsfacto_set_params or dsfacto_load_csr whose recompute
  * pass was refused: A and G are then not those of the parameters.) */
 int dsfacto_epoch(dsfacto_t *h);

@@ -2313,6 +2313,7 @@ static int load_validated(dsfacto_t *h, const int64_t *indptr, const int32_t *in
 // set is loaded after that.
 static int broke_off(dsfacto *h) {
     h->failed = true;
+    h->model_version += 1;   // (the kernels that keep the views of the model up to date may be among those left out)
     drop_epoch_graph(h);
     const size_t d = (size_t)h->d;
     cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream);
@@ -2350,9 +2351,9 @@ int dsfacto_epoch(dsfacto_t *h) {
     const int64_t launched = h->launches;
     const float w0 = h->w0;
     int rc = epoch_impl(h);
-    if (rc == DSFACTO_ERR_CUDA && !h->failed) {
-        if (h->launches != launched) rc = broke_off(h);
-        else h->w0 = w0;   // nothing has run: the handle is as it was
+    if (rc == DSFACTO_ERR_CUDA) {
+        if (!h->failed && h->launches != launched) rc = broke_off(h);   // (nothing has run: the handle is as it was)
+        h->w0 = w0;
     }
     return rc;
 }

@@ -84,3 +84,32 @@ def test_a_refused_launch_of_other_calls(m):
             assert call() == want
         assert g.epoch() == pytest.approx(o.epoch(), rel=1e-4)
         _same(g, o)
+
+
+@pytest.mark.parametrize("env", [{"DSFACTO_BANDS": "3"}, {}, {"DSFACTO_ROW_MERGE": "2"}])
+def test_parameters_left_part_of_the_way_are_scored_as_they_are(monkeypatch, env):
+    # what an epoch that broke off leaves behind is no result, but scores and a new load go by it as by any parameters
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    wl = W.make("C1")
+    ip = wl.indptr[:1001]
+    ix, v = wl.indices[: ip[-1]].copy(), wl.values[: ip[-1]].copy()
+    o = O.Oracle(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, 50.0, wl.init_seed)
+    o.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+    for k in range(2, 9):
+        with D.DSFacto(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, 50.0, wl.init_seed) as g:
+            g.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+            w0 = g.get_params()[0]
+            g.debug_set(D.DEBUG_REFUSE_LAUNCH, k)
+            if D.dsfacto_epoch(g._h) == D.OK:
+                break
+            w0_after, w, V = g.get_params()
+            assert w0_after == w0
+            o.w0, o.w[:], o.V[:] = float(w0), w, V
+            o.refresh()
+            f = o.predict(ip, ix, v)
+            np.testing.assert_allclose(g.predict(ip, ix, v), f, rtol=0, atol=2e-5 * (1 + np.abs(f).max()))
+            g.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+            assert g.objective() == pytest.approx(o.objective, rel=1e-5), k
+            A, G = g.get_aux()
+            np.testing.assert_allclose(G, o.G, rtol=0, atol=2e-5 * (1 + np.abs(o.G).max()))
