@@ -149,3 +149,38 @@ def test_many_short_rows_do_not_wait_for_copies_of_the_whole_batch():
 
         median_us(1300)
         assert min(median_us(1200) for _ in range(3)) <= 1.5 * min(median_us(1300) for _ in range(3))
+
+
+@pytest.mark.parametrize("n", [2_000, 40_000])
+def test_page_locked_arrays_belong_to_the_caller_again_on_return(n):
+    # copies of page-locked arrays are queued, not made, while a call is under way; each call has read them when it returns
+    import torch
+
+    def pinned(a):
+        t = torch.empty(a.shape, dtype=torch.from_numpy(a[:1]).dtype, pin_memory=True)
+        t.numpy()[...] = a
+        return t.numpy()
+
+    wl = W.make("C3", n=n)
+    rng = np.random.default_rng(n)
+    w, V = (0.1 * rng.standard_normal(wl.d)).astype(np.float32), (0.1 * rng.standard_normal((wl.d, wl.K))).astype(np.float32)
+    got = []
+    for make, spoil in ((np.array, False), (pinned, True)):
+        def call(f, *arrays):
+            arrays = [make(a) for a in arrays]
+            out = f(*arrays)
+            if spoil:
+                for a in arrays:
+                    a.view(np.uint8)[...] = 0xFF
+            return out
+
+        with D.DSFacto(wl.n, wl.d, wl.K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, wl.init_seed) as g:
+            call(g.load_csr, wl.indptr, wl.indices, wl.values, wl.y)
+            objective = [g.epoch() for _ in range(2)]
+            call(lambda a, b: g.set_params(0.5, a, b), w, V)
+            objective.append(g.epoch())
+            f = call(g.predict, wl.indptr, wl.indices, wl.values)
+            held = call(g.evaluate, wl.indptr, wl.indices, wl.values, wl.y)
+            got.append((objective, held, f, *g.get_params()))
+    for a, b in zip(*got):
+        assert np.array_equal(np.asarray(a), np.asarray(b))
