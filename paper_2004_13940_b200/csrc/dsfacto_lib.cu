@@ -2568,7 +2568,13 @@ int dsfacto_set_params(dsfacto_t *h, const float *w0, const float *w, const floa
         CU_TRY(h, Courier::get().move(true, {{h->d_w, const_cast<float *>(w), sizeof(float) * (size_t)h->d}}, h->stream));
         CU_TRY(h, cudaStreamSynchronize(h->stream));
     }
-    if (V) { int rc = upload_V(h, V); if (rc) return rc; }
+    if (V) {
+        const int rc = upload_V(h, V);
+        if (rc) {   // w may be new and V not, and neither is what the auxiliaries were made from
+            h->failed = h->failed || h->loaded;
+            return rc;
+        }
+    }
     if (w && V) h->failed = false;   // a handle whose SGD launch gave up is usable again once w and V are replaced
     if (h->loaded) {
         int rc = refresh_now(h);

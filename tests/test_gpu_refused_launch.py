@@ -86,6 +86,25 @@ def test_a_refused_launch_of_other_calls(m):
         _same(g, o)
 
 
+def test_a_handle_does_not_train_on_half_of_the_parameters_it_was_given():
+    wl = W.make("C1")
+    K = 7                          # padded on the device: the launch that is refused
+    o = O.Oracle(wl.n, wl.d, K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, 3)
+    o.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+    rng = np.random.default_rng(1)
+    w, V = rng.standard_normal(wl.d).astype(np.float32), rng.standard_normal((wl.d, K)).astype(np.float32)
+    with D.DSFacto(wl.n, wl.d, K, wl.p, wl.loss, wl.lambda_w, wl.lambda_v, wl.eta, 3) as g:
+        g.load_csr(wl.indptr, wl.indices, wl.values, wl.y)
+        g.debug_set(D.DEBUG_REFUSE_LAUNCH, 1)
+        assert _refused(g, D.dsfacto_set_params(g._h, None, w, V))
+        assert D.dsfacto_epoch(g._h) == D.ERR_CUDA and b"set the parameters again" in D.lib().dsfacto_last_error(g._h)
+        g.set_params(None, w, V)
+        o.w[:], o.V[:] = w, V
+        o.refresh()
+        assert g.epoch() == pytest.approx(o.epoch(), rel=1e-4)
+        _same(g, o)
+
+
 @pytest.mark.parametrize("env", [{"DSFACTO_BANDS": "3"}, {}, {"DSFACTO_ROW_MERGE": "2"}])
 def test_parameters_left_part_of_the_way_are_scored_as_they_are(monkeypatch, env):
     # what an epoch that broke off leaves behind is no result, but scores and a new load go by it as by any parameters
