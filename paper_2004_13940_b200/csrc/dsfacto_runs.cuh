@@ -83,6 +83,10 @@ __device__ __forceinline__ float4 shfl_down4(const float4 x, int o) {
     return make_float4(__shfl_down_sync(0xFFFFFFFFu, x.x, o), __shfl_down_sync(0xFFFFFFFFu, x.y, o),
                        __shfl_down_sync(0xFFFFFFFFu, x.z, o), __shfl_down_sync(0xFFFFFFFFu, x.w, o));
 }
+__device__ __forceinline__ float4 shfl4(const float4 x, int from) {
+    return make_float4(__shfl_sync(0xFFFFFFFFu, x.x, from), __shfl_sync(0xFFFFFFFFu, x.y, from),
+                       __shfl_sync(0xFFFFFFFFu, x.z, from), __shfl_sync(0xFFFFFFFFu, x.w, from));
+}
 // the sum over the lane groups, in every group
 template <int LG, int NV>
 __device__ __forceinline__ void sum_groups(float4 (&x)[NV]) {
@@ -385,16 +389,60 @@ __device__ __forceinline__ float pow_minus_1(int m, double log1m_ew) {
 // ------------------------------------------------------------------------------------------
 // runs_apply_kernel: every run of a pass acts on its column, once.  R runs per lane group, whose records and column
 // rows are requested together (the kernel waits for memory most of the time: one run per group at a time left it
-// at 1.3 TB/s), or one run per warp (COOP: few runs, each cut into many pieces; the lane groups share the pieces).
+// at 1.3 TB/s), or one run per warp (COOP: few runs, each cut into many pieces).
+// A run that lies in several CTAs of the sweep has a piece per CTA, and the most frequent column of a data set has dozens:
+// joined one after the other by the run's own lane group they were a chain of that many trips to L2 (0.7 us each), behind
+// which the kernel ended.  Rows of one float4 per lane: the whole warp joins them, a run at a time, also the two pieces of
+// a run that only crosses a border (leaving those to the lane group costs registers).  Update loop, us, before and after:
+// 2.6 M entries of 128-byte rows 46 -> 41, in four segments 96 -> 78, 11 M entries over 100 k columns 173 -> 152, 390 M
+// entries of 64-byte rows 4300 -> 4130.  Wider rows keep the chain: the join takes registers with which two CTAs fit an SM
+// instead of three (30 M entries of 512-byte rows in three bands 1240 -> 1263; 2.6 M in one band 125 -> 122).
 // ------------------------------------------------------------------------------------------
 template <int LG, int NV, bool COOP>
 struct ApplyCfg {
     static constexpr int R = COOP ? 1 : 2;                         // runs per lane group
     static constexpr int RUNS = COOP ? kThreads / 32 : R * (kThreads / LG);      // runs per CTA
 };
+// Puts a piece behind the run's part (D, W, U) so far.
+template <int NV>
+__device__ __forceinline__ void join_piece(float &D, float &W, float4 (&U)[NV], float pd, float pw, const float4 (&x)[NV]) {
+    const float inv = rcp_fast(1.0f + D);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) fma4(U[v], inv, x[v]);
+    W += pw;
+    D = fmaf(D, pd, D + pd);
+}
+// The np pieces of the run that starts in CTA c0 of the sweep, by a whole warp: a lane group takes consecutive
+// ones, AHEAD of them requested together, and a tree joins the groups' parts.  The whole is left in group 0.
+template <int LG, int NV, int AHEAD>
+__device__ __forceinline__ void join_pieces(const float4 *part, int c0, int np, float &D, float &W, float4 (&U)[NV]) {
+    constexpr int GW = 32 / LG, REC = LG * NV + 1;
+    const int lane = threadIdx.x & 31, l = lane % LG;
+    const int per = (np + GW - 1) / GW, lo = min(np, lane / LG * per), hi = min(np, lo + per);
+    D = 0.f; W = 0.f;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) U[v] = zero4();
+#pragma unroll(AHEAD)
+    for (int i = lo; i < hi; ++i) {
+        const float4 *p = part + ((size_t)(c0 + i) * 2 + (i == 0 ? 1 : 0)) * REC;
+        const float4 hd = __ldcg(p);
+        float4 x[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) x[v] = __ldcg(p + 1 + v * LG + l);
+        join_piece<NV>(D, W, U, hd.x, hd.y, x);
+    }
+#pragma unroll
+    for (int o = LG; o < 32; o <<= 1) {
+        const float Do = __shfl_down_sync(0xFFFFFFFFu, D, o), Wo = __shfl_down_sync(0xFFFFFFFFu, W, o);
+        float4 x[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) x[v] = shfl_down4(U[v], o);
+        if (lane + o < 32) join_piece<NV>(D, W, U, Do, Wo, x);
+    }
+}
 template <int LG, int NV, bool COOP>
 __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel(const RunApplyArgs a) {
-    constexpr int GW = 32 / LG, KP4 = LG * NV, REC = KP4 + 1;
+    constexpr int KP4 = LG * NV, REC = KP4 + 1;
     constexpr int R = ApplyCfg<LG, NV, COOP>::R, RUNS = ApplyCfg<LG, NV, COOP>::RUNS;
     constexpr unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, l = lane % LG, g = lane / LG;
@@ -418,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
     wait_for_previous_kernel();
     if (a.w0_step > 0.0 && blockIdx.x == 0 && threadIdx.x == 0) a.st->w0 = (float)((double)a.st->w0 - a.w0_step * a.st->g);
 
-    // ---- the column rows and the first piece of every run ----
+    // ---- the column rows, and the records of the runs that lie in one CTA of the sweep ----
     float4 y[R][NV], U[R][NV];
     float D[R], W[R], yw[R];
     int np[R];
@@ -426,8 +474,7 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
     auto w_of = [&](int r) { return ((key[r] & 1u) ? a.Tw : a.w) + (key[r] >> 1); };
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int c0 = chunk_of(s[r], a.chunk_inv);
-        np[r] = q[r] >= 0 ? chunk_of(e[r] - 1, a.chunk_inv) - c0 + 1 : 0;
+        np[r] = q[r] >= 0 ? chunk_of(e[r] - 1, a.chunk_inv) - chunk_of(s[r], a.chunk_inv) + 1 : 0;
         D[r] = 0.f; W[r] = 0.f; yw[r] = 0.f;
 #pragma unroll
         for (int v = 0; v < NV; ++v) { y[r][v] = zero4(); U[r][v] = zero4(); }
@@ -437,49 +484,46 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
             for (int v = 0; v < NV; ++v) y[r][v] = __ldcg(row_of(r) + v * LG);
             if (l == 0) yw[r] = __ldcg(w_of(r));
         }
-        if (!COOP) {
-            const float4 *p = np[r] == 1 ? a.rec + (size_t)q[r] * REC : a.part + ((size_t)c0 * 2 + 1) * REC;
+        if (np[r] == 1 ? !COOP || g == 0 : !COOP && NV > 1) {
+            const float4 *p = np[r] == 1 ? a.rec + (size_t)q[r] * REC : a.part + ((size_t)chunk_of(s[r], a.chunk_inv) * 2 + 1) * REC;
             const float4 hd = __ldcg(p);
 #pragma unroll
             for (int v = 0; v < NV; ++v) U[r][v] = __ldcg(p + 1 + v * LG + l);
             D[r] = hd.x; W[r] = hd.y;
         }
     }
-    // ---- the other pieces ----
+    // ---- runs of several pieces: joined by the warp, one run after the other, or each by its own lane group ----
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int c0 = chunk_of(s[r], a.chunk_inv);
-        int lo = 1, hi = np[r];
-        if (COOP) {
-            const int per = (np[r] + GW - 1) / GW;
-            lo = min(np[r], g * per);
-            hi = min(np[r], lo + per);
-        }
-#pragma unroll(COOP ? 4 : 1)
-        for (int i = lo; i < hi; ++i) {
-            const float4 *p = np[r] == 1 ? a.rec + (size_t)q[r] * REC : a.part + ((size_t)(c0 + i) * 2 + (i == 0 ? 1 : 0)) * REC;
-            const float4 hd = __ldcg(p);
-            float4 x[NV];
+        if (!COOP && NV > 1) {
+            for (int i = 1; i < np[r]; ++i) {
+                const float4 *p = a.part + (size_t)(c0 + i) * 2 * REC;
+                const float4 hd = __ldcg(p);
+                float4 x[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) x[v] = __ldcg(p + 1 + v * LG + l);
-            const float inv = rcp_fast(1.0f + D[r]);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) fma4(U[r][v], inv, x[v]);
-            W[r] += hd.y;
-            D[r] = fmaf(D[r], hd.x, D[r] + hd.x);
+                for (int v = 0; v < NV; ++v) x[v] = __ldcg(p + 1 + v * LG + l);
+                join_piece<NV>(D[r], W[r], U[r], hd.x, hd.y, x);
+            }
+            continue;
         }
         if (COOP) {
+            if (np[r] > 1) join_pieces<LG, NV, 4>(a.part, c0, np[r], D[r], W[r], U[r]);
+            continue;
+        }
+        for (uint32_t todo = __ballot_sync(FULL, l == 0 && np[r] > 1); todo != 0u; todo &= todo - 1u) {
+            const int owner = __ffs(todo) - 1;
+            float Dr, Wr;
+            float4 Ur[NV];
+            join_pieces<LG, NV, 2>(a.part, __shfl_sync(FULL, c0, owner), __shfl_sync(FULL, np[r], owner), Dr, Wr, Ur);
+            Dr = __shfl_sync(FULL, Dr, l);
+            Wr = __shfl_sync(FULL, Wr, l);
 #pragma unroll
-            for (int o = LG; o < 32; o <<= 1) {
-                const float Do = __shfl_down_sync(FULL, D[r], o), Wo = __shfl_down_sync(FULL, W[r], o);
-                const float inv = rcp_fast(1.0f + D[r]);
-                const bool in = lane + o < 32;
+            for (int v = 0; v < NV; ++v) Ur[v] = shfl4(Ur[v], l);
+            if (g == owner / LG) {
+                D[r] = Dr; W[r] = Wr;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const float4 Uo = shfl_down4(U[r][v], o);
-                    if (in) fma4(U[r][v], inv, Uo);
-                }
-                if (in) { W[r] += Wo; D[r] = fmaf(D[r], Do, D[r] + Do); }
+                for (int v = 0; v < NV; ++v) U[r][v] = Ur[v];
             }
         }
     }

@@ -48,6 +48,41 @@ def test_bands_units_and_widths(monkeypatch, bands, chunk, K, p, every):
         np.testing.assert_allclose(G, o.G, rtol=0, atol=2e-5)
 
 
+@pytest.mark.parametrize("K", [4, 8, 16, 30, 64, 128])
+def test_long_runs_among_many_short_ones(monkeypatch, K):
+    """More runs than a warp each is given to, and among them runs of 1 to 33 pieces (a CTA of the sweep has 128 entries
+    here), so that a warp joins pieces for some of its runs: fewer pieces than lane groups, as many, more."""
+    monkeypatch.setenv("DSFACTO_CHUNK", "32")
+    rng = np.random.default_rng(K)
+    n, short = 4200, 10000
+    rows, cols = [], []
+    for j, length in enumerate([127, 128, 129, 256, 257, 385, 512, 640, 1023, 1025, 2049, 4100, 4200]):
+        rows.append(rng.choice(n, length, replace=False))
+        cols.append(np.full(length, 700 * j + 3))
+    d = short + 700 * 13
+    taken = set(700 * j + 3 for j in range(13))
+    others = np.array([j for j in rng.permutation(d) if j not in taken][:short])
+    rows.append(rng.integers(0, n, short))
+    cols.append(others)
+    rows, cols = np.concatenate(rows), np.concatenate(cols)
+    order = np.lexsort((cols, rows))
+    indices = cols[order].astype(np.int32)
+    indptr = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=n))]).astype(np.int64)
+    values = rng.standard_normal(len(indices)).astype(np.float32)
+    y = np.where(rng.random(n) < 0.5, 1.0, -1.0).astype(np.float32)
+    o = O.Oracle(n, d, K, 3, O.LOGISTIC, 1e-2, 1e-2, 0.7, 3)
+    o.load_csr(indptr, indices, values, y)
+    with D.DSFacto(n, d, K, 3, D.LOGISTIC, 1e-2, 1e-2, 0.7, 3) as g:
+        g.load_csr(indptr, indices, values, y)
+        for _ in range(2):
+            bw, bV = o.w.copy(), o.V.copy()
+            assert g.epoch() == pytest.approx(o.epoch(), rel=1e-5)
+            w0, w, V = g.get_params()
+            assert w0 == pytest.approx(o.w0, abs=1e-6)
+            for new, ref, old in ((w, o.w, bw), (V, o.V, bV)):
+                assert np.abs(new.astype(np.float64) - ref).max() <= 1e-4 * np.abs(ref - old).max() + 1e-7
+
+
 def _wide_rows(n, d, per_row, seed):
     rng = np.random.default_rng(seed)
     idx = rng.integers(0, d // per_row, (n, per_row), dtype=np.int32) + (np.arange(per_row, dtype=np.int32) * (d // per_row))
