@@ -106,13 +106,14 @@ struct dsfacto {
 
     // scalars of an epoch on the device, and the mapped host memory its last kernel reports to
     EpochState *d_state = nullptr;
-    EpochReport *report = nullptr;
-    unsigned long long report_seq = 0, epoch_seq = 0;   // last number of a scoring or copying kernel; of a recompute pass (before_report)
+    Report *report = nullptr;
+    uint32_t call_number = 0, epoch_number = 0;   // of the last scoring or copying kernel; of the last recompute pass (before_report)
     cudaError_t launch_error = cudaSuccess;   // of the first launch that was refused since the last look (launch_status)
     int refuse_launch = 0;                    // tests: the launch that this counts down to is refused
     cudaGraphExec_t epoch_graph = nullptr;   // the launches of an epoch (all but the sweep over tiles and shards)
     int epochs_run = 0;
     int64_t epoch_launches = 0;
+    EpochBody ended{};            // the last report of a recompute pass
     char *mail = nullptr;          // the rest of that memory: small inputs and results (mail_bytes of it)
     size_t mail_bytes = 0;
     // update loop by column runs (dsfacto_runs.cuh): every load that is bucketed on the device with default settings
@@ -990,26 +991,46 @@ int run_finish(dsfacto *h) {
     return DSFACTO_OK;
 }
 
-// Waits until a kernel has delivered its report (the last thing it does): number `want` in `at`.  If a launch was
-// refused there will be none: what was launched is waited for instead.  The stream is asked now and then, so that a
+// Waits until what a kernel sends has arrived.  If a launch was
+// refused there will be nothing: what was launched is waited for instead.  The stream is asked now and then, so that a
 // kernel that failed ends the wait as well.
-int wait_report(dsfacto *h, const volatile unsigned long long &at, unsigned long long want) {
+template <class Arrived>
+int wait_for(dsfacto *h, Arrived arrived) {
     const int rc = launch_status(h);
     if (rc) {
         cudaStreamSynchronize(h->stream);
         return rc;
     }
-    for (unsigned spin = 1; at != want; ++spin) {
+    for (unsigned spin = 1; !arrived(); ++spin) {
         spin_pause();
         if ((spin & 0x3FFFu) != 0) continue;
         const cudaError_t e = cudaStreamQuery(h->stream);
         if (e == cudaErrorNotReady) continue;
-        if (e == cudaSuccess && at == want) break;
+        if (e == cudaSuccess && arrived()) break;
         h->err = std::string("report: ") + (e == cudaSuccess ? "the last kernel left none" : cudaGetErrorString(e));
         return DSFACTO_ERR_CUDA;
     }
     spin_done();
     return DSFACTO_OK;
+}
+// A word of a report: its number, and its contents once the number is there.
+uint32_t word_number(const unsigned long long &word) { return (uint32_t)(*const_cast<const volatile unsigned long long *>(&word) >> 32); }
+bool take_word(const unsigned long long &word, uint32_t number, uint32_t &contents) {
+    const unsigned long long x = *const_cast<const volatile unsigned long long *>(&word);
+    contents = (uint32_t)x;
+    return (uint32_t)(x >> 32) == number;
+}
+uint32_t next_call(dsfacto *h) { return h->call_number = h->call_number == 0xFFFFFFFFu ? 1u : h->call_number + 1; }   // (never 0)
+template <class Body>
+int wait_report(dsfacto *h, const unsigned long long *words, uint32_t number, Body &body) {
+    uint32_t contents[kReportWords<Body>];
+    int at = 0;
+    const int rc = wait_for(h, [&]() {
+        while (at < kReportWords<Body> && take_word(words[at], number, contents[at])) ++at;
+        return at == kReportWords<Body>;
+    });
+    if (!rc) std::memcpy(&body, contents, sizeof body);
+    return rc;
 }
 
 // Recompute pass with the squared norms of the objective; w0 is taken from the device.  report: the pass is the
@@ -1029,15 +1050,16 @@ int run_refresh(dsfacto *h, bool first, bool report) {
 }
 // The device counts the reports of recompute passes.  What the host waits for is the number after the one that lies in
 // the report before the launches, so a pass that never ran leaves the two counts in step.
-void before_report(dsfacto *h) { h->epoch_seq = *const_cast<const volatile unsigned long long *>(&h->report->epochs); }
+void before_report(dsfacto *h) { h->epoch_number = word_number(h->report->epoch[0]); }
 // ... and its sums on the host
 int collect(dsfacto *h) {
     if (h->nshards > 1) return DSFACTO_OK;
-    const int rc = wait_report(h, h->report->epochs, h->epoch_seq + 1);
+    EpochBody r;
+    const int rc = wait_report(h, h->report->epoch, h->epoch_number + 1, r);
     if (rc) return rc;
-    const EpochReport r = *h->report;
     h->loss_sum = r.loss; h->g_sum = r.g; h->w2 = r.w2; h->v2 = r.v2; h->w0 = r.w0;
     h->objective = r.loss / (double)h->n + 0.5 * (double)h->lambda_w * r.w2 + 0.5 * (double)h->lambda_v * r.v2;
+    h->ended = r;
     return DSFACTO_OK;
 }
 // ... with the host's w0.  If it cannot be had, the auxiliaries are not those of the parameters.
@@ -1621,10 +1643,10 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
         return fail(rc);
 
     if ((rc = dev_alloc(h, &h->d_state, 1))) return fail(rc);
-    h->report = static_cast<EpochReport *>(Mailboxes::get().take());
+    h->report = static_cast<Report *>(Mailboxes::get().take());
     if (!h->report) return fail(DSFACTO_ERR_OOM);
-    std::memset(h->report, 0, sizeof(EpochReport));
-    constexpr size_t kReportBytes = (sizeof(EpochReport) + 255) & ~(size_t)255;
+    std::memset(h->report, 0, sizeof(Report));
+    constexpr size_t kReportBytes = (sizeof(Report) + 255) & ~(size_t)255;
     h->mail = reinterpret_cast<char *>(h->report) + kReportBytes;
     h->mail_bytes = kMailboxBytes - kReportBytes;
 
@@ -2317,7 +2339,7 @@ static int broke_off(dsfacto *h) {
     drop_epoch_graph(h);
     const size_t d = (size_t)h->d;
     cudaMemsetAsync(h->d_state, 0, sizeof(EpochState), h->stream);
-    h->report->epochs = 0;
+    std::memset(h->report->epoch, 0, sizeof h->report->epoch);
     if (!h->runs) {
         cudaMemsetAsync(h->d_run_count, 0, sizeof(int) * (size_t)std::max<int64_t>(h->long_runs, 1), h->stream);
         cudaMemsetAsync(h->d_sync, 0, sizeof(int) * sync_words(h->p), h->stream);
@@ -2448,14 +2470,14 @@ static int epoch_impl(dsfacto_t *h) {
         cudaEventElapsedTime(&t12, h->ev[1], h->ev[2]);
         h->ms[0] = t01 + t12; h->ms[1] = t01; h->ms[2] = t12; h->ms[3] = 0.f;
     } else {
-        h->ms[1] = (float)(1e-6 * (double)h->report->ns[0]);
-        h->ms[2] = (float)(1e-6 * (double)h->report->ns[1]);
+        h->ms[1] = (float)(1e-6 * (double)h->ended.ns[0]);
+        h->ms[2] = (float)(1e-6 * (double)h->ended.ns[1]);
         h->ms[0] = h->ms[1] + h->ms[2];
         h->ms[3] = 0.f;
     }
     int sgd_error[3] = {0, 0, 0};  // set by the SGD kernel if a bounded wait ran out or a check of the debug build failed
     if (!h->runs) CU_TRY(h, cudaMemcpy(sgd_error, h->d_sync + kSyncError, sizeof sgd_error, cudaMemcpyDeviceToHost));
-    else if (!shard) for (int c = 0; c < 3; ++c) sgd_error[c] = h->report->err[c];
+    else if (!shard) for (int c = 0; c < 3; ++c) sgd_error[c] = h->ended.err[c];
     if (sgd_error[0]) return sgd_gave_up(h, sgd_error);
     if (shard) return DSFACTO_OK;   // the objective exists only after the shards' sums have been added up
     return std::isfinite(h->objective) ? DSFACTO_OK : DSFACTO_ERR_DIVERGED;
@@ -2547,8 +2569,9 @@ int dsfacto_get_params(dsfacto_t *h, float *w0, float *w, float *V) {
         float *mw = reinterpret_cast<float *>(h->mail), *mV = reinterpret_cast<float *>(h->mail + w_bytes);
         const int grid = (int)((std::max(w_bytes, V_bytes) / sizeof(float) + kThreads - 1) / kThreads);
         launch_overlapped(h, copy_out_kernel, grid, kThreads, 0, (const float *)h->d_w, (int64_t)h->d, (const float *)h->d_V, (int)h->K, (int)h->Kp,
-                          w ? mw : nullptr, V ? mV : nullptr, &h->d_state->done, h->report, ++h->report_seq);
-        const int rc = wait_report(h, h->report->seq, h->report_seq);
+                          w ? mw : nullptr, V ? mV : nullptr, &h->d_state->done, h->report, next_call(h));
+        CallBody r;
+        const int rc = wait_report(h, h->report->call, h->call_number, r);
         if (rc) return rc;
         if (w) std::memcpy(w, mw, w_bytes);
         if (V) std::memcpy(V, mV, V_bytes);
@@ -2684,7 +2707,7 @@ static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_
 // 21.4; of one entry, 3 x 1.5 KB 17.9 / 18.9, 10 x 6 KB 23.2 / 20.7, 38 x 24 KB 47.7 / 23.9; 8 factors, rows of 39 entries,
 // 1 x 24 KB 25.6 / 34.6; of 20 entries, 2 x 24 KB 24.8 / 28.1; of one entry, 2 x 3 KB 18.8 / 19.8, 5 x 12 KB 24.4 / 21.7.
 static bool staging_pays(size_t size, int ctas, int64_t m, int64_t nnz) {
-    return size <= (size_t)24 << 10 && (double)size * ctas <= 12288.0 + 1800.0 * (double)nnz / (double)m;
+    return size <= (size_t)kMostStaged && (double)size * ctas <= 12288.0 + 1800.0 * (double)nnz / (double)m;
 }
 
 // Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
@@ -2694,7 +2717,7 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
                       const float *values, const float *y, float *scores_out, double sums2[2]) {
     RefreshArgs a{};
     a.w0 = h->w0; a.loss = h->loss; a.n = m;
-    a.done = &h->d_state->done; a.report = h->report; a.seq = h->report_seq + 1;
+    a.done = &h->d_state->done; a.report = h->report; a.number = next_call(h);
     const int grid = refresh_grid_for(h, m);
     // everything the call allocates on the device is one block: [indptr | indices | values | y | partial sums | scores]
     char *block = nullptr;
@@ -2702,7 +2725,7 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
     auto room = [&](size_t bytes) { const size_t at = used; used += (bytes + 255) & ~(size_t)255; return at; };
     const size_t part_at = room(mode == kEvaluate ? 4 * sizeof(double) * (size_t)grid : 0);
     int rc = DSFACTO_OK;
-    bool mailed_out = false;   // the scores come through the mailbox
+    unsigned long long *mailed = nullptr;   // the scores come through the mailbox
     auto cleanup = [&]() { dev_free(block); };
     if (!indptr) {
         if (!h->loaded) return DSFACTO_ERR_NO_DATA;
@@ -2717,8 +2740,9 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         const int64_t nnz = indptr[m];
         if (nnz > 0 && (!indices || !values)) return DSFACTO_ERR_INVALID_ARG;
         const size_t ip_b = sizeof(int64_t) * ((size_t)m + 1), e_b = 4 * (size_t)nnz, y_b = sizeof(float) * (size_t)m;
-        const size_t mail = ip_b + 2 * e_b + y_b;   // (labels in, or scores out)
-        if (mail <= h->mail_bytes) {
+        const size_t mail = ip_b + 2 * e_b + (y ? y_b : 0);
+        const size_t f_b = mode == kScore ? sizeof(*mailed) * (size_t)m : 0;
+        if (((mail + 15) & ~(size_t)15) + f_b <= h->mail_bytes) {
             // A request: the kernel reads the rows from the mailbox across the link and leaves the scores there, which
             // takes less time than copies in and out before and behind it (32 rows: 60 us -> 20 us per call).
             if (!sound_rows(m, h->d, indptr, indices, values, y)) return DSFACTO_ERR_INVALID_CSR;
@@ -2728,9 +2752,13 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
             a.indptr = reinterpret_cast<int64_t *>(p);
             a.idx = reinterpret_cast<int32_t *>(p + ip_b);
             a.val = reinterpret_cast<float *>(p + ip_b + e_b);
-            float *last = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
-            if (mode == kScore) { a.f_out = last; mailed_out = true; }
-            else { std::memcpy(last, y, y_b); a.y = last; }
+            a.y = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
+            if (y) std::memcpy(p + ip_b + 2 * e_b, y, y_b);
+            if (mode == kScore) {   // the scores are their own report: words without this call's number, until they arrive
+                a.f_words = mailed = reinterpret_cast<unsigned long long *>(p + ((mail + 15) & ~(size_t)15));
+                std::memset(mailed, 0, f_b);
+                a.report = nullptr;
+            }
             if (staging_pays(mail, grid, m, nnz)) {
                 a.stage = reinterpret_cast<const uint4 *>(p);
                 a.stage_bytes = (int)((mail + 15) & ~(size_t)15);
@@ -2765,14 +2793,20 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         model_view(h, a, false);
     }
     a.partials = reinterpret_cast<double *>(block + part_at);
-    ++h->report_seq;
     if (mode == kScore) DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kScore, grid);
     else DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kEvaluate, grid);
-    rc = wait_report(h, h->report->seq, h->report_seq);
-    if (!rc && h->report->bad) rc = DSFACTO_ERR_INVALID_CSR;
-    if (!rc && mode == kScore) {
-        if (mailed_out) std::memcpy(scores_out, a.f_out, sizeof(float) * (size_t)m);
-        else {
+    CallBody r{};
+    if (mailed) {
+        int64_t at = 0;
+        uint32_t bits;
+        rc = wait_for(h, [&]() {
+            for (; at < m && take_word(mailed[at], a.number, bits); ++at) std::memcpy(scores_out + at, &bits, sizeof bits);
+            return at == m;
+        });
+    } else {
+        rc = wait_report(h, h->report->call, a.number, r);
+        if (!rc && r.bad) rc = DSFACTO_ERR_INVALID_CSR;
+        if (!rc && mode == kScore) {
             const Piece out = {a.f_out, scores_out, sizeof(float) * (size_t)m};
             const cudaError_t e = Courier::get().move(false, &out, 1, h->stream);
             if (e != cudaSuccess) { h->err = cudaGetErrorString(e); rc = DSFACTO_ERR_CUDA; }
@@ -2782,8 +2816,7 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         if (a.bad) cudaMemsetAsync(a.bad, 0, sizeof(int), h->stream);   // (the kernel that did not run would have)
         cudaStreamSynchronize(h->stream);
     }
-    h->report->bad = 0;
-    if (!rc && mode == kEvaluate) { sums2[0] = h->report->loss; sums2[1] = h->report->g; }
+    if (!rc && mode == kEvaluate) { sums2[0] = r.loss; sums2[1] = r.g; }
     cleanup();
     return rc;
 }

@@ -49,8 +49,9 @@ struct RefreshArgs {
     // end of the pass: the last CTA adds the partial sums up
     unsigned *done;        // CTAs that have delivered (zero between launches)
     EpochState *st;        // kTrain: w0 comes from here and the sums go here; NULL: w0 above
-    EpochReport *report;   // mapped host memory: the sums and, behind them, a number (NULL: not the end of an epoch)
-    unsigned long long seq;   // ... which is this one (kTrain: the number of such reports, counted on the device)
+    Report *report;        // mapped host memory (NULL: not the end of an epoch, or the scores are the report)
+    uint32_t number;       // ... the number of the report (kTrain: counted on the device)
+    unsigned long long *f_words;   // kScore: scores to mapped host memory, as words of a report each (NULL: to f_out)
     int first;             // kTrain: the first segment of an epoch (its times are set, not added)
     // STAGED: a small batch in mapped host memory, [indptr | idx | val | y]; indptr, idx, val, y are then offsets into it
     const uint4 *stage;
@@ -58,7 +59,7 @@ struct RefreshArgs {
     int *bad;              // caller rows that were checked on the device: no row is read if it is set (NULL: sound rows)
 };
 
-// Sums of the whole launch in a fixed order: thread 0 of the last CTA to get here returns true and holds them.
+// Sums of the whole launch in a fixed order: true in the last CTA to get here, whose thread 0 holds them.
 __device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, unsigned *done) {
     __shared__ bool last;
     block_sum4(s);
@@ -77,7 +78,7 @@ __device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, 
 #pragma unroll
         for (int c = 0; c < 4; ++c) s[c] += __ldcg(partials + 4 * (size_t)b + c);
     block_sum4(s);
-    return threadIdx.x == 0;
+    return true;
 }
 
 // The last thread of a kernel whose CTAs have all written their results (to memory of the host as well): thread 0
@@ -123,6 +124,7 @@ struct RefreshCfg {
     static constexpr int CTAS = STAGED ? 1 : LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
 };
+constexpr int kMostStaged = 24 << 10;   // bytes of a staged batch
 // STAGED: every CTA first copies the whole batch from the host's memory to shared memory, all of it at once: one
 // trip across the link instead of one for the row pointers and one for every two batches of entries.
 template <int LG, int NV, int MODE, bool RAW = false, bool STAGED = false>
@@ -145,9 +147,15 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     const int32_t *idx = a.idx;
     const float *val = a.val, *lab = a.y;
     if (STAGED) {
-        uint4 *to = staged;
-        for (int i = threadIdx.x; i < a.stage_bytes / 16; i += kThreads) to[i] = a.stage[i];
-        const char *p = reinterpret_cast<const char *>(to);
+        // (all requests before the first store: one trip)
+        uint4 piece[kMostStaged / 16 / kThreads];
+#pragma unroll
+        for (int i = 0; i < kMostStaged / 16 / kThreads; ++i)
+            if (i * kThreads + (int)threadIdx.x < a.stage_bytes / 16) piece[i] = a.stage[i * kThreads + threadIdx.x];
+#pragma unroll
+        for (int i = 0; i < kMostStaged / 16 / kThreads; ++i)
+            if (i * kThreads + (int)threadIdx.x < a.stage_bytes / 16) staged[i * kThreads + threadIdx.x] = piece[i];
+        const char *p = reinterpret_cast<const char *>(staged);
         indptr = reinterpret_cast<const int64_t *>(p);
         idx = reinterpret_cast<const int32_t *>(p + reinterpret_cast<size_t>(a.idx));
         val = reinterpret_cast<const float *>(p + reinterpret_cast<size_t>(a.val));
@@ -287,7 +295,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
         }
         if (l == 0 && row < n) {
             const float f = w0 + lin + 0.5f * pair;
-            if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
+            if (MODE == kScore && a.f_words) store_report_word(a.f_words + row, a.number, __float_as_uint(f));
+            else if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
             if (MODE != kScore) {
                 const float yy = lab[row];
                 float li, gi;
@@ -312,11 +321,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
         }
     }
     if (MODE == kScore && a.report && last_thread(a.done)) {
-        volatile EpochReport *r = a.report;
-        r->bad = bad;
         if (a.bad) *a.bad = 0;
-        __threadfence_system();
-        r->seq = a.seq;
+        for (int i = 0; i < kReportWords<CallBody>; ++i) store_report_word(a.report->call + i, a.number, (uint32_t)bad);   // (nothing else is looked at)
     }
     if (MODE == kTrain || MODE == kEvaluate || MODE == kScoreSums) {
         double s[4] = {l == 0 ? sums[0][g] : 0.0, l == 0 ? sums[1][g] : 0.0, 0.0, 0.0};
@@ -332,37 +338,35 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
                 s[3] += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
             }
         }
-        if (last_cta_sum4(s, a.partials, a.done)) {
-            if (TRAIN && a.st) {
-                EpochState &st = *a.st;
-                st.loss = s[0]; st.g = s[1]; st.w2 = s[2]; st.v2 = s[3];
-            }
-            if (MODE == kScoreSums) { a.sums_out[0] = s[0]; a.sums_out[1] = s[1]; }
-            if (a.report) {
-                volatile EpochReport *r = a.report;
-                r->loss = s[0]; r->g = s[1]; r->w2 = s[2]; r->v2 = s[3];
+        if (last_cta_sum4(s, a.partials, a.done) && threadIdx.x < 32) {
+            __shared__ EpochBody ended;
+            __shared__ CallBody called;
+            uint32_t number = a.number;
+            if (threadIdx.x == 0) {
+                if (MODE == kScoreSums) { a.sums_out[0] = s[0]; a.sums_out[1] = s[1]; }
                 if (MODE == kEvaluate) {
-                    r->bad = bad;
+                    called.loss = s[0]; called.g = s[1]; called.bad = bad; called.unused = 0;
                     if (a.bad) *a.bad = 0;
                 }
-            }
-            if (TRAIN && a.st) {
-                EpochState &st = *a.st;
-                const unsigned long long now = device_ns();
-                const unsigned long long ns0 = st.t1 - st.t0 + (a.first ? 0ull : st.ns[0]), ns1 = now - st.t1 + (a.first ? 0ull : st.ns[1]);
-                st.ns[0] = ns0; st.ns[1] = ns1;
-                if (a.report) {
-                    volatile EpochReport *r = a.report;
-                    r->w0 = st.w0;
-                    r->ns[0] = ns0; r->ns[1] = ns1;
-                    for (int c = 0; c < 3; ++c) r->err[c] = st.err[c];
+                if (TRAIN && a.st) {
+                    EpochState &st = *a.st;
+                    st.loss = s[0]; st.g = s[1]; st.w2 = s[2]; st.v2 = s[3];
+                    const unsigned long long now = device_ns();
+                    const unsigned long long ns0 = st.t1 - st.t0 + (a.first ? 0ull : st.ns[0]), ns1 = now - st.t1 + (a.first ? 0ull : st.ns[1]);
+                    st.ns[0] = ns0; st.ns[1] = ns1;
+                    if (a.report) {
+                        ended.loss = s[0]; ended.g = s[1]; ended.w2 = s[2]; ended.v2 = s[3];
+                        ended.w0 = st.w0;
+                        ended.ns[0] = ns0; ended.ns[1] = ns1;
+                        for (int c = 0; c < 3; ++c) ended.err[c] = st.err[c];
+                        number = ++st.epochs;
+                    }
                 }
             }
-            if (a.report) {
-                __threadfence_system();
-                volatile EpochReport *r = a.report;
-                if (TRAIN) r->epochs = ++a.st->epochs;
-                else r->seq = a.seq;
+            if (a.report && (MODE == kTrain || MODE == kEvaluate)) {
+                number = __shfl_sync(0xFFFFFFFFu, number, 0);
+                if (MODE == kTrain) store_report(a.report->epoch, number, ended);
+                else store_report(a.report->call, number, called);
             }
         }
     }

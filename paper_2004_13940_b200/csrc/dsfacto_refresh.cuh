@@ -8,7 +8,7 @@ namespace dsf {
 
 // Parameters of a small model to mapped host memory, with a report behind them.
 __global__ void __launch_bounds__(kThreads) copy_out_kernel(const float *w, int64_t d, const float *V, int K, int Kp, float *out_w, float *out_V,
-                                                            unsigned *done, EpochReport *report, unsigned long long seq) {
+                                                            unsigned *done, Report *report, uint32_t number) {
     const int64_t stride = (int64_t)gridDim.x * kThreads, first = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     let_next_kernel_start();
     wait_for_previous_kernel();
@@ -16,7 +16,8 @@ __global__ void __launch_bounds__(kThreads) copy_out_kernel(const float *w, int6
         for (int64_t i = first; i < d; i += stride) out_w[i] = w[i];
     if (out_V)
         for (int64_t i = first; i < d * K; i += stride) out_V[i] = V[i / K * Kp + i % K];
-    if (last_thread(done)) ((volatile EpochReport *)report)->seq = seq;
+    if (last_thread(done))
+        for (int i = 0; i < kReportWords<CallBody>; ++i) store_report_word(report->call + i, number, 0u);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int c0 = chunk_of(s[r], a.chunk_inv);
-        if (!COOP && NV > 1) {
+        if constexpr (!COOP && NV > 1) {
             for (int i = 1; i < np[r]; ++i) {
                 const float4 *p = a.part + (size_t)(c0 + i) * 2 * REC;
                 const float4 hd = __ldcg(p);
@@ -505,25 +505,23 @@ __global__ void __launch_bounds__(kThreads, (NV == 1 ? 4 : 2)) runs_apply_kernel
                 for (int v = 0; v < NV; ++v) x[v] = __ldcg(p + 1 + v * LG + l);
                 join_piece<NV>(D[r], W[r], U[r], hd.x, hd.y, x);
             }
-            continue;
-        }
-        if (COOP) {
+        } else if constexpr (COOP) {
             if (np[r] > 1) join_pieces<LG, NV, 4>(a.part, c0, np[r], D[r], W[r], U[r]);
-            continue;
-        }
-        for (uint32_t todo = __ballot_sync(FULL, l == 0 && np[r] > 1); todo != 0u; todo &= todo - 1u) {
-            const int owner = __ffs(todo) - 1;
-            float Dr, Wr;
-            float4 Ur[NV];
-            join_pieces<LG, NV, 2>(a.part, __shfl_sync(FULL, c0, owner), __shfl_sync(FULL, np[r], owner), Dr, Wr, Ur);
-            Dr = __shfl_sync(FULL, Dr, l);
-            Wr = __shfl_sync(FULL, Wr, l);
+        } else {
+            for (uint32_t todo = __ballot_sync(FULL, l == 0 && np[r] > 1); todo != 0u; todo &= todo - 1u) {
+                const int owner = __ffs(todo) - 1;
+                float Dr, Wr;
+                float4 Ur[NV];
+                join_pieces<LG, NV, 2>(a.part, __shfl_sync(FULL, c0, owner), __shfl_sync(FULL, np[r], owner), Dr, Wr, Ur);
+                Dr = __shfl_sync(FULL, Dr, l);
+                Wr = __shfl_sync(FULL, Wr, l);
 #pragma unroll
-            for (int v = 0; v < NV; ++v) Ur[v] = shfl4(Ur[v], l);
-            if (g == owner / LG) {
-                D[r] = Dr; W[r] = Wr;
+                for (int v = 0; v < NV; ++v) Ur[v] = shfl4(Ur[v], l);
+                if (g == owner / LG) {
+                    D[r] = Dr; W[r] = Wr;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) U[r][v] = Ur[v];
+                    for (int v = 0; v < NV; ++v) U[r][v] = Ur[v];
+                }
             }
         }
     }
