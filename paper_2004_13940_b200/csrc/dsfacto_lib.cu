@@ -5,6 +5,7 @@
 #include "dsfacto_host.cuh"
 #include "dsfacto_prepare.cuh"
 #include "dsfacto_refresh.cuh"
+#include "dsfacto_request.cuh"
 #include "dsfacto_runplan.cuh"
 #include "dsfacto_runs.cuh"
 #include "dsfacto_sgd.cuh"
@@ -476,13 +477,16 @@ void launch_sgd(dsfacto *h, const SgdArgs &a, int64_t chunks) {
 }
 template <int LG, int NV>
 void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
-    const size_t smem = a.stage ? (size_t)a.stage_bytes : 0;
-    if (a.stage && mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate, false, true>, grid, kThreads, smem, a);
-    else if (a.stage) launch_overlapped(h, refresh_kernel<LG, NV, kScore, false, true>, grid, kThreads, smem, a);
-    else if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, smem, a);
-    else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, smem, a);
-    else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, smem, a);
-    else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, smem, a);
+    if (mode == kTrain) launch_overlapped(h, refresh_kernel<LG, NV, kTrain>, grid, kThreads, 0, a);
+    else if (mode == kEvaluate) launch_overlapped(h, refresh_kernel<LG, NV, kEvaluate>, grid, kThreads, 0, a);
+    else if (mode == kPartial) launch_overlapped(h, refresh_kernel<LG, NV, kPartial>, grid, kThreads, 0, a);
+    else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, 0, a);
+}
+template <int LG, int NV>
+void launch_request(dsfacto *h, const RequestArgs &a, int mode, int grid) {
+    auto kernel = mode == kEvaluate ? request_kernel<LG, NV, kEvaluate> : request_kernel<LG, NV, kScore>;
+    if (a.stride > (47 << 10)) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMailboxBytes);   // (a refusal shows at the launch)
+    launch_overlapped(h, kernel, grid, kThreads, a.stride, a);
 }
 
 #define DSF_DISPATCH(h, FN, ...)                                   \
@@ -2700,14 +2704,39 @@ static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_
     return true;
 }
 
-// Whether a batch in the mailbox is staged: every CTA copies all of it to shared memory in one trip across the link,
-// instead of one trip for its row pointers and one for every two batches of its rows' entries.  That saves trips, the more
-// the longer the rows, and costs the link (CTAs x size).  Calls of dsfacto_predict, staged / not, in us: 32 factors, rows
-// of 39 entries, 2 CTAs x 12 KB 23.1 / 25.5, 3 x 24 KB 25.6 / 27.8; of 8 entries, 2 x 3 KB 17.6 / 18.5, 5 x 12 KB 24.1 /
-// 21.4; of one entry, 3 x 1.5 KB 17.9 / 18.9, 10 x 6 KB 23.2 / 20.7, 38 x 24 KB 47.7 / 23.9; 8 factors, rows of 39 entries,
-// 1 x 24 KB 25.6 / 34.6; of 20 entries, 2 x 24 KB 24.8 / 28.1; of one entry, 2 x 3 KB 18.8 / 19.8, 5 x 12 KB 24.4 / 21.7.
-static bool staging_pays(size_t size, int ctas, int64_t m, int64_t nnz) {
-    return size <= (size_t)kMostStaged && (double)size * ctas <= 12288.0 + 1800.0 * (double)nnz / (double)m;
+// A small batch as blocks of rows (dsfacto_request.cuh): rows of a block, and bytes from block to block (0: it does not fit).
+struct RequestLayout {
+    int rows = 0;
+    int64_t blocks = 0;
+    size_t stride = 0;
+};
+static RequestLayout request_layout(const dsfacto *h, int64_t m, const int64_t *indptr, bool labels, size_t room) {
+    RequestLayout r;
+    if ((size_t)m > room / 8) return r;
+    // a row per warp while that leaves no more CTAs than two per SM
+    const int64_t warps = kThreads / 32, per_warp = (m + 2 * warps * h->sm_count - 1) / (2 * warps * h->sm_count);
+    r.rows = (int)std::min<int64_t>(warps * per_warp, kMostBlockRows);
+    r.blocks = (m + r.rows - 1) / r.rows;
+    int64_t most = 0;
+    for (int64_t r0 = 0; r0 < m; r0 += r.rows) {
+        const int64_t e = indptr[std::min<int64_t>(m, r0 + r.rows)] - indptr[r0];
+        if (e < 0 || e > (int64_t)room / 8) return r;
+        most = std::max(most, e);
+    }
+    const size_t stride = (4 * (size_t)(r.rows + 1) + 8 * (size_t)most + (labels ? 4 * (size_t)r.rows : 0) + 15) & ~(size_t)15;
+    if (stride * (size_t)r.blocks <= room) r.stride = stride;
+    return r;
+}
+static void lay_out_request(char *to, const RequestLayout &lay, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values, const float *y) {
+    for (int64_t r0 = 0; r0 < m; r0 += lay.rows, to += lay.stride) {
+        const int64_t r1 = std::min<int64_t>(m, r0 + lay.rows), e0 = indptr[r0];
+        const size_t e = (size_t)(indptr[r1] - e0);
+        int32_t *first = reinterpret_cast<int32_t *>(to);
+        for (int r = 0; r <= lay.rows; ++r) first[r] = (int32_t)(indptr[std::min(r0 + r, r1)] - e0);
+        char *at = to + 4 * (size_t)(lay.rows + 1);
+        if (e > 0) { std::memcpy(at, indices + e0, 4 * e); std::memcpy(at + 4 * e, values + e0, 4 * e); }
+        if (y) std::memcpy(at + 8 * e, y + r0, 4 * (size_t)(r1 - r0));
+    }
 }
 
 // Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
@@ -2718,19 +2747,22 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
     RefreshArgs a{};
     a.w0 = h->w0; a.loss = h->loss; a.n = m;
     a.done = &h->d_state->done; a.report = h->report; a.number = next_call(h);
-    const int grid = refresh_grid_for(h, m);
+    int grid = refresh_grid_for(h, m);
     // everything the call allocates on the device is one block: [indptr | indices | values | y | partial sums | scores]
     char *block = nullptr;
     size_t used = 0;
     auto room = [&](size_t bytes) { const size_t at = used; used += (bytes + 255) & ~(size_t)255; return at; };
-    const size_t part_at = room(mode == kEvaluate ? 4 * sizeof(double) * (size_t)grid : 0);
+    size_t part_at = 0;
+    auto room_for_sums = [&]() { part_at = room(mode == kEvaluate ? 4 * sizeof(double) * (size_t)grid : 0); };
     int rc = DSFACTO_OK;
     unsigned long long *mailed = nullptr;   // the scores come through the mailbox
+    RequestLayout lay;                      // a request: its rows lie there too
     auto cleanup = [&]() { dev_free(block); };
     if (!indptr) {
         if (!h->loaded) return DSFACTO_ERR_NO_DATA;
         if (m != h->n) return DSFACTO_ERR_INVALID_ARG;
         a.indptr = h->d_indptr; a.idx = h->d_idx; a.val = h->d_val;
+        room_for_sums();
         const size_t f_at = room(sizeof(float) * (size_t)m);
         if ((rc = dev_alloc(h, &block, used))) return rc;
         a.f_out = reinterpret_cast<float *>(block + f_at);
@@ -2740,31 +2772,18 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         const int64_t nnz = indptr[m];
         if (nnz > 0 && (!indices || !values)) return DSFACTO_ERR_INVALID_ARG;
         const size_t ip_b = sizeof(int64_t) * ((size_t)m + 1), e_b = 4 * (size_t)nnz, y_b = sizeof(float) * (size_t)m;
-        const size_t mail = ip_b + 2 * e_b + (y ? y_b : 0);
-        const size_t f_b = mode == kScore ? sizeof(*mailed) * (size_t)m : 0;
-        if (((mail + 15) & ~(size_t)15) + f_b <= h->mail_bytes) {
-            // A request: the kernel reads the rows from the mailbox across the link and leaves the scores there, which
-            // takes less time than copies in and out before and behind it (32 rows: 60 us -> 20 us per call).
+        // A request: the kernel reads the rows from the mailbox across the link and leaves the scores there, which
+        // takes less time than copies in and out before and behind it (32 rows: 60 us -> 16 us per call).
+        const size_t f_b = mode == kScore ? (sizeof(*mailed) * (size_t)m + 15) & ~(size_t)15 : 0;
+        if (f_b < h->mail_bytes) lay = request_layout(h, m, indptr, y != nullptr, h->mail_bytes - f_b);
+        if (lay.stride > 0) grid = (int)lay.blocks;
+        room_for_sums();
+        if (lay.stride > 0) {
             if (!sound_rows(m, h->d, indptr, indices, values, y)) return DSFACTO_ERR_INVALID_CSR;
-            char *p = h->mail;
-            std::memcpy(p, indptr, ip_b);
-            if (nnz > 0) { std::memcpy(p + ip_b, indices, e_b); std::memcpy(p + ip_b + e_b, values, e_b); }
-            a.indptr = reinterpret_cast<int64_t *>(p);
-            a.idx = reinterpret_cast<int32_t *>(p + ip_b);
-            a.val = reinterpret_cast<float *>(p + ip_b + e_b);
-            a.y = reinterpret_cast<float *>(p + ip_b + 2 * e_b);
-            if (y) std::memcpy(p + ip_b + 2 * e_b, y, y_b);
+            lay_out_request(h->mail + f_b, lay, m, indptr, indices, values, y);   // (behind the scores)
             if (mode == kScore) {   // the scores are their own report: words without this call's number, until they arrive
-                a.f_words = mailed = reinterpret_cast<unsigned long long *>(p + ((mail + 15) & ~(size_t)15));
+                mailed = reinterpret_cast<unsigned long long *>(h->mail);
                 std::memset(mailed, 0, f_b);
-                a.report = nullptr;
-            }
-            if (staging_pays(mail, grid, m, nnz)) {
-                a.stage = reinterpret_cast<const uint4 *>(p);
-                a.stage_bytes = (int)((mail + 15) & ~(size_t)15);
-                a.idx = reinterpret_cast<int32_t *>(ip_b);
-                a.val = reinterpret_cast<float *>(ip_b + e_b);
-                a.y = reinterpret_cast<float *>(ip_b + 2 * e_b);
             }
             if (used > 0 && (rc = dev_alloc(h, &block, used))) return rc;
         } else {
@@ -2793,8 +2812,15 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         model_view(h, a, false);
     }
     a.partials = reinterpret_cast<double *>(block + part_at);
-    if (mode == kScore) DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kScore, grid);
-    else DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, kEvaluate, grid);
+    if (lay.stride > 0) {
+        RequestArgs q{};
+        q.blocks = reinterpret_cast<const uint4 *>(h->mail + (mailed ? (sizeof(*mailed) * (size_t)m + 15) & ~(size_t)15 : 0));
+        q.stride = (int)lay.stride; q.block_rows = lay.rows; q.rows = (int)m; q.pair = a.pair; q.V = a.V; q.w0 = a.w0; q.loss = a.loss; q.f_words = mailed;
+        q.report = a.report; q.number = a.number; q.partials = a.partials; q.done = a.done;
+        DSF_DISPATCH_REFRESH(h, launch_request, h, q, mode, grid);
+    } else {
+        DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, mode, grid);
+    }
     CallBody r{};
     if (mailed) {
         int64_t at = 0;

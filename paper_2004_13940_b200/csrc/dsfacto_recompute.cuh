@@ -49,13 +49,9 @@ struct RefreshArgs {
     // end of the pass: the last CTA adds the partial sums up
     unsigned *done;        // CTAs that have delivered (zero between launches)
     EpochState *st;        // kTrain: w0 comes from here and the sums go here; NULL: w0 above
-    Report *report;        // mapped host memory (NULL: not the end of an epoch, or the scores are the report)
+    Report *report;        // mapped host memory (NULL: not the end of an epoch)
     uint32_t number;       // ... the number of the report (kTrain: counted on the device)
-    unsigned long long *f_words;   // kScore: scores to mapped host memory, as words of a report each (NULL: to f_out)
     int first;             // kTrain: the first segment of an epoch (its times are set, not added)
-    // STAGED: a small batch in mapped host memory, [indptr | idx | val | y]; indptr, idx, val, y are then offsets into it
-    const uint4 *stage;
-    int stage_bytes;       // (a multiple of 16)
     int *bad;              // caller rows that were checked on the device: no row is read if it is set (NULL: sound rows)
 };
 
@@ -79,6 +75,22 @@ __device__ __forceinline__ bool last_cta_sum4(double (&s)[4], double *partials, 
         for (int c = 0; c < 4; ++c) s[c] += __ldcg(partials + 4 * (size_t)b + c);
     block_sum4(s);
     return true;
+}
+
+// loss of a row and dl/df, its multiplier
+__device__ __forceinline__ void loss_and_multiplier(int loss, float f, float y, float &li, float &gi) {
+    if (loss == 0) {
+        gi = f - y;
+        li = 0.5f * gi * gi;
+    } else {
+        const float m = y * f;
+        li = fmaxf(-m, 0.f) + log1pf(expf(-fabsf(m)));
+        gi = -y / (1.f + expf(m));
+    }
+}
+// what a held-out row adds to the metric: (f - y)^2 for the RMSE, or whether the sign of the score is the class
+__device__ __forceinline__ double held_out_measure(int loss, float f, float y, float gi) {
+    return loss == 0 ? (double)gi * (double)gi : y * f > 0.f ? 1.0 : 0.0;
 }
 
 // The last thread of a kernel whose CTAs have all written their results (to memory of the host as well): thread 0
@@ -110,26 +122,21 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms); rows taken longest first inside
 // blocks of 256 (text 44 -> 42.5 us, but click logs 2.97 -> 3.09 ms); two or four resident CTAs for 128-byte rows (46 and
 // 43 us).
-template <int LG, int NV, bool STAGED = false>
+template <int LG, int NV>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;
     static constexpr int E = LG == 1 ? 4 : LG <= 4 ? 2 : 1;                 // entries per lane and batch
     static constexpr int B = LG * E;
-    // entries whose rows are requested together; a small batch (STAGED) has the GPU to itself and waits for nothing
-    // but the latency of these requests, so it makes fewer and larger ones (32 rows of 39 entries: 25 -> 22 us per call)
-    static constexpr int UB = STAGED && NV <= 4 ? B / 2 : (LG == 8 && NV == 1) || LG == 4 ? 2 : 1;
+    static constexpr int UB = (LG == 8 && NV == 1) || LG == 4 ? 2 : 1;      // entries whose rows are requested together
     static constexpr int S = B / UB;                                        // steps per batch
-    static constexpr int NB = STAGED || NV >= 6 || LG == 1 || LG == 4 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
+    static constexpr int NB = NV >= 6 || LG == 1 || LG == 4 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
     static_assert(S % NB == 0, "a step keeps its registers from batch to batch");
-    static constexpr int CTAS = STAGED ? 1 : LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
+    static constexpr int CTAS = LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
 };
-constexpr int kMostStaged = 24 << 10;   // bytes of a staged batch
-// STAGED: every CTA first copies the whole batch from the host's memory to shared memory, all of it at once: one
-// trip across the link instead of one for the row pointers and one for every two batches of entries.
-template <int LG, int NV, int MODE, bool RAW = false, bool STAGED = false>
-__global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) refresh_kernel(const RefreshArgs a) {
-    typedef RefreshCfg<LG, NV, STAGED> C;
+template <int LG, int NV, int MODE, bool RAW = false>
+__global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_kernel(const RefreshArgs a) {
+    typedef RefreshCfg<LG, NV> C;
     constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, NB = C::NB, KP4 = LG * NV;
     constexpr unsigned FULL = 0xFFFFFFFFu;
     const int g = threadIdx.x / LG, l = threadIdx.x % LG, gw = (threadIdx.x & 31) / LG;
@@ -137,32 +144,11 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     float4 *A4 = reinterpret_cast<float4 *>(a.A);
     constexpr bool TRAIN = MODE == kTrain;
     constexpr bool STORE_A = MODE == kTrain || MODE == kPartial;
-    extern __shared__ __align__(16) uint4 staged[];   // STAGED: the batch
     // the fp64 sums of a lane group live in shared memory: only its first lane touches them, once per row
     __shared__ double sums[2][C::ROWS];
     if (l == 0) { sums[0][g] = 0.0; sums[1][g] = 0.0; }
     let_next_kernel_start();
 
-    const int64_t *indptr = a.indptr;
-    const int32_t *idx = a.idx;
-    const float *val = a.val, *lab = a.y;
-    if (STAGED) {
-        // (all requests before the first store: one trip)
-        uint4 piece[kMostStaged / 16 / kThreads];
-#pragma unroll
-        for (int i = 0; i < kMostStaged / 16 / kThreads; ++i)
-            if (i * kThreads + (int)threadIdx.x < a.stage_bytes / 16) piece[i] = a.stage[i * kThreads + threadIdx.x];
-#pragma unroll
-        for (int i = 0; i < kMostStaged / 16 / kThreads; ++i)
-            if (i * kThreads + (int)threadIdx.x < a.stage_bytes / 16) staged[i * kThreads + threadIdx.x] = piece[i];
-        const char *p = reinterpret_cast<const char *>(staged);
-        indptr = reinterpret_cast<const int64_t *>(p);
-        idx = reinterpret_cast<const int32_t *>(p + reinterpret_cast<size_t>(a.idx));
-        val = reinterpret_cast<const float *>(p + reinterpret_cast<size_t>(a.val));
-        lab = reinterpret_cast<const float *>(p + reinterpret_cast<size_t>(a.y));
-        __syncthreads();
-    }
-    auto fixed = [](const auto *q) { return STAGED ? *q : __ldg(q); };   // data that does not change during the kernel
     int64_t n = a.n;
     int bad = 0;
     if ((MODE == kScore || MODE == kEvaluate) && a.bad) {
@@ -179,8 +165,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
     auto next_pointers = [&](int64_t row) {
         nlen = 0;
         if (row < n) {
-            nbeg = fixed(indptr + row);
-            nlen = (int)(fixed(indptr + row + 1) - nbeg);
+            nbeg = __ldg(a.indptr + row);
+            nlen = (int)(__ldg(a.indptr + row + 1) - nbeg);
         }
     };
     auto load_entries = [&](int64_t beg, int t0, int len, int32_t (&j)[E], float (&x)[E]) {
@@ -188,8 +174,8 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
         for (int e = 0; e < E; ++e) {
             const int t = t0 + e * LG + l;
             j[e] = 0; x[e] = 0.f;
-            if (len > 0) j[e] = fixed(idx + beg + min(t, len - 1));
-            if (t < len) x[e] = fixed(val + beg + t);
+            if (len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
+            if (t < len) x[e] = __ldg(a.val + beg + t);
         }
     };
     next_pointers(base + gw);
@@ -295,32 +281,17 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV, STAGED>::CTAS)) 
         }
         if (l == 0 && row < n) {
             const float f = w0 + lin + 0.5f * pair;
-            if (MODE == kScore && a.f_words) store_report_word(a.f_words + row, a.number, __float_as_uint(f));
-            else if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
+            if (MODE == kScore || MODE == kScoreSums) a.f_out[row] = f;
             if (MODE != kScore) {
-                const float yy = lab[row];
                 float li, gi;
-                if (a.loss == 0) {
-                    gi = f - yy;
-                    li = 0.5f * gi * gi;
-                } else {
-                    const float m = yy * f;
-                    li = fmaxf(-m, 0.f) + log1pf(expf(-fabsf(m)));
-                    gi = -yy / (1.f + expf(m));
-                }
+                loss_and_multiplier(a.loss, f, a.y[row], li, gi);
                 sums[0][g] += (double)li;
                 if (TRAIN) a.G[row] = gi;
-                if (TRAIN || MODE == kScoreSums) {
-                    sums[1][g] += (double)gi;
-                } else if (a.loss == 0) {
-                    sums[1][g] += (double)gi * (double)gi;      // (f - y)^2 for the RMSE
-                } else {
-                    sums[1][g] += (yy * f > 0.f) ? 1.0 : 0.0;   // the sign of the score is the predicted class
-                }
+                sums[1][g] += TRAIN || MODE == kScoreSums ? (double)gi : held_out_measure(a.loss, f, a.y[row], gi);
             }
         }
     }
-    if (MODE == kScore && a.report && last_thread(a.done)) {
+    if (MODE == kScore && last_thread(a.done)) {
         if (a.bad) *a.bad = 0;
         for (int i = 0; i < kReportWords<CallBody>; ++i) store_report_word(a.report->call + i, a.number, (uint32_t)bad);   // (nothing else is looked at)
     }

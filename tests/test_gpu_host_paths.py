@@ -184,3 +184,55 @@ def test_page_locked_arrays_belong_to_the_caller_again_on_return(n):
             got.append((objective, held, f, *g.get_params()))
     for a, b in zip(*got):
         assert np.array_equal(np.asarray(a), np.asarray(b))
+
+
+REQUESTS = {
+    "steps": [7, 8, 9, 31, 32, 33, 63, 64, 65, 0, 127, 128, 129, 1, 0, 15, 16, 17],   # around the entries of a warp's step
+    "several rows per warp": list(np.random.default_rng(0).integers(0, 4, 2500)),
+    "more than 24 KB in a block": [0, 3100, 1, 64, 0],
+    "more than 48 KB in a block": [5, 6500, 3100, 0, 64],
+    "one row of 96 KB": [12000],
+    "too large for the mailbox": [3, 16300, 0],
+    "empty rows": [0] * 9,
+}
+
+
+@pytest.mark.parametrize("K", [4, 8, 16, 32, 64, 128, 200])
+@pytest.mark.parametrize("shape", sorted(REQUESTS))
+def test_requests_in_blocks_of_rows(K, shape):
+    lens = np.array(REQUESTS[shape])
+    rng = np.random.default_rng(K)
+    d, m = 20000, len(lens)
+    ip = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    ix = np.concatenate([np.sort(rng.choice(d, n, replace=False)) for n in lens]).astype(np.int32)
+    v = rng.standard_normal(len(ix)).astype(np.float32) / np.sqrt(np.repeat(lens, lens).clip(1)).astype(np.float32)
+    y = np.where(rng.random(m) < 0.5, 1.0, -1.0).astype(np.float32)
+    w, V = (0.1 * rng.standard_normal(d)).astype(np.float32), (0.1 * rng.standard_normal((d, K))).astype(np.float32)
+    rows = np.repeat(np.arange(m), lens)
+    x, A, q = v.astype(np.float64), np.zeros((m, K)), np.zeros(m)
+    np.add.at(A, rows, x[:, None] * V[ix])
+    np.add.at(q, rows, x * x * (V[ix].astype(np.float64) ** 2).sum(1))
+    f = 0.25 + np.bincount(rows, x * w[ix], m) + 0.5 * ((A * A).sum(1) - q)
+    # fp32 sums of up to 16300 products whose squares add up to one: error below 16300 * 2^-24 in the worst order
+    tol = 2e-5 * (1 + np.abs(f).max())
+    for loss, code in ((D.LOGISTIC, "logistic"), (D.SQUARED, "squared")):
+        with D.DSFacto(1, d, K, 1, loss, 0.0, 0.0, 0.1, 1) as g:
+            g.set_params(0.25, w, V)
+            for _ in range(2):
+                np.testing.assert_allclose(g.predict(ip, ix, v), f, rtol=0, atol=tol)
+            mean, metric = g.evaluate(ip, ix, v, y)
+            if loss == D.LOGISTIC:
+                assert mean == pytest.approx(np.logaddexp(0.0, -y * f).mean(), rel=1e-5, abs=tol)
+                assert abs(metric - np.mean(y * f > 0)) * m <= np.count_nonzero(np.abs(f) <= tol) + 1e-9
+            else:
+                assert mean == pytest.approx(0.5 * np.mean((f - y) ** 2), rel=1e-4)
+                assert metric == pytest.approx(np.sqrt(np.mean((f - y) ** 2)), rel=1e-4)
+            if len(ix) > 1 and lens.max() > 1:   # columns that do not rise inside a row, beside falls from row to row
+                t = int(ip[np.argmax(lens)]) + 1
+                bad = ix.copy()
+                bad[t] = bad[t - 1]
+                assert D.dsfacto_predict(g._h, m, ip, bad, v, np.empty(m, np.float32)) == D.ERR_INVALID_CSR
+                falling = ip.copy()
+                falling[np.argmax(lens) + 1] = ip[np.argmax(lens)] - 1 if ip[np.argmax(lens)] > 0 else len(ix) + 1
+                if m > 1 and falling[-1] == ip[-1]:
+                    assert D.dsfacto_predict(g._h, m, falling, ix, v, np.empty(m, np.float32)) == D.ERR_INVALID_CSR
