@@ -114,6 +114,7 @@ struct dsfacto {
     cudaGraphExec_t epoch_graph = nullptr;   // the launches of an epoch (all but the sweep over tiles and shards)
     int epochs_run = 0;
     int64_t epoch_launches = 0;
+    int request_smem[2] = {0, 0};   // shared memory that the request kernels of this width have been allowed
     EpochBody ended{};            // the last report of a recompute pass
     char *mail = nullptr;          // the rest of that memory: small inputs and results (mail_bytes of it)
     size_t mail_bytes = 0;
@@ -485,8 +486,13 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
 template <int LG, int NV>
 void launch_request(dsfacto *h, const RequestArgs &a, int mode, int grid) {
     auto kernel = mode == kEvaluate ? request_kernel<LG, NV, kEvaluate> : request_kernel<LG, NV, kScore>;
-    if (a.stride > (47 << 10)) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMailboxBytes);   // (a refusal shows at the launch)
-    launch_overlapped(h, kernel, grid, kThreads, a.stride, a);
+    int &most = h->request_smem[mode == kEvaluate ? 1 : 0];
+    const int smem = (int)request_smem<LG, NV>((size_t)a.stride);
+    if (smem > most && smem > (47 << 10)) {   // (a refusal shows at the launch)
+        most = (int)request_smem<LG, NV>(kMailboxBytes);
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    }
+    launch_overlapped(h, kernel, grid, kThreads, smem, a);
 }
 
 #define DSF_DISPATCH(h, FN, ...)                                   \

@@ -7,14 +7,16 @@
 namespace dsf {
 
 // A request has the GPU to itself and lasts as long as its dependent steps: the launch, the trip across the link to the rows,
-// the trip to the factor rows, the sums, the trip of the scores back.  So every row has a warp to itself, whose lane groups
-// take its entries in turn and request the rows of a whole step (32 or 64 entries up to 256-byte rows) before they use the
-// first; and the host lays the rows out in blocks, one per CTA, so that a CTA fetches what it needs, and no more, in one trip.
+// the trip to the factor rows, the sums, the trip of the scores back.  So every row has a warp to itself, which requests the
+// factor rows of a whole step (64 entries of up to 128 bytes, 8 KB of wider ones) into shared memory before it uses the first;
+// and the host lays the rows out in blocks, one per CTA, so that a CTA fetches what it needs, and no more, in one trip.
+// The sums are those of the recompute kernel, bit for bit: a row scored on its own has the score it has among others.
 // Before, a lane group of the recompute kernel went through a row eight entries at a time (two trips to L2 for each eight),
 // and either every CTA fetched the whole batch or each lane fetched its entries across the link, eight at a time.
-// Calls of dsfacto_predict, K = 16, in us, before and after: 1 row of 39 entries 17.3 -> 12.7, 32 rows 21.6 -> 15.0, 300 rows
-// 39.5 -> 31.0; 300 rows of one entry 19.0 -> 13.8, 5000 rows 33.5 -> 33.9; 1 row of 1000 entries 60 -> 28, of 8000 entries
-// 1730 -> 130.  What bounds it: 8 us for a launch and its answer, 4 us in the interpreter, then the two trips.
+// Calls of dsfacto_predict, K = 16, in us, before and after: 1 row of 39 entries 17.3 -> 13.5, 32 rows 21.6 -> 15.7, 300 rows
+// 39.5 -> 27.8; 300 rows of one entry 19.0 -> 13.6, 5000 rows 33.5 -> 31.7; 1 row of 1000 entries 60 -> 50, of 8000 entries
+// 1730 -> 315.  What bounds it: 8 us for a launch and its answer, 4 us in the interpreter, then the two trips.  (Lane groups
+// that each sum up a part of the row and add their parts at the end take 14.5 us for 32 rows, but round differently.)
 constexpr int kMostBlockRows = 64;
 // A block: first[block_rows + 1] (where the rows begin among the block's entries), then columns, values and labels.
 struct RequestArgs {
@@ -34,19 +36,28 @@ struct RequestArgs {
 };
 template <int LG, int NV>
 struct RequestCfg {
-    static constexpr int GW = 32 / LG;
-    static constexpr int UB = NV >= 6 ? 2 : NV == 4 ? 4 : LG == 1 ? 2 : LG == 2 ? 4 : 8;   // entries of a lane group per step
-    static constexpr int STEP = GW * UB;                                                 // entries of a step
-    static constexpr int E = STEP > 32 ? STEP / 32 : 1;                                  // ... per lane
+    static constexpr int KP4 = LG * NV;
+    static constexpr int STEP = KP4 <= 8 ? 64 : (512 / KP4) & ~7;      // entries whose factor rows are on their way together: 8 KB at most
+    static constexpr int F = (KP4 + 31) / 32;                          // float4s of a row per lane
 };
+// what a warp keeps in shared memory: the factor rows and the pairs (w_j, s_j) of a step
+template <int LG, int NV>
+struct RequestStep {
+    float4 rows[RequestCfg<LG, NV>::STEP * RequestCfg<LG, NV>::KP4];
+    float2 pairs[RequestCfg<LG, NV>::STEP];
+};
+template <int LG, int NV>
+constexpr size_t request_smem(size_t stride) { return sizeof(RequestStep<LG, NV>) * (kThreads / 32) + stride; }
 template <int LG, int NV, int MODE>
 __global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) {
     typedef RequestCfg<LG, NV> C;
-    constexpr int GW = C::GW, UB = C::UB, STEP = C::STEP, E = C::E, KP4 = LG * NV;
+    constexpr int STEP = C::STEP, F = C::F, KP4 = C::KP4;
     constexpr unsigned FULL = 0xFFFFFFFFu;
-    extern __shared__ __align__(16) uint4 block[];
+    extern __shared__ __align__(16) uint4 shared[];
+    RequestStep<LG, NV> &step = reinterpret_cast<RequestStep<LG, NV> *>(shared)[threadIdx.x >> 5];
+    uint4 *block = shared + sizeof(RequestStep<LG, NV>) * (kThreads / 32) / 16;
     __shared__ float scores[kMostBlockRows];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LG, g = lane / LG;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LG;
     let_next_kernel_start();
     const uint4 *from = a.blocks + (size_t)blockIdx.x * (a.stride / 16);
     constexpr int PIECES = 6;
@@ -63,65 +74,54 @@ __global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) 
     const int *first = reinterpret_cast<const int *>(block);
     const int entries = first[a.block_rows], rows = min(a.block_rows, a.rows - (int)blockIdx.x * a.block_rows);
     const int32_t *all_idx = first + a.block_rows + 1;
-    const float4 *V4 = reinterpret_cast<const float4 *>(a.V) + l;
+    const float4 *V4 = reinterpret_cast<const float4 *>(a.V);
     wait_for_previous_kernel();   // the model
 
     for (int row = warp; row < rows; row += kThreads / 32) {
         const int beg = first[row], len = first[row + 1] - beg;
         const int32_t *idx = all_idx + beg;
         const float *val = reinterpret_cast<const float *>(idx + entries);
-        float4 acc[NV];
+        float4 acc[F];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < F; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         float q = 0.f, lin = 0.f;
         for (int t0 = 0; t0 < len; t0 += STEP) {
-            float4 r[UB][NV];
-            float x[UB], xe[E];
-            float2 ws[E];
-#pragma unroll
-            for (int u = 0; u < UB; ++u) {
-                const int t = t0 + u * GW + g;
-                x[u] = 0.f;
-#pragma unroll
-                for (int v = 0; v < NV; ++v) r[u][v] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (t < len) {
-                    x[u] = val[t];
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) r[u][v] = V4[(size_t)idx[t] * KP4 + v * LG];
-                }
+            const int now = min(STEP, len - t0);
+            for (int i = lane; i < now * KP4; i += 32) {
+                const uint32_t to = (uint32_t)__cvta_generic_to_shared(step.rows + i);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(V4 + (size_t)idx[t0 + i / KP4] * KP4 + i % KP4) : "memory");
             }
+            for (int t = lane; t < now; t += 32) step.pairs[t] = a.pair[idx[t0 + t]];
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+            // in the order of the entries, a lane one part (or two) of the row
+#pragma unroll 8
+            for (int t = 0; t < now; ++t) {
+                const float x = val[t0 + t];
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int s = e * 32 + lane;
-                xe[e] = 0.f; ws[e] = make_float2(0.f, 0.f);
-                if (s < STEP && t0 + s < len) { xe[e] = val[t0 + s]; ws[e] = a.pair[idx[t0 + s]]; }
+                for (int i = 0; i < F; ++i) fma4(acc[i], x, step.rows[t * KP4 + min(lane + 32 * i, KP4 - 1)]);
             }
-#pragma unroll
-            for (int u = 0; u < UB; ++u)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) fma4(acc[v], x[u], r[u][v]);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                lin = fmaf(ws[e].x, xe[e], lin);
-                q = fmaf(xe[e] * xe[e], ws[e].y, q);
+            // ... and a lane the scalars of every LG-th entry, as the recompute kernel does
+#pragma unroll 4
+            for (int t = l; t < now; t += LG) {
+                const float x = val[t0 + t];
+                const float2 ws = step.pairs[t];
+                lin = fmaf(ws.x, x, lin);
+                q = fmaf(x * x, ws.y, q);
             }
+            __syncwarp();
         }
-#pragma unroll
-        for (int o = LG; o < 32; o <<= 1)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                acc[v].x += __shfl_xor_sync(FULL, acc[v].x, o); acc[v].y += __shfl_xor_sync(FULL, acc[v].y, o);
-                acc[v].z += __shfl_xor_sync(FULL, acc[v].z, o); acc[v].w += __shfl_xor_sync(FULL, acc[v].w, o);
-            }
         float sq = 0.f;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            sq = fmaf(acc[v].x, acc[v].x, sq); sq = fmaf(acc[v].y, acc[v].y, sq);
-            sq = fmaf(acc[v].z, acc[v].z, sq); sq = fmaf(acc[v].w, acc[v].w, sq);
+        for (int v = 0; v < NV; ++v) {   // float4 number v * LG + l of the row
+            const float4 y = acc[v * LG / 32];
+            const int from = (v * LG + l) & 31;
+            const float4 z = make_float4(__shfl_sync(FULL, y.x, from), __shfl_sync(FULL, y.y, from), __shfl_sync(FULL, y.z, from), __shfl_sync(FULL, y.w, from));
+            sq = fmaf(z.x, z.x, sq); sq = fmaf(z.y, z.y, sq); sq = fmaf(z.z, z.z, sq); sq = fmaf(z.w, z.w, sq);
         }
-        float pair = g == 0 ? sq - q : -q;
+        float pair = sq - q;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = LG / 2; o > 0; o >>= 1) {
             pair += __shfl_xor_sync(FULL, pair, o);
             lin += __shfl_xor_sync(FULL, lin, o);
         }
