@@ -947,7 +947,13 @@ int order_columns(dsfacto *h) {
     const int grid = (int)std::min<int64_t>((h->nnz + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     const int dgrid = (int)std::min<int64_t>(((int64_t)d + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     if ((e = cudaMemsetAsync(d_slot_of, 0, sizeof(int32_t) * d, h->stream)) != cudaSuccess) return fail(e);
-    launch(h, column_count_kernel, grid, kThreads, 0, h->d_idx, h->nnz, d_slot_of);
+    if (h->runs)
+        for (const RunPass &ps : h->passes) {
+            if (ps.nruns == 0) continue;
+            const int rgrid = (int)std::min<int64_t>((ps.nruns + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
+            launch(h, run_columns_kernel, rgrid, kThreads, 0, h->d_run_start + ps.run_first, h->d_run_key + ps.run_first, ps.nruns, ps.count, d_slot_of);
+        }
+    else launch(h, column_count_kernel, grid, kThreads, 0, h->d_idx, h->nnz, d_slot_of);
     launch(h, column_keys_kernel, dgrid, kThreads, 0, d_slot_of, (int64_t)d, d_key, d_col);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, d_key, d_key_out, d_col, h->d_column_of, (int64_t)d, 0, 32,
                                              h->stream)) != cudaSuccess)
@@ -1153,7 +1159,7 @@ int download_rows(dsfacto *h, float *dst, float *src_dev, int64_t rows, Fetch mo
 }
 
 void launch_validate(dsfacto *h, int64_t m, int64_t nnz, const int64_t *indptr, const int32_t *idx, const float *val, const float *y, int *bad) {
-    const int grid = (int)std::min<int64_t>((m + kThreads / 32 - 1) / (kThreads / 32), (int64_t)h->sm_count * 16);
+    const int grid = (int)std::min<int64_t>((m + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
     launch(h, validate_rows_kernel, grid, kThreads, 0, m, nnz, h->d, indptr, idx, val, y, bad);
 }
 
@@ -1866,7 +1872,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     const int wide_grid = h->sm_count * 16;
     TileKeyArgs ka{};
     ka.n = h->n; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p;
-    ka.sweep = h->sweep; ka.jbits = h->jbits; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start;
+    ka.sweep = h->sweep; ka.jbits = h->jbits; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start; ka.col_start = h->d_col_start;
     ka.rbits = h->rbits; ka.slot_rows = (int32_t)slot_rows;
     ka.key = key[0]; ka.payload = pay[0];
     launch(h, tile_keys_kernel, wide_grid, kThreads, 0, ka);
@@ -2056,9 +2062,9 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     const int wide_grid = h->sm_count * 16;
     RunKeyArgs ka{};
     ka.n = h->n; ka.nnz = nnz; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p; ka.cbits = cbits;
-    ka.bands = (int32_t)bands; ka.band_rows = (h->n + bands - 1) / bands; ka.every = (int32_t)every; ka.row_start = h->d_row_start;
+    ka.bands = (int32_t)bands; ka.band_rows = (h->n + bands - 1) / bands; ka.every = (int32_t)every; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start;
     ka.key = key[0]; ka.payload = pay[0];
-    launch(h, run_keys_kernel, (int)std::min<int64_t>((h->n + 7) / 8, wide_grid), kThreads, 0, ka);
+    launch(h, run_keys_kernel, (int)std::min<int64_t>((h->n + kThreads - 1) / kThreads, wide_grid), kThreads, 0, ka);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
     const uint32_t *sorted = kbuf.Current();
     launch(h, pass_bounds_kernel, (int)((npass + kThreads) / kThreads), kThreads, 0, nnz, sorted, low_bits, (int)npass, d_bounds);

@@ -163,3 +163,77 @@ def test_merged_row_blocks_on_the_device(monkeypatch, merge, name, kw):
     assert np.abs(w - o.w).max() <= 1e-4 * (1 + np.abs(o.w).max())
     assert np.all(np.abs(V - o.V) <= 1e-4 * (1 + np.abs(o.V)))
     assert np.all(np.abs(G - o.G) <= 1e-4 * (1 + np.abs(o.G)))
+
+
+def _uneven_rows(d, seed):
+    """70 rows of 0 to 300 entries: rows end inside, at and behind the stretches of 32 and 128 entries that warps read, some
+    of the 32 rows that a warp takes are empty, and columns fall, rise or repeat from one row to the next."""
+    rng = np.random.default_rng(seed)
+    lens = [1, 31, 32, 33, 0, 0, 127, 128, 129, 300] + list(rng.integers(0, 40, 20)) + [0, 5, 7, 0] + list(rng.integers(1, 9, 35)) + [64]
+    indptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    indices = np.concatenate([np.sort(rng.choice(d, n, replace=False)) for n in lens]).astype(np.int32)
+    return indptr, indices, rng.standard_normal(len(indices)).astype(np.float32), rng.standard_normal(len(lens)).astype(np.float32)
+
+
+def test_checks_on_the_device_agree_with_the_host():
+    """A fault planted at every kind of place is found, and what is sound is taken: the verdicts are those of the checks that
+    the host bucketer makes row by row."""
+    d = 400
+    ip, ix, v, y = _uneven_rows(d, 1)
+    n = len(y)
+    cases = [(ip, ix, v, y)]
+    nonempty = [i for i in range(n) if ip[i + 1] > ip[i]]
+    places = sorted({int(p) for i in nonempty for p in (ip[i], ip[i] + 1, ip[i + 1] - 1) if p < ip[i + 1]} | {127, 128, 129})
+    for t in places:
+        row = int(np.searchsorted(ip, t, side="right")) - 1
+        kinds = [(np.int32(-1), None), (np.int32(d), None), (None, np.nan), (None, np.inf)]
+        if t > ip[row]:
+            kinds += [(ix[t - 1], None)]                       # repeats its predecessor
+        if t > 0 and t == ip[row] and t + 1 < ip[row + 1] and ix[t - 1] < ix[t + 1]:
+            kinds += [(ix[t - 1], None)]                       # the same across a row's border is sound
+        for j, x in kinds:
+            bix, bv = ix.copy(), v.copy()
+            if j is not None:
+                bix[t] = j
+            if x is not None:
+                bv[t] = x
+            cases.append((ip, bix, bv, y))
+    pointers = []
+    for i in (1, 31, 32, 33, 64, n - 1):
+        for value in (-1, ip[i - 1] - 1, ip[i + 1] + 1, ip[n] + 1, np.iinfo(np.int64).min, np.iinfo(np.int64).max):
+            bip = ip.copy()
+            bip[i] = value
+            pointers.append(bip)
+    verdicts = set()
+    with D.DSFacto(n, d, 4, 3, D.SQUARED, 1e-3, 1e-3, 0.1, 1) as g:
+        for bip, bix, bv, by in cases:
+            want = D.dsfacto_bucket_host(n, d, 3, bip, bix, bv)[0]
+            assert D.dsfacto_load_csr(g._h, bip, bix, bv, by) == want
+            verdicts.add(want)
+        for bip in pointers:      # (the host's checks follow the pointers they are given)
+            assert D.dsfacto_load_csr(g._h, bip, ix, v, y) == D.ERR_INVALID_CSR
+        for i in (0, 31, 32, n - 1):
+            by = y.copy()
+            by[i] = np.nan
+            assert D.dsfacto_load_csr(g._h, ip, ix, v, by) == D.ERR_INVALID_CSR
+    assert verdicts == {D.OK, D.ERR_INVALID_CSR}
+
+
+@pytest.mark.parametrize("p,every", [(1, 0), (3, 0), (70, 0), (7, 2), (90, 40)])
+@pytest.mark.parametrize("bands", [1, 3])
+def test_keys_of_uneven_rows(monkeypatch, p, every, bands):
+    monkeypatch.setenv("DSFACTO_BANDS", str(bands))
+    d = 400
+    ip, ix, v, y = _uneven_rows(d, p)
+    n = len(y)
+    o = O.Oracle(n, d, 4, p, O.SQUARED, 1e-3, 1e-3, 0.1, 1)
+    o.load_csr(ip, ix, v, y)
+    with D.DSFacto(n, d, 4, p, D.SQUARED, 1e-3, 1e-3, 0.1, 1) as g:
+        g.debug_set(D.DEBUG_COLUMN_ORDER, 1)     # counts the entries of the columns from the runs
+        if every:
+            g.set_refresh_every(every)
+        g.load_csr(ip, ix, v, y)
+        tp, rows, cols, vals = g.get_tiles()
+        assert np.array_equal(tp, o.tile_ptr) and np.array_equal(rows, o.rows) and np.array_equal(cols, o.cols) and np.array_equal(vals, o.vals)
+        for _ in range(2):
+            assert g.epoch() == pytest.approx(o.epoch_segmented(every) if every else o.epoch(), rel=1e-4)
