@@ -522,6 +522,9 @@ void launch_request(dsfacto *h, const RequestArgs &a, int mode, int grid) {
         case 84: FN<8, 4>(__VA_ARGS__); break;                     \
         case 86: FN<8, 6>(__VA_ARGS__); break;                     \
         case 88: FN<8, 8>(__VA_ARGS__); break;                     \
+        case 162: FN<16, 2>(__VA_ARGS__); break;                   \
+        case 163: FN<16, 3>(__VA_ARGS__); break;                   \
+        case 164: FN<16, 4>(__VA_ARGS__); break;                   \
         default: break;                                            \
         }                                                          \
     } while (0)
@@ -1633,6 +1636,7 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
     // share the instructions that hand out columns and values.
     h->LGr = h->LG; h->NVr = h->NV;
     if (h->Kp >= 64) { h->LGr = 8; h->NVr = h->Kp / 32; }
+    if (wide_recompute_groups(h->d, h->Kp)) { h->LGr = 16; h->NVr = h->Kp / 64; }
 
     int dev = 0;
     cudaGetDevice(&dev);

@@ -85,8 +85,8 @@ extern "C" int dsfacto_score_loss_noalloc(int64_t m, int32_t d, int32_t K, int32
     case 16: launch_score_loss<4, 1>(a, st); break;
     case 32: launch_score_loss<8, 1>(a, st); break;
     case 64: launch_score_loss<8, 2>(a, st); break;
-    case 128: launch_score_loss<8, 4>(a, st); break;
-    case 256: launch_score_loss<8, 8>(a, st); break;
+    case 128: if (wide_recompute_groups(d, K)) launch_score_loss<16, 2>(a, st); else launch_score_loss<8, 4>(a, st); break;
+    case 256: if (wide_recompute_groups(d, K)) launch_score_loss<16, 4>(a, st); else launch_score_loss<8, 8>(a, st); break;
     default: return DSFACTO_ERR_INVALID_ARG;
     }
     if (cudaGetLastError() != cudaSuccess) return DSFACTO_ERR_CUDA;

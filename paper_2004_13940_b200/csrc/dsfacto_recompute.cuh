@@ -126,18 +126,27 @@ template <int LG, int NV>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;
     static constexpr int E = LG == 1 ? 4 : LG <= 4 ? 2 : 1;                 // entries per lane and batch
-    static constexpr int B = LG * E;
+    static constexpr int LANES = LG < 8 ? LG : 8;                           // lanes of a group that hold entries
+    static constexpr int B = LANES * E;                                     // entries of a row per batch
     static constexpr int UB = (LG == 8 && NV == 1) || LG == 4 ? 2 : 1;      // entries whose rows are requested together
     static constexpr int S = B / UB;                                        // steps per batch
-    static constexpr int NB = NV >= 6 || LG == 1 || LG == 4 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
+    static constexpr int NB = LG * NV >= 48 || LG == 1 || LG == 4 ? 2 : 4;         // sets of registers: NB - 1 steps are under way
     static_assert(S % NB == 0, "a step keeps its registers from batch to batch");
     static constexpr int CTAS = LG < 8 ? 4 : NV >= 4 ? 2 : 3;  // resident per SM (register cap)
     static constexpr int ROWS = kThreads / LG;                              // rows per CTA and round
 };
+// Rows of 512 bytes and more: whether 16 lanes take a row instead of 8.  With 16, a lane has half as much of a row on its way,
+// so that three CTAs fit an SM instead of two, and requests of a row are half as many; with 8, a warp has half the
+// instructions per entry.  A table of factors that one L1 holds is read as fast as instructions are issued, a larger one as
+// fast as requests are answered.  Recompute pass, us, 8 and 16 lanes: 512-byte rows, 30 M entries over 131 k columns 978 and
+// 926, 2.8 M over 50 k 128 and 119, 3.9 M over 117 k 134 and 130, 2 M over 300, 500 and 1000 columns 63 and 69, 78 and 79, 84 and 78; 1-KB rows, 7.5 M entries
+// over 131 k columns 494 and 447; 768-byte rows 379 and 357.  (Batches of 16 entries instead of 8: 905 in the first case, but
+// 140 and 79 with rows of 39 and 20 entries.)
+inline bool wide_recompute_groups(int64_t d, int Kp) { return Kp >= 128 && d * Kp * (int64_t)sizeof(float) > ((int64_t)320 << 10); }
 template <int LG, int NV, int MODE, bool RAW = false>
 __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_kernel(const RefreshArgs a) {
     typedef RefreshCfg<LG, NV> C;
-    constexpr int GW = C::GW, E = C::E, B = C::B, UB = C::UB, S = C::S, NB = C::NB, KP4 = LG * NV;
+    constexpr int GW = C::GW, E = C::E, B = C::B, LANES = C::LANES, UB = C::UB, S = C::S, NB = C::NB, KP4 = LG * NV;
     constexpr unsigned FULL = 0xFFFFFFFFu;
     const int g = threadIdx.x / LG, l = threadIdx.x % LG, gw = (threadIdx.x & 31) / LG;
     const float4 *V4 = reinterpret_cast<const float4 *>(a.V) + l;
@@ -174,6 +183,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
         for (int e = 0; e < E; ++e) {
             const int t = t0 + e * LG + l;
             j[e] = 0; x[e] = 0.f;
+            if (l >= LANES) continue;
             if (len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
             if (t < len) x[e] = __ldg(a.val + beg + t);
         }
@@ -217,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
             else if (t0 + B < longest) load_entries(nbeg, 0, nlen, jn, xn);
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                if (t0 + e * LG + l < len) {
+                if (l < LANES && t0 + e * LG + l < len) {
                     if (RAW) {
                         lin = fmaf(a.w[j0[e]], x0[e], lin);
                     } else {

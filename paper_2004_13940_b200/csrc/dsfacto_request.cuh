@@ -51,7 +51,7 @@ constexpr size_t request_smem(size_t stride) { return sizeof(RequestStep<LG, NV>
 template <int LG, int NV, int MODE>
 __global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) {
     typedef RequestCfg<LG, NV> C;
-    constexpr int STEP = C::STEP, F = C::F, KP4 = C::KP4;
+    constexpr int STEP = C::STEP, F = C::F, KP4 = C::KP4, LANES = RefreshCfg<LG, NV>::LANES;
     constexpr unsigned FULL = 0xFFFFFFFFu;
     extern __shared__ __align__(16) uint4 shared[];
     RequestStep<LG, NV> &step = reinterpret_cast<RequestStep<LG, NV> *>(shared)[threadIdx.x >> 5];
@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) 
 #pragma unroll
                 for (int i = 0; i < F; ++i) fma4(acc[i], x, step.rows[t * KP4 + min(lane + 32 * i, KP4 - 1)]);
             }
-            // ... and a lane the scalars of every LG-th entry, as the recompute kernel does
+            // ... and a lane the scalars of every eighth entry (or LG-th), as the recompute kernel does
 #pragma unroll 4
-            for (int t = l; t < now; t += LG) {
+            for (int t = l < LANES ? l : now; t < now; t += LANES) {
                 const float x = val[t0 + t];
                 const float2 ws = step.pairs[t];
                 lin = fmaf(ws.x, x, lin);

@@ -236,3 +236,20 @@ def test_requests_in_blocks_of_rows(K, shape):
                 falling[np.argmax(lens) + 1] = ip[np.argmax(lens)] - 1 if ip[np.argmax(lens)] > 0 else len(ix) + 1
                 if m > 1 and falling[-1] == ip[-1]:
                     assert D.dsfacto_predict(g._h, m, falling, ix, v, np.empty(m, np.float32)) == D.ERR_INVALID_CSR
+
+
+@pytest.mark.parametrize("K", [3, 8, 16, 20, 64, 128, 190, 256])
+@pytest.mark.parametrize("d", [150, 3000])        # 128 factors and more: both widths of the recompute kernel's lane groups
+def test_a_row_on_its_own_has_the_score_it_has_among_others(K, d):
+    rng = np.random.default_rng(K)
+    lens = np.concatenate([rng.integers(0, 140, 250), [0, 1, 7, 8, 9, 63, 64, 65, 140]])
+    m = len(lens)
+    ip = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    ix = np.concatenate([np.sort(rng.choice(d, n, replace=False)) for n in lens]).astype(np.int32)
+    v = rng.standard_normal(len(ix)).astype(np.float32)
+    with D.DSFacto(1, d, K, 1, D.LOGISTIC, 0.0, 0.0, 0.1, 1) as g:
+        g.set_params(0.25, (0.1 * rng.standard_normal(d)).astype(np.float32), (0.1 * rng.standard_normal((d, K))).astype(np.float32))
+        f = g.predict(ip, ix, v)                  # 140 KB: copied to the device and scored by the recompute kernel
+        for a, b in [(0, 20), (100, 101), (m - 9, m), (200, 230)]:
+            part = g.predict(ip[a:b + 1] - ip[a], ix[ip[a]:ip[b]], v[ip[a]:ip[b]])
+            assert np.array_equal(part, f[a:b])
