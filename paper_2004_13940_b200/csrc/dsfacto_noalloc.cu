@@ -40,12 +40,16 @@ std::atomic<unsigned *> g_done_addr[kMaxDevices];
 // The recompute kernel of the epoch (eq. (fm_model2), the multiplier G, the loss) without its stores of the
 // auxiliaries and without per-column pairs, for which there is no room: w_j and sum_k v_jk^2 come from w and V.
 template <int LG, int NV>
-void launch_score_loss(const RefreshArgs &a, cudaStream_t st) {
+void launch_score_loss(const RefreshArgs &a, int32_t d, cudaStream_t st) {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t rows = RefreshCfg<LG, NV>::ROWS;
     const int64_t grid = std::min<int64_t>((a.n + rows - 1) / rows, (int64_t)sms * RefreshCfg<LG, NV>::CTAS);
-    refresh_kernel<LG, NV, kScoreSums, true><<<(unsigned)std::min<int64_t>(grid, kMaxCtas), kThreads, 0, st>>>(a);
+    // whether nothing is requested behind the end of a row (TRIM): rows of 128 bytes and more of a table that no L1 holds
+    const bool trim = LG >= 8 && (int64_t)d * 4 * LG * NV * (int64_t)sizeof(float) > ((int64_t)320 << 10);
+    const unsigned ctas = (unsigned)std::min<int64_t>(grid, kMaxCtas);
+    if (trim) refresh_kernel<LG, NV, kScoreSums, true, true><<<ctas, kThreads, 0, st>>>(a);
+    else refresh_kernel<LG, NV, kScoreSums, true, false><<<ctas, kThreads, 0, st>>>(a);
 }
 
 }  // namespace
@@ -80,13 +84,13 @@ extern "C" int dsfacto_score_loss_noalloc(int64_t m, int32_t d, int32_t K, int32
     a.loss = loss; a.f_out = scores_dev; a.sums_out = sums_dev; a.partials = g_partials_addr[dev]; a.done = g_done_addr[dev];
     cudaStream_t st = (cudaStream_t)cuda_stream;
     switch (K) {
-    case 4: launch_score_loss<1, 1>(a, st); break;
-    case 8: launch_score_loss<2, 1>(a, st); break;
-    case 16: launch_score_loss<4, 1>(a, st); break;
-    case 32: launch_score_loss<8, 1>(a, st); break;
-    case 64: launch_score_loss<8, 2>(a, st); break;
-    case 128: if (wide_recompute_groups(d, K)) launch_score_loss<16, 2>(a, st); else launch_score_loss<8, 4>(a, st); break;
-    case 256: if (wide_recompute_groups(d, K)) launch_score_loss<16, 4>(a, st); else launch_score_loss<8, 8>(a, st); break;
+    case 4: launch_score_loss<1, 1>(a, d, st); break;
+    case 8: launch_score_loss<2, 1>(a, d, st); break;
+    case 16: launch_score_loss<4, 1>(a, d, st); break;
+    case 32: launch_score_loss<8, 1>(a, d, st); break;
+    case 64: launch_score_loss<8, 2>(a, d, st); break;
+    case 128: if (wide_recompute_groups(d, K)) launch_score_loss<16, 2>(a, d, st); else launch_score_loss<8, 4>(a, d, st); break;
+    case 256: if (wide_recompute_groups(d, K)) launch_score_loss<16, 4>(a, d, st); else launch_score_loss<8, 8>(a, d, st); break;
     default: return DSFACTO_ERR_INVALID_ARG;
     }
     if (cudaGetLastError() != cudaSuccess) return DSFACTO_ERR_CUDA;

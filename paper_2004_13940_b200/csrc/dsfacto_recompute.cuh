@@ -107,8 +107,13 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // instructions per entry of 128-byte rows, most of them for the masks and branches of the divergent groups).  A batch
 // is B = LG * E entries of each row, every lane owns E of them: it takes their (w_j, s_j) and hands column and value
 // to its group; entries are requested two batches ahead.  Factor rows are requested UB entries at a time, NB - 1 steps
-// ahead of the multiply-adds.  Behind the end of a row its last entry is repeated with
-// x = 0.
+// ahead of the multiply-adds.  Behind the end of a row x is 0, and nothing is requested (TRIM): the registers
+// keep the factors of an earlier entry of the row, whose infinities are the row's own, or zeros.  (Repeating the row's last
+// entry there found it in L1, but each repetition took the look-ups and the data of a request: recompute pass, us, repeating
+// and not: 2.6 M entries of text in 128-byte rows 42.7 and 40.9, 11 M in 96-byte rows 160 and 155, 30 M in 512-byte rows 926
+// and 894, 11.7 M of click logs in 32-byte rows 95.3 and 93.8, 390 M in 64-byte rows 2780 and 2760.  Without pairs (RAW) the
+// look at every entry costs instructions where these are short: 19 M entries of 256-byte rows over 262 k columns 400 and 365,
+// but 12 M over 300 columns 182 and 189 and of 64-byte rows 157 and 161, which therefore repeat.)
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
 // What bounds it: 64-byte rows of click logs (390 M entries, 2.8 to 2.9 ms), the data and look-up stages of L1 (85 and 89 %
 // busy: every entry costs one look-up for its row and one for its pair) at 40 % issue.  Wider rows reach no rate of any
@@ -143,7 +148,7 @@ struct RefreshCfg {
 // over 131 k columns 494 and 447; 768-byte rows 379 and 357.  (Batches of 16 entries instead of 8: 905 in the first case, but
 // 140 and 79 with rows of 39 and 20 entries.)
 inline bool wide_recompute_groups(int64_t d, int Kp) { return Kp >= 128 && d * Kp * (int64_t)sizeof(float) > ((int64_t)320 << 10); }
-template <int LG, int NV, int MODE, bool RAW = false>
+template <int LG, int NV, int MODE, bool RAW = false, bool TRIM = true>
 __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_kernel(const RefreshArgs a) {
     typedef RefreshCfg<LG, NV> C;
     constexpr int GW = C::GW, E = C::E, B = C::B, LANES = C::LANES, UB = C::UB, S = C::S, NB = C::NB, KP4 = LG * NV;
@@ -182,9 +187,10 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int t = t0 + e * LG + l;
-            j[e] = 0; x[e] = 0.f;
+            j[e] = TRIM ? -1 : 0; x[e] = 0.f;
             if (l >= LANES) continue;
-            if (len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
+            if (!TRIM && len > 0) j[e] = __ldg(a.idx + beg + min(t, len - 1));
+            if (TRIM && t < len) j[e] = __ldg(a.idx + beg + t);
             if (t < len) x[e] = __ldg(a.val + beg + t);
         }
     };
@@ -211,11 +217,20 @@ __global__ void __launch_bounds__(kThreads, (RefreshCfg<LG, NV>::CTAS)) refresh_
             for (int u = 0; u < UB; ++u) {
                 const int32_t ju = __shfl_sync(FULL, j[(u0 + u) / LG], (u0 + u) % LG, LG);
 #pragma unroll
-                for (int v = 0; v < NV; ++v) r[u][v] = V4[(size_t)ju * KP4 + v * LG];
+                for (int v = 0; v < NV; ++v)
+                    if (!TRIM || ju >= 0) r[u][v] = V4[(size_t)ju * KP4 + v * LG];
             }
         };
 #pragma unroll
         for (int e = 0; e < E; ++e) { j0[e] = jn[e]; x0[e] = xn[e]; }
+        if (TRIM && len < NB * UB) {   // (no entry of this row will have been in every register by the time they are multiplied by zero)
+#pragma unroll
+            for (int st = 0; st < NB; ++st)
+#pragma unroll
+                for (int u = 0; u < UB; ++u)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) vv[st][u][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
         for (int st = 0; st + 1 < NB; ++st) load_rows(j0, st * UB, vv[st]);
         load_entries(beg, B, len, j1, x1);

@@ -253,3 +253,31 @@ def test_a_row_on_its_own_has_the_score_it_has_among_others(K, d):
         for a, b in [(0, 20), (100, 101), (m - 9, m), (200, 230)]:
             part = g.predict(ip[a:b + 1] - ip[a], ix[ip[a]:ip[b]], v[ip[a]:ip[b]])
             assert np.array_equal(part, f[a:b])
+
+
+@pytest.mark.parametrize("K", [4, 8, 16, 32, 64, 128, 256])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_infinite_factors_stay_in_the_rows_that_have_them(K, value):
+    """Rows of very different lengths side by side, some of which have a column of infinite factors: the others' scores are
+    finite and as they are without it."""
+    rng = np.random.default_rng(K)
+    d, m = 900, 3000
+    lens = rng.choice([0, 1, 2, 3, 5, 8, 9, 17, 40], m)
+    rows = [np.sort(rng.choice(d - 1, n, replace=False) + 1) for n in lens]
+    hit = rng.random(m) < 0.2
+    rows = [np.concatenate([[0], r]) if h else r for r, h in zip(rows, hit)]      # column 0 comes first
+    lens = np.array([len(r) for r in rows])
+    ip, ix = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64), np.concatenate(rows).astype(np.int32)
+    v = rng.standard_normal(len(ix)).astype(np.float32)
+    w, V = (0.1 * rng.standard_normal(d)).astype(np.float32), (0.1 * rng.standard_normal((d, K))).astype(np.float32)
+    with D.DSFacto(1, d, K, 1, D.LOGISTIC, 0.0, 0.0, 0.1, 1) as g:
+        assert len(ix) * 8 > 128 << 10                                            # by the recompute kernel
+        g.set_params(0.25, w, V)
+        want = g.predict(ip, ix, v)
+        V[0] = value
+        g.set_params(0.25, w, V)
+        got = g.predict(ip, ix, v)
+        assert np.isfinite(got[~hit]).all() and np.array_equal(got[~hit], want[~hit])
+        few = slice(0, 40)
+        part = g.predict(ip[:41], ix[:ip[40]], v[:ip[40]])
+        assert np.array_equal(part[~hit[few]], want[few][~hit[few]])
