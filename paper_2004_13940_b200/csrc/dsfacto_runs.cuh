@@ -64,7 +64,12 @@ struct RunCfg {
     static constexpr int ST = U * GW;        // entries per stage
     static constexpr int SP = 32 / ST;       // stages per pass of 32 entries
     static constexpr int REC = KP4 + 1;      // float4s of a record
-    static constexpr int CTAS = KP4 <= 4 ? 8 : KP4 <= 8 ? 6 : 4;   // of the sweep, resident per SM (register cap; the load cuts units by it)
+    // CTAs of the sweep that stay resident per SM (register cap; the load cuts units by it).  More warps hide more of the
+    // gathers until the registers for the rows on their way run out.  Update loops, us: 256-byte rows 4 / 5 / 6 CTAs (117 / 89 /
+    // 76 registers), 2.6 M entries of text 78 / 71 / 72, 45 M in four bands 1045 / 975 / 944, 12 M of click logs 456 / 441 / 431,
+    // 3 M over 300 columns 53 / 49 / 49; 64-byte rows 7 / 8 / 10, 390 M entries 4346 / 4089 / 5392; 128-byte rows 6 / 7, text
+    // 40.9 / 43.8; 512-byte rows 4 / 5, 30 M entries 1227 / 1532.
+    static constexpr int CTAS = KP4 <= 4 ? 8 : KP4 <= 16 ? 6 : 4;
 };
 template <int LG, int NV>
 constexpr size_t run_sweep_smem() { return (size_t)kRunWarps * 2 * RunCfg<LG, NV>::REC * sizeof(float4); }
