@@ -115,18 +115,17 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // look at every entry costs instructions where these are short: 19 M entries of 256-byte rows over 262 k columns 400 and 365,
 // but 12 M over 300 columns 182 and 189 and of 64-byte rows 157 and 161, which therefore repeat.)
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
-// What bounds it: 64-byte rows of click logs (390 M entries, 2.8 to 2.9 ms), the data and look-up stages of L1 (85 and 89 %
-// busy: every entry costs one look-up for its row and one for its pair) at 40 % issue.  Wider rows reach no rate of any
-// unit: 128-byte rows (2.6 M entries, 63 -> 44 us) 52 % of the L1 data stage, 40 % issue; 256-byte rows without pairs
-// (500 k rows, 0.40 ms) 66 % and 49 %; 512-byte rows (30 M entries, 1.0 ms) 62 % and 27 %, L2 47 %, with 16 resident
-// warps that wait for their gathers.  Ragged rows pay for the common loop besides: rows of 26 to 76 and 20 to 60 entries
-// issue 1.37 and 1.39 row gathers per stored entry (1.27 and 1.29 from the longest of four rows, the rest from whole
-// batches; 39 entries in every row: 1.03).
+// What bounds it: the gathers.  A skeleton of nothing but them (rows of one length, no sums at the end) takes 0.54 ms for 78 M
+// entries of click logs in 64-byte rows where this kernel takes 0.56 (one look-up in L1 for a row, one for its pair), reaches
+// 94 G rows/s of 128 bytes, 58 G of 256 and 33 to 36 G of 512 (12, 15 and 18 TB/s, L1 and L2 hits together), and 72 k rows of
+// text in 36 to 39 us, of which this kernel's 41 are not far.
 // Not kept (each against the version it was tried on): columns and values as records of 8 bytes (2.97 -> 3.35 ms per 390 M
 // entries of click logs); the pairs of the 2048 most frequent columns in shared memory, which the L1 then lacks (2.95 ->
 // 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms); rows taken longest first inside
 // blocks of 256 (text 44 -> 42.5 us, but click logs 2.97 -> 3.09 ms); two or four resident CTAs for 128-byte rows (46 and
-// 43 us).
+// 43 us); lane groups that go on to their next row on their own (text 42.7 -> 39.5 us, click logs 2.78 -> 3.15 ms); on the
+// skeleton, row and pair in one record of 80 or 128 bytes (0.54 -> 0.72 to 0.92 ms), 32-byte loads (no faster), entries staged
+// through shared memory (0.61), hot rows and pairs there (0.55 to 0.8), hot rows kept in L1 by load policy (10 to 50 % slower).
 template <int LG, int NV>
 struct RefreshCfg {
     static constexpr int GW = 32 / LG;
