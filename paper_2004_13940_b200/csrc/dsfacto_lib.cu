@@ -1161,9 +1161,14 @@ int download_rows(dsfacto *h, float *dst, float *src_dev, int64_t rows, Fetch mo
     return rc;
 }
 
+// Rows that a warp takes at a time in the passes over a data set's rows: 32 (a lane each), fewer where that would leave an SM
+// with fewer than 32 warps (100 k rows of 39 entries checked in one go of 20 rows per warp).
+int rows_per_warp(const dsfacto *h, int64_t rows) { return (int)std::max<int64_t>(1, std::min<int64_t>(32, rows / ((int64_t)h->sm_count * 32))); }
 void launch_validate(dsfacto *h, int64_t m, int64_t nnz, const int64_t *indptr, const int32_t *idx, const float *val, const float *y, int *bad) {
-    const int grid = (int)std::min<int64_t>((m + kThreads - 1) / kThreads, (int64_t)h->sm_count * 16);
-    launch(h, validate_rows_kernel, grid, kThreads, 0, m, nnz, h->d, indptr, idx, val, y, bad);
+    const int per = rows_per_warp(h, m);
+    const int64_t rows = (int64_t)per * (kThreads / 32);
+    const int grid = (int)std::min<int64_t>((m + rows - 1) / rows, (int64_t)h->sm_count * 16);
+    launch(h, validate_rows_kernel, grid, kThreads, 0, m, nnz, h->d, indptr, idx, val, y, bad, per);
 }
 
 // CSR checks on the host (shards, the host bucketer).  Returns DSFACTO_OK or DSFACTO_ERR_INVALID_CSR.
@@ -2068,7 +2073,9 @@ static int plan_runs(dsfacto *h, int64_t nnz) {
     ka.n = h->n; ka.nnz = nnz; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p; ka.cbits = cbits;
     ka.bands = (int32_t)bands; ka.band_rows = (h->n + bands - 1) / bands; ka.every = (int32_t)every; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start;
     ka.key = key[0]; ka.payload = pay[0];
-    launch(h, run_keys_kernel, (int)std::min<int64_t>((h->n + kThreads - 1) / kThreads, wide_grid), kThreads, 0, ka);
+    ka.per = rows_per_warp(h, h->n);
+    const int64_t key_rows = (int64_t)ka.per * (kThreads / 32);
+    launch(h, run_keys_kernel, (int)std::min<int64_t>((h->n + key_rows - 1) / key_rows, wide_grid), kThreads, 0, ka);
     if ((e = cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, kbuf, pbuf, nnz, 0, kb, st)) != cudaSuccess) return fail(e);
     const uint32_t *sorted = kbuf.Current();
     launch(h, pass_bounds_kernel, (int)((npass + kThreads) / kThreads), kThreads, 0, nnz, sorted, low_bits, (int)npass, d_bounds);

@@ -45,31 +45,31 @@ __global__ void __launch_bounds__(kThreads) init_factors_kernel(uint64_t seed, i
 
 // The checks of dsfacto_load_csr, predict and evaluate on arrays that are already on the device: row pointers from 0
 // to nnz and never falling, column ids rising strictly inside a row and in [0, d), values and labels finite.
-// *bad is set if one fails.  A warp takes 32 rows at a time; once their pointers have been found sound, their entries are
+// *bad is set if one fails.  A warp takes up to 32 rows at a time (`per`: fewer while that leaves warps without any); once their pointers have been found sound, their entries are
 // one stretch that it reads 128 at a time, whatever the rows' lengths.  Columns may fall from one row to the next, so the
 // warp counts the places where they do not rise, and the rows that begin at such a place: the two are equal if no row has
 // one inside.  Nothing is read outside the arrays whatever they hold.  (One warp per row, 39 M entries: 210 us, most of it
 // waiting for one row's pointers and then its entries; now 59 us, 312 MB.)
 __global__ void __launch_bounds__(kThreads) validate_rows_kernel(int64_t m, int64_t nnz, int32_t d, const int64_t *__restrict__ indptr,
                                                                  const int32_t *__restrict__ idx, const float *__restrict__ val,
-                                                                 const float *__restrict__ y, int *bad) {
+                                                                 const float *__restrict__ y, int *bad, int per) {
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int U = 4;
     const int lane = (int)(threadIdx.x & 31u);
     const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5, warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
     bool wrong = false;
-    for (int64_t i0 = 32 * warp; i0 < m; i0 += 32 * nwarps) {
+    for (int64_t i0 = per * warp; i0 < m; i0 += per * nwarps) {
+        const int rows = (int)min((int64_t)per, m - i0);
         const int64_t i = i0 + lane;
         int64_t b = 0, e = 0;
         bool sound = true;
-        if (i < m) {
+        if (lane < rows) {
             b = indptr[i];
             e = indptr[i + 1];
             sound = b >= 0 && b <= e && e <= nnz && (i > 0 || b == 0);
             if (y && !isfinite(y[i])) wrong = true;
         }
         if (!__all_sync(FULL, sound)) { wrong = true; continue; }
-        const int rows = (int)min((int64_t)32, m - i0);
         const int64_t from = __shfl_sync(FULL, b, 0), to = __shfl_sync(FULL, e, rows - 1);
         int falls = 0;   // fewer than 2^31 in a lane: it has seen a 32nd of the entries of 32 rows
         for (int64_t t0 = from + lane; t0 < to; t0 += 32 * U) {

@@ -29,6 +29,7 @@ struct RunKeyArgs {
     int32_t every;             // rounds per segment
     const int64_t *row_start;
     const int32_t *col_start;
+    int32_t per;               // rows that a warp takes at a time, at most 32
     uint32_t *key;
     unsigned long long *payload;
 };
@@ -39,7 +40,7 @@ __device__ __forceinline__ int64_t quotient(int64_t x, int64_t d, double inv) {
     const int64_t rest = x - q * d;
     return rest < 0 ? q - 1 : rest >= d ? q + 1 : q;
 }
-// A warp takes 32 rows at a time, a lane works out where each of them goes, and the warp walks their entries as one stretch,
+// A warp takes up to 32 rows at a time, a lane works out where each of them goes, and the warp walks their entries as one stretch,
 // two windows of 32 at a time: the row of an entry is the number of row ends up to it (by bisection where rows are empty and
 // ends coincide).  Divisions by n, d and the rows of a band are products with a correction, and in the plain schedule the
 // phase of an entry is a comparison with the first column of its row's diagonal block.  (A warp per row with a 64-bit
@@ -50,8 +51,8 @@ __global__ void __launch_bounds__(kThreads) run_keys_kernel(const RunKeyArgs a) 
     const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5, nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
     const double inv_n = 1.0 / (double)a.n, inv_d = 1.0 / (double)a.d, inv_band = 1.0 / (double)a.band_rows;
     const bool plain = a.every >= a.p;    // one segment
-    for (int64_t i0 = 32 * warp; i0 < a.n; i0 += 32 * nwarps) {
-        const int rows = (int)min((int64_t)32, a.n - i0);
+    for (int64_t i0 = a.per * warp; i0 < a.n; i0 += a.per * nwarps) {
+        const int rows = (int)min((int64_t)a.per, a.n - i0);
         const int64_t i = i0 + min(lane, rows - 1);
         const int32_t r = (int32_t)quotient(i * (int64_t)a.p, a.n, inv_n);                  // row block
         const int64_t r0 = a.row_start[r], r1 = a.row_start[r + 1];
