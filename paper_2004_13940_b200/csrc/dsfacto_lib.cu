@@ -484,10 +484,10 @@ void launch_refresh(dsfacto *h, const RefreshArgs &a, int mode, int grid) {
     else launch_overlapped(h, refresh_kernel<LG, NV, kScore>, grid, kThreads, 0, a);
 }
 template <int LG, int NV>
-void launch_request(dsfacto *h, const RequestArgs &a, int mode, int grid) {
+void launch_request(dsfacto *h, const RequestArgs &a, int mode, int grid, size_t largest_block) {
     auto kernel = mode == kEvaluate ? request_kernel<LG, NV, kEvaluate> : request_kernel<LG, NV, kScore>;
     int &most = h->request_smem[mode == kEvaluate ? 1 : 0];
-    const int smem = (int)request_smem<LG, NV>((size_t)a.stride);
+    const int smem = (int)request_smem<LG, NV>(largest_block);
     if (smem > most && smem > (47 << 10)) {   // (a refusal shows at the launch)
         most = (int)request_smem<LG, NV>(kMailboxBytes);
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
@@ -2742,41 +2742,6 @@ static bool sound_rows(int64_t m, int32_t d, const int64_t *indptr, const int32_
     return falls == 0;
 }
 
-// A small batch as blocks of rows (dsfacto_request.cuh): rows of a block, and bytes from block to block (0: it does not fit).
-struct RequestLayout {
-    int rows = 0;
-    int64_t blocks = 0;
-    size_t stride = 0;
-};
-static RequestLayout request_layout(const dsfacto *h, int64_t m, const int64_t *indptr, bool labels, size_t room) {
-    RequestLayout r;
-    if ((size_t)m > room / 8) return r;
-    // a row per warp while that leaves no more CTAs than two per SM
-    const int64_t warps = kThreads / 32, per_warp = (m + 2 * warps * h->sm_count - 1) / (2 * warps * h->sm_count);
-    r.rows = (int)std::min<int64_t>(warps * per_warp, kMostBlockRows);
-    r.blocks = (m + r.rows - 1) / r.rows;
-    int64_t most = 0;
-    for (int64_t r0 = 0; r0 < m; r0 += r.rows) {
-        const int64_t e = indptr[std::min<int64_t>(m, r0 + r.rows)] - indptr[r0];
-        if (e < 0 || e > (int64_t)room / 8) return r;
-        most = std::max(most, e);
-    }
-    const size_t stride = (4 * (size_t)(r.rows + 1) + 8 * (size_t)most + (labels ? 4 * (size_t)r.rows : 0) + 15) & ~(size_t)15;
-    if (stride * (size_t)r.blocks <= room) r.stride = stride;
-    return r;
-}
-static void lay_out_request(char *to, const RequestLayout &lay, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values, const float *y) {
-    for (int64_t r0 = 0; r0 < m; r0 += lay.rows, to += lay.stride) {
-        const int64_t r1 = std::min<int64_t>(m, r0 + lay.rows), e0 = indptr[r0];
-        const size_t e = (size_t)(indptr[r1] - e0);
-        int32_t *first = reinterpret_cast<int32_t *>(to);
-        for (int r = 0; r <= lay.rows; ++r) first[r] = (int32_t)(indptr[std::min(r0 + r, r1)] - e0);
-        char *at = to + 4 * (size_t)(lay.rows + 1);
-        if (e > 0) { std::memcpy(at, indices + e0, 4 * e); std::memcpy(at + 4 * e, values + e0, 4 * e); }
-        if (y) std::memcpy(at + 8 * e, y + r0, 4 * (size_t)(r1 - r0));
-    }
-}
-
 // Scores m rows: the training rows when indptr is NULL, otherwise rows in host memory.  mode kScore: scores_out
 // fp32[m].  mode kEvaluate: labels y (host) and sums2 = {sum of losses, sum of squared errors or number of correct
 // signs}.
@@ -2795,6 +2760,8 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
     int rc = DSFACTO_OK;
     unsigned long long *mailed = nullptr;   // the scores come through the mailbox
     RequestLayout lay;                      // a request: its rows lie there too
+    RequestArgs q;
+    size_t largest_block = 0;
     auto cleanup = [&]() { dev_free(block); };
     if (!indptr) {
         if (!h->loaded) return DSFACTO_ERR_NO_DATA;
@@ -2813,12 +2780,13 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         // A request: the kernel reads the rows from the mailbox across the link and leaves the scores there, which
         // takes less time than copies in and out before and behind it (32 rows: 60 us -> 16 us per call).
         const size_t f_b = mode == kScore ? (sizeof(*mailed) * (size_t)m + 15) & ~(size_t)15 : 0;
-        if (f_b < h->mail_bytes) lay = request_layout(h, m, indptr, y != nullptr, h->mail_bytes - f_b);
-        if (lay.stride > 0) grid = (int)lay.blocks;
+        if (f_b < h->mail_bytes) lay = request_layout(m, nnz, y != nullptr, h->mail_bytes - f_b, kThreads / 32, 2 * h->sm_count);
+        if (lay.rows > 0) grid = lay.blocks;
         room_for_sums();
-        if (lay.stride > 0) {
+        if (lay.rows > 0) {
             if (!sound_rows(m, h->d, indptr, indices, values, y)) return DSFACTO_ERR_INVALID_CSR;
-            lay_out_request(h->mail + f_b, lay, m, indptr, indices, values, y);   // (behind the scores)
+            q.blocks = reinterpret_cast<const uint4 *>(h->mail + f_b);   // (behind the scores)
+            largest_block = lay_out_request(reinterpret_cast<int32_t *>(h->mail + f_b), lay, m, indptr, indices, values, y, q.at);
             if (mode == kScore) {   // the scores are their own report: words without this call's number, until they arrive
                 mailed = reinterpret_cast<unsigned long long *>(h->mail);
                 std::memset(mailed, 0, f_b);
@@ -2850,12 +2818,10 @@ static int score_rows(dsfacto_t *h, int mode, int64_t m, const int64_t *indptr, 
         model_view(h, a, false);
     }
     a.partials = reinterpret_cast<double *>(block + part_at);
-    if (lay.stride > 0) {
-        RequestArgs q{};
-        q.blocks = reinterpret_cast<const uint4 *>(h->mail + (mailed ? (sizeof(*mailed) * (size_t)m + 15) & ~(size_t)15 : 0));
-        q.stride = (int)lay.stride; q.block_rows = lay.rows; q.rows = (int)m; q.pair = a.pair; q.V = a.V; q.w0 = a.w0; q.loss = a.loss; q.f_words = mailed;
+    if (lay.rows > 0) {
+        q.block_rows = lay.rows; q.rows = (int)m; q.pair = a.pair; q.V = a.V; q.w0 = a.w0; q.loss = a.loss; q.f_words = mailed;
         q.report = a.report; q.number = a.number; q.partials = a.partials; q.done = a.done;
-        DSF_DISPATCH_REFRESH(h, launch_request, h, q, mode, grid);
+        DSF_DISPATCH_REFRESH(h, launch_request, h, q, mode, grid, largest_block);
     } else {
         DSF_DISPATCH_REFRESH(h, launch_refresh, h, a, mode, grid);
     }

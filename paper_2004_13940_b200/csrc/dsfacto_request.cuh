@@ -3,6 +3,7 @@
 #include "dsfacto_common.cuh"
 #include "dsfacto_epoch.cuh"
 #include "dsfacto_recompute.cuh"
+#include "dsfacto_request.h"
 
 namespace dsf {
 
@@ -17,11 +18,8 @@ namespace dsf {
 // 39.5 -> 27.8; 300 rows of one entry 19.0 -> 13.6, 5000 rows 33.5 -> 31.7; 1 row of 1000 entries 60 -> 50, of 8000 entries
 // 1730 -> 315.  What bounds it: 8 us for a launch and its answer, 4 us in the interpreter, then the two trips.  (Lane groups
 // that each sum up a part of the row and add their parts at the end take 14.5 us for 32 rows, but round differently.)
-constexpr int kMostBlockRows = 64;
-// A block: first[block_rows + 1] (where the rows begin among the block's entries), then columns, values and labels.
 struct RequestArgs {
-    const uint4 *blocks;       // mapped host memory
-    int stride;                // bytes from block to block (a multiple of 16)
+    const uint4 *blocks;       // mapped host memory, laid out by lay_out_request
     int block_rows;            // rows of a block (at most kMostBlockRows)
     int rows;                  // of the batch
     const float2 *pair;        // per column (w_j, s_j = sum_k v_jk^2)
@@ -33,6 +31,7 @@ struct RequestArgs {
     uint32_t number;           // of the words
     double *partials;          // kEvaluate: 4 per CTA
     unsigned *done;            // CTAs that have delivered (zero between launches)
+    uint16_t at[kMostBlocks + 1];  // first word of every block, and the word behind the last one
 };
 template <int LG, int NV>
 struct RequestCfg {
@@ -47,9 +46,9 @@ struct RequestStep {
     float2 pairs[RequestCfg<LG, NV>::STEP];
 };
 template <int LG, int NV>
-constexpr size_t request_smem(size_t stride) { return sizeof(RequestStep<LG, NV>) * (kThreads / 32) + stride; }
+constexpr size_t request_smem(size_t largest_block) { return sizeof(RequestStep<LG, NV>) * (kThreads / 32) + largest_block; }
 template <int LG, int NV, int MODE>
-__global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) {
+__global__ void __launch_bounds__(kThreads) request_kernel(const __grid_constant__ RequestArgs a) {
     typedef RequestCfg<LG, NV> C;
     constexpr int STEP = C::STEP, F = C::F, KP4 = C::KP4, LANES = RefreshCfg<LG, NV>::LANES;
     constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -59,26 +58,28 @@ __global__ void __launch_bounds__(kThreads) request_kernel(const RequestArgs a) 
     __shared__ float scores[kMostBlockRows];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LG;
     let_next_kernel_start();
-    const uint4 *from = a.blocks + (size_t)blockIdx.x * (a.stride / 16);
+    const int word = a.at[blockIdx.x];                                          // the 16-byte units that hold the block
+    const uint4 *from = a.blocks + word / 4;
+    const int units = (a.at[blockIdx.x + 1] + 3) / 4 - word / 4;
     constexpr int PIECES = 6;
-    for (int i0 = threadIdx.x; i0 < a.stride / 16; i0 += PIECES * kThreads) {   // one trip across the link for up to 24 KB
+    for (int i0 = threadIdx.x; i0 < units; i0 += PIECES * kThreads) {           // one trip across the link for up to 24 KB
         uint4 piece[PIECES];
 #pragma unroll
         for (int i = 0; i < PIECES; ++i)
-            if (i0 + i * kThreads < a.stride / 16) piece[i] = from[i0 + i * kThreads];
+            if (i0 + i * kThreads < units) piece[i] = from[i0 + i * kThreads];
 #pragma unroll
         for (int i = 0; i < PIECES; ++i)
-            if (i0 + i * kThreads < a.stride / 16) block[i0 + i * kThreads] = piece[i];
+            if (i0 + i * kThreads < units) block[i0 + i * kThreads] = piece[i];
     }
     __syncthreads();
-    const int *first = reinterpret_cast<const int *>(block);
-    const int entries = first[a.block_rows], rows = min(a.block_rows, a.rows - (int)blockIdx.x * a.block_rows);
-    const int32_t *all_idx = first + a.block_rows + 1;
+    const int *ends = reinterpret_cast<const int *>(block) + word % 4;
+    const int rows = min(a.block_rows, a.rows - (int)blockIdx.x * a.block_rows), entries = ends[rows - 1];
+    const int32_t *all_idx = ends + rows;
     const float4 *V4 = reinterpret_cast<const float4 *>(a.V);
     wait_for_previous_kernel();   // the model
 
     for (int row = warp; row < rows; row += kThreads / 32) {
-        const int beg = first[row], len = first[row + 1] - beg;
+        const int beg = row > 0 ? ends[row - 1] : 0, len = ends[row] - beg;
         const int32_t *idx = all_idx + beg;
         const float *val = reinterpret_cast<const float *>(idx + entries);
         float4 acc[F];

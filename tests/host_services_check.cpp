@@ -2,6 +2,7 @@
 // that they make are defined here, device memory is ordinary memory.  Built and run by test_host_services.py; the
 // argument names the check, exit status 0 means that it holds.
 #include "dsfacto_host.cuh"
+#include "dsfacto_request.h"
 
 #include <chrono>
 #include <cstdio>
@@ -176,11 +177,71 @@ static int no_host_memory() {
     return 0;
 }
 
+// Small batches whose own bytes fit the mailbox are laid out in it, however unequal their rows, and every block, read as
+// request_kernel reads it, holds its rows.
+static int requests() {
+    using namespace dsf;
+    std::mt19937 rng(7);
+    std::lognormal_distribution<double> uneven(2.0, 1.2);
+    const size_t mail = kMailboxBytes - 256;
+    int fitted = 0;
+    for (int round = 0; round < 3000; ++round) {
+        const bool labels = round % 2 == 1;
+        const int64_t m = round < 40 ? 1 + round / 2 : 1 + (int64_t)(rng() % (1u << (4 + rng() % 11)));
+        std::vector<int64_t> indptr(1, 0);
+        for (int64_t i = 0; i < m; ++i) {
+            int64_t len = round % 5 == 0 ? 8 : round % 5 == 1 ? (int64_t)uneven(rng) : round % 5 == 2 ? (int64_t)(rng() % 3) : round % 5 == 3 ? 0 : 26 + rng() % 51;
+            if (i == m / 2) len += round % 3 == 0 ? 400 : round % 3 == 1 ? 0 : 1 + rng() % 9000;   // one long row
+            indptr.push_back(indptr.back() + len);
+        }
+        const int64_t nnz = indptr.back();
+        const size_t scores = labels ? 0 : ((size_t)m * 8 + 15) / 16 * 16;
+        const size_t own = 8 * (size_t)(m + 1) + 8 * (size_t)nnz + 4 * (size_t)m;   // row pointers, entries, labels or scores
+        const RequestLayout lay = scores < mail ? request_layout(m, nnz, labels, mail - scores, 8, 296) : RequestLayout();
+        if (own <= mail) NEED(lay.rows > 0);
+        if (lay.rows == 0) continue;
+        ++fitted;
+        NEED(lay.rows <= kMostBlockRows && lay.blocks <= kMostBlocks && (int64_t)lay.rows * lay.blocks >= m && (int64_t)lay.rows * (lay.blocks - 1) < m);
+        std::vector<int32_t> indices((size_t)nnz), box((mail - scores) / 4 + 64, -1);
+        std::vector<float> values((size_t)nnz), y((size_t)m);
+        for (int32_t &j : indices) j = (int32_t)(rng() >> 1);
+        for (float &x : values) x = (float)rng();
+        for (float &x : y) x = (float)rng();
+        uint16_t at[kMostBlocks + 1];
+        const size_t largest = lay_out_request(box.data(), lay, m, indptr.data(), indices.data(), values.data(), labels ? y.data() : nullptr, at);
+        size_t most = 0;
+        for (size_t k = at[lay.blocks]; k < box.size(); ++k) NEED(box[k] == -1);   // nothing behind the last word
+        NEED(4 * (size_t)((at[lay.blocks] + 3) / 4 * 4) <= mail - scores);         // nor is read, with the unit it lies in
+        for (int b = 0; b < lay.blocks; ++b) {
+            const int units = (at[b + 1] + 3) / 4 - at[b] / 4;
+            most = std::max(most, (size_t)units * 16);
+            std::vector<int32_t> block(box.begin() + at[b] / 4 * 4, box.begin() + at[b] / 4 * 4 + units * 4);
+            const int64_t r0 = (int64_t)b * lay.rows;
+            const int rows = (int)std::min<int64_t>(lay.rows, m - r0);
+            const int32_t *ends = block.data() + at[b] % 4, *idx = ends + rows;
+            const int entries = ends[rows - 1];
+            NEED(entries == indptr[r0 + rows] - indptr[r0] && at[b + 1] - at[b] == rows * (labels ? 2 : 1) + 2 * entries);
+            for (int r = 0; r < rows; ++r) {
+                const int beg = r > 0 ? ends[r - 1] : 0, len = ends[r] - beg;
+                NEED(len == indptr[r0 + r + 1] - indptr[r0 + r]);
+                if (len == 0) continue;
+                NEED(std::memcmp(idx + beg, indices.data() + indptr[r0 + r], 4 * (size_t)len) == 0);
+                NEED(std::memcmp(idx + entries + beg, values.data() + indptr[r0 + r], 4 * (size_t)len) == 0);
+            }
+            if (labels) NEED(std::memcmp(idx + 2 * entries, y.data() + r0, 4 * (size_t)rows) == 0);
+        }
+        NEED(most == largest);
+    }
+    NEED(fitted > 1000);
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "transfers-in") return transfers(true);
     if (what == "transfers-out") return transfers(false);
     if (what == "threads") return threads();
     if (what == "no-host-memory") return no_host_memory();
+    if (what == "requests") return requests();
     return 2;
 }

@@ -186,6 +186,49 @@ def test_page_locked_arrays_belong_to_the_caller_again_on_return(n):
         assert np.array_equal(np.asarray(a), np.asarray(b))
 
 
+def _batch(lens, d, seed):
+    lens, rng = np.asarray(lens), np.random.default_rng(seed)
+    ip = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    ix = np.concatenate([np.sort(rng.choice(d, n, replace=False)) for n in lens]).astype(np.int32)
+    return ip, ix, rng.standard_normal(len(ix)).astype(np.float32), np.where(rng.random(len(lens)) < 0.5, 1.0, -1.0).astype(np.float32)
+
+
+_uneven = np.random.default_rng(5)
+RAGGED = {
+    "one of 400 among 8s": [8] * 500 + [400] + [8] * 500,
+    "one long among 8s, to the last bytes": [8] * 800 + [408] + [8] * 878,                # 12 m + 8 + 8 nnz: 128 KB less the reports
+    "log-normal, mean 40": _uneven.lognormal(np.log(40) - 0.5, 1.0, 300).astype(int).clip(1, 2000),
+    "log-normal, mean 8": _uneven.lognormal(np.log(8) - 0.5, 1.0, 700).astype(int).clip(1, 2000),
+    "26 to 76": _uneven.integers(26, 77, 300),
+    "a long row and 2000 empty ones": [0] * 1000 + [9000] + [0] * 1000,
+}
+
+
+@pytest.mark.parametrize("K", [8, 32, 128])
+@pytest.mark.parametrize("shape", sorted(RAGGED))
+def test_ragged_batches_go_through_the_mailbox(K, shape):
+    """One launch, whatever the longest row, while the batch's own bytes fit; and the scores that its rows have in a batch
+    that is too large for it."""
+    d = 20000
+    ip, ix, v, y = _batch(RAGGED[shape], d, K)
+    m = len(y)
+    assert 12 * m + 8 + 8 * len(ix) <= (128 << 10) - 256
+    rng = np.random.default_rng(K)
+    with D.DSFacto(1, d, K, 1, D.LOGISTIC, 0.0, 0.0, 0.1, 1) as g:
+        w, V = (0.1 * rng.standard_normal(d)).astype(np.float32), (0.1 * rng.standard_normal((d, K))).astype(np.float32)
+        g.set_params(0.25, w, V)
+        copied = g.predict(np.concatenate([ip, ip[-1] + ip[1:], 2 * ip[-1] + np.arange(1, 12001)]),
+                           np.concatenate([ix, ix, np.arange(12000, dtype=np.int32) % d]), np.concatenate([v, v, np.ones(12000, np.float32)]))
+        before = g.launch_count()
+        f = g.predict(ip, ix, v)
+        assert g.launch_count() - before == 1
+        assert np.array_equal(f, copied[:m]) and np.array_equal(f, copied[m:2 * m])
+        loss, acc = g.evaluate(ip, ix, v, y)
+        assert g.launch_count() - before == 2
+        assert loss == pytest.approx(np.logaddexp(0.0, -y * f.astype(np.float64)).mean(), rel=1e-5)
+        assert acc == pytest.approx(np.mean(y * f > 0), abs=1e-12)
+
+
 REQUESTS = {
     "steps": [7, 8, 9, 31, 32, 33, 63, 64, 65, 0, 127, 128, 129, 1, 0, 15, 16, 17],   # around the entries of a warp's step
     "several rows per warp": list(np.random.default_rng(0).integers(0, 4, 2500)),
