@@ -42,7 +42,7 @@ inline RequestLayout request_layout(int64_t m, int64_t nnz, bool labels, size_t 
 }
 // Rows that are known to be sound.  at[b]: the first word of block b, at[blocks]: the number of words.  Returns the bytes that
 // the largest block takes with the 16-byte units it begins and ends in.
-inline size_t lay_out_request(int32_t *to, const RequestLayout &lay, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values,
+__attribute__((noinline)) inline size_t lay_out_request(int32_t *to, const RequestLayout &lay, int64_t m, const int64_t *indptr, const int32_t *indices, const float *values,
                               const float *y, uint16_t *at) {
     size_t largest = 0;
     int64_t word = 0;

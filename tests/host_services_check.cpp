@@ -3,6 +3,7 @@
 // argument names the check, exit status 0 means that it holds.
 #include "dsfacto_host.cuh"
 #include "dsfacto_request.h"
+#include "dsfacto_words.h"
 
 #include <chrono>
 #include <cstdio>
@@ -236,6 +237,31 @@ static int requests() {
     return 0;
 }
 
+// Scores that arrive one by one: the caller has all of them, or, where the kernel fails in between, none.
+static int scores_in_words() {
+    const int64_t m = 1000;
+    const uint32_t number = 77;
+    for (int64_t arriving : {(int64_t)0, (int64_t)1, m / 2, m - 1, m}) {
+        std::vector<unsigned long long> words((size_t)m, (unsigned long long)(number - 1) << 32 | 5);
+        std::vector<float> scores((size_t)m, -1.0f);
+        const int rc = dsf::take_scores(words.data(), m, number, scores.data(), [&](auto arrived) {
+            for (int64_t k = 0; k < arriving; ++k) {      // the last one first: order is nobody's promise
+                const int64_t i = arriving == m ? m - 1 - k : k;
+                const float f = (float)i + 0.5f;
+                uint32_t bits;
+                std::memcpy(&bits, &f, sizeof bits);
+                const bool all = arrived();
+                if (all) return 1;                        // too early
+                words[(size_t)i] = (unsigned long long)number << 32 | bits;
+            }
+            return arrived() ? 0 : -5;
+        });
+        NEED(rc == (arriving == m ? 0 : -5));
+        for (int64_t i = 0; i < m; ++i) NEED(scores[(size_t)i] == (arriving == m ? (float)i + 0.5f : -1.0f));
+    }
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "transfers-in") return transfers(true);
@@ -243,5 +269,6 @@ int main(int argc, char **argv) {
     if (what == "threads") return threads();
     if (what == "no-host-memory") return no_host_memory();
     if (what == "requests") return requests();
+    if (what == "scores") return scores_in_words();
     return 2;
 }

@@ -1,5 +1,6 @@
 """The library's host-side services (device memory pool, transfers, result buffers, mailboxes) under several threads and
-without host memory, and the layout of small scoring batches, on the CPU: host_services_check.cpp defines the CUDA runtime calls they make."""
+without host memory, and the layout of small scoring batches and their answers, on the CPU: host_services_check.cpp defines
+the CUDA runtime calls they make."""
 import subprocess
 from pathlib import Path
 
@@ -17,7 +18,7 @@ def check(tmp_path_factory):
     return lambda what: subprocess.run([str(exe), what], capture_output=True, text=True, timeout=120)
 
 
-@pytest.mark.parametrize("what", ["transfers-in", "transfers-out", "threads", "no-host-memory", "requests"])
+@pytest.mark.parametrize("what", ["transfers-in", "transfers-out", "threads", "no-host-memory", "requests", "scores"])
 def test_host_services(check, what):
     r = check(what)
     assert r.returncode == 0, r.stdout + r.stderr
