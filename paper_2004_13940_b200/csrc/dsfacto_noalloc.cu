@@ -45,11 +45,22 @@ void launch_score_loss(const RefreshArgs &a, int32_t d, cudaStream_t st) {
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t rows = RefreshCfg<LG, NV>::ROWS;
     const int64_t grid = std::min<int64_t>((a.n + rows - 1) / rows, (int64_t)sms * RefreshCfg<LG, NV>::CTAS);
-    // whether nothing is requested behind the end of a row (TRIM): rows of 128 bytes and more of a table that no L1 holds
-    const bool trim = LG >= 8 && (int64_t)d * 4 * LG * NV * (int64_t)sizeof(float) > ((int64_t)320 << 10);
     const unsigned ctas = (unsigned)std::min<int64_t>(grid, kMaxCtas);
-    if (trim) refresh_kernel<LG, NV, kScoreSums, true, true><<<ctas, kThreads, 0, st>>>(a);
-    else refresh_kernel<LG, NV, kScoreSums, true, false><<<ctas, kThreads, 0, st>>>(a);
+    // Whether nothing is requested behind the end of a row (TRIM), or its last entry again.  Not requesting saves look-ups and
+    // data where the rows that a warp takes side by side differ in length, and costs a look at every entry.  12 M entries over
+    // 50 to 1 M columns, rows of 39, 20 to 60, 1 to 77 and 1 to 12 entries, columns drawn evenly and by a power law: the time
+    // that repeating takes, over the time without, is 0.96 to 1.20 for 32-byte rows, 0.98 to 1.22 for 64-byte, 0.99 to 1.13 for
+    // 128-byte and 1.00 to 1.09 for 512-byte rows.  256-byte rows: 0.97 to 1.00 over tables of up to 150 KB, which an L1 holds
+    // whole, 0.98 to 1.03 over 175 to 225 KB, 0.99 to 1.27 over larger ones.  Two widths are better off repeating more often
+    // than not: 16-byte rows (0.86 to 1.11, below 1 in 16 of 24 cases) and 1-KB rows over up to 320 KB (0.96 to 1.12, in 21 of 32).
+    constexpr bool repeats = (LG == 1 && NV == 1) || (LG == 8 && NV == 8), by_table = LG == 8 && NV == 2;
+    if constexpr (!repeats) {
+        if (!by_table || (int64_t)d * 4 * LG * NV * (int64_t)sizeof(float) > ((int64_t)192 << 10)) {
+            refresh_kernel<LG, NV, kScoreSums, true, true><<<ctas, kThreads, 0, st>>>(a);
+            return;
+        }
+    }
+    if constexpr (repeats || by_table) refresh_kernel<LG, NV, kScoreSums, true, false><<<ctas, kThreads, 0, st>>>(a);
 }
 
 }  // namespace

@@ -110,10 +110,10 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // ahead of the multiply-adds.  Behind the end of a row x is 0, and nothing is requested (TRIM): the registers
 // keep the factors of an earlier entry of the row, whose infinities are the row's own, or zeros.  (Repeating the row's last
 // entry there found it in L1, but each repetition took the look-ups and the data of a request: recompute pass, us, repeating
-// and not: 2.6 M entries of text in 128-byte rows 42.7 and 40.9, 11 M in 96-byte rows 160 and 155, 30 M in 512-byte rows 926
-// and 894, 11.7 M of click logs in 32-byte rows 95.3 and 93.8, 390 M in 64-byte rows 2780 and 2760.  Without pairs (RAW) the
-// look at every entry costs instructions where these are short: 19 M entries of 256-byte rows over 262 k columns 400 and 365,
-// but 12 M over 300 columns 182 and 189 and of 64-byte rows 157 and 161, which therefore repeat.)
+// and not: 2.6 M entries of text in 128-byte rows 42.7 and 40.9, 30 M in 512-byte rows 926 and 894, 11.7 M of click logs in
+// 32-byte rows 95.3 and 93.8, 390 M in 64-byte rows 2780 and 2760.  Training passes over 12 M entries of tables, text and click
+// logs with 3 to 128 factors: time repeating over time not 0.98 to 1.15, but for 3 factors and rows of 1 to 12 entries 0.95.
+// Without pairs (RAW) some widths repeat: see launch_score_loss.)
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
 // What bounds it: the gathers.  A skeleton of nothing but them (rows of one length, no sums at the end) takes 0.54 ms for 78 M
 // entries of click logs in 64-byte rows where this kernel takes 0.56 (one look-up in L1 for a row, one for its pair), reaches

@@ -324,3 +324,40 @@ def test_infinite_factors_stay_in_the_rows_that_have_them(K, value):
         few = slice(0, 40)
         part = g.predict(ip[:41], ix[:ip[40]], v[:ip[40]])
         assert np.array_equal(part[~hit[few]], want[few][~hit[few]])
+
+
+# columns on both sides of the line between 8 and 16 lanes for wide rows (320 KB), and of the one between repeating the last
+# entry of a row and not (192 KB, 256-byte rows only)
+@pytest.mark.parametrize("K,d", [(4, 900), (8, 900), (16, 900), (32, 900), (64, 768), (64, 769), (128, 640), (128, 641), (256, 320), (256, 321)])
+@pytest.mark.parametrize("value", [0.25, np.inf, np.nan])
+def test_allocation_free_scoring_of_uneven_rows(K, d, value):
+    """Rows of very different lengths side by side, against 64 bits; a column of infinite factors spoils the rows that have it
+    and no other."""
+    import torch
+
+    rng = np.random.default_rng(K + d)
+    m = 3000
+    lens = rng.choice([0, 1, 2, 3, 5, 8, 9, 17, 40, 90], m)
+    rows = [np.sort(rng.choice(d - 1, n, replace=False) + 1) for n in lens]
+    hit = rng.random(m) < 0.2
+    rows = [np.concatenate([[0], r]) if h else r for r, h in zip(rows, hit)]      # column 0 comes first
+    lens = np.array([len(r) for r in rows])
+    ip, ix = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64), np.concatenate(rows).astype(np.int32)
+    v = rng.standard_normal(len(ix)).astype(np.float32) / np.sqrt(np.repeat(lens, lens)).astype(np.float32)
+    y = np.where(rng.random(m) < 0.5, 1.0, -1.0).astype(np.float32)
+    w, V = (0.1 * rng.standard_normal(d)).astype(np.float32), (0.1 * rng.standard_normal((d, K))).astype(np.float32)
+    V[0] = value
+    t = [torch.from_numpy(a).cuda() for a in (ip, ix, v, y, w, V)]
+    scores, sums = torch.empty(m, device="cuda"), torch.empty(2, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    assert D.dsfacto_score_loss_noalloc(m, d, K, D.LOGISTIC, *[a.data_ptr() for a in t[:4]], 0.25, t[4].data_ptr(),
+                                        t[5].data_ptr(), scores.data_ptr(), sums.data_ptr()) == D.OK
+    got = scores.cpu().numpy()
+    f = O.score(ip, ix, v, 0.25, w.astype(np.float64), np.where(np.isfinite(V), V, 0).astype(np.float64))
+    sound = ~hit if value != 0.25 else np.ones(m, bool)
+    # fp32 sums of up to 91 products whose squares add up to about one: error below 91 * 2^-24 in the worst order
+    np.testing.assert_allclose(got[sound], f[sound], rtol=0, atol=2e-5 * (1 + np.abs(f).max()))
+    if value == 0.25:
+        assert float(sums[0]) == pytest.approx(np.logaddexp(0.0, -y * f).sum(), rel=1e-5)
+    else:
+        assert not np.isfinite(got[hit]).any()
