@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kThreads) unit_runs_kernel(const int *__restri
 // themselves takes as long as the adds to the most frequent columns take one after the other: 39 M entries 566 us, now 5 us.)
 __global__ void __launch_bounds__(kThreads) run_columns_kernel(const int *__restrict__ run_start, const uint32_t *__restrict__ run_key, int nruns, int count,
                                                                int32_t *__restrict__ entries) {
-    for (int q = blockIdx.x * kThreads + threadIdx.x; q < nruns; q += gridDim.x * kThreads)
+    for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < nruns; q += (int64_t)gridDim.x * kThreads)   // (nearly 2^31 runs at most)
         atomicAdd(entries + (run_key[q] >> 1), (q + 1 < nruns ? run_start[q + 1] : count) - run_start[q]);
 }
 

@@ -117,6 +117,18 @@ def test_host_code_builds_on_other_processors_than_x86():
     assert r.returncode == 0 and "yield" in r.stdout, r.stderr
 
 
+def test_loops_over_a_whole_grid_count_in_64_bits_unless_their_bound_is_small():
+    # a pass may have nearly 2^31 runs, and a grid takes steps of some 600,000: 32 bits overflow behind the last step
+    from paper_2004_13940_b200 import build as B
+    small = {"npasses": "a part of a 32-bit key, a thread each", "units": "of a pass, 32 entries or more each"}
+    loops = 0
+    for f in sorted(B.CSRC.glob("*.cu*")):
+        for kind, name, bound in re.findall(r"for \((\w+) (\w+) = [^;]*blockIdx[^;]*; \w+ <=? ([^;]+);", f.read_text()):
+            loops += 1
+            assert kind == "int64_t" or bound in small, (f.name, name, bound)
+    assert loops > 8
+
+
 def test_result_arrays_while_another_thread_empties_the_count_of_sizes(monkeypatch):
     class Emptied(dict):        # the other thread comes in at the worst moment
         def __setitem__(self, key, value):
