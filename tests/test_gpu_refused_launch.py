@@ -49,7 +49,7 @@ def test_a_refused_launch_of_an_epoch(monkeypatch, env, every, before):
             _same(g, o)
 
 
-@pytest.mark.parametrize("m", [10, 300, 3000])      # staged, mapped, copied and checked on the device
+@pytest.mark.parametrize("m", [10, 300, 3000])      # through the mailbox in two and in many blocks; copied and checked on the device
 def test_a_refused_launch_of_other_calls(m):
     wl = W.make("C3", n=3000)
     ip = wl.indptr[: m + 1].copy()
