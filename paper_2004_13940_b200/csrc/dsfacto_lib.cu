@@ -1632,7 +1632,8 @@ static int create_handle(dsfacto_t **out, int64_t n, int32_t d, int32_t K, int32
     h->NV = (q4 + LG - 1) / LG;
     h->Kp = 4 * h->LG * h->NV;
     // The recompute kernel gives a row of 128 bytes and more to 8 lanes, a 128-byte line per load and row: four rows
-    // share the instructions that hand out columns and values.
+    // share the instructions that hand out columns and values.  Rows of 512 bytes and more of a table that no L1 holds go
+    // to 16 (wide_recompute_groups).
     h->LGr = h->LG; h->NVr = h->NV;
     if (h->Kp >= 64) { h->LGr = 8; h->NVr = h->Kp / 32; }
     if (wide_recompute_groups(h->d, h->Kp)) { h->LGr = 16; h->NVr = h->Kp / 64; }
@@ -1875,7 +1876,7 @@ static int device_bucket_tiles(dsfacto *h, int64_t nnz, SgdPlanBuild &pb) {
     const int wide_grid = h->sm_count * 16;
     TileKeyArgs ka{};
     ka.n = h->n; ka.indptr = h->d_indptr; ka.idx = h->d_idx; ka.val = h->d_val; ka.d = h->d; ka.p = h->p;
-    ka.sweep = h->sweep; ka.jbits = h->jbits; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start; ka.col_start = h->d_col_start;
+    ka.sweep = h->sweep; ka.jbits = h->jbits; ka.row_start = h->d_row_start; ka.col_start = h->d_col_start;
     ka.rbits = h->rbits; ka.slot_rows = (int32_t)slot_rows;
     ka.key = key[0]; ka.payload = pay[0];
     launch(h, tile_keys_kernel, wide_grid, kThreads, 0, ka);

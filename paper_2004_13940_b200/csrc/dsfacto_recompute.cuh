@@ -115,10 +115,10 @@ __device__ __forceinline__ bool last_thread(unsigned *done) {
 // logs with 3 to 128 factors: time repeating over time not 0.98 to 1.15, but for 3 factors and rows of 1 to 12 entries 0.95.
 // Without pairs (RAW) some widths repeat: see launch_score_loss.)
 // RAW: no pairs are at hand (the entry point that allocates nothing): w_j from w, s_j from the row itself.
-// What bounds it: the gathers.  A skeleton of nothing but them (rows of one length, no sums at the end) takes 0.54 ms for 78 M
-// entries of click logs in 64-byte rows where this kernel takes 0.56 (one look-up in L1 for a row, one for its pair), reaches
-// 94 G rows/s of 128 bytes, 58 G of 256 and 33 to 36 G of 512 (12, 15 and 18 TB/s, L1 and L2 hits together), and 72 k rows of
-// text in 36 to 39 us, of which this kernel's 41 are not far.
+// What bounds it: the gathers.  A skeleton of nothing but them (rows of one length, no sums at the end; the best of several
+// widths of lane groups and depths) takes 2.57 ms for 390 M entries of click logs in 64-byte rows where this kernel takes 2.76,
+// 38 us for 2.6 M of text in 128-byte rows (41), 0.31 ms for 17 M in 256-byte rows (0.37 for a call without pairs), 0.84 ms for
+// 30 M in 512-byte rows (0.89): 152, 69, 54 and 36 G rows/s, 9 to 19 TB/s of L1 and L2 hits together.
 // Not kept (each against the version it was tried on): columns and values as records of 8 bytes (2.97 -> 3.35 ms per 390 M
 // entries of click logs); the pairs of the 2048 most frequent columns in shared memory, which the L1 then lacks (2.95 ->
 // 2.98 ms); 64-byte rows requested three steps ahead instead of one (2.93 -> 2.98 ms); rows taken longest first inside
